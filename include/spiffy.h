@@ -94,6 +94,14 @@ typedef enum { SPIFFY_RULE_TOPS = 0, SPIFFY_RULE_THRESHOLD = 1 } spiffy_rule;
 #define SPIFFY_DEV_BADGRAPH 2  /* parent list malformed (offsets or indices)   */
 #define SPIFFY_DEV_TIMEOUT 4   /* a bounded on-chip wait gave up               */
 
+/* Flag, OR-ed into the logits_dtype of a decision or drafting descriptor: the
+ * call's status words arrive with arbitrary contents and are cleared by its own
+ * first kernel, so that on return they hold this call's bits alone.  Without it
+ * the bits are OR-ed into what the caller left there.  (The drafting call then
+ * also writes 0 to the entries of parent_idx behind its lists.)  Spares a caller
+ * that allocates its outputs for the call the clearing of them. */
+#define SPIFFY_FRESH_STATUS 0x100
+
 /* Attention kernel selection (spiffy_attn_desc.kernel). */
 #define SPIFFY_ATTN_AUTO 0   /* tensor-core kernel when the shape allows it   */
 #define SPIFFY_ATTN_SIMT 1   /* fp32 CUDA-core kernel (any supported shape)   */
@@ -183,7 +191,7 @@ typedef struct {
   int32_t n_nodes;       /* N                                                */
   int32_t block_len;     /* L in [1, 64]                                     */
   int32_t vocab;         /* V >= 1                                           */
-  int32_t logits_dtype;  /* spiffy_dtype                                     */
+  int32_t logits_dtype;  /* spiffy_dtype, | SPIFFY_FRESH_STATUS              */
   int64_t row_stride;    /* elements between consecutive logits rows, >= V;
                             row_stride * sizeof(element) must be a multiple
                             of 16                                            */
@@ -326,7 +334,8 @@ spiffy_status spiffy_unmask_decide_sampled(const spiffy_decide_desc* desc,
  *                 unmasked positions are computed and ignored
  *   weight        [V][hidden] bf16 (the output embedding, one row per token)
  *   desc          batch, n_nodes, block_len, vocab, mask_token_id, rule, top_s,
- *                 threshold are used; logits_dtype and row_stride are ignored
+ *                 threshold are used; of logits_dtype only SPIFFY_FRESH_STATUS;
+ *                 row_stride is ignored
  * Limit: hidden a multiple of 128, else SPIFFY_EUNSUPPORTED.  Rows are taken 256 at a
  * time and every such pass reads the weight matrix again: the call is made for
  * the few hundred rows of one verification step.
@@ -518,7 +527,7 @@ typedef struct {
   int32_t batch;         /* B                                                */
   int32_t block_len;     /* L in [1, 64]                                     */
   int32_t vocab;         /* V                                                */
-  int32_t logits_dtype;  /* spiffy_dtype                                     */
+  int32_t logits_dtype;  /* spiffy_dtype, | SPIFFY_FRESH_STATUS              */
   int64_t row_stride;    /* elements between logits rows, as in the decision */
   int32_t mask_token_id;
   int32_t n_formulas;    /* D draft formulas of the calibrated graph, <= 1024 */

@@ -50,9 +50,10 @@ spiffy_status check_decide_desc(const spiffy_decide_desc* d, bool need_vocab) {
   if ((int64_t)d->batch * d->n_nodes * d->block_len > 65535) return SPIFFY_EUNSUPPORTED;
   if (!need_vocab) return SPIFFY_OK;
   if (d->vocab < 1) return SPIFFY_EINVAL;
-  if (d->logits_dtype != SPIFFY_F32 && d->logits_dtype != SPIFFY_BF16) return SPIFFY_EINVAL;
+  const int dtype = d->logits_dtype & ~SPIFFY_FRESH_STATUS;
+  if (dtype != SPIFFY_F32 && dtype != SPIFFY_BF16) return SPIFFY_EINVAL;
   if (d->row_stride < d->vocab) return SPIFFY_EINVAL;
-  const int64_t esize = d->logits_dtype == SPIFFY_BF16 ? 2 : 4;
+  const int64_t esize = dtype == SPIFFY_BF16 ? 2 : 4;
   if ((d->row_stride * esize) % 16 != 0) return SPIFFY_EINVAL;
   if (d->rule != SPIFFY_RULE_TOPS && d->rule != SPIFFY_RULE_THRESHOLD) return SPIFFY_EINVAL;
   if (d->rule == SPIFFY_RULE_TOPS && d->top_s < 1) return SPIFFY_EINVAL;
@@ -60,12 +61,22 @@ spiffy_status check_decide_desc(const spiffy_decide_desc* d, bool need_vocab) {
   return SPIFFY_OK;
 }
 
+// The descriptor as the kernels' launchers take it: the flag in its own variable.
+template <typename Desc>
+Desc split_flags(const Desc* desc, bool* fresh) {
+  Desc d = *desc;
+  *fresh = (d.logits_dtype & SPIFFY_FRESH_STATUS) != 0;
+  d.logits_dtype &= ~SPIFFY_FRESH_STATUS;
+  return d;
+}
+
 spiffy_status check_draft_desc(const spiffy_draft_desc* d) {
   if (!d) return SPIFFY_EINVAL;
   if (d->batch < 1 || d->block_len < 1 || d->vocab < 1 || d->n_formulas < 1) return SPIFFY_EINVAL;
-  if (d->logits_dtype != SPIFFY_F32 && d->logits_dtype != SPIFFY_BF16) return SPIFFY_EINVAL;
+  const int dtype = d->logits_dtype & ~SPIFFY_FRESH_STATUS;
+  if (dtype != SPIFFY_F32 && dtype != SPIFFY_BF16) return SPIFFY_EINVAL;
   if (d->row_stride < d->vocab) return SPIFFY_EINVAL;
-  if ((d->row_stride * (d->logits_dtype == SPIFFY_BF16 ? 2 : 4)) % 16 != 0) return SPIFFY_EINVAL;
+  if ((d->row_stride * (dtype == SPIFFY_BF16 ? 2 : 4)) % 16 != 0) return SPIFFY_EINVAL;
   if (d->top_k < 1 || d->budget < 1 || d->budget > d->n_formulas || d->parent_cap < 1) return SPIFFY_EINVAL;
   if (d->block_len > 64 || d->top_k > 4 || d->n_formulas > 1024) return SPIFFY_EUNSUPPORTED;
   if ((int64_t)d->batch * d->block_len > 65535) return SPIFFY_EUNSUPPORTED;
@@ -171,7 +182,9 @@ spiffy_status spiffy_full_sequence_attention(const spiffy_attn_desc* desc, int32
 
 size_t spiffy_unmask_decide_workspace(const spiffy_decide_desc* desc) {
   if (check_decide_desc(desc, true) != SPIFFY_OK) return 0;
-  return decide_workspace_bytes(*desc);
+  bool fresh;
+  const spiffy_decide_desc d = split_flags(desc, &fresh);
+  return decide_workspace_bytes(d);
 }
 
 spiffy_status spiffy_unmask_decide(const spiffy_decide_desc* desc,
@@ -186,11 +199,13 @@ spiffy_status spiffy_unmask_decide(const spiffy_decide_desc* desc,
   if (!logits || !block_tokens || !conf || !top_tok || !unmask_bits || !n_unmask)
     return SPIFFY_EINVAL;
   if (!aligned16(logits)) return SPIFFY_EINVAL;
-  const size_t need = decide_workspace_bytes(*desc);
+  bool fresh;
+  const spiffy_decide_desc d = split_flags(desc, &fresh);
+  const size_t need = decide_workspace_bytes(d);
   if (!workspace || workspace_bytes < need || !aligned16(workspace)) return SPIFFY_EWORKSPACE;
-  return launch_decide(*desc, logits, block_tokens, conf, top_tok, unmask_bits,
+  return launch_decide(d, logits, block_tokens, conf, top_tok, unmask_bits,
                        n_unmask, dev_status, workspace,
-                       static_cast<cudaStream_t>(cuda_stream));
+                       fresh, static_cast<cudaStream_t>(cuda_stream));
 }
 
 spiffy_status spiffy_accept_walk(const spiffy_decide_desc* desc,
@@ -208,9 +223,11 @@ spiffy_status spiffy_accept_walk(const spiffy_decide_desc* desc,
       !accepted_node || !n_accepted || !path || !next_block)
     return SPIFFY_EINVAL;
   if (parent_cap < 0) return SPIFFY_EINVAL;
-  return launch_walk(*desc, block_tokens, parent_off, parent_idx, parent_cap,
+  bool fresh;
+  const spiffy_decide_desc d = split_flags(desc, &fresh);
+  return launch_walk(d, block_tokens, parent_off, parent_idx, parent_cap,
                      top_tok, unmask_bits, accepted_node, n_accepted, path,
-                     next_block, dev_status, static_cast<cudaStream_t>(cuda_stream));
+                     next_block, dev_status, fresh, static_cast<cudaStream_t>(cuda_stream));
 }
 
 spiffy_status spiffy_decide_walk(const spiffy_decide_desc* desc, const void* logits,
@@ -227,17 +244,21 @@ spiffy_status spiffy_decide_walk(const spiffy_decide_desc* desc, const void* log
       !parent_idx || !accepted_node || !n_accepted || !path || !next_block)
     return SPIFFY_EINVAL;
   if (!aligned16(logits) || parent_cap < 0) return SPIFFY_EINVAL;
-  const size_t need = decide_workspace_bytes(*desc);
+  bool fresh;
+  const spiffy_decide_desc d = split_flags(desc, &fresh);
+  const size_t need = decide_workspace_bytes(d);
   if (!workspace || workspace_bytes < need || !aligned16(workspace)) return SPIFFY_EWORKSPACE;
-  return launch_decide_walk(*desc, logits, block_tokens, conf, top_tok, unmask_bits, n_unmask,
+  return launch_decide_walk(d, logits, block_tokens, conf, top_tok, unmask_bits, n_unmask,
                             decide_status, parent_off, parent_idx, parent_cap, accepted_node,
                             n_accepted, path, next_block, walk_status, workspace,
-                            static_cast<cudaStream_t>(cuda_stream));
+                            fresh, static_cast<cudaStream_t>(cuda_stream));
 }
 
 size_t spiffy_decide_walk_lazy_workspace(const spiffy_decide_desc* desc) {
   if (check_decide_desc(desc, true) != SPIFFY_OK) return 0;
-  return decide_lazy_workspace_bytes(*desc);
+  bool fresh;
+  const spiffy_decide_desc d = split_flags(desc, &fresh);
+  return decide_lazy_workspace_bytes(d);
 }
 
 spiffy_status spiffy_decide_walk_lazy(const spiffy_decide_desc* desc, const void* logits,
@@ -254,12 +275,14 @@ spiffy_status spiffy_decide_walk_lazy(const spiffy_decide_desc* desc, const void
       !parent_idx || !accepted_node || !n_accepted || !path || !next_block)
     return SPIFFY_EINVAL;
   if (!aligned16(logits) || parent_cap < 0) return SPIFFY_EINVAL;
-  const size_t need = decide_lazy_workspace_bytes(*desc);
+  bool fresh;
+  const spiffy_decide_desc d = split_flags(desc, &fresh);
+  const size_t need = decide_lazy_workspace_bytes(d);
   if (!workspace || workspace_bytes < need || !aligned16(workspace)) return SPIFFY_EWORKSPACE;
-  return launch_decide_walk_lazy(*desc, logits, block_tokens, conf, top_tok, unmask_bits, n_unmask,
+  return launch_decide_walk_lazy(d, logits, block_tokens, conf, top_tok, unmask_bits, n_unmask,
                                  decide_status, parent_off, parent_idx, parent_cap, accepted_node,
                                  n_accepted, path, next_block, walk_status, workspace,
-                                 static_cast<cudaStream_t>(cuda_stream));
+                                 fresh, static_cast<cudaStream_t>(cuda_stream));
 }
 
 spiffy_status spiffy_stage_masked_rows(const void* src_rows, void* dst_rows, int64_t row_bytes,
@@ -275,13 +298,17 @@ spiffy_status spiffy_stage_masked_rows(const void* src_rows, void* dst_rows, int
 
 size_t spiffy_unmask_decide_sampled_workspace(const spiffy_decide_desc* desc) {
   if (check_decide_desc(desc, true) != SPIFFY_OK) return 0;
-  return decide_sampled_workspace_bytes(*desc);
+  bool fresh;
+  const spiffy_decide_desc d = split_flags(desc, &fresh);
+  return decide_sampled_workspace_bytes(d);
 }
 
 int64_t spiffy_sampled_slice_width(const spiffy_decide_desc* desc) {
   if (check_decide_desc(desc, true) != SPIFFY_OK) return 0;
+  bool fresh;
+  const spiffy_decide_desc d = split_flags(desc, &fresh);
   int64_t chunk = 0;
-  decide_splits(*desc, &chunk);
+  decide_splits(d, &chunk);
   return chunk;
 }
 
@@ -298,19 +325,21 @@ spiffy_status spiffy_unmask_decide_sampled(const spiffy_decide_desc* desc,
   if (!logits || !block_tokens || !conf || !top_tok || !unmask_bits || !n_unmask)
     return SPIFFY_EINVAL;
   if (!aligned16(logits)) return SPIFFY_EINVAL;
-  const size_t need = decide_sampled_workspace_bytes(*desc);
+  bool fresh;
+  const spiffy_decide_desc d = split_flags(desc, &fresh);
+  const size_t need = decide_sampled_workspace_bytes(d);
   if (!workspace || workspace_bytes < need || !aligned16(workspace)) return SPIFFY_EWORKSPACE;
-  return launch_decide_sampled(*desc, sample->temperature, sample->seed, logits, block_tokens, conf,
+  return launch_decide_sampled(d, sample->temperature, sample->seed, logits, block_tokens, conf,
                                top_tok, unmask_bits, n_unmask, dev_status, workspace,
-                               static_cast<cudaStream_t>(cuda_stream));
+                               fresh, static_cast<cudaStream_t>(cuda_stream));
 }
 
 namespace {
 // The descriptor of the fused call names no logits: fill those fields in so that the
 // common checks apply.
-spiffy_status lmhead_desc(const spiffy_decide_desc* desc, int32_t hidden, spiffy_decide_desc* out) {
+spiffy_status lmhead_desc(const spiffy_decide_desc* desc, int32_t hidden, spiffy_decide_desc* out, bool* fresh) {
   if (!desc) return SPIFFY_EINVAL;
-  *out = *desc;
+  *out = split_flags(desc, fresh);
   out->logits_dtype = SPIFFY_BF16;
   out->row_stride = ((int64_t)desc->vocab + 7) / 8 * 8;
   const spiffy_status st = check_decide_desc(out, true);
@@ -322,7 +351,8 @@ spiffy_status lmhead_desc(const spiffy_decide_desc* desc, int32_t hidden, spiffy
 
 size_t spiffy_lmhead_decide_workspace(const spiffy_decide_desc* desc, int32_t hidden) {
   spiffy_decide_desc d;
-  if (lmhead_desc(desc, hidden, &d) != SPIFFY_OK) return 0;
+  bool fresh;
+  if (lmhead_desc(desc, hidden, &d, &fresh) != SPIFFY_OK) return 0;
   const int grid = lmhead_grid(d);
   return grid > 0 ? lmhead_workspace_bytes(d, grid) : 0;
 }
@@ -333,7 +363,8 @@ spiffy_status spiffy_lmhead_decide(const spiffy_decide_desc* desc, int32_t hidde
                                    uint64_t* unmask_bits, int32_t* n_unmask, int32_t* dev_status,
                                    void* workspace, size_t workspace_bytes, void* cuda_stream) {
   spiffy_decide_desc d;
-  const spiffy_status st = lmhead_desc(desc, hidden, &d);
+  bool fresh;
+  const spiffy_status st = lmhead_desc(desc, hidden, &d, &fresh);
   if (st != SPIFFY_OK) return st;
   if (!hidden_states || !weight || !block_tokens || !conf || !top_tok || !unmask_bits || !n_unmask)
     return SPIFFY_EINVAL;
@@ -344,12 +375,13 @@ spiffy_status spiffy_lmhead_decide(const spiffy_decide_desc* desc, int32_t hidde
   if (!workspace || workspace_bytes < need || !aligned16(workspace)) return SPIFFY_EWORKSPACE;
   return launch_lmhead_decide(d, hidden, hidden_states, weight, block_tokens, conf, top_tok,
                               unmask_bits, n_unmask, dev_status, workspace,
-                              static_cast<cudaStream_t>(cuda_stream));
+                              fresh, static_cast<cudaStream_t>(cuda_stream));
 }
 
 size_t spiffy_draft_blocks_workspace(const spiffy_draft_desc* desc) {
   if (check_draft_desc(desc) != SPIFFY_OK) return 0;
-  return draft_workspace_bytes(*desc);
+  bool fresh;
+  return draft_workspace_bytes(split_flags(desc, &fresh));
 }
 
 spiffy_status spiffy_draft_blocks(const spiffy_draft_desc* desc, const void* logits,
@@ -366,11 +398,13 @@ spiffy_status spiffy_draft_blocks(const spiffy_draft_desc* desc, const void* log
       !draft_tokens || !kept || !score || !parent_off || !parent_idx)
     return SPIFFY_EINVAL;
   if (!aligned16(logits)) return SPIFFY_EINVAL;
-  const size_t need = draft_workspace_bytes(*desc);
+  bool fresh;
+  const spiffy_draft_desc d = split_flags(desc, &fresh);
+  const size_t need = draft_workspace_bytes(d);
   if (!workspace || workspace_bytes < need || !aligned16(workspace)) return SPIFFY_EWORKSPACE;
-  return launch_draft(*desc, logits, state, formula_off, formula_i, formula_j, child_off, child_idx,
+  return launch_draft(d, logits, state, formula_off, formula_i, formula_j, child_off, child_idx,
                       draft_tokens, kept, score, parent_off, parent_idx, dev_status, workspace,
-                      static_cast<cudaStream_t>(cuda_stream));
+                      fresh, static_cast<cudaStream_t>(cuda_stream));
 }
 
 const char* spiffy_status_string(spiffy_status status) {

@@ -860,13 +860,10 @@ spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const void* q, cons
   p.spin_limit = mbar_poll_limit();
   p.early_trigger = (d.kernel & SPIFFY_ATTN_EARLY_DEPENDENTS) ? 1 : 0;
 
-  if (cudaFuncSetAttribute(graph_attention_tc_kernel<1>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess ||
-      cudaFuncSetAttribute(graph_attention_tc_kernel<2>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
-    return SPIFFY_ECUDA;
+  static std::atomic<bool> smem_allowed[2][64];
   const dim3 grid((pl.MT + pl.nq - 1) / pl.nq, d.batch * d.n_kv_heads, pl.splits);
   auto kern = pl.nq == 2 ? graph_attention_tc_kernel<2> : graph_attention_tc_kernel<1>;
+  if (!allow_smem(kern, kSmemBytes, smem_allowed[pl.nq - 1])) return SPIFFY_ECUDA;
   {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "spiffy.h"
 
 namespace spiffy {
@@ -58,10 +60,13 @@ uint32_t flag_poll_limit();   // polls of one wait on a global-memory word (lazy
 int32_t lazy_extra_arrivals();  // arrivals sequence 0's tail expects beyond those that can come
 
 // Entry points implemented in the kernel files; all validated by the caller.
+// `fresh`: the call's first kernel clears the status words (SPIFFY_FRESH_STATUS);
+// the descriptors arrive without that flag.
 spiffy_status launch_decide(const spiffy_decide_desc& d, const void* logits,
                             const int32_t* block_tokens, float* conf,
                             int32_t* top_tok, uint64_t* unmask_bits,
                             int32_t* n_unmask, int32_t* dev_status, void* ws,
+                            bool fresh,
                             cudaStream_t stream);
 size_t decide_workspace_bytes(const spiffy_decide_desc& d);
 int decide_splits(const spiffy_decide_desc& d, int64_t* chunk_elems);
@@ -73,7 +78,8 @@ spiffy_status launch_walk(const spiffy_decide_desc& d,
                           const uint64_t* unmask_bits, int32_t* accepted_node,
                           int32_t* n_accepted, int32_t* path,
                           int32_t* next_block, int32_t* dev_status,
-                          cudaStream_t stream);
+                          bool fresh,
+                            cudaStream_t stream);
 
 spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits,
                                  const int32_t* block_tokens, float* conf, int32_t* top_tok,
@@ -82,7 +88,8 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
                                  const int32_t* parent_idx, int32_t parent_cap,
                                  int32_t* accepted_node, int32_t* n_accepted, int32_t* path,
                                  int32_t* next_block, int32_t* walk_status, void* ws,
-                                 cudaStream_t stream);
+                                 bool fresh,
+                            cudaStream_t stream);
 
 size_t decide_lazy_workspace_bytes(const spiffy_decide_desc& d);
 spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc& d, const void* logits,
@@ -92,7 +99,8 @@ spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc& d, const void* l
                                       const int32_t* parent_idx, int32_t parent_cap,
                                       int32_t* accepted_node, int32_t* n_accepted, int32_t* path,
                                       int32_t* next_block, int32_t* walk_status, void* ws,
-                                      cudaStream_t stream);
+                                      bool fresh,
+                            cudaStream_t stream);
 
 spiffy_status launch_stage_masked_rows(const void* src, void* dst, int64_t row_bytes,
                                        const int32_t* tokens, int32_t mask_id, int64_t n_rows,
@@ -102,7 +110,8 @@ size_t decide_sampled_workspace_bytes(const spiffy_decide_desc& d);
 spiffy_status launch_decide_sampled(const spiffy_decide_desc& d, float temperature, uint64_t seed,
                                     const void* logits, const int32_t* block_tokens, float* conf,
                                     int32_t* top_tok, uint64_t* unmask_bits, int32_t* n_unmask,
-                                    int32_t* dev_status, void* ws, cudaStream_t stream);
+                                    int32_t* dev_status, void* ws, bool fresh,
+                            cudaStream_t stream);
 
 spiffy_status launch_decide_finalize(const spiffy_decide_desc& d, const void* partials, int splits,
                                      const int32_t* block_tokens, float* conf, int32_t* top_tok,
@@ -113,7 +122,8 @@ size_t lmhead_workspace_bytes(const spiffy_decide_desc& d, int grid);
 spiffy_status launch_lmhead_decide(const spiffy_decide_desc& d, int hidden, const void* hstates,
                                    const void* weight, const int32_t* block_tokens, float* conf,
                                    int32_t* top_tok, uint64_t* unmask_bits, int32_t* n_unmask,
-                                   int32_t* dev_status, void* ws, cudaStream_t stream);
+                                   int32_t* dev_status, void* ws, bool fresh,
+                            cudaStream_t stream);
 
 spiffy_status launch_attention_simt(const spiffy_attn_desc& d, const void* q,
                                     const void* kp, const void* vp,
@@ -126,7 +136,8 @@ spiffy_status launch_draft(const spiffy_draft_desc& d, const void* logits, const
                            const int32_t* formula_j, const int32_t* child_off,
                            const int32_t* child_idx, int32_t* tokens, int32_t* kept, float* score,
                            int32_t* parent_off, int32_t* parent_idx, int32_t* dev_status, void* ws,
-                           cudaStream_t stream);
+                           bool fresh,
+                            cudaStream_t stream);
 
 // tcgen05 path: shape support query, workspace and launch.  The cached context
 // comes as up to two segments of keys/values, [B][len][Hkv][d] each, whose
@@ -177,6 +188,19 @@ __device__ __forceinline__ void pdl_launch_dependents() {
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900
   cudaTriggerProgrammaticLaunchCompletion();
 #endif
+}
+
+// Lets `kern` use `bytes` of dynamic shared memory on the current device.  Asked
+// for once per kernel and device (the attribute sticks to the kernel); `done` is
+// the kernel's own table, all false at first.
+template <typename Kernel>
+bool allow_smem(Kernel kern, int bytes, std::atomic<bool> (&done)[64]) {
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return false;
+  if (done[device].load(std::memory_order_acquire)) return true;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+  done[device].store(true, std::memory_order_release);
+  return true;
 }
 
 inline spiffy_status check_launch() {

@@ -29,6 +29,22 @@ struct __align__(16) Partial {
   int pad;
 };
 
+// Clears the status words of a call whose caller left them arbitrary
+// (SPIFFY_FRESH_STATUS); part of the call's first kernel, which sets no bit itself.
+struct StatusClear {
+  int32_t* a;  // [B], null when there is nothing to clear
+  int32_t* b;
+  int rows_per_seq;
+  __device__ __forceinline__ void run(int row) const {
+    if (blockIdx.x != 0 || threadIdx.x != 0 || rows_per_seq == 0 || row % rows_per_seq != 0) return;
+    if (a) a[row / rows_per_seq] = 0;
+    if (b) b[row / rows_per_seq] = 0;
+  }
+};
+inline StatusClear status_clear(const spiffy_decide_desc& d, bool fresh, int32_t* a, int32_t* b) {
+  return fresh ? StatusClear{a, b, d.n_nodes * d.block_len} : StatusClear{nullptr, nullptr, 0};
+}
+
 // acc += {2^(x0 * log2e - ml), 2^(x1 * log2e - ml)}; k2 = {log2e, log2e}, nml2 = {-ml, -ml}
 __device__ __forceinline__ uint64_t add_exp2(uint64_t acc, float x0, float x1, uint64_t k2,
                                              uint64_t nml2) {

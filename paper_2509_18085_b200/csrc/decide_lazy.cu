@@ -56,6 +56,7 @@ struct LazyParams {
   unsigned* arrivals;  // [B] slices of b reduced so far, over all levels
   int32_t* epoch;      // [B] levels of b whose tail has finished
   int32_t* cur;        // [B] node b stands on at level epoch[b], -1 once its walk has ended
+  int clear_status;    // the status words arrive with arbitrary contents
   int stage_graph;     // the sequence's states and parent lists fit shared memory
   unsigned wait_spins;   // polls of one wait before it gives up
   unsigned extra_arrivals;  // test hook: sequence 0 expects this many arrivals that never come
@@ -133,7 +134,13 @@ decide_walk_lazy_kernel(const LazyParams p) {
       p.n_unmask[(int64_t)b_own * N + i] = -1;  // not evaluated (yet)
     }
   }
-  if (tid == 0) s_bad = 0;
+  if (tid == 0) {
+    s_bad = 0;
+    if (b_own >= 0 && p.clear_status) {  // only this CTA touches its sequence's words
+      if (p.decide_status) p.decide_status[b_own] = 0;
+      if (p.walk_status) p.walk_status[b_own] = 0;
+    }
+  }
   int own_node = b_own >= 0 ? 0 : -1;  // uniform over the CTA
   int own_hops = 0;
   // arrivals[b_own] once the current level is reduced
@@ -315,7 +322,7 @@ spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc& d, const void* l
                                       const int32_t* parent_idx, int32_t parent_cap,
                                       int32_t* accepted_node, int32_t* n_accepted, int32_t* path,
                                       int32_t* next_block, int32_t* walk_status, void* ws,
-                                      cudaStream_t stream) {
+                                      bool fresh, cudaStream_t stream) {
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess) return SPIFFY_ECUDA;
   const bool bf16 = d.logits_dtype == SPIFFY_BF16;
@@ -357,6 +364,7 @@ spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc& d, const void* l
   p.arrivals = reinterpret_cast<unsigned*>(p.header + 1);
   p.epoch = reinterpret_cast<int32_t*>(p.arrivals + d.batch);
   p.cur = p.epoch + d.batch;
+  p.clear_status = fresh ? 1 : 0;
   p.stage_graph = stage_graph;
   p.wait_spins = flag_poll_limit();
   p.extra_arrivals = (unsigned)lazy_extra_arrivals();

@@ -89,11 +89,13 @@ template <typename T>
 __global__ void __launch_bounds__(kReduceThreads, 8)
 decide_sampled_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V, int64_t chunk,
                              int splits, int L, const int32_t* __restrict__ block_tokens, int mask_id,
-                             float k, Partial* __restrict__ partials, int* __restrict__ node_count) {
+                             float k, Partial* __restrict__ partials, int* __restrict__ node_count,
+                             StatusClear clear) {
 #if __CUDA_ARCH__ >= 900
   cudaGridDependencySynchronize();
 #endif
   const int row = blockIdx.y;
+  clear.run(row);
   if (blockIdx.x == 0 && threadIdx.x == 0 && row % L == 0) node_count[row / L] = 0;
   if (block_tokens[row] != mask_id) return;  // already unmasked: never read
   reduce_slice(logits + (int64_t)row * row_stride, V, chunk, (int)blockIdx.x,
@@ -333,7 +335,7 @@ size_t decide_sampled_workspace_bytes(const spiffy_decide_desc& d) {
 spiffy_status launch_decide_sampled(const spiffy_decide_desc& d, float temperature, uint64_t seed,
                                     const void* logits, const int32_t* block_tokens, float* conf,
                                     int32_t* top_tok, uint64_t* unmask_bits, int32_t* n_unmask,
-                                    int32_t* dev_status, void* ws, cudaStream_t stream) {
+                                    int32_t* dev_status, void* ws, bool fresh, cudaStream_t stream) {
   int64_t chunk = 0;
   const int splits = decide_splits(d, &chunk);
   const int rows = d.batch * d.n_nodes * d.block_len;
@@ -348,7 +350,7 @@ spiffy_status launch_decide_sampled(const spiffy_decide_desc& d, float temperatu
     cudaError_t r = launch_pdl(decide_sampled_reduce_kernel<T>, dim3(splits, rows), dim3(kReduceThreads),
                                (size_t)0, stream, typed, (int64_t)d.row_stride, (int)d.vocab, chunk, splits,
                                (int)d.block_len, block_tokens, (int)d.mask_token_id, inv_t * kLog2e, partials,
-                               node_count);
+                               node_count, status_clear(d, fresh, dev_status, nullptr));
     count_launch();
     if (r != cudaSuccess) return r;
     r = launch_pdl(decide_sampled_select_kernel<T>, dim3(rows), dim3(kReduceThreads), (size_t)0, stream,

@@ -67,12 +67,13 @@ template <typename T>
 __global__ void __launch_bounds__(kThreads)
 draft_topk_kernel(const T* __restrict__ logits, int64_t row_stride, int V, int64_t chunk,
                   int splits, int K, const int32_t* __restrict__ state, int mask_id,
-                  TopPartial* __restrict__ partials) {
+                  TopPartial* __restrict__ partials, int32_t* __restrict__ clear_status, int L) {
 #if __CUDA_ARCH__ >= 900
   cudaGridDependencySynchronize();
   pdl_launch_dependents();  // the build kernel (one CTA per sequence) may take its SM and stage the graph
 #endif
   const int row = blockIdx.y;
+  if (clear_status && blockIdx.x == 0 && threadIdx.x == 0 && row % L == 0) clear_status[row / L] = 0;
   if (state[row] != mask_id) return;
   const int split = blockIdx.x;
   const int64_t begin = (int64_t)split * chunk;
@@ -195,6 +196,7 @@ struct BuildArgs {
   int32_t* parent_off;  // [B][budget+2]
   int32_t* parent_idx;  // [B][parent_cap]
   int32_t* dev_status;  // [B]
+  int fill_parents;     // entries of parent_idx past the lists are written as 0
 };
 
 // Is the candidate set of formula a a strict subset of formula c's?  a < 0 is
@@ -442,6 +444,8 @@ draft_build_kernel(BuildArgs g) {
       if (c == g.budget) off[c + 1] = min(start + n_parents[c], g.parent_cap);
       if (start + n_parents[c] > g.parent_cap && g.dev_status) atomicOr(g.dev_status + b, SPIFFY_DEV_BADGRAPH);
     }
+    if (g.fill_parents && c == g.budget)
+      for (int i = start + n_parents[c] + lane; i < g.parent_cap; i += 32) idx[i] = 0;
     if (c > 0 && node_formula[c] >= 0) {
       int w = start;
       for (int a0 = 0; a0 < c; a0 += 32) {
@@ -478,20 +482,21 @@ spiffy_status launch_draft(const spiffy_draft_desc& d, const void* logits, const
                            const int32_t* formula_j, const int32_t* child_off,
                            const int32_t* child_idx, int32_t* tokens, int32_t* kept, float* score,
                            int32_t* parent_off, int32_t* parent_idx, int32_t* dev_status, void* ws,
-                           cudaStream_t stream) {
+                           bool fresh, cudaStream_t stream) {
   int splits = 1;
   const int64_t chunk = draft_chunk(d, &splits);
   TopPartial* partials = static_cast<TopPartial*>(ws);
+  int32_t* clear = fresh ? dev_status : nullptr;
   const dim3 grid(splits, d.batch * d.block_len);
   cudaError_t e;
   if (d.logits_dtype == SPIFFY_BF16)
     e = launch_pdl(draft_topk_kernel<__nv_bfloat16>, grid, dim3(kThreads), (size_t)0, stream,
                    static_cast<const __nv_bfloat16*>(logits), (int64_t)d.row_stride, (int)d.vocab, chunk,
-                   splits, (int)d.top_k, state, (int)d.mask_token_id, partials);
+                   splits, (int)d.top_k, state, (int)d.mask_token_id, partials, clear, (int)d.block_len);
   else
     e = launch_pdl(draft_topk_kernel<float>, grid, dim3(kThreads), (size_t)0, stream,
                    static_cast<const float*>(logits), (int64_t)d.row_stride, (int)d.vocab, chunk, splits,
-                   (int)d.top_k, state, (int)d.mask_token_id, partials);
+                   (int)d.top_k, state, (int)d.mask_token_id, partials, clear, (int)d.block_len);
   count_launch();
   if (e != cudaSuccess) return SPIFFY_ECUDA;
   BuildArgs g;
@@ -499,7 +504,7 @@ spiffy_status launch_draft(const spiffy_draft_desc& d, const void* logits, const
   g.budget = d.budget; g.parent_cap = d.parent_cap; g.mask_id = d.mask_token_id;
   g.state = state; g.formula_off = formula_off; g.formula_i = formula_i; g.formula_j = formula_j;
   g.child_off = child_off; g.child_idx = child_idx; g.tokens = tokens; g.kept = kept; g.score = score;
-  g.parent_off = parent_off; g.parent_idx = parent_idx; g.dev_status = dev_status;
+  g.parent_off = parent_off; g.parent_idx = parent_idx; g.dev_status = dev_status; g.fill_parents = fresh ? 1 : 0;
   const size_t smem = (size_t)d.block_len * kMaxK * 8 + (size_t)d.block_len * 4 +
                       (size_t)d.n_formulas * 12 + (size_t)(d.budget + 1) * 8 + 16;
   e = launch_pdl(draft_build_kernel, dim3(d.batch), dim3(kBuildThreads), smem, stream, g);

@@ -255,7 +255,7 @@ size_t lmhead_workspace_bytes(const spiffy_decide_desc& d, int grid) {
 spiffy_status launch_lmhead_decide(const spiffy_decide_desc& d, int hidden, const void* hstates,
                                    const void* weight, const int32_t* block_tokens, float* conf,
                                    int32_t* top_tok, uint64_t* unmask_bits, int32_t* n_unmask,
-                                   int32_t* dev_status, void* ws, cudaStream_t stream) {
+                                   int32_t* dev_status, void* ws, bool fresh, cudaStream_t stream) {
   const int rows = d.batch * d.n_nodes * d.block_len;
   const int grid = lmhead_grid(d);
   if (grid <= 0) return SPIFFY_ECUDA;
@@ -268,15 +268,8 @@ spiffy_status launch_lmhead_decide(const spiffy_decide_desc& d, int hidden, cons
   if (!make_map(&tm_h, hstates, hidden / 128, rows, 1, 1, 128) ||
       !make_map(&tm_w, weight, hidden / 128, d.vocab, 1, 1, n_tile))
     return SPIFFY_ECUDA;
-  static bool attr_set[64];
-  int device = 0;
-  cudaGetDevice(&device);
-  if (device >= 0 && device < 64 && !attr_set[device]) {
-    if (cudaFuncSetAttribute(lmhead_reduce_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLmSmem) !=
-        cudaSuccess)
-      return SPIFFY_ECUDA;
-    attr_set[device] = true;
-  }
+  static std::atomic<bool> smem_allowed[64];
+  if (!allow_smem(lmhead_reduce_kernel, kLmSmem, smem_allowed)) return SPIFFY_ECUDA;
   LmParams p;
   p.rows = rows;
   p.hidden = hidden;
@@ -286,6 +279,9 @@ spiffy_status launch_lmhead_decide(const spiffy_decide_desc& d, int hidden, cons
   p.status = dev_status;
   p.n_status = d.batch;
   p.spin_limit = mbar_poll_limit();
+  // any CTA of the first kernel may set a bit: cleared ahead of it
+  if (fresh && dev_status && cudaMemsetAsync(dev_status, 0, (size_t)d.batch * 4, stream) != cudaSuccess)
+    return SPIFFY_ECUDA;
   cudaError_t e = launch_pdl(lmhead_reduce_kernel, dim3(grid), dim3(kLmThreads), (size_t)kLmSmem, stream,
                              tm_h, tm_w, p);
   count_launch();

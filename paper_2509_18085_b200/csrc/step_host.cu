@@ -29,7 +29,7 @@ struct Layout {
 Layout layout_of(const spiffy_step_desc& s) {
   const spiffy_attn_desc& a = s.attn;
   const spiffy_decide_desc& d = s.decide;
-  const size_t e = a.dtype == SPIFFY_BF16 ? 2 : 4, le = d.logits_dtype == SPIFFY_BF16 ? 2 : 4;
+  const size_t e = a.dtype == SPIFFY_BF16 ? 2 : 4, le = (d.logits_dtype & ~SPIFFY_FRESH_STATUS) == SPIFFY_BF16 ? 2 : 4;
   const size_t B = a.batch, N = a.n_nodes, L = a.block_len;
   Layout l;
   l.qn = B * N * L * a.n_q_heads * a.head_dim * e;
@@ -48,7 +48,7 @@ Layout layout_of(const spiffy_step_desc& s) {
   l.accepted = take(B * 4); l.n_accepted = take(B * 4); l.path = take(B * N * 4); l.next_block = take(B * L * 4);
   l.status = take((1 + 2 * B) * 4);
   l.attn_ws = take(spiffy_graph_attention_workspace(&a));
-  l.decide_ws = take(decide_workspace_bytes(d));
+  l.decide_ws = take(spiffy_unmask_decide_workspace(&d));
   l.total = o;
   return l;
 }
@@ -117,7 +117,8 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
                                       size_t workspace_bytes, void* cuda_stream) {
   spiffy_status st = check(desc);
   if (st != SPIFFY_OK) return st;
-  const spiffy_step_desc s = *desc;
+  spiffy_step_desc s = *desc;
+  s.decide.logits_dtype &= ~SPIFFY_FRESH_STATUS;  // the call clears all its status words
   if (!q || !k_block || !v_block || !logits || !block_tokens || !parent_off || !parent_idx ||
       !accepted_node || !n_accepted || !path || !next_block || !status)
     return SPIFFY_EINVAL;

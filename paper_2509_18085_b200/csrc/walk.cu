@@ -18,7 +18,8 @@ accept_walk_kernel(int N, int L, const int32_t* __restrict__ block_tokens,
                    int32_t* __restrict__ accepted_node,
                    int32_t* __restrict__ n_accepted, int32_t* __restrict__ path,
                    int32_t* __restrict__ next_block,
-                   int32_t* __restrict__ dev_status, int stage_in_smem, int link_in_smem) {
+                   int32_t* __restrict__ dev_status, int stage_in_smem, int link_in_smem,
+                   int clear_status) {
   const int b = blockIdx.x;
   const int tid = threadIdx.x;
   const int32_t* state = block_tokens + (int64_t)b * N * L;
@@ -54,6 +55,7 @@ accept_walk_kernel(int N, int L, const int32_t* __restrict__ block_tokens,
   pdl_launch_dependents();
   cudaGridDependencySynchronize();  // the decision kernel's outputs are visible
 #endif
+  if (clear_status && tid == 0 && dev_status) dev_status[b] = 0;
   for (int i = tid; i < N; i += kWalkThreads) link[i] = kNoLink;
   if (stage_in_smem) {
     for (int i = tid; i < N * L; i += kWalkThreads) copy4(s_top + i, top + i);
@@ -81,7 +83,7 @@ spiffy_status launch_walk(const spiffy_decide_desc& d,
                           int32_t parent_cap, const int32_t* top_tok,
                           const uint64_t* unmask_bits, int32_t* accepted_node,
                           int32_t* n_accepted, int32_t* path,
-                          int32_t* next_block, int32_t* dev_status,
+                          int32_t* next_block, int32_t* dev_status, bool fresh,
                           cudaStream_t stream) {
   const size_t graph = (size_t)d.n_nodes * 8 +
                        ((size_t)2 * d.n_nodes * d.block_len + d.n_nodes + 1 + parent_cap) * 4;
@@ -93,7 +95,7 @@ spiffy_status launch_walk(const spiffy_decide_desc& d,
       accept_walk_kernel, dim3(d.batch), dim3(kWalkThreads), smem, stream,
       (int)d.n_nodes, (int)d.block_len, block_tokens, parent_off, parent_idx, (int)parent_cap,
       top_tok, unmask_bits, accepted_node, n_accepted, path, next_block, dev_status,
-      stage_in_smem, link_in_smem);
+      stage_in_smem, link_in_smem, fresh ? 1 : 0);
   count_launch();
   return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
 }

@@ -1,4 +1,6 @@
-"""ctypes binding of ``libspiffy.so`` -- argument marshalling only.
+"""Python side of ``libspiffy.so`` -- argument marshalling only, most of it in the
+native module ``_binding`` (csrc/binding.cpp); the calls that take microseconds
+anyway go through ctypes.
 
 The three entry points carry the names of the C ABI (``include/spiffy.h``) and
 take torch CUDA tensors; every step of the path runs in the library's kernels.
@@ -66,6 +68,7 @@ class DraftDesc(ctypes.Structure):
 
 
 _lib = None
+_nat = None
 
 
 def lib() -> ctypes.CDLL:
@@ -131,6 +134,21 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _native():
+    """The native binding; raises when it has not been built."""
+    global _nat
+    if _nat is None:
+        lib()  # says what is missing; the binding uses this very library
+        try:
+            from . import _binding
+        except ImportError as e:
+            raise RuntimeError("the native binding is missing: build it with "
+                               "`python -m paper_2509_18085_b200.build`") from e
+        _binding.set_classes(SpiffyError, Decision, Walk, Drafts)
+        _nat = _binding
+    return _nat
+
+
 def launch_count() -> int:
     return int(lib().spiffy_launch_count())
 
@@ -188,21 +206,8 @@ def spiffy_graph_attention(q, k_prefix, v_prefix, k_block, v_block, out=None,
                            dev_status=None, workspace=None, stream=None):
     """Packed draft-graph attention.  q [B,N,L,Hq,d]; k/v_prefix [B,P,Hkv,d];
     k/v_block [B,N,L,Hkv,d]; returns out [B,N,L,Hq,d] (allocated when None)."""
-    desc = attn_desc(q, k_prefix, k_block, scale, kernel)
-    if out is None:
-        out = torch.empty_like(q)
-    need = spiffy_graph_attention_workspace(desc)
-    if need and workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    st = lib().spiffy_graph_attention(
-        ctypes.byref(desc), _dev(q, "q"), _dev(k_prefix, "k_prefix", q.dtype),
-        _dev(v_prefix, "v_prefix", q.dtype), _dev(k_block, "k_block", q.dtype),
-        _dev(v_block, "v_block", q.dtype), _dev(out, "out", q.dtype),
-        _dev(dev_status, "dev_status", torch.int32), _dev(workspace, "workspace"),
-        ws_bytes, _stream(stream))
-    _check(st, "spiffy_graph_attention")
-    return out
+    return _native().graph_attention(q, k_prefix, v_prefix, k_block, v_block, out, scale, kernel, dev_status,
+                                     workspace, stream)
 
 
 def decide_desc(logits, block_tokens, mask_token_id, rule, top_s=1, threshold=0.9) -> DecideDesc:
@@ -227,25 +232,9 @@ def spiffy_full_sequence_attention(q_nodes, q_suffix, k_prefix, v_prefix, k_suff
     q_nodes [B,N,L,Hq,d], q_suffix [B,S,Hq,d], k/v_prefix [B,P,Hkv,d], k/v_suffix
     [B,S,Hkv,d], k/v_block [B,N,L,Hkv,d], all bf16, d = 128, S <= 1024.
     Returns (out_nodes [B,N,L,Hq,d], out_suffix [B,S,Hq,d])."""
-    desc = attn_desc(q_nodes, k_prefix, k_block, scale, ATTN_TCGEN05)
-    S = int(q_suffix.shape[1])
-    if out_nodes is None:
-        out_nodes = torch.empty_like(q_nodes)
-    if out_suffix is None:
-        out_suffix = torch.empty_like(q_suffix)
-    need = int(lib().spiffy_full_sequence_attention_workspace(ctypes.byref(desc), S))
-    if need and workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=q_nodes.device)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    dt = q_nodes.dtype
-    st = lib().spiffy_full_sequence_attention(
-        ctypes.byref(desc), S, _dev(q_nodes, "q_nodes"), _dev(q_suffix, "q_suffix", dt),
-        _dev(k_prefix, "k_prefix", dt), _dev(v_prefix, "v_prefix", dt), _dev(k_suffix, "k_suffix", dt),
-        _dev(v_suffix, "v_suffix", dt), _dev(k_block, "k_block", dt), _dev(v_block, "v_block", dt),
-        _dev(out_nodes, "out_nodes", dt), _dev(out_suffix, "out_suffix", dt),
-        _dev(dev_status, "dev_status", torch.int32), _dev(workspace, "workspace"), ws_bytes, _stream(stream))
-    _check(st, "spiffy_full_sequence_attention")
-    return out_nodes, out_suffix
+    return _native().full_sequence_attention(q_nodes, q_suffix, k_prefix, v_prefix, k_suffix, v_suffix, k_block,
+                                             v_block, scale, ATTN_TCGEN05, out_nodes, out_suffix, dev_status,
+                                             workspace, stream)
 
 
 @dataclass
@@ -275,23 +264,8 @@ def spiffy_unmask_decide(logits, block_tokens, mask_token_id: int, rule: int,
                          workspace=None, stream=None) -> Decision:
     """Steps 1-4 of Algorithm 1 for every node.  logits [B,N,L,V] (rows may be
     a strided view of a wider buffer), block_tokens [B,N,L] int32."""
-    desc = decide_desc(logits, block_tokens, mask_token_id, rule, top_s, threshold)
-    B, N, L = block_tokens.shape
-    dev = logits.device
-    if out is None:
-        out = _new_decision(B, N, L, dev)
-    need = spiffy_unmask_decide_workspace(desc)
-    if workspace is None:
-        workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
-    st = lib().spiffy_unmask_decide(
-        ctypes.byref(desc), _logits_ptr(logits), _dev(block_tokens, "block_tokens", torch.int32),
-        _dev(out.conf, "conf", torch.float32), _dev(out.top_tok, "top_tok", torch.int32),
-        _dev(out.unmask_bits, "unmask_bits", torch.int64),
-        _dev(out.n_unmask, "n_unmask", torch.int32),
-        _dev(out.dev_status, "dev_status", torch.int32), _dev(workspace, "workspace"),
-        workspace.numel() * workspace.element_size(), _stream(stream))
-    _check(st, "spiffy_unmask_decide")
-    return out
+    return _native().unmask_decide(logits, block_tokens, mask_token_id, rule, top_s, threshold, out, workspace,
+                                   stream)
 
 
 def spiffy_unmask_decide_sampled(logits, block_tokens, mask_token_id: int, rule: int, temperature: float,
@@ -302,25 +276,8 @@ def spiffy_unmask_decide_sampled(logits, block_tokens, mask_token_id: int, rule:
     of the running sum inside the chosen slice) with Philox4x32-10 noise that
     follows the block's state (sequence, position, slice, masked count), never
     the node's index; conf is the drawn token's probability."""
-    desc = decide_desc(logits, block_tokens, mask_token_id, rule, top_s, threshold)
-    sample = SampleDesc(float(temperature), 0, int(seed) & 0xFFFFFFFFFFFFFFFF)
-    B, N, L = block_tokens.shape
-    dev = logits.device
-    if out is None:
-        out = _new_decision(B, N, L, dev)
-    if workspace is None:
-        need = int(lib().spiffy_unmask_decide_sampled_workspace(ctypes.byref(desc)))
-        workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
-    st = lib().spiffy_unmask_decide_sampled(
-        ctypes.byref(desc), ctypes.byref(sample), _logits_ptr(logits),
-        _dev(block_tokens, "block_tokens", torch.int32),
-        _dev(out.conf, "conf", torch.float32), _dev(out.top_tok, "top_tok", torch.int32),
-        _dev(out.unmask_bits, "unmask_bits", torch.int64),
-        _dev(out.n_unmask, "n_unmask", torch.int32),
-        _dev(out.dev_status, "dev_status", torch.int32), _dev(workspace, "workspace"),
-        workspace.numel() * workspace.element_size(), _stream(stream))
-    _check(st, "spiffy_unmask_decide_sampled")
-    return out
+    return _native().unmask_decide_sampled(logits, block_tokens, mask_token_id, rule, top_s, threshold, temperature,
+                                           seed, out, workspace, stream)
 
 
 def spiffy_sampled_slice_width(desc: DecideDesc) -> int:
@@ -335,32 +292,8 @@ def spiffy_lmhead_decide(hidden_states, weight, block_tokens, mask_token_id: int
     hidden_states @ weight.T are formed and reduced on the tensor cores without
     ever being written.  hidden_states [B,N,L,H] bf16 (H a multiple of 128),
     weight [V,H] bf16, block_tokens [B,N,L] int32."""
-    B, N, L = block_tokens.shape
-    H = hidden_states.shape[-1]
-    V = weight.shape[0]
-    if hidden_states.dtype != torch.bfloat16 or weight.dtype != torch.bfloat16:
-        raise ValueError("hidden_states and weight must be bf16")
-    if tuple(hidden_states.shape) != (B, N, L, H) or weight.shape[1] != H:
-        raise ValueError("hidden_states must be [B,N,L,H] and weight [V,H]")
-    if not hidden_states.is_contiguous() or not weight.is_contiguous():
-        raise ValueError("hidden_states and weight must be contiguous")
-    desc = DecideDesc(B, N, L, V, BF16, V, int(mask_token_id), int(rule), int(top_s), float(threshold))
-    dev = hidden_states.device
-    if out is None:
-        out = _new_decision(B, N, L, dev)
-    if workspace is None:
-        need = int(lib().spiffy_lmhead_decide_workspace(ctypes.byref(desc), int(H)))
-        workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
-    st = lib().spiffy_lmhead_decide(
-        ctypes.byref(desc), int(H), _dev(hidden_states, "hidden_states"), _dev(weight, "weight"),
-        _dev(block_tokens, "block_tokens", torch.int32),
-        _dev(out.conf, "conf", torch.float32), _dev(out.top_tok, "top_tok", torch.int32),
-        _dev(out.unmask_bits, "unmask_bits", torch.int64),
-        _dev(out.n_unmask, "n_unmask", torch.int32),
-        _dev(out.dev_status, "dev_status", torch.int32), _dev(workspace, "workspace"),
-        workspace.numel() * workspace.element_size(), _stream(stream))
-    _check(st, "spiffy_lmhead_decide")
-    return out
+    return _native().lmhead_decide(hidden_states, weight, block_tokens, mask_token_id, rule, top_s, threshold, out,
+                                   workspace, stream)
 
 
 def spiffy_unmask_decide_static(logits, block_tokens, mask_token_id: int, rule: int, out: Decision,
@@ -394,40 +327,7 @@ class Walk:
 def spiffy_accept_walk(block_tokens, parent_off, parent_idx, top_tok, unmask_bits,
                        out: Optional[Walk] = None, stream=None) -> Walk:
     """Step 5 of Algorithm 1.  parent_off [B,N+1], parent_idx [B,cap] int32."""
-    B, N, L = block_tokens.shape
-    dev = block_tokens.device
-    desc = DecideDesc(B, N, L, 0, F32, 0, 0, 0, 1, 0.0)
-    if out is None:
-        out = _new_walk(B, N, L, dev)
-    if tuple(parent_off.shape) != (B, N + 1) or parent_idx.dim() != 2 or parent_idx.shape[0] != B:
-        raise ValueError("parent_off must be [B,N+1] and parent_idx [B,cap]")
-    st = lib().spiffy_accept_walk(
-        ctypes.byref(desc), _dev(block_tokens, "block_tokens", torch.int32),
-        _dev(parent_off, "parent_off", torch.int32), _dev(parent_idx, "parent_idx", torch.int32),
-        int(parent_idx.shape[1]), _dev(top_tok, "top_tok", torch.int32),
-        _dev(unmask_bits, "unmask_bits", torch.int64),
-        _dev(out.accepted_node, "accepted_node", torch.int32),
-        _dev(out.n_accepted, "n_accepted", torch.int32), _dev(out.path, "path", torch.int32),
-        _dev(out.next_block, "next_block", torch.int32),
-        _dev(out.dev_status, "dev_status", torch.int32), _stream(stream))
-    _check(st, "spiffy_accept_walk")
-    return out
-
-
-def _new_decision(B, N, L, dev) -> Decision:
-    return Decision(torch.empty((B, N, L), dtype=torch.float32, device=dev),
-                    torch.empty((B, N, L), dtype=torch.int32, device=dev),
-                    torch.empty((B, N), dtype=torch.int64, device=dev),
-                    torch.empty((B, N), dtype=torch.int32, device=dev),
-                    torch.zeros((B,), dtype=torch.int32, device=dev))
-
-
-def _new_walk(B, N, L, dev) -> Walk:
-    return Walk(torch.empty((B,), dtype=torch.int32, device=dev),
-                torch.empty((B,), dtype=torch.int32, device=dev),
-                torch.empty((B, N), dtype=torch.int32, device=dev),
-                torch.empty((B, L), dtype=torch.int32, device=dev),
-                torch.zeros((B,), dtype=torch.int32, device=dev))
+    return _native().accept_walk(block_tokens, parent_off, parent_idx, top_tok, unmask_bits, out, stream)
 
 
 def spiffy_decide_walk_lazy_workspace(desc: DecideDesc) -> int:
@@ -442,32 +342,8 @@ def spiffy_decide_walk(logits, block_tokens, parent_off, parent_idx, mask_token_
     decision is evaluated only for the nodes the walk reaches
     (spiffy_decide_walk_lazy): the Decision then holds those nodes' entries and
     n_unmask = -1 everywhere else.  Returns (Decision, Walk)."""
-    desc = decide_desc(logits, block_tokens, mask_token_id, rule, top_s, threshold)
-    B, N, L = block_tokens.shape
-    dev = logits.device
-    decision = decision or _new_decision(B, N, L, dev)
-    walk = walk or _new_walk(B, N, L, dev)
-    if tuple(parent_off.shape) != (B, N + 1) or parent_idx.dim() != 2 or parent_idx.shape[0] != B:
-        raise ValueError("parent_off must be [B,N+1] and parent_idx [B,cap]")
-    need = spiffy_decide_walk_lazy_workspace(desc) if lazy else spiffy_unmask_decide_workspace(desc)
-    if workspace is None:
-        workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
-    entry = lib().spiffy_decide_walk_lazy if lazy else lib().spiffy_decide_walk
-    st = entry(
-        ctypes.byref(desc), _logits_ptr(logits), _dev(block_tokens, "block_tokens", torch.int32),
-        _dev(parent_off, "parent_off", torch.int32), _dev(parent_idx, "parent_idx", torch.int32),
-        int(parent_idx.shape[1]),
-        _dev(decision.conf, "conf", torch.float32), _dev(decision.top_tok, "top_tok", torch.int32),
-        _dev(decision.unmask_bits, "unmask_bits", torch.int64),
-        _dev(decision.n_unmask, "n_unmask", torch.int32),
-        _dev(decision.dev_status, "decide_status", torch.int32),
-        _dev(walk.accepted_node, "accepted_node", torch.int32),
-        _dev(walk.n_accepted, "n_accepted", torch.int32), _dev(walk.path, "path", torch.int32),
-        _dev(walk.next_block, "next_block", torch.int32),
-        _dev(walk.dev_status, "walk_status", torch.int32), _dev(workspace, "workspace"),
-        workspace.numel() * workspace.element_size(), _stream(stream))
-    _check(st, "spiffy_decide_walk_lazy" if lazy else "spiffy_decide_walk")
-    return decision, walk
+    return _native().decide_walk(logits, block_tokens, mask_token_id, rule, top_s, threshold, parent_off, parent_idx,
+                                 decision, walk, workspace, stream, lazy)
 
 
 def spiffy_stage_masked_rows(src_logits, dst_logits, tokens, mask_token_id: int, stream=None):
@@ -579,35 +455,5 @@ def spiffy_draft_blocks(logits, state, mask_token_id: int, graph: DraftGraph, bu
                         parent_cap: int = 0, out: Optional[Drafts] = None, workspace=None,
                         stream=None) -> Drafts:
     """Drafting and pruning.  logits [B,L,V] (rows may be a strided view), state [B,L] int32."""
-    B, L = state.shape
-    V = logits.shape[-1]
-    D = graph.n_formulas
-    cap = parent_cap or max(4, (budget + 1) * budget // 2)
-    row_stride = logits.stride(-2)
-    if B > 1 and logits.stride(0) != L * row_stride:
-        raise ValueError("logits rows must be equally spaced")
-    desc = DraftDesc(B, L, V, _dtype_code(logits), int(row_stride), int(mask_token_id), D, int(top_k),
-                     int(budget), int(cap))
-    dev = logits.device
-    if out is None:
-        out = Drafts(torch.empty((B, budget + 1, L), dtype=torch.int32, device=dev),
-                     torch.empty((B, budget), dtype=torch.int32, device=dev),
-                     torch.empty((B, D), dtype=torch.float32, device=dev),
-                     torch.empty((B, budget + 2), dtype=torch.int32, device=dev),
-                     torch.zeros((B, cap), dtype=torch.int32, device=dev),
-                     torch.zeros((B,), dtype=torch.int32, device=dev))
-    need = int(lib().spiffy_draft_blocks_workspace(ctypes.byref(desc)))
-    if workspace is None:
-        workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
-    i32 = torch.int32
-    st = lib().spiffy_draft_blocks(
-        ctypes.byref(desc), _logits_ptr(logits) if logits.dim() == 4 else logits.data_ptr(),
-        _dev(state, "state", i32), _dev(graph.formula_off, "formula_off", i32),
-        _dev(graph.formula_i, "formula_i", i32), _dev(graph.formula_j, "formula_j", i32),
-        _dev(graph.child_off, "child_off", i32), _dev(graph.child_idx, "child_idx", i32),
-        _dev(out.tokens, "tokens", i32), _dev(out.kept, "kept", i32),
-        _dev(out.score, "score", torch.float32), _dev(out.parent_off, "parent_off", i32),
-        _dev(out.parent_idx, "parent_idx", i32), _dev(out.dev_status, "dev_status", i32),
-        _dev(workspace, "workspace"), workspace.numel() * workspace.element_size(), _stream(stream))
-    _check(st, "spiffy_draft_blocks")
-    return out
+    return _native().draft_blocks(logits, state, mask_token_id, graph, budget, top_k, parent_cap, out, workspace,
+                                  stream)
