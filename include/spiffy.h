@@ -103,9 +103,11 @@ typedef enum { SPIFFY_RULE_TOPS = 0, SPIFFY_RULE_THRESHOLD = 1 } spiffy_rule;
 #define SPIFFY_FRESH_STATUS 0x100
 
 /* Attention kernel selection (spiffy_attn_desc.kernel). */
-#define SPIFFY_ATTN_AUTO 0   /* tensor-core kernel when the shape allows it   */
+#define SPIFFY_ATTN_AUTO 0   /* tensor-core kernel when the shape allows it: bf16,
+                                at most 128 query heads per kv head           */
 #define SPIFFY_ATTN_SIMT 1   /* fp32 CUDA-core kernel (any supported shape)   */
-#define SPIFFY_ATTN_TCGEN05 2 /* tcgen05/TMEM kernel or SPIFFY_EUNSUPPORTED   */
+#define SPIFFY_ATTN_TCGEN05 2 /* tcgen05/TMEM kernel of head_dim 128 or
+                                 SPIFFY_EUNSUPPORTED                          */
 /* Flag, OR-ed into spiffy_attn_desc.kernel: the next kernel of the stream may be
  * scheduled while this call's kernel still runs (it is launched as soon as every
  * thread block of this kernel has started; kernels that order themselves with

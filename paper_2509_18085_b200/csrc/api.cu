@@ -39,6 +39,8 @@ spiffy_status check_attn_desc(const spiffy_attn_desc* d) {
 
 bool use_tc(const spiffy_attn_desc& d) {
   if ((d.kernel & 0xff) == SPIFFY_ATTN_SIMT) return false;
+  // asked for by name, the tensor-core kernel is the one of head dimension 128
+  if ((d.kernel & 0xff) == SPIFFY_ATTN_TCGEN05 && d.head_dim != 128) return false;
   return attention_tc_supported(d);
 }
 
@@ -136,7 +138,7 @@ spiffy_status check_full_sequence(const spiffy_attn_desc* desc, int32_t suffix_l
   if (st != SPIFFY_OK) return st;
   if (suffix_len < 0) return SPIFFY_EINVAL;
   if (suffix_len > 1024) return SPIFFY_EUNSUPPORTED;
-  if (!use_tc(*desc)) return SPIFFY_EUNSUPPORTED;  // bf16, head dimension 128 only
+  if (!use_tc(*desc) || desc->head_dim != 128) return SPIFFY_EUNSUPPORTED;  // bf16, head dimension 128 only
   return SPIFFY_OK;
 }
 }  // namespace

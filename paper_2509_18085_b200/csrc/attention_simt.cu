@@ -1,7 +1,7 @@
 // Packed draft-graph attention (Sec. 4.3; mask of Fig. 3) on the fp32 CUDA
 // cores.  This is the kernel for fp32 inputs (tensor cores would need TF32,
-// whose 10-bit mantissa cannot hold a 1e-4 tolerance) and for shapes the
-// tcgen05 kernel does not take.  The mask is never materialised: a CTA works
+// whose 10-bit mantissa cannot hold a 1e-4 tolerance), and for bf16 where it is
+// asked for by name or more than 128 query heads share a kv head.  The mask is never materialised: a CTA works
 // on one (sequence, node, query head) and simply iterates over the context
 // keys followed by that node's own block keys.
 #include <math.h>

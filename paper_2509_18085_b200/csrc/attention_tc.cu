@@ -1,5 +1,5 @@
 // Packed draft-graph attention (Sec. 4.3; mask of Fig. 3) on the sm_100a tensor
-// cores: bf16 operands, head dimension 128.
+// cores: bf16 operands, head dimension 128 or 64.
 //
 // Work decomposition.  For one sequence b and one key/value head g, the query
 // rows are all (node n, position l, query head of the group) triples; they all
@@ -15,8 +15,9 @@
 //
 // Pipeline inside a CTA (320 threads):
 //   warp 0      TMA producer: Q once, then K and V tiles into two rings (seven
-//               32 KB tiles of shared memory in all); its first loads go out
-//               before the rest of the CTA has finished setting up
+//               32 KB tiles of shared memory in all, or fourteen of 16 KB at
+//               head dimension 64); its first loads go out before the rest of
+//               the CTA has finished setting up
 //   warp 1      allocates tensor memory; one lane issues tcgen05.mma:
 //               S = Q K^T (fp32 in TMEM, double buffered), O += P V
 //   warps 2-9   two softmax warpgroups, one thread per row each.  With one
@@ -35,6 +36,11 @@
 // slices store unnormalised partials (O, reference maximum, sum) that a second
 // kernel merges.
 //
+// Head dimension 64 halves every tile (one 64-column half instead of two) and the
+// products, not the exponentials: the softmax warps bound it.  3 sequences of 100
+// positions x 24 heads over 777 + 20 keys: 215 us on the CUDA cores, about 13 us
+// here.
+//
 // Every wait is bounded; a wait that gives up raises SPIFFY_DEV_TIMEOUT in the
 // caller's status word and the CTA winds down without touching its output.
 #include <math.h>
@@ -50,35 +56,35 @@ using namespace sm100;
 
 constexpr int BM = 128;       // rows of an M-tile (TMEM lanes)
 constexpr int BN = 128;       // keys per key tile
-constexpr int HD = 128;       // head dimension
-constexpr int kMaxStages = 3;  // most stages a K or V ring has
 constexpr int kThreads = 320;  // producer warp, MMA warp, two softmax warpgroups
 constexpr int kHalfBytes = BN * 128;           // one 64-column half of a tile: 128 rows x 128 B
-constexpr int kTileBytes = 2 * kHalfBytes;     // 32 KB
 constexpr uint32_t kTmemCols = 512;
 // S: 2 x 128 columns (P, as bf16 pairs, overwrites the first 64 columns of its S);
-// O: 2 x 128 columns, one accumulator per softmax warpgroup
+// O: 2 x 128 (or 64) columns, one accumulator per softmax warpgroup
 constexpr uint32_t kColS = 0, kColO = 256;
 constexpr float kRescaleLog2 = 8.0f;
-// bytes a CTA of a pair receives from its peer: 128 rows x 64 columns of partial O, and (max, sum) per row
-constexpr uint32_t kXchgBytes = BM * 64 * 4 + BM * 8;
 
 // NQ M-tiles per CTA: NQ Q tiles, a K ring of 3 stages and a V ring of 4 - NQ
-// stages: 7 tiles of 32 KB either way.
-template <int NQ>
+// stages, seven tiles of 32 KB either way; at head dimension 64 twice as many
+// tiles of half the size.  (The same amount for both: two CTAs must not share an
+// SM, each holds all of its tensor memory until it exits.)
+template <int NQ, int HD>
 struct Smem {
-  static constexpr int ks = 3, vs = 4 - NQ;
+  static constexpr int tile = BN * HD * 2;  // bytes
+  static constexpr int ks = HD == 128 ? 3 : 6, vs = 14 * 64 / HD - NQ - ks;
   static constexpr int q = 0;
-  static constexpr int k = q + NQ * kTileBytes;
-  static constexpr int v = k + ks * kTileBytes;
-  static constexpr int bars = v + vs * kTileBytes;
-  static constexpr int n_bars = 1 + 4 * kMaxStages + 2 + 2 + 2 + 2;
+  static constexpr int k = q + NQ * tile;
+  static constexpr int v = k + ks * tile;
+  static constexpr int bars = v + vs * tile;
+  static constexpr int n_bars = 1 + 2 * ks + 2 * vs + 2 + 2 + 2 + 2;
   static constexpr int tmem = bars + 8 * n_bars;
   static constexpr int abort_flag = tmem + 8;
   static constexpr int total = abort_flag + 8;
 };
-constexpr int kSmemBytes = Smem<1>::total + 1024;  // slack for 1024-byte alignment
-static_assert(Smem<1>::total == Smem<2>::total, "both layouts use the same amount");
+constexpr int kSmemBytes = Smem<1, 64>::total + 1024;  // slack for 1024-byte alignment
+static_assert(Smem<1, 64>::total >= Smem<2, 64>::total && Smem<1, 64>::total >= Smem<1, 128>::total &&
+                  Smem<1, 64>::total >= Smem<2, 128>::total && kSmemBytes <= 227 * 1024,
+              "one amount for all layouts");
 
 struct Params {
   int B, N, L, Hq, Hkv, group;
@@ -91,7 +97,7 @@ struct Params {
   int pair;  // the two splits are the two CTAs of a cluster and merge through shared memory
   float scale_log2;
   __nv_bfloat16* out;
-  float* part_o;   // [splits][B*Hkv][MT][128][128]
+  float* part_o;   // [splits][B*Hkv][MT][128][head dim]
   float* part_ml;  // [splits][B*Hkv][MT][128][2]
   int32_t* status;
   uint32_t spin_limit;  // polls of one mbarrier wait
@@ -189,7 +195,7 @@ __device__ __forceinline__ Window visible_window(const Params& p, int t, int kb_
 // NQ = 2: the CTA owns two neighbouring M-tiles, one per warpgroup, and every
 // K/V tile brought into shared memory serves both, which halves the L2-to-SM
 // traffic per flop.
-template <int NQ>
+template <int NQ, int HD>
 __global__ void __launch_bounds__(kThreads, 1)
 graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                           const __grid_constant__ CUtensorMap tm_kp,
@@ -201,8 +207,11 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  using SM = Smem<NQ>;
-  constexpr int KS = SM::ks, VS = SM::vs;
+  using SM = Smem<NQ, HD>;
+  constexpr int KS = SM::ks, VS = SM::vs, kTileBytes = SM::tile;
+  constexpr int kHalves = HD / 64;  // 64-column halves of a tile
+  // bytes a CTA of a pair receives from its peer: half the columns of a partial O, and (max, sum) per row
+  constexpr uint32_t kXchgBytes = BM * (HD / 2) * 4 + BM * 8;
   uint8_t* sq = smem + SM::q;
   uint8_t* sk = smem + SM::k;
   uint8_t* sv = smem + SM::v;
@@ -272,7 +281,7 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
     uint8_t* dst = (is_k ? sk : sv) + stage * kTileBytes;
     mbar_arrive_expect_tx(full, kTileBytes);
     tma_load_4d(dst, m, full, 0, g, key0, b);
-    tma_load_4d(dst + kHalfBytes, m, full, 64, g, key0, b);
+    if constexpr (kHalves == 2) tma_load_4d(dst + kHalfBytes, m, full, 64, g, key0, b);
     if (is_k) issued_k = j + 1; else issued_v = j + 1;
     return true;
   };
@@ -292,12 +301,13 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
     if (pair) mbar_arrive_expect_tx(xchg_full, kXchgBytes);  // what the peer will send in the epilogue
     cudaGridDependencySynchronize();
     if (T > 0) {
-      mbar_arrive_expect_tx(q_full, (uint32_t)NQ * 2u * rows_box * 128u);
+      mbar_arrive_expect_tx(q_full, (uint32_t)(NQ * kHalves) * rows_box * 128u);
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {  // an M-tile beyond the last one reads as zeros
         tma_load_4d(sq + q * kTileBytes, &tm_q, q_full, 0, g * p.group, nl0 + q * p.TNL, b);
-        tma_load_4d(sq + q * kTileBytes + kHalfBytes, &tm_q, q_full, 64, g * p.group,
-                    nl0 + q * p.TNL, b);
+        if constexpr (kHalves == 2)
+          tma_load_4d(sq + q * kTileBytes + kHalfBytes, &tm_q, q_full, 64, g * p.group,
+                      nl0 + q * p.TNL, b);
       }
       while (issued_k < T && produce(true, issued_k, false)) {}
     }
@@ -312,7 +322,7 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
   for (int i = rows_box * 8 + threadIdx.x; i < BM * 8; i += kThreads) {
     const uint4 z = make_uint4(0, 0, 0, 0);
 #pragma unroll
-    for (int h = 0; h < 2 * NQ; ++h) reinterpret_cast<uint4*>(sq + h * kHalfBytes)[i] = z;
+    for (int h = 0; h < kHalves * NQ; ++h) reinterpret_cast<uint4*>(sq + h * kHalfBytes)[i] = z;
   }
   fence_proxy_async_smem();
   if (warp == 1) tmem_alloc(tmem_slot, kTmemCols);
@@ -360,8 +370,11 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
       bool ok = mbar_wait(q_full, 0, abort_flag, p.spin_limit);
       // S = Q K^T of key tile j into S buffer `buf`, from Q tile `qt`
       auto issue_s = [&](int j, int buf, int qt) {
-        umma_ss_k128(tmem + kColS + (uint32_t)buf * BN, q_lo + (uint32_t)qt * (kTileBytes >> 4),
-                     k_lo + (uint32_t)(j % KS) * (kTileBytes >> 4), hi, idesc_s, 0u);
+        const uint32_t d = tmem + kColS + (uint32_t)buf * BN;
+        const uint32_t qa = q_lo + (uint32_t)qt * (kTileBytes >> 4);
+        const uint32_t kb = k_lo + (uint32_t)(j % KS) * (kTileBytes >> 4);
+        if constexpr (HD == 128) umma_ss_k128(d, qa, kb, hi, idesc_s, 0u);
+        else umma_ss_k64(d, qa, kb, hi, idesc_s, 0u);
         umma_commit(s_full + buf);
       };
       auto wait_k = [&](int j) {
@@ -619,20 +632,27 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
       const float w_a = has_a ? ex2(m_a - m_all) : 0.f;
       const float w_b = has_b ? ex2(m_b - m_all) : 0.f;
       const float l_all = w_a * l_a + w_b * l_b;
-      // 32 columns of this CTA's two accumulators, merged against m_all and scaled by f
-      auto merged = [&](int c0, float f, float (&o)[32]) {
-        uint32_t oa[32], ob[32];
-        tmem_ld_x32(tmem_addr(tmem, lane_base, kColO + c0), oa);
-        tmem_ld_x32(tmem_addr(tmem, lane_base, kColO + HD + c0), ob);
+      // W columns of this CTA's two accumulators, merged against m_all and scaled by f; a
+      // warpgroup handles a quarter of the columns at a time
+      constexpr int W = HD / 4;
+      auto merged = [&](int c0, float f, float (&o)[W]) {
+        uint32_t oa[W], ob[W];
+        if constexpr (W == 32) {
+          tmem_ld_x32(tmem_addr(tmem, lane_base, kColO + c0), oa);
+          tmem_ld_x32(tmem_addr(tmem, lane_base, kColO + HD + c0), ob);
+        } else {
+          tmem_ld_x16(tmem_addr(tmem, lane_base, kColO + c0), oa);
+          tmem_ld_x16(tmem_addr(tmem, lane_base, kColO + HD + c0), ob);
+        }
         const float f_a = w_a * f, f_b = w_b * f;
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
+        for (int c = 0; c < W; ++c)
           o[c] = (has_a ? __uint_as_float(oa[c]) * f_a : 0.f) +
                  (has_b ? __uint_as_float(ob[c]) * f_b : 0.f);
       };
-      auto store_bf16 = [&](__nv_bfloat16* at, const float (&o)[32]) {
+      auto store_bf16 = [&](__nv_bfloat16* at, const float (&o)[W]) {
 #pragma unroll
-        for (int c = 0; c < 32; c += 8) {
+        for (int c = 0; c < W; c += 8) {
           uint4 w;
           w.x = pack_bf16(o[c], o[c + 1]);
           w.y = pack_bf16(o[c + 2], o[c + 3]);
@@ -643,7 +663,7 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
       };
       if (pair) {
         // The other half of the key tiles went to the peer CTA of the cluster.  Each of the
-        // two finishes 64 of the 128 output columns: it sends its partial of the peer's
+        // two finishes half of the output columns: it sends its partial of the peer's
         // columns into the peer's shared memory (the Q tile and the first K stage, idle
         // since the last S) and merges what it gets.  Hand-over by mbarriers: xchg_ready =
         // "my buffers are free" (sent from the tile loop), xchg_full = "your partial has
@@ -654,18 +674,18 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
           tc_fence_after_sync();
           const uint32_t q_peer = map_to_cta(smem_u32(sq), peer);
           const uint32_t bar_peer = map_to_cta(smem_u32(xchg_full), peer);
-          float o[32];
-          merged(64 * (int)peer + 32 * wg, 1.0f, o);
+          float o[W];
+          merged(HD / 2 * (int)peer + W * wg, 1.0f, o);
 #pragma unroll
-          for (int k = 0; k < 8; ++k)  // 16-byte chunk (8 wg + k) of row r: chunk-major, rows contiguous
-            st_async_f4(q_peer + (uint32_t)(8 * wg + k) * 2048u + (uint32_t)r * 16u, bar_peer, o[4 * k],
+          for (int k = 0; k < W / 4; ++k)  // 16-byte chunk (W / 4 wg + k) of row r: chunk-major, rows contiguous
+            st_async_f4(q_peer + (uint32_t)(W / 4 * wg + k) * 2048u + (uint32_t)r * 16u, bar_peer, o[4 * k],
                         o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
           if (wg == 0) st_async_f2(map_to_cta(smem_u32(sk), peer) + (uint32_t)r * 8u, bar_peer, m_all, l_all);
         }
         cluster_arrive();  // phase 2: this thread issues nothing more towards the peer
         // this CTA's own share of its output columns, read while the peer's partial travels
-        float o[32];
-        merged(64 * (int)rank + 32 * wg, 1.0f, o);
+        float o[W];
+        merged(HD / 2 * (int)rank + W * wg, 1.0f, o);
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait_cluster(xchg_full, 0, abort_flag, p.spin_limit));
         if (ok) {
           const float2 mlp = *reinterpret_cast<const float2*>(sk + r * 8);
@@ -676,29 +696,29 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
           const float inv = 1.0f / (w_l * l_all + w_p * l_p);
           const float f_l = w_l * inv, f_p = w_p * inv;
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const float4 q4 = *reinterpret_cast<const float4*>(sq + (8 * wg + k) * 2048 + r * 16);
+          for (int k = 0; k < W / 4; ++k) {
+            const float4 q4 = *reinterpret_cast<const float4*>(sq + (W / 4 * wg + k) * 2048 + r * 16);
             o[4 * k] = o[4 * k] * f_l + (w_p != 0.f ? q4.x * f_p : 0.f);
             o[4 * k + 1] = o[4 * k + 1] * f_l + (w_p != 0.f ? q4.y * f_p : 0.f);
             o[4 * k + 2] = o[4 * k + 2] * f_l + (w_p != 0.f ? q4.z * f_p : 0.f);
             o[4 * k + 3] = o[4 * k + 3] * f_l + (w_p != 0.f ? q4.w * f_p : 0.f);
           }
-          if (row_ok) store_bf16(dst + 64 * (int)rank + 32 * wg, o);
+          if (row_ok) store_bf16(dst + HD / 2 * (int)rank + W * wg, o);
         }
       } else if (ok) {
         tc_fence_after_sync();
         const float inv = p.splits == 1 ? 1.0f / l_all : 1.0f;
         const int64_t tile = ((int64_t)split * gridDim.y + bg) * p.MT + mt;
         float* po = p.part_o + (tile * BM + r) * HD;
-        for (int c0 = wg * 64; c0 < wg * 64 + 64; c0 += 32) {  // each warpgroup stores one half
-          float o[32];
+        for (int c0 = wg * (HD / 2); c0 < (wg + 1) * (HD / 2); c0 += W) {  // each warpgroup stores one half
+          float o[W];
           merged(c0, inv, o);
           if (row_ok) {
             if (p.splits == 1) {
               store_bf16(dst + c0, o);
             } else {
 #pragma unroll
-              for (int c = 0; c < 32; c += 4)
+              for (int c = 0; c < W; c += 4)
                 *reinterpret_cast<float4*>(po + c0 + c) = make_float4(o[c], o[c + 1], o[c + 2], o[c + 3]);
             }
           }
@@ -731,12 +751,14 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
   if (threadIdx.x == 0 && *abort_flag && p.status) atomicOr(p.status, SPIFFY_DEV_TIMEOUT);
 }
 
-// Merge of the per-split partials: one warp per output row, lane = 4 columns.
+// Merge of the per-split partials: HD / 4 lanes per output row, lane = 4 columns.
+template <int HD>
 __global__ void __launch_bounds__(256)
 graph_attention_combine_kernel(const Params p) {
   cudaGridDependencySynchronize();  // the partials are visible
-  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);  // (b, nl, h)
-  const int lane = threadIdx.x & 31;
+  constexpr int kLanes = HD / 4;
+  const int64_t row = (int64_t)blockIdx.x * (256 / kLanes) + threadIdx.x / kLanes;  // (b, nl, h)
+  const int lane = threadIdx.x % kLanes;
   const int64_t rows = (int64_t)p.B * p.NL * p.Hq;
   if (row >= rows) return;
   const int h = (int)(row % p.Hq);
@@ -775,10 +797,12 @@ struct Plan {
   int nq;    // M-tiles per CTA
   int pair;  // key tiles split over the two CTAs of a cluster (no workspace, no merge kernel)
   int64_t tiles;  // B * Hkv * MT
+  int hd;
 };
 
 Plan make_plan(const spiffy_attn_desc& d, int ctx2_len) {
   Plan pl;
+  pl.hd = d.head_dim;
   pl.group = d.n_q_heads / d.n_kv_heads;
   pl.TNL = BM / pl.group;
   pl.NL = d.n_nodes * d.block_len;
@@ -809,7 +833,7 @@ Plan make_plan(const spiffy_attn_desc& d, int ctx2_len) {
 }  // namespace
 
 bool attention_tc_supported(const spiffy_attn_desc& d) {
-  if (d.dtype != SPIFFY_BF16 || d.head_dim != HD) return false;
+  if (d.dtype != SPIFFY_BF16 || (d.head_dim != 128 && d.head_dim != 64)) return false;
   const int group = d.n_q_heads / d.n_kv_heads;
   if (group > BM) return false;
   if ((int64_t)d.batch * d.n_kv_heads > 65535) return false;
@@ -819,7 +843,7 @@ bool attention_tc_supported(const spiffy_attn_desc& d) {
 size_t attention_tc_workspace_bytes(const spiffy_attn_desc& d, int ctx2_len) {
   const Plan pl = make_plan(d, ctx2_len);
   if (pl.splits == 1 || pl.pair) return 0;
-  return (size_t)pl.splits * pl.tiles * BM * (HD + 2) * sizeof(float);
+  return (size_t)pl.splits * pl.tiles * BM * (pl.hd + 2) * sizeof(float);
 }
 
 spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const void* q, const AttnContext& ctx,
@@ -827,19 +851,23 @@ spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const void* q, cons
                                   int32_t* dev_status, void* ws, cudaStream_t stream) {
   const Plan pl = make_plan(d, ctx2.len);
   CUtensorMap tm_q, tm_kp, tm_vp, tm_kp2, tm_vp2, tm_kb, tm_vb;
-  bool ok = make_map(&tm_q, q, d.n_q_heads, pl.NL, d.batch, pl.group, pl.TNL);
-  ok = ok && make_map(&tm_kb, kb, d.n_kv_heads, pl.NL, d.batch, 1, BN);
-  ok = ok && make_map(&tm_vb, vb, d.n_kv_heads, pl.NL, d.batch, 1, BN);
+  bool ok = make_map(&tm_q, q, d.n_q_heads, pl.NL, d.batch, pl.group, pl.TNL, 0, pl.hd);
+  ok = ok && make_map(&tm_kb, kb, d.n_kv_heads, pl.NL, d.batch, 1, BN, 0, pl.hd);
+  ok = ok && make_map(&tm_vb, vb, d.n_kv_heads, pl.NL, d.batch, 1, BN, 0, pl.hd);
   if (ctx.len > 0) {
-    ok = ok && make_map(&tm_kp, ctx.k, d.n_kv_heads, ctx.len, d.batch, 1, BN, ctx.batch_stride_rows);
-    ok = ok && make_map(&tm_vp, ctx.v, d.n_kv_heads, ctx.len, d.batch, 1, BN, ctx.batch_stride_rows);
+    ok = ok && make_map(&tm_kp, ctx.k, d.n_kv_heads, ctx.len, d.batch, 1, BN, ctx.batch_stride_rows,
+                        pl.hd);
+    ok = ok && make_map(&tm_vp, ctx.v, d.n_kv_heads, ctx.len, d.batch, 1, BN, ctx.batch_stride_rows,
+                        pl.hd);
   } else {  // never dereferenced: the segment has no tile
     tm_kp = tm_kb;
     tm_vp = tm_vb;
   }
   if (ctx2.len > 0) {
-    ok = ok && make_map(&tm_kp2, ctx2.k, d.n_kv_heads, ctx2.len, d.batch, 1, BN, ctx2.batch_stride_rows);
-    ok = ok && make_map(&tm_vp2, ctx2.v, d.n_kv_heads, ctx2.len, d.batch, 1, BN, ctx2.batch_stride_rows);
+    ok = ok && make_map(&tm_kp2, ctx2.k, d.n_kv_heads, ctx2.len, d.batch, 1, BN, ctx2.batch_stride_rows,
+                        pl.hd);
+    ok = ok && make_map(&tm_vp2, ctx2.v, d.n_kv_heads, ctx2.len, d.batch, 1, BN, ctx2.batch_stride_rows,
+                        pl.hd);
   } else {
     tm_kp2 = tm_kb;
     tm_vp2 = tm_vb;
@@ -855,15 +883,16 @@ spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const void* q, cons
   p.scale_log2 = scale * kLog2e;
   p.out = static_cast<__nv_bfloat16*>(out);
   p.part_o = static_cast<float*>(ws);
-  p.part_ml = p.part_o ? p.part_o + (size_t)pl.splits * pl.tiles * BM * HD : nullptr;
+  p.part_ml = p.part_o ? p.part_o + (size_t)pl.splits * pl.tiles * BM * pl.hd : nullptr;
   p.status = dev_status;
   p.spin_limit = mbar_poll_limit();
   p.early_trigger = (d.kernel & SPIFFY_ATTN_EARLY_DEPENDENTS) ? 1 : 0;
 
-  static std::atomic<bool> smem_allowed[2][64];
+  static std::atomic<bool> smem_allowed[4][64];
   const dim3 grid((pl.MT + pl.nq - 1) / pl.nq, d.batch * d.n_kv_heads, pl.splits);
-  auto kern = pl.nq == 2 ? graph_attention_tc_kernel<2> : graph_attention_tc_kernel<1>;
-  if (!allow_smem(kern, kSmemBytes, smem_allowed[pl.nq - 1])) return SPIFFY_ECUDA;
+  auto kern = pl.hd == 128 ? (pl.nq == 2 ? graph_attention_tc_kernel<2, 128> : graph_attention_tc_kernel<1, 128>)
+                           : (pl.nq == 2 ? graph_attention_tc_kernel<2, 64> : graph_attention_tc_kernel<1, 64>);
+  if (!allow_smem(kern, kSmemBytes, smem_allowed[(pl.hd == 128 ? 0 : 2) + pl.nq - 1])) return SPIFFY_ECUDA;
   {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -885,8 +914,10 @@ spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const void* q, cons
   count_launch();
   if (pl.splits > 1 && !pl.pair) {
     const int64_t rows = (int64_t)d.batch * pl.NL * d.n_q_heads;
-    if (launch_pdl(graph_attention_combine_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256),
-                   (size_t)0, stream, p) != cudaSuccess)
+    const int per_cta = 256 / (pl.hd / 4);
+    auto combine = pl.hd == 128 ? graph_attention_combine_kernel<128> : graph_attention_combine_kernel<64>;
+    if (launch_pdl(combine, dim3((unsigned)((rows + per_cta - 1) / per_cta)), dim3(256), (size_t)0, stream, p) !=
+        cudaSuccess)
       return SPIFFY_ECUDA;
     count_launch();
   }
