@@ -133,7 +133,8 @@ typedef struct {
   int32_t kernel;     /* SPIFFY_ATTN_AUTO/SIMT/TCGEN05, | SPIFFY_ATTN_EARLY_DEPENDENTS */
 } spiffy_attn_desc;
 
-/* Bytes of scratch spiffy_graph_attention needs for this shape (may be 0). */
+/* Bytes of scratch spiffy_graph_attention needs for this shape: 0 for every shape
+ * of this version (key tiles split over CTAs are merged through shared memory). */
 size_t spiffy_graph_attention_workspace(const spiffy_attn_desc* desc);
 
 /*
@@ -172,8 +173,7 @@ spiffy_status spiffy_graph_attention(const spiffy_attn_desc* desc,
  *   suffix_len S in [0, 1024]; 0 makes this spiffy_graph_attention
  *   q_nodes, out_nodes   [B][N][L][Hq][d]     q_suffix, out_suffix [B][S][Hq][d]
  *   k/v_prefix [B][P][Hkv][d]   k/v_suffix [B][S][Hkv][d]   k/v_block [B][N][L][Hkv][d]
- * dev_status, stream and error behaviour as in spiffy_graph_attention; the
- * workspace (spiffy_full_sequence_attention_workspace) serves both launches.
+ * dev_status, workspace, stream and error behaviour as in spiffy_graph_attention.
  */
 size_t spiffy_full_sequence_attention_workspace(const spiffy_attn_desc* desc, int32_t suffix_len);
 spiffy_status spiffy_full_sequence_attention(const spiffy_attn_desc* desc, int32_t suffix_len,

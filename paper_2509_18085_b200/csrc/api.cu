@@ -93,8 +93,8 @@ using namespace spiffy;
 extern "C" {
 
 size_t spiffy_graph_attention_workspace(const spiffy_attn_desc* desc) {
-  if (check_attn_desc(desc) != SPIFFY_OK) return 0;
-  return use_tc(*desc) ? attention_tc_workspace_bytes(*desc, 0) : 0;
+  (void)desc;  // key tiles split over CTAs are merged through shared memory
+  return 0;
 }
 
 spiffy_status spiffy_graph_attention(const spiffy_attn_desc* desc, const void* q,
@@ -103,6 +103,8 @@ spiffy_status spiffy_graph_attention(const spiffy_attn_desc* desc, const void* q
                                      void* out, int32_t* dev_status,
                                      void* workspace, size_t workspace_bytes,
                                      void* cuda_stream) {
+  (void)workspace;
+  (void)workspace_bytes;
   const spiffy_status st = check_attn_desc(desc);
   if (st != SPIFFY_OK) return st;
   const spiffy_attn_desc d = *desc;
@@ -113,12 +115,9 @@ spiffy_status spiffy_graph_attention(const spiffy_attn_desc* desc, const void* q
     return SPIFFY_EINVAL;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   if (use_tc(d)) {
-    const size_t need = attention_tc_workspace_bytes(d, 0);
-    if (need > 0 && (!workspace || workspace_bytes < need || !aligned16(workspace)))
-      return SPIFFY_EWORKSPACE;
     const AttnContext ctx = {k_prefix, v_prefix, d.prefix_len, 0};
     const AttnContext none = {nullptr, nullptr, 0, 0};
-    return launch_attention_tc(d, q, ctx, none, k_block, v_block, out, dev_status, workspace, stream);
+    return launch_attention_tc(d, q, ctx, none, k_block, v_block, out, dev_status, stream);
   }
   if ((d.kernel & 0xff) == SPIFFY_ATTN_TCGEN05) return SPIFFY_EUNSUPPORTED;
   if (d.block_len > 64) return SPIFFY_EUNSUPPORTED;  // the CUDA-core kernel keeps a block's rows in registers
@@ -144,10 +143,9 @@ spiffy_status check_full_sequence(const spiffy_attn_desc* desc, int32_t suffix_l
 }  // namespace
 
 size_t spiffy_full_sequence_attention_workspace(const spiffy_attn_desc* desc, int32_t suffix_len) {
-  if (check_full_sequence(desc, suffix_len) != SPIFFY_OK) return 0;
-  const size_t nodes = attention_tc_workspace_bytes(*desc, suffix_len);
-  const size_t suffix = suffix_len > 0 ? attention_tc_workspace_bytes(suffix_desc(*desc, suffix_len), desc->block_len) : 0;
-  return nodes > suffix ? nodes : suffix;
+  (void)desc;
+  (void)suffix_len;
+  return 0;
 }
 
 spiffy_status spiffy_full_sequence_attention(const spiffy_attn_desc* desc, int32_t suffix_len,
@@ -166,20 +164,18 @@ spiffy_status spiffy_full_sequence_attention(const spiffy_attn_desc* desc, int32
   const void* all[] = {q_nodes, q_suffix, k_prefix, v_prefix, k_suffix, v_suffix, k_block, v_block, out_nodes, out_suffix};
   for (const void* ptr : all)
     if (!aligned16(ptr)) return SPIFFY_EINVAL;
-  const size_t need = spiffy_full_sequence_attention_workspace(desc, suffix_len);
-  if (need > 0 && (!workspace || workspace_bytes < need || !aligned16(workspace))) return SPIFFY_EWORKSPACE;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   const AttnContext prefix = {k_prefix, v_prefix, d.prefix_len, 0};
   // nodes: context = [prefix ; suffix]; every node's own block as always
   const AttnContext suffix = {k_suffix, v_suffix, suffix_len, 0};
   spiffy_status rc = launch_attention_tc(d, q_nodes, prefix, suffix, k_block, v_block, out_nodes, dev_status,
-                                         workspace, stream);
+                                         stream);
   if (rc != SPIFFY_OK || suffix_len == 0) return rc;
   // suffix rows: one node whose block is the suffix; context = [prefix ; the true block], the
   // latter being node 0 of every sequence's blocks (sequences N * L rows apart)
   const AttnContext true_block = {k_block, v_block, d.block_len, (int64_t)d.n_nodes * d.block_len};
   return launch_attention_tc(suffix_desc(d, suffix_len), q_suffix, prefix, true_block, k_suffix, v_suffix,
-                             out_suffix, dev_status, workspace, stream);
+                             out_suffix, dev_status, stream);
 }
 
 size_t spiffy_unmask_decide_workspace(const spiffy_decide_desc* desc) {

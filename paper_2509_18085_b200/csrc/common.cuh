@@ -49,6 +49,16 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
   return v;
 }
 
+// Stores to global memory that order nothing else: a store through a pointer whose
+// address space the compiler cannot tell would hold up the shared-memory loads of
+// the next turn of a loop.
+__device__ __forceinline__ void st_global(void* p, uint2 v) {
+  asm volatile("st.global.v2.u32 [%0], {%1, %2};" ::"l"(p), "r"(v.x), "r"(v.y));
+}
+__device__ __forceinline__ void st_global(void* p, uint4 v) {
+  asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
+}
+
 // Every launch of the library goes through this counter (spiffy_launch_count).
 void count_launch(int n = 1);
 
@@ -139,7 +149,7 @@ spiffy_status launch_draft(const spiffy_draft_desc& d, const void* logits, const
                            bool fresh,
                             cudaStream_t stream);
 
-// tcgen05 path: shape support query, workspace and launch.  The cached context
+// tcgen05 path: shape support query and launch.  The cached context
 // comes as up to two segments of keys/values, [B][len][Hkv][d] each, whose
 // sequences may lie `batch_stride_rows` rows apart (0: densely packed).
 struct AttnContext {
@@ -149,10 +159,9 @@ struct AttnContext {
   int64_t batch_stride_rows;
 };
 bool attention_tc_supported(const spiffy_attn_desc& d);
-size_t attention_tc_workspace_bytes(const spiffy_attn_desc& d, int ctx2_len);
 spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const void* q, const AttnContext& ctx,
                                   const AttnContext& ctx2, const void* kb, const void* vb, void* out,
-                                  int32_t* dev_status, void* ws, cudaStream_t stream);
+                                  int32_t* dev_status, cudaStream_t stream);
 
 // Launch with programmatic stream serialisation: the kernel may be scheduled
 // while its predecessor in the stream is still draining.  Every kernel launched

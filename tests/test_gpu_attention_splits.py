@@ -1,0 +1,47 @@
+"""How the tensor-core attention kernel shares out its key tiles: one unit in all,
+odd and even numbers of them between the two softmax warpgroups, clusters of 2, 4
+and 8 CTAs with as few as one key tile each, two M-tiles per CTA."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2509_18085_b200 import spiffy
+from paper_2509_18085_b200 import workloads as W
+import gpu_util as G
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,N,L,P,Hq,Hkv", [
+    (1, 2, 16, 0, 2, 2),          # one unit: the second warpgroup has none
+    (1, 4, 32, 100, 4, 4),        # two units
+    (1, 4, 32, 128 * 2, 64, 64),  # three
+    (1, 1, 7, 128 * 6, 2, 1),     # a cluster of 8 over seven tiles is not taken, 4 or 2 are
+    (1, 1, 7, 128 * 7, 2, 1), (1, 1, 7, 128 * 7 + 1, 2, 1),  # one tile each and one more
+    (1, 6, 32, 2562, 8, 1), (1, 2, 32, 1746, 28, 4),          # clusters of 8
+    (1, 4, 32, 900, 30, 30),      # clusters of 4
+    (1, 7, 32, 777, 32, 32),      # clusters of 2
+    (2, 9, 32, 500, 40, 40),      # two M-tiles per CTA, an odd number of M-tiles
+    (4, 32, 32, 140, 16, 8)])
+def test_parity(B, N, L, P, Hq, Hkv):
+    cfg = W.Config("splits", B, N, L, P, Hq, Hkv, 128, "bf16", 16, 0)
+    w = W.make(cfg, 11 + P, decision=False)
+    got = G.gpu_attention(w, spiffy.ATTN_TCGEN05)
+    want = oracle.graph_attention(w.q, w.k_prefix, w.v_prefix, w.k_block, w.v_block)
+    assert np.max(np.abs(got - want)) <= G.TOL["bf16"]
+    assert np.sqrt(np.mean((got - want) ** 2)) < 4e-3
+    assert np.array_equal(got, G.gpu_attention(w, spiffy.ATTN_TCGEN05))
+
+
+def test_late_maximum_in_another_slice():
+    """The largest scores sit in the last slice of a cluster, and in tiles of one
+    warpgroup only: partials with very different reference maxima are merged."""
+    cfg = W.Config("splits", 1, 2, 16, 128 * 16, 2, 1, 128, "bf16", 16, 0)
+    w = W.make(cfg, 5, decision=False)
+    w.q *= 6.0
+    w.k_prefix[:, 128 * 14:128 * 15] *= 3.0
+    for a in ("q", "k_prefix"):
+        setattr(w, a, W.round_to(getattr(w, a), "bf16"))
+    got = G.gpu_attention(w, spiffy.ATTN_TCGEN05)
+    want = oracle.graph_attention(w.q, w.k_prefix, w.v_prefix, w.k_block, w.v_block)
+    assert np.all(np.isfinite(got)) and np.max(np.abs(got - want)) <= G.TOL["bf16"]
