@@ -164,9 +164,10 @@ spiffy_status spiffy_graph_attention(const spiffy_attn_desc* desc,
  * and the S trailing, still fully masked positions attend to the whole true
  * sequence -- prefix, true block, suffix --, every draft block to the prefix, the
  * suffix and itself (every block of the true sequence except the one it is a
- * draft of).  Two launches of the tensor-core kernel, no copy: the nodes with
- * the context given as two segments [prefix ; suffix], then the suffix rows as
- * one node whose block is the suffix and whose context is [prefix ; true block].
+ * draft of).  One launch of the tensor-core kernel on two problems, no copy: the
+ * nodes with the context given as two segments [prefix ; suffix], and the suffix
+ * rows as one node whose block is the suffix and whose context is [prefix ; true
+ * block].
  *
  *   desc      batch, n_nodes, block_len, prefix_len, heads, head_dim, scale of the
  *             nodes' call; dtype bf16 and head_dim 128 (else SPIFFY_EUNSUPPORTED)

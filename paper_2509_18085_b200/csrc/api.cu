@@ -115,9 +115,8 @@ spiffy_status spiffy_graph_attention(const spiffy_attn_desc* desc, const void* q
     return SPIFFY_EINVAL;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   if (use_tc(d)) {
-    const AttnContext ctx = {k_prefix, v_prefix, d.prefix_len, 0};
-    const AttnContext none = {nullptr, nullptr, 0, 0};
-    return launch_attention_tc(d, q, ctx, none, k_block, v_block, out, dev_status, stream);
+    const AttnProblem a = {q, {k_prefix, v_prefix, d.prefix_len, 0}, {nullptr, nullptr, 0, 0}, k_block, v_block, out};
+    return launch_attention_tc(d, a, dev_status, stream);
   }
   if ((d.kernel & 0xff) == SPIFFY_ATTN_TCGEN05) return SPIFFY_EUNSUPPORTED;
   if (d.block_len > 64) return SPIFFY_EUNSUPPORTED;  // the CUDA-core kernel keeps a block's rows in registers
@@ -125,7 +124,7 @@ spiffy_status spiffy_graph_attention(const spiffy_attn_desc* desc, const void* q
 }
 
 namespace {
-// The second launch of the full-sequence call: the suffix rows as one node whose block is the suffix.
+// The second problem of the full-sequence call: the suffix rows as one node whose block is the suffix.
 spiffy_attn_desc suffix_desc(const spiffy_attn_desc& d, int32_t suffix_len) {
   spiffy_attn_desc s = d;
   s.n_nodes = 1;
@@ -167,15 +166,13 @@ spiffy_status spiffy_full_sequence_attention(const spiffy_attn_desc* desc, int32
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   const AttnContext prefix = {k_prefix, v_prefix, d.prefix_len, 0};
   // nodes: context = [prefix ; suffix]; every node's own block as always
-  const AttnContext suffix = {k_suffix, v_suffix, suffix_len, 0};
-  spiffy_status rc = launch_attention_tc(d, q_nodes, prefix, suffix, k_block, v_block, out_nodes, dev_status,
-                                         stream);
-  if (rc != SPIFFY_OK || suffix_len == 0) return rc;
+  const AttnProblem nodes = {q_nodes, prefix, {k_suffix, v_suffix, suffix_len, 0}, k_block, v_block, out_nodes};
+  if (suffix_len == 0) return launch_attention_tc(d, nodes, dev_status, stream);
   // suffix rows: one node whose block is the suffix; context = [prefix ; the true block], the
   // latter being node 0 of every sequence's blocks (sequences N * L rows apart)
-  const AttnContext true_block = {k_block, v_block, d.block_len, (int64_t)d.n_nodes * d.block_len};
-  return launch_attention_tc(suffix_desc(d, suffix_len), q_suffix, prefix, true_block, k_suffix, v_suffix,
-                             out_suffix, dev_status, stream);
+  const AttnProblem suffix = {q_suffix, prefix, {k_block, v_block, d.block_len, (int64_t)d.n_nodes * d.block_len},
+                              k_suffix, v_suffix, out_suffix};
+  return launch_attention_tc_dual(d, nodes, suffix_desc(d, suffix_len), suffix, dev_status, stream);
 }
 
 size_t spiffy_unmask_decide_workspace(const spiffy_decide_desc* desc) {

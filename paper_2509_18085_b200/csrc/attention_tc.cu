@@ -122,6 +122,19 @@ struct Params {
   int early_trigger;    // let the next kernel of the stream begin its set-up while this one runs
 };
 
+// The operands of one attention problem: Q, two context segments, block keys.
+struct Maps {
+  CUtensorMap q, kp, vp, kp2, vp2, kb, vb;
+};
+// One launch runs one problem, or two side by side (the nodes and the trailing rows of a
+// full-sequence model): the CTAs from x_split on along grid.x work on the second.
+template <int NP>
+struct Problems {
+  Maps maps[NP];
+  Params p[NP];
+  int x_split;
+};
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
@@ -205,15 +218,9 @@ __device__ __forceinline__ Window visible_window(const Params& p, int t, int kb_
 // u >> 1.  Every K/V tile brought into shared memory serves both, which halves the
 // L2-to-SM traffic per flop.
 // Unit u belongs to warpgroup u & 1 and to accumulator u & 1 either way.
-template <int NQ, int HD>
+template <int NQ, int HD, int NP>
 __global__ void __launch_bounds__(kThreads, 1)
-graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
-                          const __grid_constant__ CUtensorMap tm_kp,
-                          const __grid_constant__ CUtensorMap tm_vp,
-                          const __grid_constant__ CUtensorMap tm_kp2,
-                          const __grid_constant__ CUtensorMap tm_vp2,
-                          const __grid_constant__ CUtensorMap tm_kb,
-                          const __grid_constant__ CUtensorMap tm_vb, const Params p) {
+graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
   extern __shared__ uint8_t smem_raw[];
   // an offset, not a rounded address: the compiler still knows that this is shared memory
   uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);
@@ -242,12 +249,15 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
   int* rows = reinterpret_cast<int*>(smem + SM::rows);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int which = NP == 2 && (int)blockIdx.x >= problems.x_split ? 1 : 0;
+  const Maps& maps = problems.maps[which];
+  const Params& p = problems.p[which];
   if (threadIdx.x == 0) {
-    prefetch_tensormap(&tm_q);  // the descriptors are kernel parameters
-    prefetch_tensormap(p.TP1 > 0 ? &tm_kp : (p.TP > 0 ? &tm_kp2 : &tm_kb));
-    prefetch_tensormap(p.TP1 > 0 ? &tm_vp : (p.TP > 0 ? &tm_vp2 : &tm_vb));
+    prefetch_tensormap(&maps.q);  // the descriptors are kernel parameters
+    prefetch_tensormap(p.TP1 > 0 ? &maps.kp : (p.TP > 0 ? &maps.kp2 : &maps.kb));
+    prefetch_tensormap(p.TP1 > 0 ? &maps.vp : (p.TP > 0 ? &maps.vp2 : &maps.vb));
   }
-  const int mt = blockIdx.x * NQ;  // first M-tile of this CTA
+  const int mt = ((int)blockIdx.x - (which ? problems.x_split : 0)) * NQ;  // first M-tile of this CTA
   const int bg = blockIdx.y;
   const int b = bg / p.Hkv, g = bg % p.Hkv;
   const int cs = NQ == 1 ? p.cs : 1;
@@ -279,8 +289,8 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
     const int t = t_begin + j;
     // key tiles in order: first context segment, second context segment, block keys
     const int seg = t < p.TP1 ? 0 : (t < p.TP ? 1 : 2);
-    const CUtensorMap* m = is_k ? (seg == 0 ? &tm_kp : seg == 1 ? &tm_kp2 : &tm_kb)
-                                : (seg == 0 ? &tm_vp : seg == 1 ? &tm_vp2 : &tm_vb);
+    const CUtensorMap* m = is_k ? (seg == 0 ? &maps.kp : seg == 1 ? &maps.kp2 : &maps.kb)
+                                : (seg == 0 ? &maps.vp : seg == 1 ? &maps.vp2 : &maps.vb);
     const int key0 = seg == 0 ? t * BN : seg == 1 ? (t - p.TP1) * BN : kb_start + (t - p.TP) * BN;
     uint8_t* dst = (is_k ? sk : sv) + stage * kTileBytes;
     mbar_arrive_expect_tx(full, kTileBytes);
@@ -311,9 +321,9 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
     mbar_arrive_expect_tx(q_full, (uint32_t)(NQ * kHalves) * rows_box * 128u);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {  // an M-tile beyond the last one reads as zeros
-      tma_load_4d(sq + q * kTileBytes, &tm_q, q_full, 0, g * p.group, nl0 + q * p.TNL, b);
+      tma_load_4d(sq + q * kTileBytes, &maps.q, q_full, 0, g * p.group, nl0 + q * p.TNL, b);
       if constexpr (kHalves == 2)
-        tma_load_4d(sq + q * kTileBytes + kHalfBytes, &tm_q, q_full, 64, g * p.group,
+        tma_load_4d(sq + q * kTileBytes + kHalfBytes, &maps.q, q_full, 64, g * p.group,
                     nl0 + q * p.TNL, b);
     }
     produce(true, 0);
@@ -707,16 +717,37 @@ graph_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
 }
 
 // ------------------------------------------------------------------ host ----
+// What one problem's descriptor and segment lengths amount to.
+struct Shape {
+  int group, TNL, NL, MT, TP1, TP;
+  int T;  // key tiles of an M-tile, at least
+};
+Shape shape_of(const spiffy_attn_desc& d, const AttnContext& ctx, const AttnContext& ctx2) {
+  Shape s;
+  s.group = d.n_q_heads / d.n_kv_heads;
+  s.TNL = BM / s.group;
+  s.NL = d.n_nodes * d.block_len;
+  s.MT = (s.NL + s.TNL - 1) / s.TNL;
+  s.TP1 = (ctx.len + BN - 1) / BN;
+  s.TP = s.TP1 + (ctx2.len + BN - 1) / BN;
+  s.T = s.TP + (d.block_len + BN - 1) / BN;
+  return s;
+}
+
 struct Plan {
-  int group, TNL, NL, MT, TP1, TP, hd;
   int nq;  // M-tiles per CTA
   int cs;  // CTAs of a cluster that share an M-tile's key tiles (nq = 1)
 };
 
-using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, Params);
-Kernel kernel_of(int hd, int nq) {
-  return hd == 128 ? (nq == 2 ? graph_attention_tc_kernel<2, 128> : graph_attention_tc_kernel<1, 128>)
-                   : (nq == 2 ? graph_attention_tc_kernel<2, 64> : graph_attention_tc_kernel<1, 64>);
+template <int NP>
+using Kernel = void (*)(Problems<NP>);
+template <int NP>
+Kernel<NP> kernel_of(int hd, int nq) {
+  if constexpr (NP == 2)  // the full-sequence call takes head dimension 128 only
+    return nq == 2 ? graph_attention_tc_kernel<2, 128, 2> : graph_attention_tc_kernel<1, 128, 2>;
+  else
+    return hd == 128 ? (nq == 2 ? graph_attention_tc_kernel<2, 128, 1> : graph_attention_tc_kernel<1, 128, 1>)
+                     : (nq == 2 ? graph_attention_tc_kernel<2, 64, 1> : graph_attention_tc_kernel<1, 64, 1>);
 }
 
 // Clusters of `cs` CTAs that the current device can hold at once (a GPU cluster's SMs are no
@@ -738,7 +769,7 @@ int resident_clusters(int hd, int cs) {
     attr[0].val.clusterDim.z = (unsigned)cs;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel_of(hd, 1), &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, kernel_of<1>(hd, 1), &cfg) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
@@ -753,88 +784,90 @@ int resident_clusters(int hd, int cs) {
 // round of CTAs (148, each holds its SM) takes 7 us plus 0.85 us per key tile with one
 // M-tile, 1.6 us with two; handing the partials around a cluster costs 2 us and a
 // little more in larger clusters, so that a second CTA pays from about six key tiles.
-Plan make_plan(const spiffy_attn_desc& d, int ctx2_len) {
-  Plan pl;
-  pl.hd = d.head_dim;
-  pl.group = d.n_q_heads / d.n_kv_heads;
-  pl.TNL = BM / pl.group;
-  pl.NL = d.n_nodes * d.block_len;
-  pl.MT = (pl.NL + pl.TNL - 1) / pl.TNL;
-  pl.TP1 = (d.prefix_len + BN - 1) / BN;
-  pl.TP = pl.TP1 + (ctx2_len + BN - 1) / BN;
+// `tiles` counts the M-tiles of all problems of the launch, `pairs` the CTAs that take two
+// of them, T is the key tiles of the longer problem.
+Plan make_plan(int64_t tiles, int64_t pairs, int T, int hd) {
   constexpr int kSms = 148;
-  const int64_t bg = (int64_t)d.batch * d.n_kv_heads;
-  const int T = pl.TP + 1;  // key tiles of an M-tile, at least
   auto rounds = [](int64_t ctas) { return (float)((ctas + kSms - 1) / kSms); };
-  float best = rounds(bg * ((pl.MT + 1) / 2)) * (7.0f + 1.6f * (float)T);
-  pl.nq = 2;
-  pl.cs = 1;
+  Plan pl = {2, 1};
+  float best = rounds(pairs) * (7.0f + 1.6f * (float)T);
   for (int cs = 1; cs <= 8 && cs <= T; cs *= 2) {
     // clusters only where all of them run at once
-    if (cs > 1 && (bg * pl.MT * cs > kSms || bg * pl.MT > resident_clusters(pl.hd, cs))) continue;
+    if (cs > 1 && (tiles * cs > kSms || tiles > resident_clusters(hd, cs))) continue;
     const float exchange = cs == 1 ? 0.f : 1.9f + 0.07f * (float)cs;
-    const float cost = rounds(bg * pl.MT * cs) * (7.0f + exchange + 0.85f * (float)((T + cs - 1) / cs));
+    const float cost = rounds(tiles * cs) * (7.0f + exchange + 0.85f * (float)((T + cs - 1) / cs));
     if (cost < best) {
       best = cost;
-      pl.nq = 1;
-      pl.cs = cs;
+      pl = {1, cs};
     }
   }
   return pl;
 }
 
-}  // namespace
-
-bool attention_tc_supported(const spiffy_attn_desc& d) {
-  if (d.dtype != SPIFFY_BF16 || (d.head_dim != 128 && d.head_dim != 64)) return false;
-  const int group = d.n_q_heads / d.n_kv_heads;
-  if (group > BM) return false;
-  if ((int64_t)d.batch * d.n_kv_heads > 65535) return false;
-  return true;
+bool make_problem(const spiffy_attn_desc& d, const Shape& sh, const AttnProblem& a, Maps* m, Params* p, int cs,
+                  int32_t* dev_status) {
+  const int hd = d.head_dim;
+  bool ok = make_map(&m->q, a.q, d.n_q_heads, sh.NL, d.batch, sh.group, sh.TNL, 0, hd);
+  ok = ok && make_map(&m->kb, a.kb, d.n_kv_heads, sh.NL, d.batch, 1, BN, 0, hd);
+  ok = ok && make_map(&m->vb, a.vb, d.n_kv_heads, sh.NL, d.batch, 1, BN, 0, hd);
+  if (a.ctx.len > 0) {
+    ok = ok && make_map(&m->kp, a.ctx.k, d.n_kv_heads, a.ctx.len, d.batch, 1, BN, a.ctx.batch_stride_rows, hd);
+    ok = ok && make_map(&m->vp, a.ctx.v, d.n_kv_heads, a.ctx.len, d.batch, 1, BN, a.ctx.batch_stride_rows, hd);
+  } else {  // never dereferenced: the segment has no tile
+    m->kp = m->kb;
+    m->vp = m->vb;
+  }
+  if (a.ctx2.len > 0) {
+    ok = ok && make_map(&m->kp2, a.ctx2.k, d.n_kv_heads, a.ctx2.len, d.batch, 1, BN, a.ctx2.batch_stride_rows, hd);
+    ok = ok && make_map(&m->vp2, a.ctx2.v, d.n_kv_heads, a.ctx2.len, d.batch, 1, BN, a.ctx2.batch_stride_rows, hd);
+  } else {
+    m->kp2 = m->kb;
+    m->vp2 = m->vb;
+  }
+  p->B = d.batch; p->N = d.n_nodes; p->L = d.block_len; p->P = a.ctx.len; p->P2 = a.ctx2.len;
+  p->Hq = d.n_q_heads; p->Hkv = d.n_kv_heads; p->group = sh.group;
+  p->TNL = sh.TNL; p->NL = sh.NL; p->TP1 = sh.TP1; p->TP = sh.TP; p->cs = cs;
+  const float scale = d.scale != 0.f ? d.scale : 1.0f / sqrtf((float)d.head_dim);
+  p->scale_log2 = scale * kLog2e;
+  p->out = static_cast<__nv_bfloat16*>(a.out);
+  p->status = dev_status;
+  p->spin_limit = mbar_poll_limit();
+  p->early_trigger = (d.kernel & SPIFFY_ATTN_EARLY_DEPENDENTS) ? 1 : 0;
+  return ok;
 }
 
-spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const void* q, const AttnContext& ctx,
-                                  const AttnContext& ctx2, const void* kb, const void* vb, void* out,
-                                  int32_t* dev_status, cudaStream_t stream) {
+template <int NP>
+spiffy_status launch(const spiffy_attn_desc* const (&d)[NP], const AttnProblem* const (&a)[NP], int32_t* dev_status,
+                     cudaStream_t stream) {
+  const int hd = d[0]->head_dim;
   static std::atomic<bool> smem_allowed[4][64];
   for (int nq = 1; nq <= 2; ++nq)
-    if (!allow_smem(kernel_of(d.head_dim, nq), kSmemBytes, smem_allowed[(d.head_dim == 128 ? 0 : 2) + nq - 1]))
+    if (!allow_smem(kernel_of<NP>(hd, nq), kSmemBytes, smem_allowed[(hd == 128 ? 0 : 2) + nq - 1]))
       return SPIFFY_ECUDA;
-  const Plan pl = make_plan(d, ctx2.len);
-  CUtensorMap tm_q, tm_kp, tm_vp, tm_kp2, tm_vp2, tm_kb, tm_vb;
-  bool ok = make_map(&tm_q, q, d.n_q_heads, pl.NL, d.batch, pl.group, pl.TNL, 0, pl.hd);
-  ok = ok && make_map(&tm_kb, kb, d.n_kv_heads, pl.NL, d.batch, 1, BN, 0, pl.hd);
-  ok = ok && make_map(&tm_vb, vb, d.n_kv_heads, pl.NL, d.batch, 1, BN, 0, pl.hd);
-  if (ctx.len > 0) {
-    ok = ok && make_map(&tm_kp, ctx.k, d.n_kv_heads, ctx.len, d.batch, 1, BN, ctx.batch_stride_rows, pl.hd);
-    ok = ok && make_map(&tm_vp, ctx.v, d.n_kv_heads, ctx.len, d.batch, 1, BN, ctx.batch_stride_rows, pl.hd);
-  } else {  // never dereferenced: the segment has no tile
-    tm_kp = tm_kb;
-    tm_vp = tm_vb;
+  if constexpr (NP == 2) {  // make_plan asks about the one-problem kernel
+    static std::atomic<bool> allowed[64];
+    if (!allow_smem(kernel_of<1>(hd, 1), kSmemBytes, allowed)) return SPIFFY_ECUDA;
   }
-  if (ctx2.len > 0) {
-    ok = ok && make_map(&tm_kp2, ctx2.k, d.n_kv_heads, ctx2.len, d.batch, 1, BN, ctx2.batch_stride_rows, pl.hd);
-    ok = ok && make_map(&tm_vp2, ctx2.v, d.n_kv_heads, ctx2.len, d.batch, 1, BN, ctx2.batch_stride_rows, pl.hd);
-  } else {
-    tm_kp2 = tm_kb;
-    tm_vp2 = tm_vb;
+  const int64_t bg = (int64_t)d[0]->batch * d[0]->n_kv_heads;
+  Shape sh[NP];
+  int64_t tiles = 0, pairs = 0;
+  int T = 0;
+  for (int i = 0; i < NP; ++i) {
+    sh[i] = shape_of(*d[i], a[i]->ctx, a[i]->ctx2);
+    tiles += bg * sh[i].MT;
+    pairs += bg * ((sh[i].MT + 1) / 2);
+    T = sh[i].T > T ? sh[i].T : T;
   }
-  if (!ok) return SPIFFY_ECUDA;
-
-  Params p;
-  p.B = d.batch; p.N = d.n_nodes; p.L = d.block_len; p.P = ctx.len; p.P2 = ctx2.len;
-  p.Hq = d.n_q_heads; p.Hkv = d.n_kv_heads; p.group = pl.group;
-  p.TNL = pl.TNL; p.NL = pl.NL; p.TP1 = pl.TP1; p.TP = pl.TP; p.cs = pl.cs;
-  const float scale = d.scale != 0.f ? d.scale : 1.0f / sqrtf((float)d.head_dim);
-  p.scale_log2 = scale * kLog2e;
-  p.out = static_cast<__nv_bfloat16*>(out);
-  p.status = dev_status;
-  p.spin_limit = mbar_poll_limit();
-  p.early_trigger = (d.kernel & SPIFFY_ATTN_EARLY_DEPENDENTS) ? 1 : 0;
-
-  const Kernel kern = kernel_of(pl.hd, pl.nq);
+  const Plan pl = make_plan(tiles, pairs, T, hd);
+  Problems<NP> pr;
+  int x = 0;
+  for (int i = 0; i < NP; ++i) {
+    if (!make_problem(*d[i], sh[i], *a[i], &pr.maps[i], &pr.p[i], pl.cs, dev_status)) return SPIFFY_ECUDA;
+    if (i == 1) pr.x_split = x;
+    x += (sh[i].MT + pl.nq - 1) / pl.nq;
+  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((pl.MT + pl.nq - 1) / pl.nq, d.batch * d.n_kv_heads, pl.cs);
+  cfg.gridDim = dim3((unsigned)x, (unsigned)bg, (unsigned)pl.cs);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = stream;
@@ -847,9 +880,29 @@ spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const void* q, cons
   attr[1].val.clusterDim.z = (unsigned)pl.cs;
   cfg.attrs = attr;
   cfg.numAttrs = pl.cs > 1 ? 2 : 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tm_q, tm_kp, tm_vp, tm_kp2, tm_vp2, tm_kb, tm_vb, p);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel_of<NP>(hd, pl.nq), pr);
   count_launch();
   return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
+}
+
+}  // namespace
+
+bool attention_tc_supported(const spiffy_attn_desc& d) {
+  if (d.dtype != SPIFFY_BF16 || (d.head_dim != 128 && d.head_dim != 64)) return false;
+  const int group = d.n_q_heads / d.n_kv_heads;
+  if (group > BM) return false;
+  if ((int64_t)d.batch * d.n_kv_heads > 65535) return false;
+  return true;
+}
+
+spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const AttnProblem& a, int32_t* dev_status,
+                                  cudaStream_t stream) {
+  return launch<1>({&d}, {&a}, dev_status, stream);
+}
+
+spiffy_status launch_attention_tc_dual(const spiffy_attn_desc& d0, const AttnProblem& a0, const spiffy_attn_desc& d1,
+                                       const AttnProblem& a1, int32_t* dev_status, cudaStream_t stream) {
+  return launch<2>({&d0, &d1}, {&a0, &a1}, dev_status, stream);
 }
 
 }  // namespace spiffy

@@ -158,10 +158,20 @@ struct AttnContext {
   int len;
   int64_t batch_stride_rows;
 };
+// One attention problem's tensors: queries, two context segments, block keys/values, output.
+struct AttnProblem {
+  const void* q;
+  AttnContext ctx, ctx2;
+  const void* kb;
+  const void* vb;
+  void* out;
+};
 bool attention_tc_supported(const spiffy_attn_desc& d);
-spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const void* q, const AttnContext& ctx,
-                                  const AttnContext& ctx2, const void* kb, const void* vb, void* out,
-                                  int32_t* dev_status, cudaStream_t stream);
+spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const AttnProblem& a, int32_t* dev_status,
+                                  cudaStream_t stream);
+// Two problems of the same batch, heads and head dimension (128) in one launch.
+spiffy_status launch_attention_tc_dual(const spiffy_attn_desc& d0, const AttnProblem& a0, const spiffy_attn_desc& d1,
+                                       const AttnProblem& a1, int32_t* dev_status, cudaStream_t stream);
 
 // Launch with programmatic stream serialisation: the kernel may be scheduled
 // while its predecessor in the stream is still draining.  Every kernel launched
