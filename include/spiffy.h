@@ -334,14 +334,14 @@ spiffy_status spiffy_unmask_decide_sampled(const spiffy_decide_desc* desc,
  * [rows x V] logits are never written to memory; the result is what
  * spiffy_unmask_decide gives on those (unrounded, fp32) logits.
  *   hidden_states [B*N*L][hidden] bf16, row r = (b * N + n) * L + l; rows of
- *                 unmasked positions are computed and ignored
+ *                 unmasked positions are not used
  *   weight        [V][hidden] bf16 (the output embedding, one row per token)
  *   desc          batch, n_nodes, block_len, vocab, mask_token_id, rule, top_s,
  *                 threshold are used; of logits_dtype only SPIFFY_FRESH_STATUS;
  *                 row_stride is ignored
- * Limit: hidden a multiple of 128, else SPIFFY_EUNSUPPORTED.  Rows are taken 256 at a
- * time and every such pass reads the weight matrix again: the call is made for
- * the few hundred rows of one verification step.
+ * Limit: hidden a multiple of 128, else SPIFFY_EUNSUPPORTED.  Still-masked rows are
+ * taken 256 at a time and every such pass reads the weight matrix again: the call
+ * is made for the few hundred rows of one verification step.
  * Outputs, status bits and the finalize step are those of spiffy_unmask_decide.
  * The paper evaluates the decision on materialised logits; fusing it into the
  * output projection is this library's addition.

@@ -349,7 +349,7 @@ size_t spiffy_lmhead_decide_workspace(const spiffy_decide_desc* desc, int32_t hi
   bool fresh;
   if (lmhead_desc(desc, hidden, &d, &fresh) != SPIFFY_OK) return 0;
   const int grid = lmhead_grid(d);
-  return grid > 0 ? lmhead_workspace_bytes(d, grid) : 0;
+  return grid > 0 ? lmhead_workspace_bytes(d, hidden, grid) : 0;
 }
 
 spiffy_status spiffy_lmhead_decide(const spiffy_decide_desc* desc, int32_t hidden,
@@ -366,7 +366,7 @@ spiffy_status spiffy_lmhead_decide(const spiffy_decide_desc* desc, int32_t hidde
   if (!aligned16(hidden_states) || !aligned16(weight)) return SPIFFY_EINVAL;
   const int grid = lmhead_grid(d);
   if (grid <= 0) return SPIFFY_ECUDA;
-  const size_t need = lmhead_workspace_bytes(d, grid);
+  const size_t need = lmhead_workspace_bytes(d, hidden, grid);
   if (!workspace || workspace_bytes < need || !aligned16(workspace)) return SPIFFY_EWORKSPACE;
   return launch_lmhead_decide(d, hidden, hidden_states, weight, block_tokens, conf, top_tok,
                               unmask_bits, n_unmask, dev_status, workspace,

@@ -128,7 +128,7 @@ spiffy_status launch_decide_finalize(const spiffy_decide_desc& d, const void* pa
                                      uint64_t* unmask_bits, int32_t* n_unmask, int32_t* dev_status,
                                      cudaStream_t stream);
 int lmhead_grid(const spiffy_decide_desc& d);
-size_t lmhead_workspace_bytes(const spiffy_decide_desc& d, int grid);
+size_t lmhead_workspace_bytes(const spiffy_decide_desc& d, int hidden, int grid);
 spiffy_status launch_lmhead_decide(const spiffy_decide_desc& d, int hidden, const void* hstates,
                                    const void* weight, const int32_t* block_tokens, float* conf,
                                    int32_t* top_tok, uint64_t* unmask_bits, int32_t* n_unmask,

@@ -5,24 +5,33 @@
 // Sec. 3.1 before it is materialised).
 //
 // H: [rows][hidden] bf16 hidden states of the B*N*L positions,
-// W: [vocabulary][hidden] bf16 output embedding.  A CTA owns vocabulary tiles of
-// up to 256 entries (tile n, n + grid, ...), two M-tiles of 128 rows at once, and
-// runs the K loop over `hidden` in chunks of 64 (more than 256 rows are taken 256
-// at a time, each pass reading the weight matrix again):
-//   warp 0      TMA producer: per chunk the two H tiles and the W tile (64 KB)
-//               into a three-stage ring
-//   warp 1      allocates tensor memory; one lane issues tcgen05.mma, M = 128,
-//               N = 256 (the shape that runs near the tensor pipe's peak: 75-88 ns
-//               per K = 16 step against 64 ns for N = 128), four steps per chunk
-//               and M-tile; the two fp32 accumulators fill the 512 TMEM columns
-//   warps 2-9   one thread per row: reads a finished accumulator (the logits of
-//               256 vocabulary entries), updates its running maximum, sum of
-//               exponentials and arg-max (ties to the lower token), hands the
-//               buffer back
-// Each CTA leaves one partial result per row; the decision's finalize kernel
-// merges them (in a fixed order) and applies the unmasking rule.
+// W: [vocabulary][hidden] bf16 output embedding.
 //
-// Every wait is bounded; a wait that gives up raises SPIFFY_DEV_TIMEOUT.
+//   lmhead_gather_kernel   copies the hidden states of the still-masked positions,
+//                          the only ones the decision needs, one after another
+//   lmhead_reduce_kernel   D[vocabulary, position] = W H^T.  The vocabulary is the M
+//                          side of the products and the masked positions are N, so
+//                          that the work follows their number in steps of 16 (up to
+//                          256 at a time; beyond that, passes that read W again).  A
+//                          CTA owns a contiguous share of the vocabulary, cut into
+//                          tiles of 256 entries, and runs the K loop over `hidden`
+//                          in chunks of 64:
+//     warp 0      TMA producer: per chunk 256 rows of W and the positions' rows
+//                 of H into a ring
+//     warp 1      allocates tensor memory; one lane issues tcgen05.mma, M = 128,
+//                 two M-tiles per chunk
+//     warps 2-9   one thread per vocabulary entry (TMEM lane): for every position
+//                 (column) the warp's 32 entries are reduced across lanes
+//
+// Bound: the weights, read once (1.04 GB, 159 us at the measured copy rate, for
+// 126464 x 4096).  What an SM takes in is 32 KB of W and 128 bytes per position per
+// chunk, and 48.7 bytes per clock is what TMA delivers: with 256 positions as M and
+// a vocabulary tile of 224 as N, as it was, that came to 1232 cycles per chunk and
+// 238-277 us per call; with 166 masked positions as N to about 1110 per 256 entries.
+//
+// Each CTA leaves one partial result per position; the decision's finalize kernel
+// merges them (in a fixed order) and applies the unmasking rule.  Every wait is
+// bounded; a wait that gives up raises SPIFFY_DEV_TIMEOUT.
 #include <math.h>
 
 #include "common.cuh"
@@ -36,47 +45,109 @@ namespace {
 using namespace sm100;
 
 constexpr int kLmThreads = 320;
-constexpr int kLmStages = 3;
-constexpr int kTile = 128 * 128;        // one operand tile of a stage: 128 rows x 64 bf16 = 16 KB
-constexpr int kLmN = 256;               // most vocabulary entries per tile
-constexpr int kStageBytes = 4 * kTile;  // H tile 0 | H tile 1 | W tile (256 rows)
-constexpr int kLmBars = 2 * kLmStages + 4;
-constexpr int kLmSmem = kLmStages * kStageBytes + 8 * kLmBars + 16 + 1024;
-constexpr uint32_t kLmTmemCols = 512;   // M-tile t -> columns 256 t .. 256 t + 255
+constexpr int kGatherThreads = 128;
+constexpr int kPass = 256;              // positions per pass
+constexpr int kBox = 32;                // rows of H per TMA box (and of W in a tile that is not whole)
+constexpr int kTileV = 256;             // vocabulary entries per tile: two M-tiles
+constexpr int kWBytes = kTileV * 128;   // W part of a stage: 256 rows x 64 bf16
+constexpr int kRing = 192 * 1024;
+constexpr int kMaxStages = 5;           // at 32 positions or fewer: 36 KB per stage
+constexpr uint32_t kLmTmemCols = 512;
+
+// Running reduction of one column over one warp's vocabulary entries.
+struct ColumnState {
+  float m[8][kPass];  // [warp][column] maximum
+  float s[8][kPass];  // sum of exp(x - m)
+  int idx[8][kPass];  // lowest entry attaining m
+};
+constexpr int kLmBars = 2 * kMaxStages + 4;
+constexpr int kLmSmem = kRing + (int)sizeof(ColumnState) + 8 * kLmBars + 16 + 1024;
 
 struct LmParams {
-  int rows, hidden, vocab;
-  int n_tile;                   // vocabulary entries per tile: a multiple of 32, at most kLmN
-  Partial* partials;            // [rows][gridDim.x]
-  int32_t* status;              // [B], may be null
+  int hidden, vocab;
+  const int* list;       // [0] number of masked positions, [1 + i] row of the i-th
+  Partial* partials;     // [rows][gridDim.x]
+  int32_t* status;       // [B], may be null
   int n_status;
-  uint32_t spin_limit;          // polls of one mbarrier wait
+  uint32_t spin_limit;   // polls of one mbarrier wait
 };
+
+// grid = rows.  Block r copies row r, if its position is masked, behind the masked rows before it.
+__global__ void __launch_bounds__(kGatherThreads)
+lmhead_gather_kernel(const uint4* __restrict__ h, int row_vecs, const int32_t* __restrict__ tokens, int mask_id,
+                     uint4* __restrict__ packed, int* __restrict__ list, StatusClear clear) {
+  cudaGridDependencySynchronize();
+  pdl_launch_dependents();
+  const int row = blockIdx.x, tid = threadIdx.x;
+  const bool last = row + 1 == (int)gridDim.x;
+  if (clear.rows_per_seq > 0 && tid == 0 && row % clear.rows_per_seq == 0 && clear.a) clear.a[row / clear.rows_per_seq] = 0;
+  const bool masked = tokens[row] == mask_id;
+  if (!masked && !last) return;
+  int before = 0;
+  for (int i = tid; i < row; i += kGatherThreads) before += tokens[i] == mask_id;
+  before = __reduce_add_sync(0xffffffffu, before);
+  __shared__ int part[kGatherThreads / 32];
+  if ((tid & 31) == 0) part[tid >> 5] = before;
+  __syncthreads();
+  before = 0;
+#pragma unroll
+  for (int w = 0; w < kGatherThreads / 32; ++w) before += part[w];
+  if (tid == 0) {
+    if (masked) list[1 + before] = row;
+    if (last) list[0] = before + (masked ? 1 : 0);
+  }
+  if (!masked) return;
+  for (int i = tid; i < row_vecs; i += kGatherThreads)
+    packed[(int64_t)before * row_vecs + i] = h[(int64_t)row * row_vecs + i];
+}
+
+// Reduction across the 32 lanes of 32 columns at once: lane i ends with column i.  At each step a
+// lane gives away the half of the columns that is not its own: 31 exchanges instead of 160.
+template <typename Op>
+__device__ __forceinline__ float reduce_columns(float (&v)[32], int lane, Op op) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const bool upper = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (i < off) {
+        const float give = upper ? v[i] : v[i + off];
+        const float keep = upper ? v[i + off] : v[i];
+        v[i] = op(keep, __shfl_xor_sync(0xffffffffu, give, off));
+      }
+    }
+  }
+  return v[0];
+}
 
 __global__ void __launch_bounds__(kLmThreads, 1)
 lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w,
-                     const LmParams p) {
+                     const __grid_constant__ CUtensorMap tm_w32, const LmParams p) {
   extern __shared__ uint8_t lm_smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>(
-      (reinterpret_cast<uintptr_t>(lm_smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kLmStages * kStageBytes);
+  uint8_t* smem = lm_smem_raw + ((0u - smem_u32(lm_smem_raw)) & 1023u);
+  ColumnState& state = *reinterpret_cast<ColumnState*>(smem + kRing);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kRing + sizeof(ColumnState));
   uint64_t* full = bars;
-  uint64_t* empty = full + kLmStages;
-  uint64_t* acc_full = empty + kLmStages;  // the accumulators hold a finished tile
-  uint64_t* acc_empty = acc_full + 2;      // the epilogue has read them
+  uint64_t* empty = full + kMaxStages;
+  uint64_t* acc_full = empty + kMaxStages;  // [2] an accumulator pair holds a finished tile
+  uint64_t* acc_empty = acc_full + 2;       // [2] ... and has been read
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kLmBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_tiles = (p.vocab + p.n_tile - 1) / p.n_tile;
-  const int my_tiles = (int)blockIdx.x < n_tiles ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  // this CTA's share of the vocabulary, in steps of 32 entries
+  const int64_t units = (p.vocab + kBox - 1) / kBox;
+  const int v_begin = (int)(units * blockIdx.x / gridDim.x) * kBox;
+  const int v_end = (int)(units * (blockIdx.x + 1) / gridDim.x) * kBox;
+  const int tiles = (v_end - v_begin + kTileV - 1) / kTileV;
   const int kc_count = p.hidden / 64;
-  const int passes = (p.rows + 255) / 256;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kLmStages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 1); }
-    mbar_init(acc_full, 1);
-    mbar_init(acc_empty, 256u);  // every epilogue thread, also those of an M-tile beyond the rows
+    prefetch_tensormap(&tm_h);
+    prefetch_tensormap(&tm_w);
+    prefetch_tensormap(&tm_w32);
+    for (int i = 0; i < kMaxStages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(acc_full + i, 1); mbar_init(acc_empty + i, 8); }  // the epilogue warps
     *abort_flag = 0;
     mbar_fence_init();
   }
@@ -85,125 +156,165 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  if (threadIdx.x == 0) {
-    prefetch_tensormap(&tm_h);
-    prefetch_tensormap(&tm_w);
-  }
-  cudaGridDependencySynchronize();  // H (and the tokens the finalize kernel reads) are visible
+  cudaGridDependencySynchronize();  // the packed rows (and everything before them) are visible
+
+  const int count = *reinterpret_cast<const volatile int*>(p.list);
+  const int passes = (count + kPass - 1) / kPass;
+  auto positions = [&](int pass) { return min(kPass, count - pass * kPass); };
+  auto boxes = [&](int pass) { return (positions(pass) + kBox - 1) / kBox; };
+  // the ring is cut for the first pass, the one with the most positions
+  const int stage_bytes = kWBytes + (passes > 0 ? boxes(0) : 0) * kBox * 128;
+  const int stages = min(kMaxStages, kRing / stage_bytes);
+  // accumulator pairs that fit tensor memory: two (columns 0 and 256 on) up to 128 positions
+  const int bufs = count <= 128 ? 2 : 1;
+  const uint32_t acc_step = bufs == 2 ? 128u : 256u;  // columns between the accumulators of a pair
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer --
     if (lane == 0) {
       bool ok = true;
-      int it = 0, issued = 0;
-      for (int g = 0; g < passes * my_tiles && ok; ++g) {
-        const int pass = g / my_tiles, i = g - pass * my_tiles;
-        const int n = (int)blockIdx.x + i * (int)gridDim.x;
-        const int row0 = pass * 256, mt = p.rows - row0 > 128 ? 2 : 1;
-        for (int kc = 0; kc < kc_count; ++kc, ++it) {
-          const int stage = it % kLmStages;
-          if (!mbar_wait(empty + stage, (((uint32_t)(it / kLmStages)) & 1u) ^ 1u, abort_flag, p.spin_limit)) { ok = false; break; }
-          uint8_t* dst = smem + stage * kStageBytes;
-          mbar_arrive_expect_tx(full + stage, (uint32_t)mt * kTile + (uint32_t)p.n_tile * 128u);
-          const int c0 = (kc & 1) * 64, head = kc >> 1;
-          tma_load_4d(dst, &tm_h, full + stage, c0, head, row0, 0);
-          if (mt > 1) tma_load_4d(dst + kTile, &tm_h, full + stage, c0, head, row0 + 128, 0);
-          tma_load_4d(dst + 2 * kTile, &tm_w, full + stage, c0, head, n * p.n_tile, 0);
-          issued = it + 1;
+      int stage = 0;
+      uint32_t phase = 0, used = 0;  // `used`: stages that hold a copy this thread has issued
+      for (int pass = 0; pass < passes && ok; ++pass) {
+        const int nb = boxes(pass);
+        for (int i = 0; i < tiles && ok; ++i) {
+          const int v0 = v_begin + i * kTileV, rows = min(kTileV, v_end - v0);
+          for (int kc = 0; kc < kc_count; ++kc) {
+            if (!mbar_wait(empty + stage, phase ^ 1u, abort_flag, p.spin_limit)) { ok = false; break; }
+            uint8_t* dst = smem + stage * stage_bytes;
+            mbar_arrive_expect_tx(full + stage, (uint32_t)(rows + nb * kBox) * 128u);
+            used |= 1u << stage;
+            const int c0 = (kc & 1) * 64, head = kc >> 1;
+            if (rows == kTileV) {
+              tma_load_4d(dst, &tm_w, full + stage, c0, head, v0, 0);
+              tma_load_4d(dst + kWBytes / 2, &tm_w, full + stage, c0, head, v0 + 128, 0);
+            } else {
+              for (int q = 0; q < rows / kBox; ++q)
+                tma_load_4d(dst + q * kBox * 128, &tm_w32, full + stage, c0, head, v0 + q * kBox, 0);
+            }
+            for (int q = 0; q < nb; ++q)
+              tma_load_4d(dst + kWBytes + q * kBox * 128, &tm_h, full + stage, c0, head, pass * kPass + q * kBox, 0);
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
+          }
         }
       }
       if (!ok) {  // winding down: let the copies already in flight land before exit
-        for (int j = max(0, issued - kLmStages); j < issued; ++j)
-          for (uint32_t s = 0; s < kSpinLimit; ++s)
-            if (mbar_try_wait(full + j % kLmStages, (uint32_t)(j / kLmStages) & 1u)) break;
+        for (int q = 0; q < kMaxStages; ++q)
+          if ((used >> q) & 1u)
+            for (uint32_t s = 0; s < kSpinLimit; ++s)
+              if (mbar_try_wait(full + q, q < stage ? phase : phase ^ 1u)) break;
       }
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------- MMA issuer --
     if (lane == 0) {
-      const uint32_t idesc = idesc_bf16_f32(128, p.n_tile, false, false);
+      constexpr uint32_t hi = desc_hi_sw128(1024);
       bool ok = true;
-      int it = 0;
-      for (int g = 0; g < passes * my_tiles && ok; ++g) {
-        const int mt = p.rows - (g / my_tiles) * 256 > 128 ? 2 : 1;
-        if (!mbar_wait(acc_empty, ((uint32_t)g & 1u) ^ 1u, abort_flag, p.spin_limit)) { ok = false; break; }
-        tc_fence_after_sync();
-        for (int kc = 0; kc < kc_count; ++kc, ++it) {
-          const int stage = it % kLmStages;
-          if (!mbar_wait(full + stage, (uint32_t)(it / kLmStages) & 1u, abort_flag, p.spin_limit)) { ok = false; break; }
+      int stage = 0, g = 0;
+      uint32_t phase = 0;
+      for (int pass = 0; pass < passes && ok; ++pass) {
+        const int n16 = (positions(pass) + 15) / 16 * 16;
+        const uint32_t idesc = idesc_bf16_f32(128, n16, false, false);
+        for (int i = 0; i < tiles && ok; ++i, ++g) {
+          const int m_tiles = v_end - (v_begin + i * kTileV) > 128 ? 2 : 1;
+          const int buf = bufs == 2 ? g & 1 : 0;
+          const uint32_t round = (uint32_t)(bufs == 2 ? g >> 1 : g);
+          ok = mbar_wait(acc_empty + buf, (round & 1u) ^ 1u, abort_flag, p.spin_limit);
+          if (!ok) break;
           tc_fence_after_sync();
-          const uint32_t h0 = smem_u32(smem + stage * kStageBytes);
-          const uint32_t w0 = h0 + 2 * kTile;
-#pragma unroll
-          for (int t = 0; t < 2; ++t) {
-            if (t < mt) {
-              const uint32_t d = tmem + (uint32_t)t * (uint32_t)kLmN;
-#pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                umma_ss(d, smem_desc_sw128(h0 + (uint32_t)t * kTile + (uint32_t)kk * 32u, 16, 1024),
-                        smem_desc_sw128(w0 + (uint32_t)kk * 32u, 16, 1024), idesc, (kc > 0 || kk > 0) ? 1u : 0u);
-            }
+          const uint32_t d = tmem + (uint32_t)buf * 256u;
+          for (int kc = 0; kc < kc_count; ++kc) {
+            if (!mbar_wait(full + stage, phase, abort_flag, p.spin_limit)) { ok = false; break; }
+            tc_fence_after_sync();
+            const uint32_t w_lo = desc_lo_sw128(smem_u32(smem + stage * stage_bytes), 16);
+            const uint32_t h_lo = w_lo + (kWBytes >> 4);
+            for (int t = 0; t < m_tiles; ++t)
+              umma_ss_k64(d + (uint32_t)t * acc_step, w_lo + (uint32_t)t * (kWBytes >> 5), h_lo, hi, idesc, kc > 0 ? 1u : 0u);
+            umma_commit(empty + stage);  // the stage is free once these products have read it
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
-          umma_commit(empty + stage);  // the stage is free once these products have read it
+          if (ok) umma_commit(acc_full + buf);
         }
-        if (ok) umma_commit(acc_full);
       }
     }
   } else {
     // ------------------------------------------------------------ epilogue --
-    const int quad = warp & 3;
-    const int t = (warp - 2) >> 2;  // M-tile of this warpgroup
-    const int r = quad * 32 + lane;
+    const int quad = warp & 3, ew = warp - 2;
+    const int t = ew >> 2;  // M-tile of this warp
     const uint32_t lane_base = (uint32_t)(quad * 32);
     bool ok = true;
+    int g = 0;
     for (int pass = 0; pass < passes && ok; ++pass) {
-      const int row = pass * 256 + t * 128 + r;
-      const bool live = pass * 256 + t * 128 < p.rows;  // this warpgroup's M-tile holds rows in this pass
-      float m_run = -INFINITY, s_run = 0.f, best = -INFINITY;
-      int best_idx = 0x7fffffff;
-      for (int i = 0; i < my_tiles && ok; ++i) {
-        const int n = (int)blockIdx.x + i * (int)gridDim.x;
-        const int g = pass * my_tiles + i;
-        ok = __all_sync(0xffffffffu, mbar_wait(acc_full, (uint32_t)g & 1u, abort_flag, p.spin_limit));
+      const int nb = boxes(pass);
+      for (int c = lane; c < nb * 32; c += 32) {
+        state.m[ew][c] = -INFINITY;
+        state.s[ew][c] = 0.f;
+        state.idx[ew][c] = 0x7fffffff;
+      }
+      __syncwarp();
+      for (int i = 0; i < tiles && ok; ++i, ++g) {
+        const int buf = bufs == 2 ? g & 1 : 0;
+        const uint32_t round = (uint32_t)(bufs == 2 ? g >> 1 : g);
+        ok = __all_sync(0xffffffffu, mbar_wait(acc_full + buf, round & 1u, abort_flag, p.spin_limit));
         if (!ok) break;
         tc_fence_after_sync();
-        const uint32_t col0 = (uint32_t)t * (uint32_t)kLmN;
+        const int v = v_begin + i * kTileV + t * 128 + quad * 32;  // first vocabulary entry of this warp
+        const bool live = v < v_end && v < p.vocab;
+        const bool valid = v + lane < p.vocab;
 #pragma unroll 1
-        for (int c0 = 0; live && c0 < p.n_tile; c0 += 32) {
-          uint32_t v[32];
-          tmem_ld_x32(tmem_addr(tmem, lane_base, col0 + (uint32_t)c0), v);
-          const int v0 = n * p.n_tile + c0;
-          float cm = -INFINITY;
+        for (int q = 0; live && q < nb; ++q) {
+          uint32_t x[32];
+          tmem_ld_x32(tmem_addr(tmem, lane_base, (uint32_t)buf * 256u + (uint32_t)t * acc_step + (uint32_t)q * 32u), x);
+          float f[32];
 #pragma unroll
           for (int c = 0; c < 32; ++c) {
-            const float x = (v0 + c < p.vocab) ? __uint_as_float(v[c]) : -INFINITY;
-            v[c] = __float_as_uint(x);
-            cm = fmaxf(cm, x);
+            if (!valid) x[c] = 0xff800000u;  // -inf
+            f[c] = __uint_as_float(x[c]);
           }
-          if (cm > m_run) {  // new reference maximum: rescale the sum
-            s_run *= (m_run == -INFINITY) ? 0.f : ex2((m_run - cm) * kLog2e);
-            m_run = cm;
-          }
-          const float ml = (m_run == -INFINITY) ? 0.f : m_run * kLog2e;
+          // lane c: the maximum of column 32 q + c over the warp's entries, then the running one
+          const float cm = reduce_columns(f, lane, [](float a, float b) { return fmaxf(a, b); });
+          const int at = q * 32 + lane;
+          const float m_old = state.m[ew][at];
+          const bool better = cm > m_old;  // strictly: tiles come in ascending token order
+          const float m_new = better ? cm : m_old;
+          const float ref = m_new == -INFINITY ? 0.f : m_new * kLog2e;
 #pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            const float x = __uint_as_float(v[c]);
-            s_run += ex2(fmaf(x, kLog2e, -ml));
-            if (x > best) {  // strictly: tiles and columns come in ascending token order
-              best = x;
-              best_idx = v0 + c;
+          for (int c = 0; c < 32; ++c)
+            f[c] = ex2(fmaf(__uint_as_float(x[c]), kLog2e, -__shfl_sync(0xffffffffu, ref, c)));
+          const float cs = reduce_columns(f, lane, [](float a, float b) { return a + b; });
+          state.s[ew][at] = fmaf(state.s[ew][at], better ? ex2((m_old - m_new) * kLog2e) : 1.f, cs);
+          const unsigned improved = __ballot_sync(0xffffffffu, better);
+          if (improved) {  // the lowest entry that attains the new maximum: rare after the first tiles
+            int found = 0;
+#pragma unroll
+            for (int c = 0; c < 32; ++c) {
+              if ((improved >> c) & 1u) {
+                const unsigned who = __ballot_sync(0xffffffffu, __uint_as_float(x[c]) == __shfl_sync(0xffffffffu, cm, c));
+                if (lane == c) found = __ffs(who) - 1;
+              }
+            }
+            if (better) {
+              state.m[ew][at] = m_new;
+              state.idx[ew][at] = v + found;
             }
           }
         }
         tc_fence_before_sync();
-        mbar_arrive(acc_empty);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty + buf);
       }
-      if (ok && row < p.rows) {
+      asm volatile("bar.sync 1, 256;" ::: "memory");  // every warp's columns, whatever `ok` says
+      const int c = (int)threadIdx.x - 64;
+      if (ok && c < positions(pass)) {
+        float m = -INFINITY, sum = 0.f;
+        int idx = 0x7fffffff;
+#pragma unroll 1
+        for (int w = 0; w < 8; ++w) merge(m, sum, idx, state.m[w][c], state.s[w][c], state.idx[w][c]);
         // NaN logits never win a comparison: report them through the maximum
-        if (!(s_run == s_run)) m_run = s_run;
-        p.partials[(int64_t)row * gridDim.x + blockIdx.x] =
-            Partial{m_run, s_run, best == -INFINITY ? 0x7fffffff : best_idx, 0};
+        if (!(sum == sum)) m = sum;
+        p.partials[(int64_t)p.list[1 + pass * kPass + c] * gridDim.x + blockIdx.x] = Partial{m, sum, idx, 0};
       }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
     }
   }
 
@@ -217,39 +328,31 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
     for (int b = 0; b < p.n_status; ++b) atomicOr(p.status + b, SPIFFY_DEV_TIMEOUT);
 }
 
+size_t up256(size_t n) { return (n + 255) / 256 * 256; }
+size_t partial_bytes(const spiffy_decide_desc& d, int grid) {
+  return up256((size_t)d.batch * d.n_nodes * d.block_len * (size_t)grid * sizeof(Partial));
+}
+size_t list_bytes(const spiffy_decide_desc& d) { return up256(((size_t)d.batch * d.n_nodes * d.block_len + 1) * sizeof(int)); }
+
 }  // namespace
 
-// Vocabulary entries per tile: the multiple of 32 (at most 256, at least 128) for which
-// rounds of tiles x tile width is smallest -- a narrower tile can fill the last round.
-int lmhead_tile(int vocab, int sms) {
-  int best = kLmN;
-  int64_t best_cost = -1;
-  for (int n = kLmN; n >= 128; n -= 32) {
-    const int64_t tiles = (vocab + n - 1) / n;
-    const int64_t rounds = (tiles + sms - 1) / sms;
-    const int64_t cost = rounds * (n + 64);  // a tile costs about its width plus a fixed part
-    if (best_cost < 0 || cost < best_cost) {
-      best = n;
-      best_cost = cost;
-    }
-  }
-  return best;
-}
-
+// One CTA per SM, or fewer for a vocabulary of fewer than 32 entries each.
 int lmhead_grid(const spiffy_decide_desc& d) {
-  static int sms[64];
+  static std::atomic<int> sms[64];
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return 0;
-  if (sms[device] == 0 &&
-      cudaDeviceGetAttribute(&sms[device], cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
-    return 0;
-  const int n = lmhead_tile(d.vocab, sms[device]);
-  const int n_tiles = (d.vocab + n - 1) / n;
-  return n_tiles < sms[device] ? n_tiles : sms[device];
+  int n = sms[device].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
+    sms[device].store(n, std::memory_order_relaxed);
+  }
+  const int units = (d.vocab + kBox - 1) / kBox;
+  return units < n ? units : n;
 }
 
-size_t lmhead_workspace_bytes(const spiffy_decide_desc& d, int grid) {
-  return (size_t)d.batch * d.n_nodes * d.block_len * (size_t)grid * sizeof(Partial);
+// partial results | list of masked rows | their hidden states
+size_t lmhead_workspace_bytes(const spiffy_decide_desc& d, int hidden, int grid) {
+  return partial_bytes(d, grid) + list_bytes(d) + (size_t)d.batch * d.n_nodes * d.block_len * (size_t)hidden * 2;
 }
 
 spiffy_status launch_lmhead_decide(const spiffy_decide_desc& d, int hidden, const void* hstates,
@@ -259,31 +362,30 @@ spiffy_status launch_lmhead_decide(const spiffy_decide_desc& d, int hidden, cons
   const int rows = d.batch * d.n_nodes * d.block_len;
   const int grid = lmhead_grid(d);
   if (grid <= 0) return SPIFFY_ECUDA;
-  int sm_count = 0, dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return SPIFFY_ECUDA;
-  const int n_tile = lmhead_tile(d.vocab, sm_count);
-  CUtensorMap tm_h, tm_w;
-  if (!make_map(&tm_h, hstates, hidden / 128, rows, 1, 1, 128) ||
-      !make_map(&tm_w, weight, hidden / 128, d.vocab, 1, 1, n_tile))
+  char* at = static_cast<char*>(ws);
+  int* list = reinterpret_cast<int*>(at + partial_bytes(d, grid));
+  uint4* packed = reinterpret_cast<uint4*>(at + partial_bytes(d, grid) + list_bytes(d));
+  CUtensorMap tm_h, tm_w, tm_w32;
+  if (!make_map(&tm_h, packed, hidden / 128, rows, 1, 1, kBox) ||
+      !make_map(&tm_w, weight, hidden / 128, d.vocab, 1, 1, 128) ||
+      !make_map(&tm_w32, weight, hidden / 128, d.vocab, 1, 1, kBox))
     return SPIFFY_ECUDA;
   static std::atomic<bool> smem_allowed[64];
   if (!allow_smem(lmhead_reduce_kernel, kLmSmem, smem_allowed)) return SPIFFY_ECUDA;
+  cudaError_t e = launch_pdl(lmhead_gather_kernel, dim3(rows), dim3(kGatherThreads), (size_t)0, stream,
+                             static_cast<const uint4*>(hstates), hidden / 8, block_tokens, (int)d.mask_token_id,
+                             packed, list, status_clear(d, fresh, dev_status, nullptr));
+  count_launch();
+  if (e != cudaSuccess) return SPIFFY_ECUDA;
   LmParams p;
-  p.rows = rows;
   p.hidden = hidden;
   p.vocab = d.vocab;
-  p.n_tile = n_tile;
+  p.list = list;
   p.partials = static_cast<Partial*>(ws);
   p.status = dev_status;
   p.n_status = d.batch;
   p.spin_limit = mbar_poll_limit();
-  // any CTA of the first kernel may set a bit: cleared ahead of it
-  if (fresh && dev_status && cudaMemsetAsync(dev_status, 0, (size_t)d.batch * 4, stream) != cudaSuccess)
-    return SPIFFY_ECUDA;
-  cudaError_t e = launch_pdl(lmhead_reduce_kernel, dim3(grid), dim3(kLmThreads), (size_t)kLmSmem, stream,
-                             tm_h, tm_w, p);
+  e = launch_pdl(lmhead_reduce_kernel, dim3(grid), dim3(kLmThreads), (size_t)kLmSmem, stream, tm_h, tm_w, tm_w32, p);
   count_launch();
   if (e != cudaSuccess) return SPIFFY_ECUDA;
   return launch_decide_finalize(d, ws, grid, block_tokens, conf, top_tok, unmask_bits, n_unmask, dev_status,
