@@ -8,7 +8,8 @@
 // W: [vocabulary][hidden] bf16 output embedding.
 //
 //   lmhead_gather_kernel   copies the hidden states of the still-masked positions,
-//                          the only ones the decision needs, one after another
+//                          the only ones the decision needs, one after another;
+//                          left out when there are few positions anyhow
 //   lmhead_reduce_kernel   D[vocabulary, position] = W H^T.  The vocabulary is the M
 //                          side of the products and the masked positions are N, so
 //                          that the work follows their number in steps of 16 (up to
@@ -20,7 +21,7 @@
 //                 of H into a ring
 //     warp 1      allocates tensor memory; one lane issues tcgen05.mma, M = 128,
 //                 two M-tiles per chunk
-//     warps 2-9   one thread per vocabulary entry (TMEM lane): for every position
+//     warps 4-11  one thread per vocabulary entry (TMEM lane): for every position
 //                 (column) the warp's 32 entries are reduced across lanes
 //
 // Bound: the weights, read once (1.04 GB, 159 us at the measured copy rate, for
@@ -28,6 +29,10 @@
 // chunk, and 48.7 bytes per clock is what TMA delivers: with 256 positions as M and
 // a vocabulary tile of 224 as N, as it was, that came to 1232 cycles per chunk and
 // 238-277 us per call; with 166 masked positions as N to about 1110 per 256 entries.
+// The reduction across lanes takes 6.6 us a tile there, and tensor memory has no room
+// for a second accumulator pair: the epilogue empties the first into registers (192 a
+// thread, which is why its warps take the others' share) and gives it back, so that
+// the next tile's products run meanwhile: 237 -> 206-214 us.
 //
 // Each CTA leaves one partial result per position; the decision's finalize kernel
 // merges them (in a fixed order) and applies the unmasking rule.  Every wait is
@@ -44,14 +49,19 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kLmThreads = 320;
+constexpr int kLmThreads = 384;
 constexpr int kGatherThreads = 128;
 constexpr int kPass = 256;              // positions per pass
+// Up to this many positions are taken as they are, masked or not: they cost less time as columns
+// (their part of what an SM takes in stays below the weights' third) than the launch that packs.
+constexpr int kDirectRows = 128;
 constexpr int kBox = 32;                // rows of H per TMA box (and of W in a tile that is not whole)
 constexpr int kTileV = 256;             // vocabulary entries per tile: two M-tiles
-constexpr int kWBytes = kTileV * 128;   // W part of a stage: 256 rows x 64 bf16
-constexpr int kRing = 192 * 1024;
-constexpr int kMaxStages = 5;           // at 32 positions or fewer: 36 KB per stage
+constexpr int kRing = 200 * 1024;
+constexpr int kMaxStages = 12;          // at least three: 64 KB per stage at 256 positions
+constexpr int kHeld = 6;                // blocks of 32 columns that the epilogue holds in registers
+constexpr int kRegsIssue = 40, kRegsEpilogue = 232;
+static_assert(kRegsIssue + 2 * kRegsEpilogue <= 3 * 168, "within what the block was launched with");
 constexpr uint32_t kLmTmemCols = 512;
 
 // Running reduction of one column over one warp's vocabulary entries.
@@ -65,10 +75,12 @@ constexpr int kLmSmem = kRing + (int)sizeof(ColumnState) + 8 * kLmBars + 16 + 10
 
 struct LmParams {
   int hidden, vocab;
-  const int* list;       // [0] number of masked positions, [1 + i] row of the i-th
+  int rows;              // positions, when all of them are taken in their own order ...
+  const int* list;       // ... which is when this is null: [0] number of masked positions, [1 + i] row of the i-th
   Partial* partials;     // [rows][gridDim.x]
   int32_t* status;       // [B], may be null
   int n_status;
+  int clear_status;      // the status words arrive with arbitrary contents (without a list only)
   uint32_t spin_limit;   // polls of one mbarrier wait
 };
 
@@ -104,20 +116,56 @@ lmhead_gather_kernel(const uint4* __restrict__ h, int row_vecs, const int32_t* _
 // Reduction across the 32 lanes of 32 columns at once: lane i ends with column i.  At each step a
 // lane gives away the half of the columns that is not its own: 31 exchanges instead of 160.
 template <typename Op>
-__device__ __forceinline__ float reduce_columns(float (&v)[32], int lane, Op op) {
+__device__ __forceinline__ float reduce_columns(uint32_t (&v)[32], int lane, Op op) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     const bool upper = (lane & off) != 0;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      if (i < off) {
-        const float give = upper ? v[i] : v[i + off];
-        const float keep = upper ? v[i + off] : v[i];
-        v[i] = op(keep, __shfl_xor_sync(0xffffffffu, give, off));
-      }
+    for (int i = 0; i < off; ++i) {
+      const uint32_t give = upper ? v[i] : v[i + off];
+      const uint32_t keep = upper ? v[i + off] : v[i];
+      v[i] = __float_as_uint(op(__uint_as_float(keep), __uint_as_float(__shfl_xor_sync(0xffffffffu, give, off))));
     }
   }
-  return v[0];
+  return __uint_as_float(v[0]);
+}
+
+// Adds 32 columns (state column `at` belongs to this lane), one of them per register and one
+// vocabulary entry (v0 + lane) per lane, to the state of warp `ew`.  Uses x up.
+__device__ __forceinline__ void add_columns(ColumnState& state, int ew, int at, uint32_t (&x)[32], int v0,
+                                            bool valid, int lane) {
+  uint32_t f[32];
+#pragma unroll
+  for (int c = 0; c < 32; ++c) {
+    if (!valid) x[c] = 0xff800000u;  // -inf
+    f[c] = x[c];
+  }
+  // lane c: the maximum of column c over the warp's entries
+  const float cm = reduce_columns(f, lane, [](float a, float b) { return fmaxf(a, b); });
+  const float m_old = state.m[ew][at];
+  const bool better = cm > m_old;  // strictly: tiles come in ascending token order
+  const float m_new = better ? cm : m_old;
+  const unsigned improved = __ballot_sync(0xffffffffu, better);
+  if (improved) {  // the lowest entry that attains the new maximum: rare after the first tiles
+    int found = 0;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      if ((improved >> c) & 1u) {
+        const unsigned who = __ballot_sync(0xffffffffu, __uint_as_float(x[c]) == __shfl_sync(0xffffffffu, cm, c));
+        if (lane == c) found = __ffs(who) - 1;
+      }
+    }
+    if (better) {
+      state.m[ew][at] = m_new;
+      state.idx[ew][at] = v0 + found;
+    }
+  }
+  const float ref = m_new == -INFINITY ? 0.f : m_new * kLog2e;
+#pragma unroll
+  for (int c = 0; c < 32; ++c)
+    x[c] = __float_as_uint(ex2(fmaf(__uint_as_float(x[c]), kLog2e, -__shfl_sync(0xffffffffu, ref, c))));
+  const float cs = reduce_columns(x, lane, [](float a, float b) { return a + b; });
+  state.s[ew][at] = fmaf(state.s[ew][at], better ? ex2((m_old - m_new) * kLog2e) : 1.f, cs);
 }
 
 __global__ void __launch_bounds__(kLmThreads, 1)
@@ -158,20 +206,27 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
   const uint32_t tmem = *tmem_slot;
   cudaGridDependencySynchronize();  // the packed rows (and everything before them) are visible
 
-  const int count = *reinterpret_cast<const volatile int*>(p.list);
+  const int count = p.list ? *reinterpret_cast<const volatile int*>(p.list) : p.rows;
+  if (p.clear_status && blockIdx.x == 0 && threadIdx.x == 0 && p.status)
+    for (int b = 0; b < p.n_status; ++b) p.status[b] = 0;
   const int passes = (count + kPass - 1) / kPass;
   auto positions = [&](int pass) { return min(kPass, count - pass * kPass); };
   auto boxes = [&](int pass) { return (positions(pass) + kBox - 1) / kBox; };
-  // the ring is cut for the first pass, the one with the most positions
-  const int stage_bytes = kWBytes + (passes > 0 ? boxes(0) : 0) * kBox * 128;
-  const int stages = min(kMaxStages, kRing / stage_bytes);
+  // The ring is cut for the longest tile of this CTA and the first pass, the one with the most
+  // positions: a CTA whose share of the vocabulary is a short tile has more chunks in flight.
+  const int w_bytes = min(kTileV, v_end - v_begin) * 128;
+  const int stage_bytes = w_bytes + (passes > 0 ? boxes(0) : 0) * kBox * 128;
+  // (the products read whole M-tiles, so the last stage is followed by as much of the ring)
+  const int reach = w_bytes > 128 * 128 ? kTileV * 128 : 128 * 128;
+  const int stages = min(kMaxStages, min(kRing / stage_bytes, (kRing - reach) / stage_bytes + 1));
   // accumulator pairs that fit tensor memory: two (columns 0 and 256 on) up to 128 positions
   const int bufs = count <= 128 ? 2 : 1;
   const uint32_t acc_step = bufs == 2 ? 128u : 256u;  // columns between the accumulators of a pair
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ producer --
-    if (lane == 0) {
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
+    if (warp == 0 && lane == 0) {
+      // ---------------------------------------------------------- producer --
       bool ok = true;
       int stage = 0;
       uint32_t phase = 0, used = 0;  // `used`: stages that hold a copy this thread has issued
@@ -187,13 +242,13 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
             const int c0 = (kc & 1) * 64, head = kc >> 1;
             if (rows == kTileV) {
               tma_load_4d(dst, &tm_w, full + stage, c0, head, v0, 0);
-              tma_load_4d(dst + kWBytes / 2, &tm_w, full + stage, c0, head, v0 + 128, 0);
+              tma_load_4d(dst + 128 * 128, &tm_w, full + stage, c0, head, v0 + 128, 0);
             } else {
               for (int q = 0; q < rows / kBox; ++q)
                 tma_load_4d(dst + q * kBox * 128, &tm_w32, full + stage, c0, head, v0 + q * kBox, 0);
             }
             for (int q = 0; q < nb; ++q)
-              tma_load_4d(dst + kWBytes + q * kBox * 128, &tm_h, full + stage, c0, head, pass * kPass + q * kBox, 0);
+              tma_load_4d(dst + w_bytes + q * kBox * 128, &tm_h, full + stage, c0, head, pass * kPass + q * kBox, 0);
             if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
         }
@@ -204,10 +259,8 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
             for (uint32_t s = 0; s < kSpinLimit; ++s)
               if (mbar_try_wait(full + q, q < stage ? phase : phase ^ 1u)) break;
       }
-    }
-  } else if (warp == 1) {
-    // ---------------------------------------------------------- MMA issuer --
-    if (lane == 0) {
+    } else if (warp == 1 && lane == 0) {
+      // -------------------------------------------------------- MMA issuer --
       constexpr uint32_t hi = desc_hi_sw128(1024);
       bool ok = true;
       int stage = 0, g = 0;
@@ -227,9 +280,9 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
             if (!mbar_wait(full + stage, phase, abort_flag, p.spin_limit)) { ok = false; break; }
             tc_fence_after_sync();
             const uint32_t w_lo = desc_lo_sw128(smem_u32(smem + stage * stage_bytes), 16);
-            const uint32_t h_lo = w_lo + (kWBytes >> 4);
+            const uint32_t h_lo = w_lo + ((uint32_t)w_bytes >> 4);
             for (int t = 0; t < m_tiles; ++t)
-              umma_ss_k64(d + (uint32_t)t * acc_step, w_lo + (uint32_t)t * (kWBytes >> 5), h_lo, hi, idesc, kc > 0 ? 1u : 0u);
+              umma_ss_k64(d + (uint32_t)t * acc_step, w_lo + (uint32_t)t * (128 * 128 >> 4), h_lo, hi, idesc, kc > 0 ? 1u : 0u);
             umma_commit(empty + stage);  // the stage is free once these products have read it
             if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
@@ -239,9 +292,9 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
     }
   } else {
     // ------------------------------------------------------------ epilogue --
-    const int quad = warp & 3, ew = warp - 2;
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpilogue));
+    const int quad = warp & 3, ew = warp - 4;
     const int t = ew >> 2;  // M-tile of this warp
-    const uint32_t lane_base = (uint32_t)(quad * 32);
     bool ok = true;
     int g = 0;
     for (int pass = 0; pass < passes && ok; ++pass) {
@@ -258,53 +311,42 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
         ok = __all_sync(0xffffffffu, mbar_wait(acc_full + buf, round & 1u, abort_flag, p.spin_limit));
         if (!ok) break;
         tc_fence_after_sync();
-        const int v = v_begin + i * kTileV + t * 128 + quad * 32;  // first vocabulary entry of this warp
-        const bool live = v < v_end && v < p.vocab;
-        const bool valid = v + lane < p.vocab;
+        const int v0 = v_begin + i * kTileV + t * 128 + quad * 32;  // first vocabulary entry of this warp
+        const bool live = v0 < v_end && v0 < p.vocab;
+        const bool valid = v0 + lane < p.vocab;
+        const uint32_t acc = tmem_addr(tmem, (uint32_t)quad * 32u, (uint32_t)buf * 256u + (uint32_t)t * acc_step);
+        // What the issuer waits for is emptied into registers and given back before any of the
+        // arithmetic, which then runs under the next tile's products.  Behind the last tile, or with a
+        // second pair, nothing waits: there the loop takes all of it, whose few instructions are
+        // fetched sooner (3 us less at a single tile).
+        const int q0 = bufs == 2 || (i + 1 == tiles && pass + 1 == passes) ? 0 : kHeld;
+        uint32_t x[kHeld][32];
+        if (live) {
 #pragma unroll 1
-        for (int q = 0; live && q < nb; ++q) {
-          uint32_t x[32];
-          tmem_ld_x32(tmem_addr(tmem, lane_base, (uint32_t)buf * 256u + (uint32_t)t * acc_step + (uint32_t)q * 32u), x);
-          float f[32];
-#pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            if (!valid) x[c] = 0xff800000u;  // -inf
-            f[c] = __uint_as_float(x[c]);
+          for (int q = q0; q < nb; ++q) {
+            tmem_ld_x32(acc + (uint32_t)q * 32u, x[0]);
+            add_columns(state, ew, q * 32 + lane, x[0], v0, valid, lane);
           }
-          // lane c: the maximum of column 32 q + c over the warp's entries, then the running one
-          const float cm = reduce_columns(f, lane, [](float a, float b) { return fmaxf(a, b); });
-          const int at = q * 32 + lane;
-          const float m_old = state.m[ew][at];
-          const bool better = cm > m_old;  // strictly: tiles come in ascending token order
-          const float m_new = better ? cm : m_old;
-          const float ref = m_new == -INFINITY ? 0.f : m_new * kLog2e;
+          if (q0 == kHeld) {
 #pragma unroll
-          for (int c = 0; c < 32; ++c)
-            f[c] = ex2(fmaf(__uint_as_float(x[c]), kLog2e, -__shfl_sync(0xffffffffu, ref, c)));
-          const float cs = reduce_columns(f, lane, [](float a, float b) { return a + b; });
-          state.s[ew][at] = fmaf(state.s[ew][at], better ? ex2((m_old - m_new) * kLog2e) : 1.f, cs);
-          const unsigned improved = __ballot_sync(0xffffffffu, better);
-          if (improved) {  // the lowest entry that attains the new maximum: rare after the first tiles
-            int found = 0;
+            for (int q = 0; q < kHeld; ++q)
+              if (q < nb) tmem_ld_async(acc + (uint32_t)q * 32u, x[q]);
+            tmem_wait_ld();
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              if ((improved >> c) & 1u) {
-                const unsigned who = __ballot_sync(0xffffffffu, __uint_as_float(x[c]) == __shfl_sync(0xffffffffu, cm, c));
-                if (lane == c) found = __ffs(who) - 1;
-              }
-            }
-            if (better) {
-              state.m[ew][at] = m_new;
-              state.idx[ew][at] = v + found;
-            }
+            for (int q = 0; q < kHeld; ++q) tmem_loaded(x[q]);
           }
         }
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(acc_empty + buf);
+        if (live && q0 == kHeld) {
+#pragma unroll
+          for (int q = 0; q < kHeld; ++q)
+            if (q < nb) add_columns(state, ew, q * 32 + lane, x[q], v0, valid, lane);
+        }
       }
       asm volatile("bar.sync 1, 256;" ::: "memory");  // every warp's columns, whatever `ok` says
-      const int c = (int)threadIdx.x - 64;
+      const int c = (int)threadIdx.x - 128;
       if (ok && c < positions(pass)) {
         float m = -INFINITY, sum = 0.f;
         int idx = 0x7fffffff;
@@ -312,7 +354,8 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
         for (int w = 0; w < 8; ++w) merge(m, sum, idx, state.m[w][c], state.s[w][c], state.idx[w][c]);
         // NaN logits never win a comparison: report them through the maximum
         if (!(sum == sum)) m = sum;
-        p.partials[(int64_t)p.list[1 + pass * kPass + c] * gridDim.x + blockIdx.x] = Partial{m, sum, idx, 0};
+        const int at = pass * kPass + c, row = p.list ? p.list[1 + at] : at;
+        p.partials[(int64_t)row * gridDim.x + blockIdx.x] = Partial{m, sum, idx, 0};
       }
       asm volatile("bar.sync 1, 256;" ::: "memory");
     }
@@ -366,21 +409,27 @@ spiffy_status launch_lmhead_decide(const spiffy_decide_desc& d, int hidden, cons
   int* list = reinterpret_cast<int*>(at + partial_bytes(d, grid));
   uint4* packed = reinterpret_cast<uint4*>(at + partial_bytes(d, grid) + list_bytes(d));
   CUtensorMap tm_h, tm_w, tm_w32;
-  if (!make_map(&tm_h, packed, hidden / 128, rows, 1, 1, kBox) ||
+  const bool pack = rows > kDirectRows;
+  if (!make_map(&tm_h, pack ? static_cast<const void*>(packed) : hstates, hidden / 128, rows, 1, 1, kBox) ||
       !make_map(&tm_w, weight, hidden / 128, d.vocab, 1, 1, 128) ||
       !make_map(&tm_w32, weight, hidden / 128, d.vocab, 1, 1, kBox))
     return SPIFFY_ECUDA;
   static std::atomic<bool> smem_allowed[64];
   if (!allow_smem(lmhead_reduce_kernel, kLmSmem, smem_allowed)) return SPIFFY_ECUDA;
-  cudaError_t e = launch_pdl(lmhead_gather_kernel, dim3(rows), dim3(kGatherThreads), (size_t)0, stream,
-                             static_cast<const uint4*>(hstates), hidden / 8, block_tokens, (int)d.mask_token_id,
-                             packed, list, status_clear(d, fresh, dev_status, nullptr));
-  count_launch();
-  if (e != cudaSuccess) return SPIFFY_ECUDA;
+  cudaError_t e = cudaSuccess;
+  if (pack) {
+    e = launch_pdl(lmhead_gather_kernel, dim3(rows), dim3(kGatherThreads), (size_t)0, stream,
+                   static_cast<const uint4*>(hstates), hidden / 8, block_tokens, (int)d.mask_token_id,
+                   packed, list, status_clear(d, fresh, dev_status, nullptr));
+    count_launch();
+    if (e != cudaSuccess) return SPIFFY_ECUDA;
+  }
   LmParams p;
   p.hidden = hidden;
   p.vocab = d.vocab;
-  p.list = list;
+  p.rows = rows;
+  p.list = pack ? list : nullptr;
+  p.clear_status = !pack && fresh ? 1 : 0;
   p.partials = static_cast<Partial*>(ws);
   p.status = dev_status;
   p.n_status = d.batch;

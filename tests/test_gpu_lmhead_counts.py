@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("count,V,H", [(0, 500, 128), (1, 31, 128), (15, 33, 256), (16, 4736, 128), (17, 4737, 640),
                                        (33, 40000, 128), (127, 9000, 256), (128, 9001, 256), (129, 9002, 256),
-                                       (255, 38000, 384), (256, 1000, 128), (257, 5000, 128), (600, 300, 256)])
+                                       (255, 38000, 384), (256, 1000, 128), (257, 5000, 128), (600, 300, 256), (166, 80000, 128),
+                                       (300, 45000, 128)])
 def test_every_count_of_masked_positions(count, V, H):
     g = torch.Generator().manual_seed(count + V)
     L = 40
