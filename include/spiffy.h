@@ -101,6 +101,11 @@ typedef enum { SPIFFY_RULE_TOPS = 0, SPIFFY_RULE_THRESHOLD = 1 } spiffy_rule;
  * also writes 0 to the entries of parent_idx behind its lists.)  Spares a caller
  * that allocates its outputs for the call the clearing of them. */
 #define SPIFFY_FRESH_STATUS 0x100
+/* Flag, OR-ed into spiffy_decide_desc.logits_dtype of spiffy_decide_walk: none of
+ * the call's inputs is written by the call before it in the stream, which is an
+ * attention call with SPIFFY_ATTN_INDEPENDENT_NEXT.  The two then run side by
+ * side.  What follows in the stream still follows both.  Other calls ignore it. */
+#define SPIFFY_INDEPENDENT 0x200
 
 /* Attention kernel selection (spiffy_attn_desc.kernel). */
 #define SPIFFY_ATTN_AUTO 0   /* tensor-core kernel when the shape allows it: bf16,
@@ -115,6 +120,10 @@ typedef enum { SPIFFY_RULE_TOPS = 0, SPIFFY_RULE_THRESHOLD = 1 } spiffy_rule;
  * this call's complete output).  For the layer loop of a model, where the next
  * kernel's set-up then overlaps this kernel's tail.  Tensor-core kernel only. */
 #define SPIFFY_ATTN_EARLY_DEPENDENTS 0x100
+/* Flag, OR-ed into spiffy_attn_desc.kernel: the next call of the stream is a
+ * decision with SPIFFY_INDEPENDENT.  Such a decision may start as soon as what
+ * precedes this call is complete. */
+#define SPIFFY_ATTN_INDEPENDENT_NEXT 0x200
 
 /* ------------------------------------------------------------------------- */
 /* Packed draft-graph attention (Sec. 4.3; mask semantics: caption of Fig. 3) */
@@ -130,7 +139,7 @@ typedef struct {
   int32_t head_dim;   /* d in {64, 128}                                      */
   int32_t dtype;      /* spiffy_dtype of q, k, v and out                     */
   float scale;        /* softmax scale; 0 means 1/sqrt(d)                    */
-  int32_t kernel;     /* SPIFFY_ATTN_AUTO/SIMT/TCGEN05, | SPIFFY_ATTN_EARLY_DEPENDENTS */
+  int32_t kernel;     /* SPIFFY_ATTN_AUTO/SIMT/TCGEN05, | the SPIFFY_ATTN_ flags */
 } spiffy_attn_desc;
 
 /* Bytes of scratch spiffy_graph_attention needs for this shape: 0 for every shape
@@ -194,7 +203,7 @@ typedef struct {
   int32_t n_nodes;       /* N                                                */
   int32_t block_len;     /* L in [1, 64]                                     */
   int32_t vocab;         /* V >= 1                                           */
-  int32_t logits_dtype;  /* spiffy_dtype, | SPIFFY_FRESH_STATUS              */
+  int32_t logits_dtype;  /* spiffy_dtype, | SPIFFY_FRESH_STATUS, SPIFFY_INDEPENDENT */
   int64_t row_stride;    /* elements between consecutive logits rows, >= V;
                             row_stride * sizeof(element) must be a multiple
                             of 16                                            */

@@ -119,7 +119,9 @@ struct Params {
   __nv_bfloat16* out;
   int32_t* status;
   uint32_t spin_limit;  // polls of one mbarrier wait
-  int early_trigger;    // let the next kernel of the stream begin its set-up while this one runs
+  // Lets the next kernel of the stream start while this one runs: 1 as soon as may be (it waits for
+  // this one by itself), 2 once what precedes this one is complete (it does not); 0 not.
+  int trigger;
 };
 
 // The operands of one attention problem: Q, two context segments, block keys.
@@ -342,9 +344,10 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
   const uint32_t tmem = *tmem_slot;
   // all CTAs' barriers exist before any touches another's (waited for in the epilogue)
   if (cs > 1) cluster_arrive_relaxed();
-  if (p.early_trigger) pdl_launch_dependents();
+  if (p.trigger == 1) pdl_launch_dependents();
   // everything above is on-chip set-up (thread 0 aside); global memory is touched from here on
   cudaGridDependencySynchronize();
+  if (p.trigger == 2) pdl_launch_dependents();
 
   const int U = T << kLogNQ;  // units of this CTA
   if (warp < 4) {
@@ -832,7 +835,7 @@ bool make_problem(const spiffy_attn_desc& d, const Shape& sh, const AttnProblem&
   p->out = static_cast<__nv_bfloat16*>(a.out);
   p->status = dev_status;
   p->spin_limit = mbar_poll_limit();
-  p->early_trigger = (d.kernel & SPIFFY_ATTN_EARLY_DEPENDENTS) ? 1 : 0;
+  p->trigger = (d.kernel & SPIFFY_ATTN_INDEPENDENT_NEXT) ? 2 : (d.kernel & SPIFFY_ATTN_EARLY_DEPENDENTS) ? 1 : 0;
   return ok;
 }
 
@@ -866,6 +869,11 @@ spiffy_status launch(const spiffy_attn_desc* const (&d)[NP], const AttnProblem* 
     if (i == 1) pr.x_split = x;
     x += (sh[i].MT + pl.nq - 1) / pl.nq;
   }
+  // An independent kernel next finds few SMs when one round of CTAs fills nearly all: it then gains
+  // nothing and its first CTAs pile up on those few (144 CTAs: a step of 19.9 us took 20.6).
+  const int64_t ctas = (int64_t)x * bg * pl.cs;
+  for (int i = 0; i < NP; ++i)
+    if (pr.p[i].trigger == 2 && ctas > 132 && ctas <= 148) pr.p[i].trigger = 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)x, (unsigned)bg, (unsigned)pl.cs);
   cfg.blockDim = dim3(kThreads);

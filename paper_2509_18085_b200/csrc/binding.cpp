@@ -460,7 +460,7 @@ PyObject* accept_walk(PyObject* const* a) {
 }
 
 // logits, block_tokens, mask_token_id, rule, top_s, threshold, parent_off, parent_idx, decision, walk, workspace,
-// stream, lazy
+// stream, lazy, independent
 PyObject* decide_walk(PyObject* const* a) {
   const at::Tensor& logits = tensor(a[0], "logits");
   const at::Tensor& tokens = tensor(a[1], "block_tokens");
@@ -470,7 +470,9 @@ PyObject* decide_walk(PyObject* const* a) {
   const int64_t B = d.batch, N = d.n_nodes, L = d.block_len;
   const int32_t cap = parent_cap(off, idx, B, N);
   const int lazy = PyObject_IsTrue(a[12]);
-  if (lazy < 0) throw PyError{};
+  const int independent = PyObject_IsTrue(a[13]);
+  if (lazy < 0 || independent < 0) throw PyError{};
+  if (independent) d.logits_dtype |= SPIFFY_INDEPENDENT;
   const void* lp = logits_ptr(logits);
   const int32_t* tp = (const int32_t*)device_ptr(tokens, "block_tokens", at::kInt);
   const int32_t* op = (const int32_t*)device_ptr(off, "parent_off", at::kInt);
@@ -620,7 +622,7 @@ PyMethodDef g_methods[] = {
     method<unmask_decide_sampled, 11>("unmask_decide_sampled"),
     method<lmhead_decide, 10>("lmhead_decide"),
     method<accept_walk, 7>("accept_walk"),
-    method<decide_walk, 13>("decide_walk"),
+    method<decide_walk, 14>("decide_walk"),
     method<draft_blocks, 10>("draft_blocks"),
     {nullptr, nullptr, 0, nullptr},
 };

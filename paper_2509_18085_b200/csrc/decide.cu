@@ -27,18 +27,24 @@ __global__ void __launch_bounds__(kReduceThreads, 8)  // 64 registers: eight CTA
 decide_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V,
                      int64_t chunk, int splits,
                      const int32_t* __restrict__ block_tokens, int mask_id,
-                     Partial* __restrict__ partials, int early_trigger, StatusClear clear) {
+                     Partial* __restrict__ partials, int early_trigger, int independent, StatusClear clear) {
 #if __CUDA_ARCH__ >= 900
-  cudaGridDependencySynchronize();  // inputs written by earlier kernels are visible
+  // Inputs written by earlier kernels are visible; the kernel before this one may write none of
+  // them and have let this one start only when all others were complete.
+  if (!independent) cudaGridDependencySynchronize();
   // The one-CTA-per-sequence tail kernel may take its SM while this grid still
   // runs (it waits there for this grid to finish): its launch latency is hidden.
   if (early_trigger) pdl_launch_dependents();
 #endif
   const int row = blockIdx.y;
   clear.run(row);
-  if (block_tokens[row] != mask_id) return;  // already unmasked: never read
-  reduce_slice(logits + (int64_t)row * row_stride, V, chunk, (int)blockIdx.x,
-               partials + (int64_t)row * splits + blockIdx.x);
+  if (__ldcg(block_tokens + row) == mask_id)  // already unmasked: never read
+    reduce_slice(logits + (int64_t)row * row_stride, V, chunk, (int)blockIdx.x,
+                 partials + (int64_t)row * splits + blockIdx.x);
+#if __CUDA_ARCH__ >= 900
+  // This grid is complete, for all that wait for it, no sooner than the one before it.
+  if (independent && blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y) cudaGridDependencySynchronize();
+#endif
 }
 
 // grid = B*N nodes, 512 threads: eight threads per position merge the slices of
@@ -200,33 +206,33 @@ namespace {
 
 spiffy_status launch_reduce(const spiffy_decide_desc& d, const void* logits,
                             const int32_t* block_tokens, Partial* partials, int splits,
-                            int64_t chunk, int early_trigger, StatusClear clear, cudaStream_t stream) {
+                            int64_t chunk, int early_trigger, bool independent, StatusClear clear,
+                            cudaStream_t stream) {
   const int rows = d.batch * d.n_nodes * d.block_len;
   const dim3 grid(splits, rows);
   cudaError_t e;
   if (d.logits_dtype == SPIFFY_BF16)
     e = launch_pdl(decide_reduce_kernel<__nv_bfloat16>, grid, dim3(kReduceThreads), (size_t)0, stream,
                    static_cast<const __nv_bfloat16*>(logits), (int64_t)d.row_stride, (int)d.vocab,
-                   chunk, splits, block_tokens, (int)d.mask_token_id, partials, early_trigger, clear);
+                   chunk, splits, block_tokens, (int)d.mask_token_id, partials, early_trigger,
+                   (int)independent, clear);
   else
     e = launch_pdl(decide_reduce_kernel<float>, grid, dim3(kReduceThreads), (size_t)0, stream,
                    static_cast<const float*>(logits), (int64_t)d.row_stride, (int)d.vocab, chunk,
-                   splits, block_tokens, (int)d.mask_token_id, partials, early_trigger, clear);
+                   splits, block_tokens, (int)d.mask_token_id, partials, early_trigger, (int)independent, clear);
   count_launch();
   return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
 }
 
-}  // namespace
-
-spiffy_status launch_decide(const spiffy_decide_desc& d, const void* logits,
-                            const int32_t* block_tokens, float* conf,
-                            int32_t* top_tok, uint64_t* unmask_bits,
-                            int32_t* n_unmask, int32_t* dev_status, void* ws, bool fresh,
-                            cudaStream_t stream) {
+spiffy_status decide_only(const spiffy_decide_desc& d, const void* logits,
+                          const int32_t* block_tokens, float* conf,
+                          int32_t* top_tok, uint64_t* unmask_bits,
+                          int32_t* n_unmask, int32_t* dev_status, void* ws, bool fresh, bool independent,
+                          cudaStream_t stream) {
   int64_t chunk = 0;
   const int splits = decide_splits(d, &chunk);
   Partial* partials = static_cast<Partial*>(ws);
-  const spiffy_status st = launch_reduce(d, logits, block_tokens, partials, splits, chunk, 0,
+  const spiffy_status st = launch_reduce(d, logits, block_tokens, partials, splits, chunk, 0, independent,
                                          status_clear(d, fresh, dev_status, nullptr), stream);
   if (st != SPIFFY_OK) return st;
   // The finalize kernel's launch overlaps the tail of the reduce kernel; it
@@ -239,6 +245,15 @@ spiffy_status launch_decide(const spiffy_decide_desc& d, const void* logits,
                  unmask_bits, n_unmask, dev_status);
   count_launch();
   return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
+}
+
+}  // namespace
+
+spiffy_status launch_decide(const spiffy_decide_desc& d, const void* logits, const int32_t* block_tokens,
+                            float* conf, int32_t* top_tok, uint64_t* unmask_bits, int32_t* n_unmask,
+                            int32_t* dev_status, void* ws, bool fresh, cudaStream_t stream) {
+  return decide_only(d, logits, block_tokens, conf, top_tok, unmask_bits, n_unmask, dev_status, ws, fresh, false,
+                     stream);
 }
 
 // The finalize kernel alone, on partial results another kernel produced
@@ -269,11 +284,11 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
                                  const int32_t* parent_idx, int32_t parent_cap,
                                  int32_t* accepted_node, int32_t* n_accepted, int32_t* path,
                                  int32_t* next_block, int32_t* walk_status, void* ws,
-                                 bool fresh, cudaStream_t stream) {
+                                 bool fresh, bool independent, cudaStream_t stream) {
   const size_t smem = tail_smem_bytes(d, parent_cap);
   if ((int64_t)d.n_nodes * d.block_len > kTailRows || smem > 48 * 1024) {
-    const spiffy_status st = launch_decide(d, logits, block_tokens, conf, top_tok, unmask_bits,
-                                           n_unmask, decide_status, ws, fresh, stream);
+    const spiffy_status st = decide_only(d, logits, block_tokens, conf, top_tok, unmask_bits,
+                                         n_unmask, decide_status, ws, fresh, independent, stream);
     if (st != SPIFFY_OK) return st;
     return launch_walk(d, block_tokens, parent_off, parent_idx, parent_cap, top_tok, unmask_bits,
                        accepted_node, n_accepted, path, next_block, walk_status, fresh, stream);
@@ -281,7 +296,7 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
   int64_t chunk = 0;
   const int splits = decide_splits(d, &chunk);
   Partial* partials = static_cast<Partial*>(ws);
-  const spiffy_status st = launch_reduce(d, logits, block_tokens, partials, splits, chunk, 1,
+  const spiffy_status st = launch_reduce(d, logits, block_tokens, partials, splits, chunk, 1, independent,
                                          status_clear(d, fresh, decide_status, walk_status), stream);
   if (st != SPIFFY_OK) return st;
   const Partial* cpart = partials;

@@ -86,6 +86,13 @@ class VerifyStep:
             torch.empty((B, N), dtype=torch.int32, device=dev),
             torch.empty((B, L), dtype=torch.int32, device=dev),
             torch.zeros((B,), dtype=torch.int32, device=dev))
+        # The decision takes nothing from the attention, so a step runs the two side by side.  Not so
+        # where the attention is one round of CTAs that hold whole SMs and the decision long: begun on
+        # the SMs left over, it spreads badly over the others later (16 nodes x 32 positions x 28 heads
+        # and 156 MB of logits: 43.4 us one after the other, 45.5 side by side; at 19 MB 19.4 and 15.1).
+        m_tiles = B * cfg.n_kv_heads * -(-N * L * cfg.n_q_heads // (cfg.n_kv_heads * 128))
+        logits_bytes = B * N * L * cfg.vocab * self.attn_out.element_size()
+        self.side_by_side = cfg.dtype != "bf16" or m_tiles > 2 * 148 or logits_bytes <= 40 << 20
         self.host_ws = None
         self.host_desc = None
         self.host_verdict = None
@@ -139,8 +146,17 @@ class VerifyStep:
         return self.walk
 
     def run(self, x: StepInputs):
-        self.attention(x)
-        return self.decide_accept(x)
+        if not self.side_by_side:
+            self.attention(x)
+            return self.decide_accept(x)
+        c = self.cfg
+        spiffy.spiffy_graph_attention(x.q, x.k_prefix, x.v_prefix, x.k_block, x.v_block, out=self.attn_out,
+                                      kernel=self.attn_kernel | spiffy.ATTN_INDEPENDENT_NEXT,
+                                      dev_status=self.attn_status, workspace=self.attn_ws)
+        spiffy.spiffy_decide_walk(x.logits, x.block_tokens, x.parent_off, x.parent_idx, c.mask_id,
+                                  c.rule, c.top_s, c.threshold, decision=self.decision,
+                                  walk=self.walk, workspace=self.decide_ws, independent=True)
+        return self.walk
 
     def run_host(self, host: StepInputs):
         """End to end from pinned host memory through the C ABI's host-buffer

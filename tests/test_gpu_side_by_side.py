@@ -1,0 +1,47 @@
+"""VerifyStep.run, where the decision starts beside the attention, against the
+same calls one after the other: bit-identical on every path the two kernels
+have (tail in one CTA, separate finalize and walk, both attention kernels, one
+and several rounds of CTAs), many steps back to back on alternating inputs."""
+import dataclasses
+
+import pytest
+import torch
+
+from paper_2509_18085_b200 import spiffy
+from paper_2509_18085_b200 import workloads as W
+from paper_2509_18085_b200.step import VerifyStep, inputs_from_workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,N,L,P,Hq,Hkv,d,V,dtype", [
+    (1, 2, 4, 0, 4, 4, 128, 1000, "bf16"),      # nothing to share the machine with
+    (3, 24, 4, 764, 24, 8, 128, 4000, "bf16"),  # one nearly full round of clusters
+    (1, 54, 32, 300, 28, 4, 64, 4072, "bf16"),  # more than 512 rows: finalize and walk kernels
+    (2, 16, 32, 2000, 32, 32, 128, 8192, "bf16"),  # several rounds
+    (2, 3, 32, 500, 5, 5, 128, 2864, "f32"),
+])
+def test_same_bits_as_one_after_the_other(B, N, L, P, Hq, Hkv, d, V, dtype):
+    cfg = W.Config("t", B, N, L, P, Hq, Hkv, d, dtype, V, spiffy.RULE_THRESHOLD)
+    step, apart = VerifyStep(cfg), VerifyStep(cfg)
+    step.side_by_side = True
+    xs = [inputs_from_workload(W.make(cfg, s)) for s in (1, 2, 3)]
+    want = []
+    for x in xs:
+        apart.attention(x)
+        apart.decide_accept(x)
+        want.append(_results(apart))
+    for i in range(30):
+        step.run(xs[i % 3])
+        if i % 7 == 0 or i > 26:
+            for a, b in zip(_results(step), want[i % 3]):
+                assert torch.equal(a, b)
+
+
+def _results(s):
+    out = [s.attn_out, s.attn_status] + list(_fields(s.decision)) + list(_fields(s.walk))
+    return [t.clone().view(torch.uint8) for t in out]
+
+
+def _fields(x):
+    return [getattr(x, f.name) for f in dataclasses.fields(x)] if dataclasses.is_dataclass(x) else list(x)
