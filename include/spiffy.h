@@ -101,11 +101,16 @@ typedef enum { SPIFFY_RULE_TOPS = 0, SPIFFY_RULE_THRESHOLD = 1 } spiffy_rule;
  * also writes 0 to the entries of parent_idx behind its lists.)  Spares a caller
  * that allocates its outputs for the call the clearing of them. */
 #define SPIFFY_FRESH_STATUS 0x100
-/* Flag, OR-ed into spiffy_decide_desc.logits_dtype of spiffy_decide_walk: none of
- * the call's inputs is written by the call before it in the stream, which is an
- * attention call with SPIFFY_ATTN_INDEPENDENT_NEXT.  The two then run side by
- * side.  What follows in the stream still follows both.  Other calls ignore it. */
+/* Flags, OR-ed into spiffy_decide_desc.logits_dtype of spiffy_decide_walk (other
+ * calls ignore them), for a decision and an attention that take nothing from one
+ * another and follow one another in a stream: they then run side by side, and
+ * what follows in the stream still follows both.
+ * SPIFFY_INDEPENDENT: the call before this one is an attention call on the
+ * CUDA-core kernel and writes none of this call's inputs.
+ * SPIFFY_INDEPENDENT_NEXT: the next call is an attention call with
+ * SPIFFY_ATTN_INDEPENDENT. */
 #define SPIFFY_INDEPENDENT 0x200
+#define SPIFFY_INDEPENDENT_NEXT 0x400
 
 /* Attention kernel selection (spiffy_attn_desc.kernel). */
 #define SPIFFY_ATTN_AUTO 0   /* tensor-core kernel when the shape allows it: bf16,
@@ -120,10 +125,10 @@ typedef enum { SPIFFY_RULE_TOPS = 0, SPIFFY_RULE_THRESHOLD = 1 } spiffy_rule;
  * this call's complete output).  For the layer loop of a model, where the next
  * kernel's set-up then overlaps this kernel's tail.  Tensor-core kernel only. */
 #define SPIFFY_ATTN_EARLY_DEPENDENTS 0x100
-/* Flag, OR-ed into spiffy_attn_desc.kernel: the next call of the stream is a
- * decision with SPIFFY_INDEPENDENT.  Such a decision may start as soon as what
- * precedes this call is complete. */
-#define SPIFFY_ATTN_INDEPENDENT_NEXT 0x200
+/* Flag, OR-ed into spiffy_attn_desc.kernel: the call before this one in the stream
+ * is spiffy_decide_walk with SPIFFY_INDEPENDENT_NEXT, and none of this call's
+ * inputs or outputs is touched by it.  Tensor-core kernel only. */
+#define SPIFFY_ATTN_INDEPENDENT 0x200
 
 /* ------------------------------------------------------------------------- */
 /* Packed draft-graph attention (Sec. 4.3; mask semantics: caption of Fig. 3) */
@@ -203,7 +208,7 @@ typedef struct {
   int32_t n_nodes;       /* N                                                */
   int32_t block_len;     /* L in [1, 64]                                     */
   int32_t vocab;         /* V >= 1                                           */
-  int32_t logits_dtype;  /* spiffy_dtype, | SPIFFY_FRESH_STATUS, SPIFFY_INDEPENDENT */
+  int32_t logits_dtype;  /* spiffy_dtype, | the flags above          */
   int64_t row_stride;    /* elements between consecutive logits rows, >= V;
                             row_stride * sizeof(element) must be a multiple
                             of 16                                            */

@@ -29,7 +29,7 @@ spiffy_status check_attn_desc(const spiffy_attn_desc* d) {
   if (d->n_q_heads % d->n_kv_heads != 0) return SPIFFY_EINVAL;
   if (d->dtype != SPIFFY_F32 && d->dtype != SPIFFY_BF16) return SPIFFY_EINVAL;
   if (!(d->scale >= 0.f) || !(d->scale < INFINITY)) return SPIFFY_EINVAL;
-  if (d->kernel & ~(0xff | SPIFFY_ATTN_EARLY_DEPENDENTS | SPIFFY_ATTN_INDEPENDENT_NEXT)) return SPIFFY_EINVAL;
+  if (d->kernel & ~(0xff | SPIFFY_ATTN_EARLY_DEPENDENTS | SPIFFY_ATTN_INDEPENDENT)) return SPIFFY_EINVAL;
   if ((d->kernel & 0xff) > SPIFFY_ATTN_TCGEN05) return SPIFFY_EINVAL;
   if (d->block_len > 1024) return SPIFFY_EUNSUPPORTED;
   if (d->head_dim != 64 && d->head_dim != 128) return SPIFFY_EUNSUPPORTED;
@@ -52,7 +52,7 @@ spiffy_status check_decide_desc(const spiffy_decide_desc* d, bool need_vocab) {
   if ((int64_t)d->batch * d->n_nodes * d->block_len > 65535) return SPIFFY_EUNSUPPORTED;
   if (!need_vocab) return SPIFFY_OK;
   if (d->vocab < 1) return SPIFFY_EINVAL;
-  const int dtype = d->logits_dtype & ~(SPIFFY_FRESH_STATUS | SPIFFY_INDEPENDENT);
+  const int dtype = d->logits_dtype & ~(SPIFFY_FRESH_STATUS | SPIFFY_INDEPENDENT | SPIFFY_INDEPENDENT_NEXT);
   if (dtype != SPIFFY_F32 && dtype != SPIFFY_BF16) return SPIFFY_EINVAL;
   if (d->row_stride < d->vocab) return SPIFFY_EINVAL;
   const int64_t esize = dtype == SPIFFY_BF16 ? 2 : 4;
@@ -65,11 +65,12 @@ spiffy_status check_decide_desc(const spiffy_decide_desc* d, bool need_vocab) {
 
 // The descriptor as the kernels' launchers take it: the flags in variables of their own.
 template <typename Desc>
-Desc split_flags(const Desc* desc, bool* fresh, bool* independent = nullptr) {
+Desc split_flags(const Desc* desc, bool* fresh, bool* independent = nullptr, bool* next = nullptr) {
   Desc d = *desc;
   *fresh = (d.logits_dtype & SPIFFY_FRESH_STATUS) != 0;
   if (independent) *independent = (d.logits_dtype & SPIFFY_INDEPENDENT) != 0;
-  d.logits_dtype &= ~(SPIFFY_FRESH_STATUS | SPIFFY_INDEPENDENT);
+  if (next) *next = (d.logits_dtype & SPIFFY_INDEPENDENT_NEXT) != 0;
+  d.logits_dtype &= ~(SPIFFY_FRESH_STATUS | SPIFFY_INDEPENDENT | SPIFFY_INDEPENDENT_NEXT);
   return d;
 }
 
@@ -240,14 +241,14 @@ spiffy_status spiffy_decide_walk(const spiffy_decide_desc* desc, const void* log
       !parent_idx || !accepted_node || !n_accepted || !path || !next_block)
     return SPIFFY_EINVAL;
   if (!aligned16(logits) || parent_cap < 0) return SPIFFY_EINVAL;
-  bool fresh, independent;
-  const spiffy_decide_desc d = split_flags(desc, &fresh, &independent);
+  bool fresh, independent, next;
+  const spiffy_decide_desc d = split_flags(desc, &fresh, &independent, &next);
   const size_t need = decide_workspace_bytes(d);
   if (!workspace || workspace_bytes < need || !aligned16(workspace)) return SPIFFY_EWORKSPACE;
   return launch_decide_walk(d, logits, block_tokens, conf, top_tok, unmask_bits, n_unmask,
                             decide_status, parent_off, parent_idx, parent_cap, accepted_node,
                             n_accepted, path, next_block, walk_status, workspace,
-                            fresh, independent, static_cast<cudaStream_t>(cuda_stream));
+                            fresh, independent, next, static_cast<cudaStream_t>(cuda_stream));
 }
 
 size_t spiffy_decide_walk_lazy_workspace(const spiffy_decide_desc* desc) {

@@ -119,9 +119,8 @@ struct Params {
   __nv_bfloat16* out;
   int32_t* status;
   uint32_t spin_limit;  // polls of one mbarrier wait
-  // Lets the next kernel of the stream start while this one runs: 1 as soon as may be (it waits for
-  // this one by itself), 2 once what precedes this one is complete (it does not); 0 not.
-  int trigger;
+  int early_trigger;    // let the next kernel of the stream begin its set-up while this one runs
+  int independent;      // the kernel before this one writes none of its inputs: waited for at the end
 };
 
 // The operands of one attention problem: Q, two context segments, block keys.
@@ -319,7 +318,7 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
   if (threadIdx.x == 0) {
     // what the others will send in the epilogue: this CTA's rows, and (maximum, sum) of each
     if (cs > 1) mbar_arrive_expect_tx(xchg_full, (uint32_t)((cs - 1) * (BM / cs) * (kRowBytes + 8)));
-    cudaGridDependencySynchronize();
+    if (!p.independent) cudaGridDependencySynchronize();
     mbar_arrive_expect_tx(q_full, (uint32_t)(NQ * kHalves) * rows_box * 128u);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {  // an M-tile beyond the last one reads as zeros
@@ -344,10 +343,9 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
   const uint32_t tmem = *tmem_slot;
   // all CTAs' barriers exist before any touches another's (waited for in the epilogue)
   if (cs > 1) cluster_arrive_relaxed();
-  if (p.trigger == 1) pdl_launch_dependents();
+  if (p.early_trigger) pdl_launch_dependents();
   // everything above is on-chip set-up (thread 0 aside); global memory is touched from here on
-  cudaGridDependencySynchronize();
-  if (p.trigger == 2) pdl_launch_dependents();
+  if (!p.independent) cudaGridDependencySynchronize();
 
   const int U = T << kLogNQ;  // units of this CTA
   if (warp < 4) {
@@ -716,6 +714,7 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
   }
+  if (p.independent) cudaGridDependencySynchronize();  // complete no sooner than the kernel before
   if (threadIdx.x == 0 && *abort_flag && p.status) atomicOr(p.status, SPIFFY_DEV_TIMEOUT);
 }
 
@@ -835,7 +834,8 @@ bool make_problem(const spiffy_attn_desc& d, const Shape& sh, const AttnProblem&
   p->out = static_cast<__nv_bfloat16*>(a.out);
   p->status = dev_status;
   p->spin_limit = mbar_poll_limit();
-  p->trigger = (d.kernel & SPIFFY_ATTN_INDEPENDENT_NEXT) ? 2 : (d.kernel & SPIFFY_ATTN_EARLY_DEPENDENTS) ? 1 : 0;
+  p->early_trigger = (d.kernel & SPIFFY_ATTN_EARLY_DEPENDENTS) ? 1 : 0;
+  p->independent = (d.kernel & SPIFFY_ATTN_INDEPENDENT) ? 1 : 0;
   return ok;
 }
 
@@ -869,11 +869,6 @@ spiffy_status launch(const spiffy_attn_desc* const (&d)[NP], const AttnProblem* 
     if (i == 1) pr.x_split = x;
     x += (sh[i].MT + pl.nq - 1) / pl.nq;
   }
-  // An independent kernel next finds few SMs when one round of CTAs fills nearly all: it then gains
-  // nothing and its first CTAs pile up on those few (144 CTAs: a step of 19.9 us took 20.6).
-  const int64_t ctas = (int64_t)x * bg * pl.cs;
-  for (int i = 0; i < NP; ++i)
-    if (pr.p[i].trigger == 2 && ctas > 132 && ctas <= 148) pr.p[i].trigger = 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)x, (unsigned)bg, (unsigned)pl.cs);
   cfg.blockDim = dim3(kThreads);

@@ -460,7 +460,7 @@ PyObject* accept_walk(PyObject* const* a) {
 }
 
 // logits, block_tokens, mask_token_id, rule, top_s, threshold, parent_off, parent_idx, decision, walk, workspace,
-// stream, lazy, independent
+// stream, lazy, flags
 PyObject* decide_walk(PyObject* const* a) {
   const at::Tensor& logits = tensor(a[0], "logits");
   const at::Tensor& tokens = tensor(a[1], "block_tokens");
@@ -470,9 +470,9 @@ PyObject* decide_walk(PyObject* const* a) {
   const int64_t B = d.batch, N = d.n_nodes, L = d.block_len;
   const int32_t cap = parent_cap(off, idx, B, N);
   const int lazy = PyObject_IsTrue(a[12]);
-  const int independent = PyObject_IsTrue(a[13]);
-  if (lazy < 0 || independent < 0) throw PyError{};
-  if (independent) d.logits_dtype |= SPIFFY_INDEPENDENT;
+  const long flags = PyLong_AsLong(a[13]);
+  if (lazy < 0 || (flags == -1 && PyErr_Occurred())) throw PyError{};
+  d.logits_dtype |= (int32_t)flags & (SPIFFY_INDEPENDENT | SPIFFY_INDEPENDENT_NEXT);
   const void* lp = logits_ptr(logits);
   const int32_t* tp = (const int32_t*)device_ptr(tokens, "block_tokens", at::kInt);
   const int32_t* op = (const int32_t*)device_ptr(off, "parent_off", at::kInt);

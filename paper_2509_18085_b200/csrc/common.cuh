@@ -98,7 +98,7 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
                                  const int32_t* parent_idx, int32_t parent_cap,
                                  int32_t* accepted_node, int32_t* n_accepted, int32_t* path,
                                  int32_t* next_block, int32_t* walk_status, void* ws,
-                                 bool fresh, bool independent, cudaStream_t stream);
+                                 bool fresh, bool independent, bool next, cudaStream_t stream);
 
 size_t decide_lazy_workspace_bytes(const spiffy_decide_desc& d);
 spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc& d, const void* logits,

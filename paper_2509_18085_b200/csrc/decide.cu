@@ -107,7 +107,7 @@ decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int 
                    const int32_t* __restrict__ parent_off, const int32_t* __restrict__ parent_idx,
                    int parent_cap, int32_t* __restrict__ accepted_node,
                    int32_t* __restrict__ n_accepted, int32_t* __restrict__ path,
-                   int32_t* __restrict__ next_block, int32_t* __restrict__ walk_status) {
+                   int32_t* __restrict__ next_block, int32_t* __restrict__ walk_status, int early_trigger) {
   extern __shared__ __align__(8) unsigned char tail_smem[];
   const int b = blockIdx.x;
   const int rows = N * L;
@@ -134,6 +134,7 @@ decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int 
     for (int i = threadIdx.x; i < N; i += kTailThreads) s_link[i] = kNoLink;
   }
 #if __CUDA_ARCH__ >= 900
+  if (early_trigger) pdl_launch_dependents();  // an independent kernel comes next, and takes the SMs the reduce leaves
   cudaGridDependencySynchronize();  // the reduce kernel's partials are visible
   pdl_launch_dependents();          // only now: this CTA was resident during the reduce, the next kernel's need not be
 #endif
@@ -284,7 +285,7 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
                                  const int32_t* parent_idx, int32_t parent_cap,
                                  int32_t* accepted_node, int32_t* n_accepted, int32_t* path,
                                  int32_t* next_block, int32_t* walk_status, void* ws,
-                                 bool fresh, bool independent, cudaStream_t stream) {
+                                 bool fresh, bool independent, bool next, cudaStream_t stream) {
   const size_t smem = tail_smem_bytes(d, parent_cap);
   if ((int64_t)d.n_nodes * d.block_len > kTailRows || smem > 48 * 1024) {
     const spiffy_status st = decide_only(d, logits, block_tokens, conf, top_tok, unmask_bits,
@@ -306,7 +307,7 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
                       (int)d.n_nodes, (int)d.block_len, block_tokens, (int)d.mask_token_id,
                       (int)d.rule, (int)d.top_s, d.threshold, conf, top_tok, unmask_bits, n_unmask,
                       decide_status, parent_off, parent_idx, (int)parent_cap, accepted_node,
-                      n_accepted, path, next_block, walk_status);
+                      n_accepted, path, next_block, walk_status, (int)next);
   };
   const cudaError_t e = rows <= kTailThreads / 8   ? launch(decide_tail_kernel<8>)
                         : rows <= kTailThreads / 4 ? launch(decide_tail_kernel<4>)

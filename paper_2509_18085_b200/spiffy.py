@@ -25,7 +25,9 @@ RULE_TOPS, RULE_THRESHOLD = 0, 1
 DEV_NONFINITE, DEV_BADGRAPH, DEV_TIMEOUT = 1, 2, 4
 ATTN_AUTO, ATTN_SIMT, ATTN_TCGEN05 = 0, 1, 2
 ATTN_EARLY_DEPENDENTS = 0x100  # flags OR-ed into the kernel selection
-ATTN_INDEPENDENT_NEXT = 0x200
+ATTN_INDEPENDENT = 0x200
+INDEPENDENT = 0x200            # flags of spiffy_decide_walk
+INDEPENDENT_NEXT = 0x400
 
 DECIDE_STATIC_BYTES = 2 << 20
 
@@ -338,17 +340,17 @@ def spiffy_decide_walk_lazy_workspace(desc: DecideDesc) -> int:
 def spiffy_decide_walk(logits, block_tokens, parent_off, parent_idx, mask_token_id: int, rule: int,
                        top_s: int = 1, threshold: float = 0.9, decision: Optional[Decision] = None,
                        walk: Optional[Walk] = None, workspace=None, stream=None, lazy: bool = False,
-                       independent: bool = False):
+                       flags: int = 0):
     """Steps 1-5 of Algorithm 1 in one call: spiffy_unmask_decide followed by
     spiffy_accept_walk, fused on the device for small graphs.  With ``lazy`` the
     decision is evaluated only for the nodes the walk reaches
     (spiffy_decide_walk_lazy): the Decision then holds those nodes' entries and
-    n_unmask = -1 everywhere else.  ``independent``: the call before this one in
-    the stream is an attention with ATTN_INDEPENDENT_NEXT and writes none of
-    this call's inputs, so that the two run side by side.
+    n_unmask = -1 everywhere else.  ``flags``: INDEPENDENT (of the
+    CUDA-core attention call before this one) or INDEPENDENT_NEXT (an attention
+    with ATTN_INDEPENDENT comes next), so that the two run side by side.
     Returns (Decision, Walk)."""
     return _native().decide_walk(logits, block_tokens, mask_token_id, rule, top_s, threshold, parent_off, parent_idx,
-                                 decision, walk, workspace, stream, lazy, independent)
+                                 decision, walk, workspace, stream, lazy, flags)
 
 
 def spiffy_stage_masked_rows(src_logits, dst_logits, tokens, mask_token_id: int, stream=None):

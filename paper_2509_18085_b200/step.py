@@ -86,13 +86,14 @@ class VerifyStep:
             torch.empty((B, N), dtype=torch.int32, device=dev),
             torch.empty((B, L), dtype=torch.int32, device=dev),
             torch.zeros((B,), dtype=torch.int32, device=dev))
-        # The decision takes nothing from the attention, so a step runs the two side by side.  Not so
-        # where the attention is one round of CTAs that hold whole SMs and the decision long: begun on
-        # the SMs left over, it spreads badly over the others later (16 nodes x 32 positions x 28 heads
-        # and 156 MB of logits: 43.4 us one after the other, 45.5 side by side; at 19 MB 19.4 and 15.1).
-        m_tiles = B * cfg.n_kv_heads * -(-N * L * cfg.n_q_heads // (cfg.n_kv_heads * 128))
-        logits_bytes = B * N * L * cfg.vocab * self.attn_out.element_size()
-        self.side_by_side = cfg.dtype != "bf16" or m_tiles > 2 * 148 or logits_bytes <= 40 << 20
+        # A step's attention and decision take nothing from one another and run side by side.  The
+        # tensor-core kernel's CTAs hold whole SMs: they come second and move in as the reduce kernel
+        # lets go, the decision's tail runs beside them (16 nodes x 32 positions x 28 heads, 156 MB of
+        # logits: 44 -> 36 us; attention first: 45).  The CUDA-core kernel's come several to an SM and
+        # would crowd the first ones that are free: there the decision comes second (8 positions x 24
+        # heads over 3249 keys: 38 -> 34 us; attention second: 42).
+        self.attention_second = (cfg.dtype == "bf16" and attn_kernel != spiffy.ATTN_SIMT
+                                 and cfg.n_q_heads <= 128 * cfg.n_kv_heads)
         self.host_ws = None
         self.host_desc = None
         self.host_verdict = None
@@ -100,10 +101,13 @@ class VerifyStep:
         self.sampled_ws = None
 
     # the three calls of one step, asynchronous on the current stream
-    def attention(self, x: StepInputs):
+    def _attention(self, x: StepInputs, flags=0):
         return spiffy.spiffy_graph_attention(x.q, x.k_prefix, x.v_prefix, x.k_block, x.v_block,
-                                             out=self.attn_out, kernel=self.attn_kernel,
+                                             out=self.attn_out, kernel=self.attn_kernel | flags,
                                              dev_status=self.attn_status, workspace=self.attn_ws)
+
+    def attention(self, x: StepInputs):
+        return self._attention(x)
 
     def decide(self, x: StepInputs):
         c = self.cfg
@@ -115,12 +119,15 @@ class VerifyStep:
                                          self.decision.top_tok, self.decision.unmask_bits,
                                          out=self.walk)
 
-    def decide_accept(self, x: StepInputs):
+    def _decide_walk(self, x: StepInputs, flags=0):
         c = self.cfg
         spiffy.spiffy_decide_walk(x.logits, x.block_tokens, x.parent_off, x.parent_idx, c.mask_id,
                                   c.rule, c.top_s, c.threshold, decision=self.decision,
-                                  walk=self.walk, workspace=self.decide_ws)
+                                  walk=self.walk, workspace=self.decide_ws, flags=flags)
         return self.walk
+
+    def decide_accept(self, x: StepInputs):
+        return self._decide_walk(x)
 
     def decide_sampled(self, x: StepInputs, temperature: float = 1.0, seed: int = 1):
         """The decision at sampling temperature T > 0 (spiffy_unmask_decide_sampled)."""
@@ -146,16 +153,12 @@ class VerifyStep:
         return self.walk
 
     def run(self, x: StepInputs):
-        if not self.side_by_side:
-            self.attention(x)
-            return self.decide_accept(x)
-        c = self.cfg
-        spiffy.spiffy_graph_attention(x.q, x.k_prefix, x.v_prefix, x.k_block, x.v_block, out=self.attn_out,
-                                      kernel=self.attn_kernel | spiffy.ATTN_INDEPENDENT_NEXT,
-                                      dev_status=self.attn_status, workspace=self.attn_ws)
-        spiffy.spiffy_decide_walk(x.logits, x.block_tokens, x.parent_off, x.parent_idx, c.mask_id,
-                                  c.rule, c.top_s, c.threshold, decision=self.decision,
-                                  walk=self.walk, workspace=self.decide_ws, independent=True)
+        if self.attention_second:
+            self._decide_walk(x, spiffy.INDEPENDENT_NEXT)
+            self._attention(x, spiffy.ATTN_INDEPENDENT)
+        else:
+            self._attention(x)
+            self._decide_walk(x, spiffy.INDEPENDENT)
         return self.walk
 
     def run_host(self, host: StepInputs):

@@ -1,4 +1,4 @@
-"""VerifyStep.run, where the decision starts beside the attention, against the
+"""VerifyStep.run, where decision and attention run side by side, against the
 same calls one after the other: bit-identical on every path the two kernels
 have (tail in one CTA, separate finalize and walk, both attention kernels, one
 and several rounds of CTAs), many steps back to back on alternating inputs."""
@@ -24,7 +24,6 @@ pytestmark = pytest.mark.gpu
 def test_same_bits_as_one_after_the_other(B, N, L, P, Hq, Hkv, d, V, dtype):
     cfg = W.Config("t", B, N, L, P, Hq, Hkv, d, dtype, V, spiffy.RULE_THRESHOLD)
     step, apart = VerifyStep(cfg), VerifyStep(cfg)
-    step.side_by_side = True
     xs = [inputs_from_workload(W.make(cfg, s)) for s in (1, 2, 3)]
     want = []
     for x in xs:
