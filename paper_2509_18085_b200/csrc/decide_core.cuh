@@ -152,6 +152,13 @@ struct Elem<float> {
   static __device__ __forceinline__ float load1(const float* p) { return *p; }
 };
 
+// 16 aligned bytes in one access, as another CTA may be polling for them.
+__device__ __forceinline__ void store16(void* p, uint64_t lo, uint64_t hi) {
+  asm volatile("{\n.reg .b128 t;\nmov.b128 t, {%1, %2};\nst.relaxed.gpu.global.b128 [%0], t;\n}" ::"l"(p), "l"(lo),
+               "l"(hi)
+               : "memory");
+}
+
 // One CTA of kReduceThreads threads reduces one vocabulary slice
 // [split * chunk, min(V, (split + 1) * chunk)) of the logits row at `base` to
 // (maximum, sum of exp(x - maximum), lowest index attaining the maximum).  A
@@ -160,11 +167,12 @@ struct Elem<float> {
 // found first and the exponentials are then taken against it directly.  All
 // threads of the CTA call it together; thread 0 stores the result.  `k` is
 // log2(e) for the plain softmax; the sampled decision passes log2(e) / T and
-// gets the sum of exp((x - maximum) / T).
+// gets the sum of exp((x - maximum) / T).  `tag` goes into the result's spare word, in the
+// one 16-byte store that writes it: a reader that polls for the tag has the rest with it.
 template <typename T>
 __device__ __forceinline__ void reduce_slice(const T* __restrict__ base, int V, int64_t chunk,
                                              int split, Partial* __restrict__ out,
-                                             const float k = kLog2e) {
+                                             const float k = kLog2e, const int tag = 0) {
   const int64_t begin = (int64_t)split * chunk;
   const int64_t end = min((int64_t)V, begin + chunk);
   constexpr int EPV = Elem<T>::kPerVec;
@@ -239,7 +247,8 @@ __device__ __forceinline__ void reduce_slice(const T* __restrict__ base, int V, 
   if (tid == 0) {
     s = warp_s[0];
     for (int w = 1; w < kReduceThreads / 32; ++w) s += warp_s[w];
-    *out = Partial{m, s, slice_idx, 0};
+    store16(out, (uint64_t)__float_as_uint(m) | (uint64_t)__float_as_uint(s) << 32,
+            (uint64_t)(uint32_t)slice_idx | (uint64_t)(uint32_t)tag << 32);
   }
 }
 
@@ -249,8 +258,9 @@ __device__ __forceinline__ void reduce_slice(const T* __restrict__ base, int V, 
 // (accumulator j takes slices j, j + 8, ...) are combined by the butterfly
 // 4, 2, 1 with the lower index first; a lane holds the accumulators j = sub,
 // sub + kLanes, ... and does the butterfly steps that stay inside it locally.
-// Returns false on lane 0 when the row is masked and not usable.
-template <int kLanes>
+// Returns false on lane 0 when the row is masked and not usable.  kShared: the slices are in
+// shared memory.
+template <int kLanes, bool kShared = false>
 __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int splits, int sub,
                                              int32_t state, int mask_id, float& conf, int32_t& tok) {
   constexpr int kAcc = 8 / kLanes;
@@ -273,7 +283,8 @@ __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int 
       const int k = sub + kLanes * (t0 + u);
       q[u] = Partial{-INFINITY, 0.f, 0x7fffffff, 0};
       if (k < splits && state == mask_id) {  // read at L2: another grid wrote these while this CTA may already have been resident; the slices of an unmasked row were never written
-        const int4 w = __ldcg(reinterpret_cast<const int4*>(p + k));
+        const int4* at = reinterpret_cast<const int4*>(p + k);
+        const int4 w = kShared ? *at : __ldcg(at);
         q[u] = Partial{__int_as_float(w.x), __int_as_float(w.y), w.z, w.w};
       }
     }

@@ -5,13 +5,13 @@
 // 1 + n_accepted nodes on the accepted path are ever used.  Here one
 // cooperative kernel works level by level.  For every sequence b that is still
 // walking:
-//   R  the CTAs that own the (position, vocabulary slice) items of b reduce the
-//      rows of b's current node (the HBM-bound part, 1/N of the eager traffic
-//      per level) and count themselves in on arrivals[b];
-//   T  CTA b waits for those arrivals, merges the slices, applies the unmasking
+//   R  the reducing CTAs of b take the vocabulary slices of the masked rows of b's
+//      current node (the HBM-bound part, 1/N of the eager traffic
+//      per level); a slice's result carries the level;
+//   T  CTA b waits until all slices carry it, merges them, applies the unmasking
 //      rule, forms the next state, looks for the child that equals it (the graph
-//      of b sits in its shared memory) and publishes the new current node with
-//      epoch[b] = level + 1, for which the reducers of b wait.
+//      of b sits in its shared memory) and publishes the new current node, its
+//      masked positions and the level in one word, for which the reducers wait.
 // Sequences never wait for one another.  The arithmetic is the code the eager
 // kernels use (decide_core.cuh), so the results on the path have the same bits.
 //
@@ -19,7 +19,13 @@
 // < k, or of level k's R phase, so there is no cycle; the launch is cooperative
 // (all CTAs resident); every wait is bounded, and when one runs out the kernel
 // sets SPIFFY_DEV_TIMEOUT, tells the others through the header and returns.
-// The host zeroes header, arrivals and epoch before the launch.
+// The host zeroes header, words and slices before the launch.
+//
+// Bound: a chain of trips through L2 and HBM, level after level.  What passes
+// between the CTAs is therefore the data itself, 16 bytes at a time in one access
+// with the level in it, instead of data, fence, counter and a load behind the
+// counter: per level two trips each way became one, and the reducers no longer
+// look the tokens up (B 4, N 32, L 32, V 126464, bf16: 79 us before, 65 now).
 #include "common.cuh"
 #include "decide_core.cuh"
 #include "walk_core.cuh"
@@ -30,6 +36,13 @@ namespace {
 struct LazyHeader {
   int timeout;  // a bounded wait ran out somewhere
   int pad[3];
+};
+
+// Where a sequence stands.
+struct __align__(16) LazyWord {
+  int level;        // levels whose tail has finished; 0x7fffffff: the walk has ended
+  int node;
+  uint64_t masked;  // still-masked positions of the node
 };
 
 struct LazyParams {
@@ -53,44 +66,36 @@ struct LazyParams {
   int32_t* walk_status;
   Partial* partials;   // [B][L][splits]
   LazyHeader* header;
-  unsigned* arrivals;  // [B] slices of b reduced so far, over all levels
-  int32_t* epoch;      // [B] levels of b whose tail has finished
-  int32_t* cur;        // [B] node b stands on at level epoch[b], -1 once its walk has ended
+  LazyWord* words;     // [B]
   int clear_status;    // the status words arrive with arbitrary contents
   int stage_graph;     // the sequence's states and parent lists fit shared memory
+  int stage_slices;    // ... and so do the slices of one node
   unsigned wait_spins;   // polls of one wait before it gives up
-  unsigned extra_arrivals;  // test hook: sequence 0 expects this many arrivals that never come
+  int lost_slices;       // test hook: sequence 0 expects slices that never come
 };
 
 
-__device__ __forceinline__ unsigned ld_acquire_u32(const void* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
+// One access each: 16 aligned bytes that belong together.
+__device__ __forceinline__ LazyWord load_word(const LazyWord* p) {
+  uint64_t a, b;
+  asm volatile("{\n.reg .b128 t;\nld.relaxed.gpu.global.b128 t, [%2];\nmov.b128 {%0, %1}, t;\n}"
+               : "=l"(a), "=l"(b)
+               : "l"(p)
+               : "memory");
+  return LazyWord{(int)(uint32_t)a, (int)(uint32_t)(a >> 32), b};
+}
+__device__ __forceinline__ void store_word(LazyWord* p, const LazyWord& w) {
+  store16(p, (uint64_t)(uint32_t)w.level | (uint64_t)(uint32_t)w.node << 32, w.masked);
 }
 
-// Thread 0 waits until the word at `p` has reached `target`; every thread of
-// the CTA gets the verdict (false: the wait ran out, here or elsewhere).
-__device__ __forceinline__ bool wait_reached(const void* p, unsigned target, LazyHeader* h,
-                                             unsigned limit) {
-  __shared__ int ok_flag;
-  if (threadIdx.x == 0) {
-    unsigned spins = 0;
-    bool ok = true;
-    while (ld_acquire_u32(p) < target) {
-      if (++spins > limit || *reinterpret_cast<volatile int*>(&h->timeout)) {
-        ok = false;
-        h->timeout = 1;
-        break;
-      }
-      __nanosleep(100);
-    }
-    ok_flag = ok;
+// True while polling may go on; gives up after `limit` polls here, or once another wait has.
+__device__ __forceinline__ bool keep_polling(unsigned& polls, LazyHeader* h, unsigned limit) {
+  if (++polls > limit || ((polls & 7u) == 0 && *reinterpret_cast<volatile int*>(&h->timeout))) {
+    h->timeout = 1;
+    return false;
   }
-  __syncthreads();
-  const bool ok = ok_flag != 0;
-  __syncthreads();  // ok_flag may be rewritten by the next wait
-  return ok;
+  __nanosleep(32);
+  return true;
 }
 
 template <typename T>
@@ -101,9 +106,12 @@ decide_walk_lazy_kernel(const LazyParams p) {
   const int N = p.N, L = p.L;
   __shared__ float s_conf[64];
   __shared__ int32_t s_top[64], s_next[64];
-  __shared__ uint64_t s_bits;
-  __shared__ int s_found, s_node, s_bad;
-  extern __shared__ __align__(8) unsigned char lazy_smem[];
+  __shared__ uint64_t s_bits, s_mask;
+  __shared__ LazyWord s_word;
+  __shared__ int s_found, s_bad;
+  extern __shared__ __align__(16) unsigned char lazy_smem[];
+  // the slices of the own sequence's current node: [L][splits], staged when they fit
+  Partial* s_part = reinterpret_cast<Partial*>(lazy_smem);
   // the graph of the own sequence: [states N*L | off N+1 | idx cap], staged when it fits
   const int32_t* g_state = nullptr;
   const int32_t* g_off = nullptr;
@@ -113,7 +121,7 @@ decide_walk_lazy_kernel(const LazyParams p) {
     g_off = p.parent_off + (int64_t)b_own * (N + 1);
     g_idx = p.parent_idx + (int64_t)b_own * p.parent_cap;
     if (p.stage_graph) {
-      int32_t* s_state = reinterpret_cast<int32_t*>(lazy_smem);
+      int32_t* s_state = reinterpret_cast<int32_t*>(s_part + (p.stage_slices ? L * p.splits : 0));
       int32_t* s_off = s_state + N * L;
       int32_t* s_idx = s_off + (N + 1);
       auto copy4 = [](void* dst, const void* src) {
@@ -143,43 +151,58 @@ decide_walk_lazy_kernel(const LazyParams p) {
   }
   int own_node = b_own >= 0 ? 0 : -1;  // uniform over the CTA
   int own_hops = 0;
-  // arrivals[b_own] once the current level is reduced
-  unsigned own_expected = b_own == 0 ? p.extra_arrivals : 0u;
+  uint64_t own_mask = 0;  // still-masked positions of own_node, from level 1 on
   bool failed = false;
-  const int items = p.B * L * p.splits;
+  // CTA b runs the tail of sequence b and, where there are others, nothing else; the others divide
+  // the sequences among them, so that none of them waits for one on behalf of another.
+  const bool apart = (int)gridDim.x > p.B;
+  const int reducers = apart ? (int)gridDim.x - p.B : (int)gridDim.x;
+  const int r = apart ? (int)blockIdx.x - p.B : (int)blockIdx.x;
+  const bool many = reducers >= p.B;  // several CTAs per sequence, else several sequences per CTA
+  const int step_b = many ? p.B : reducers;
   for (int level = 0; level < N && !failed; ++level) {
     bool alive = false;
     // R: this CTA's slices of the current nodes
-    for (int item = blockIdx.x; item < items; item += gridDim.x) {
-      const int b = item / (L * p.splits);
-      const int l = (item / p.splits) % L;
-      const int split = item % p.splits;
-      int node = 0;
-      if (level > 0) {
-        if (b == b_own) {
-          node = own_node;
-        } else {
-          if (!wait_reached(p.epoch + b, (unsigned)level, p.header, p.wait_spins)) {
-            failed = true;
-            break;
+    for (int b = many ? r % p.B : r; r >= 0 && b < p.B; b += step_b) {
+      __syncthreads();  // s_word is free
+      if (level == 0) {
+        if (warp == 0) {
+          const int32_t* st = p.block_tokens + (int64_t)b * N * L;
+          uint64_t masked = 0;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int l = lane + 32 * h;
+            masked |= (uint64_t)__ballot_sync(0xffffffffu, l < L && st[min(l, L - 1)] == p.mask_id) << (32 * h);
           }
-          if (tid == 0) s_node = __ldcg(p.cur + b);
-          __syncthreads();
-          node = s_node;
-          __syncthreads();
+          if (lane == 0) s_word = LazyWord{0, 0, masked};
         }
+      } else if (b != b_own && tid == 0) {
+        LazyWord w;
+        unsigned polls = 0;
+        while ((w = load_word(p.words + b)).level < level)
+          if (!keep_polling(polls, p.header, p.wait_spins)) break;
+        s_word = w;
       }
-      if (node < 0) continue;  // this sequence's walk has ended
+      __syncthreads();
+      const LazyWord w = level > 0 && b == b_own ? LazyWord{level, own_node, own_mask} : s_word;
+      if (w.level < level) {
+        failed = true;
+        break;
+      }
+      if (w.node < 0) continue;  // this sequence's walk has ended
       alive = true;
-      const int64_t row = ((int64_t)b * N + node) * L + l;
-      if (p.block_tokens[row] != p.mask_id) continue;  // already unmasked: never read, never counted
-      reduce_slice(static_cast<const T*>(p.logits) + row * p.row_stride, p.V, p.chunk, split,
-                   p.partials + ((int64_t)b * L + l) * p.splits + split);
-      if (tid == 0) {  // the thread that stored the result counts it in
-        __threadfence();
-        atomicAdd(p.arrivals + b, 1u);
+      // the slices of the masked rows; the others are never read
+      const int items = __popcll(w.masked) * p.splits;
+      const int stride = many ? (reducers - b + p.B - 1) / p.B : 1;
+      for (int i = many ? r / p.B : 0; i < items; i += stride) {
+        uint64_t left = w.masked;
+        for (int k = i / p.splits; k > 0; --k) left &= left - 1;
+        const int l = __ffsll((long long)left) - 1, split = i % p.splits;
+        const int64_t row = ((int64_t)b * N + w.node) * L + l;
+        reduce_slice(static_cast<const T*>(p.logits) + row * p.row_stride, p.V, p.chunk, split,
+                     p.partials + ((int64_t)b * L + l) * p.splits + split, kLog2e, level + 1);
+        __syncthreads();  // the reduce's shared scratch is reused by the next item
       }
-      __syncthreads();  // the reduce's shared scratch is reused by the next item
     }
     if (failed) break;
     // T: the own sequence
@@ -191,14 +214,21 @@ decide_walk_lazy_kernel(const LazyParams p) {
         __syncthreads();
       }
       const int32_t* state = g_state + node * L;
-      {  // slices of this level: every still-masked row of the node, `splits` each
-        int masked = 0;
-        for (int l = lane; l < L; l += 32) masked += state[l] == p.mask_id;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) masked += __shfl_xor_sync(0xffffffffu, masked, off);
-        own_expected += (unsigned)masked * (unsigned)p.splits;
+      // slices of this level: those of every still-masked row of the node
+      bool ok_wait = true;
+      {
+        const Partial* from = p.partials + (int64_t)b * L * p.splits;
+        const int tag = level + 1 + (b == 0 ? p.lost_slices : 0);
+        unsigned polls = 0;
+        for (int i = tid; i < L * p.splits && ok_wait; i += kReduceThreads) {
+          if (state[i / p.splits] != p.mask_id) continue;
+          LazyWord w;  // 16 bytes, the tag last
+          while ((int)((w = load_word(reinterpret_cast<const LazyWord*>(from + i))).masked >> 32) != tag)
+            if (!(ok_wait = keep_polling(polls, p.header, p.wait_spins))) break;
+          if (p.stage_slices) reinterpret_cast<LazyWord*>(s_part)[i] = w;
+        }
       }
-      if (!wait_reached(p.arrivals + b, own_expected, p.header, p.wait_spins)) {
+      if (__syncthreads_or(!ok_wait)) {
         failed = true;
         break;
       }
@@ -207,8 +237,9 @@ decide_walk_lazy_kernel(const LazyParams p) {
         const int32_t st = state[l];
         float conf;
         int32_t tok;
-        const bool ok = finalize_row<2>(p.partials + ((int64_t)b * L + l) * p.splits, p.splits, sub, st,
-                                        p.mask_id, conf, tok);
+        const bool ok = p.stage_slices ? finalize_row<2, true>(s_part + l * p.splits, p.splits, sub, st, p.mask_id, conf, tok)
+                                       : finalize_row<2>(p.partials + ((int64_t)b * L + l) * p.splits, p.splits, sub, st,
+                                                         p.mask_id, conf, tok);
         if (sub == 0 && r < L) {
           const int64_t row = ((int64_t)b * N + node) * L + l;
           p.conf[row] = conf;
@@ -231,6 +262,16 @@ decide_walk_lazy_kernel(const LazyParams p) {
       __syncthreads();
       const uint64_t bits = s_bits;
       if (tid < L) s_next[tid] = ((bits >> tid) & 1ull) ? s_top[tid] : state[tid];
+      if (warp == 0) {  // positions the next state still masks
+        uint64_t left = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int l = lane + 32 * h;
+          const bool m = l < L && (((bits >> l) & 1ull) ? s_top[l] : state[l]) == p.mask_id;
+          left |= (uint64_t)__ballot_sync(0xffffffffu, m) << (32 * h);
+        }
+        if (lane == 0) s_mask = left;
+      }
       __syncthreads();
       const bool may_go_on = bits != 0 && own_hops < N - 1;
       if (may_go_on) {
@@ -272,11 +313,9 @@ decide_walk_lazy_kernel(const LazyParams p) {
         }
         own_node = -1;
       }
-      if (tid == 0) {  // publish: the reducers of b wait for epoch[b] > level, then read cur[b]
-        p.cur[b] = own_node;
-        __threadfence();
-        atomicExch(p.epoch + b, own_node < 0 ? 0x7fffffff : level + 1);
-      }
+      own_mask = s_mask;
+      if (tid == 0)  // what the reducers of b wait for
+        store_word(p.words + b, LazyWord{own_node < 0 ? 0x7fffffff : level + 1, own_node, own_mask});
       __syncthreads();
     }
     if (!alive) return;  // every sequence this CTA works for has ended
@@ -311,8 +350,8 @@ int resident_ctas(int device, size_t smem) {
 
 size_t decide_lazy_workspace_bytes(const spiffy_decide_desc& d) {
   const size_t partials = (size_t)d.batch * d.block_len * decide_splits(d, nullptr) * sizeof(Partial);
-  // header | arrivals[B] | epoch[B] | cur[B], the first three zeroed by every call
-  return partials + sizeof(LazyHeader) + (((size_t)d.batch * 12 + 15) / 16) * 16;
+  // slices | header | words[B], all zeroed by every call
+  return partials + sizeof(LazyHeader) + (size_t)d.batch * sizeof(LazyWord);
 }
 
 spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc& d, const void* logits,
@@ -328,7 +367,9 @@ spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc& d, const void* l
   const bool bf16 = d.logits_dtype == SPIFFY_BF16;
   const size_t graph = lazy_graph_bytes(d, parent_cap);
   const int stage_graph = graph <= 16 * 1024;  // beyond that it would cost resident CTAs
-  const size_t smem = stage_graph ? graph : 0;
+  const size_t slices = (size_t)d.block_len * decide_splits(d, nullptr) * sizeof(Partial);
+  const int stage_slices = slices <= 20 * 1024;
+  const size_t smem = (stage_graph ? graph : 0) + (stage_slices ? slices : 0);
   const int resident = bf16 ? resident_ctas<__nv_bfloat16>(device, smem) : resident_ctas<float>(device, smem);
   if (resident <= 0) return SPIFFY_ECUDA;
   if (d.batch > resident) return SPIFFY_EUNSUPPORTED;  // one resident CTA per sequence runs its tail
@@ -361,17 +402,15 @@ spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc& d, const void* l
   const size_t partial_bytes = (size_t)d.batch * d.block_len * p.splits * sizeof(Partial);
   p.partials = static_cast<Partial*>(ws);
   p.header = reinterpret_cast<LazyHeader*>(static_cast<char*>(ws) + partial_bytes);
-  p.arrivals = reinterpret_cast<unsigned*>(p.header + 1);
-  p.epoch = reinterpret_cast<int32_t*>(p.arrivals + d.batch);
-  p.cur = p.epoch + d.batch;
+  p.words = reinterpret_cast<LazyWord*>(p.header + 1);
   p.clear_status = fresh ? 1 : 0;
   p.stage_graph = stage_graph;
+  p.stage_slices = stage_slices;
   p.wait_spins = flag_poll_limit();
-  p.extra_arrivals = (unsigned)lazy_extra_arrivals();
+  p.lost_slices = lazy_extra_arrivals();
   const int64_t items = (int64_t)d.batch * d.block_len * p.splits;
-  int grid = (int)(items < resident ? items : resident);
-  if (grid < d.batch) grid = d.batch;
-  if (cudaMemsetAsync(p.header, 0, sizeof(LazyHeader) + (size_t)d.batch * 8, stream) != cudaSuccess)
+  int grid = (int)(items + d.batch < resident ? items + d.batch : resident);
+  if (cudaMemsetAsync(ws, 0, decide_lazy_workspace_bytes(d), stream) != cudaSuccess)
     return SPIFFY_ECUDA;
   void* args[] = {&p};
   const void* fn = bf16 ? (const void*)decide_walk_lazy_kernel<__nv_bfloat16>
