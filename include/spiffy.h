@@ -449,9 +449,9 @@ spiffy_status spiffy_decide_walk(const spiffy_decide_desc* desc, const void* log
  *     SPIFFY_DEV_TIMEOUT in both status words when a bounded wait between the
  *     levels ran out (results are then unspecified).
  * There is no grid-wide barrier: per sequence, the thread blocks that reduce
- * the current node's rows count themselves in on an arrival counter, the block
- * that owns the sequence waits for that count, decides, and publishes the next
- * node under an epoch number the reducers wait for; sequences never wait for one
+ * the current node's rows tag their results with the level, the block that owns
+ * the sequence waits for those tags, decides, and publishes the next node with
+ * its level, for which the reducers wait; sequences never wait for one
  * another.  A level still costs two such round trips through memory, so the
  * call pays off when one node's share of the logits is large (long
  * vocabularies, batches) and loses to spiffy_decide_walk on a single short
@@ -613,8 +613,8 @@ spiffy_status spiffy_draft_blocks(const spiffy_draft_desc* desc, const void* log
  *                        and no tensor-core product); < 0 restores the default
  *   flag_polls           polls (about 100 ns apart) per wait of the lazy call;
  *                        < 0 restores the default
- *   lazy_extra_arrivals  sequence 0 of the lazy call waits for this many
- *                        arrivals more than can come (0 = normal operation)
+ *   lazy_extra_arrivals  other than 0: sequence 0 of the lazy call waits for
+ *                        results that cannot come
  * Values above the defaults are clamped to them.  Not for production use.
  */
 void spiffy_set_wait_limits(int64_t mbarrier_polls, int64_t flag_polls,

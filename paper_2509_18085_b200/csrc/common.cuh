@@ -67,7 +67,7 @@ void count_launch(int n = 1);
 // which exists so that the give-up paths can be exercised.
 uint32_t mbar_poll_limit();   // polls of one mbarrier wait (tensor-core kernels)
 uint32_t flag_poll_limit();   // polls of one wait on a global-memory word (lazy call)
-int32_t lazy_extra_arrivals();  // arrivals sequence 0's tail expects beyond those that can come
+int32_t lazy_extra_arrivals();  // not 0: sequence 0's tail waits for results that cannot come
 
 // Entry points implemented in the kernel files; all validated by the caller.
 // `fresh`: the call's first kernel clears the status words (SPIFFY_FRESH_STATUS);

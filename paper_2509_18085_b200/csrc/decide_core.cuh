@@ -169,10 +169,13 @@ __device__ __forceinline__ void store16(void* p, uint64_t lo, uint64_t hi) {
 // log2(e) for the plain softmax; the sampled decision passes log2(e) / T and
 // gets the sum of exp((x - maximum) / T).  `tag` goes into the result's spare word, in the
 // one 16-byte store that writes it: a reader that polls for the tag has the rest with it.
+// `out` may be null: thread 0 has the result anyway.  `keep`, in shared memory, gets the slice's
+// vectors, number i at kept_at(i).
+__device__ __forceinline__ int kept_at(int i) { return i ^ ((i >> 3) & 7); }  // no bank conflicts at stride 8 either
 template <typename T>
-__device__ __forceinline__ void reduce_slice(const T* __restrict__ base, int V, int64_t chunk,
+__device__ __forceinline__ Partial reduce_slice(const T* __restrict__ base, int V, int64_t chunk,
                                              int split, Partial* __restrict__ out,
-                                             const float k = kLog2e, const int tag = 0) {
+                                             const float k = kLog2e, const int tag = 0, uint4* keep = nullptr) {
   const int64_t begin = (int64_t)split * chunk;
   const int64_t end = min((int64_t)V, begin + chunk);
   constexpr int EPV = Elem<T>::kPerVec;
@@ -192,6 +195,10 @@ __device__ __forceinline__ void reduce_slice(const T* __restrict__ base, int V, 
 #pragma unroll
   for (int e = 0; e < EPV; ++e)
     tail[e] = (tid == 0 && e < ntail) ? Elem<T>::load1(base + begin + (int64_t)nvec * EPV + e) : -INFINITY;
+  if (keep) {
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) keep[kept_at(tid + u * kReduceThreads)] = v[u];
+  }
   // 2. slice maximum: lanes, warps
   float m = Elem<T>::gmax(v);
 #pragma unroll
@@ -244,12 +251,16 @@ __device__ __forceinline__ void reduce_slice(const T* __restrict__ base, int V, 
     if (idx != 0x7fffffff) atomicMin(&slice_idx, idx);
   }
   __syncthreads();
+  Partial r = {m, s, 0, tag};
   if (tid == 0) {
     s = warp_s[0];
     for (int w = 1; w < kReduceThreads / 32; ++w) s += warp_s[w];
-    store16(out, (uint64_t)__float_as_uint(m) | (uint64_t)__float_as_uint(s) << 32,
-            (uint64_t)(uint32_t)slice_idx | (uint64_t)(uint32_t)tag << 32);
+    r = Partial{m, s, slice_idx, tag};
+    if (out)
+      store16(out, (uint64_t)__float_as_uint(m) | (uint64_t)__float_as_uint(s) << 32,
+              (uint64_t)(uint32_t)slice_idx | (uint64_t)(uint32_t)tag << 32);
   }
+  return r;
 }
 
 // kLanes (8, 4, 2 or 1) neighbouring lanes merge the slices of one row and lane

@@ -218,7 +218,7 @@ decide_walk_lazy_kernel(const LazyParams p) {
       bool ok_wait = true;
       {
         const Partial* from = p.partials + (int64_t)b * L * p.splits;
-        const int tag = level + 1 + (b == 0 ? p.lost_slices : 0);
+        const int tag = b == 0 && p.lost_slices != 0 ? -1 : level + 1;
         unsigned polls = 0;
         for (int i = tid; i < L * p.splits && ok_wait; i += kReduceThreads) {
           if (state[i / p.splits] != p.mask_id) continue;
