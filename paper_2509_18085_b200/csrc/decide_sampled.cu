@@ -166,6 +166,14 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
     const bool m1 = lane + 32 < L && st[min(lane + 32, L - 1)] == mask_id;
     masked_count = __popc(__ballot_sync(0xffffffffu, m0)) + __popc(__ballot_sync(0xffffffffu, m1));
   }
+  // so is the noise of the first 32 slices, lane s that of slice s
+  const Philox rng{seed_lo, seed_hi, (uint32_t)l, (uint32_t)b, (uint32_t)masked_count};
+  uint32_t first_w[4] = {0u, 0u, 0u, 0u};
+  float first_g = 0.f;
+  if (warp == 0 && state == mask_id) {
+    rng.draw((uint32_t)lane, first_w);
+    first_g = gumbel(first_w[0]);
+  }
 #if __CUDA_ARCH__ >= 900
   pdl_launch_dependents();
   if (!kWhole) cudaGridDependencySynchronize();  // the reduce kernel's partials and cleared counters are visible
@@ -178,13 +186,10 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
   __shared__ uint4 kept[kWhole ? kReduceThreads * kUnroll : 1];  // the row, when it is one slice
   if (state == mask_id) {  // the whole CTA takes the same branch
     if (kWhole) {
-      uint32_t w[4];
-      if (warp == 0) Philox{seed_lo, seed_hi, (uint32_t)l, (uint32_t)b, (uint32_t)masked_count}.draw(0u, w);
       const Partial r = reduce_slice(logits + (int64_t)row * row_stride, V, chunk, 0, nullptr, k, 0, kept);
-      if (tid == 0) choice = SliceChoice{r.s > 0.f && r.m > -INFINITY ? 0 : 0x7fffffff, w[1], r.m, r.s, r.m, r.s};
+      if (tid == 0) choice = SliceChoice{r.s > 0.f && r.m > -INFINITY ? 0 : 0x7fffffff, first_w[1], r.m, r.s, r.m, r.s};
     } else if (warp == 0) {
       // level 1: lanes over slices
-      const Philox rng{seed_lo, seed_hi, (uint32_t)l, (uint32_t)b, (uint32_t)masked_count};
       float rm = -INFINITY, rs = 0.f;      // row maximum of x and sum of exp((x - rm) / T)
       float best = -INFINITY, bm = 0.f, bz = 0.f;
       int bs = 0x7fffffff;
@@ -195,11 +200,17 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
         const float m = __int_as_float(raw.x), z = __int_as_float(raw.y);
         merge_t(rm, rs, m, z, k);
         if (z > 0.f && m > -INFINITY) {
-          uint32_t w[4];
-          rng.draw((uint32_t)s, w);
-          const float score = fmaf(m, inv_t, 0.6931471805599453f * lg2(z)) + gumbel(w[0]);
+          float g = first_g;
+          uint32_t w1 = first_w[1];
+          if (s >= 32) {
+            uint32_t w[4];
+            rng.draw((uint32_t)s, w);
+            g = gumbel(w[0]);
+            w1 = w[1];
+          }
+          const float score = fmaf(m, inv_t, 0.6931471805599453f * lg2(z)) + g;
           if (score > best || (score == best && s < bs)) {
-            best = score; bs = s; bw = w[1]; bm = m; bz = z;
+            best = score; bs = s; bw = w1; bm = m; bz = z;
           }
         }
       }
@@ -257,12 +268,14 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
         }
       };
       float local = 0.f;  // weight of this thread's entries, summed in ascending order
+      float upto[kUnroll];  // ... up to the end of each vector
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
         float x[EPV];
         slot(u, x);
 #pragma unroll
         for (int e = 0; e < EPV; ++e) local += ex2(fmaf(x[e], k, nml));
+        upto[u] = local;
       }
       // running sums across threads, in double: thread t's exclusive sum is thread t - 1's inclusive one, bit for bit
       double in_warp = (double)local;
@@ -287,30 +300,43 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
       if (mine) {
         // excl + run >= target for a float run is run >= (target - excl) rounded up to a float
         const float need = __double2float_ru(target - excl);
-        int first_reach = -1, last_weight = -1;
-        float x_reach = 0.f, x_weight = 0.f, run = 0.f;
+        int at = 0;  // the vector in which the running sum reaches it
+        float run = 0.f;
+        float x[EPV] = {};
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          float x[EPV];
-          slot(u, x);
+        for (int u = kUnroll - 1; u >= 0; --u)
+          if (upto[u] >= need) {
+            at = u;
+            run = u > 0 ? upto[u > 0 ? u - 1 : 0] : 0.f;
+            slot(u, x);
+          }
+        int pick = 0;
+        float x_pick = 0.f;
+        bool found = false;
 #pragma unroll
-          for (int e = 0; e < EPV; ++e) {
-            const float w = ex2(fmaf(x[e], k, nml));
-            run += w;  // the order of `local`
-            if (first_reach < 0 && w > 0.f && run >= need) {
-              first_reach = (tid * kUnroll + u) * EPV + e;
-              x_reach = x[e];
-            }
-            if (w > 0.f) {
-              last_weight = (tid * kUnroll + u) * EPV + e;
-              x_weight = x[e];
+        for (int e = 0; e < EPV; ++e) {
+          const float w = ex2(fmaf(x[e], k, nml));
+          run += w;  // the order of `local`
+          if (!found && w > 0.f && run >= need) {
+            found = true;
+            pick = (tid * kUnroll + at) * EPV + e;
+            x_pick = x[e];
+          }
+        }
+        if (!(local >= need)) {
+          // the thread's own sums end at `local`, which can miss incl by a rounding of the scan: the last
+          // entry of any weight
+          pick = 0;
+          x_pick = 0.f;
+          const int first = tid * kUnroll * EPV, past = min(first + kUnroll * EPV, (int)(end - begin));
+          for (int j = first; j < past; ++j) {
+            const float xj = Elem<T>::load1(base + j);
+            if (ex2(fmaf(xj, k, nml)) > 0.f) {
+              pick = j;
+              x_pick = xj;
             }
           }
         }
-        // the thread's own partial sums end at `local`, which can miss incl by a rounding of the scan
-        const bool reach = first_reach >= 0;
-        const int pick = reach ? first_reach : max(last_weight, 0);
-        const float x_pick = reach ? x_reach : x_weight;
         conf_out[row] = fminf(1.0f, ex2((x_pick - c.row_m) * k) / c.row_s);
         tok_out[row] = (int32_t)begin + pick;
         __threadfence();
