@@ -23,6 +23,7 @@ constexpr int kThreads = 128;  // top-k kernel
 constexpr int kVecs = 8;       // 128-bit vectors per thread
 constexpr int kMaxK = 4;       // vocabulary ranks
 constexpr int kBuildThreads = 1024;  // a warp per block position
+constexpr int kRelated = 64;         // formulas whose subset relation fits its table
 constexpr int kGraphInts = 6144;     // shared-memory copy of the draft graph (24 KB)
 
 struct __align__(16) TopPartial {
@@ -31,6 +32,13 @@ struct __align__(16) TopPartial {
   int idx[kMaxK];      // their token ids
   int pad[2];
 };
+
+// The maximum over the warp's lanes, on every lane (NaN loses).
+__device__ __forceinline__ float warp_max(float x) {
+  float m;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+  return m;
+}
 
 // (value desc, id asc): is (v2, i2) ahead of (v1, i1)?
 __device__ __forceinline__ bool ahead(float v2, int i2, float v1, int i1) {
@@ -104,79 +112,100 @@ draft_topk_kernel(const T* __restrict__ logits, int64_t row_stride, int V, int64
   for (int e = 0; e < EPV; ++e)
     x[kVecs * EPV + e] =
         (tid == 0 && e < ntail) ? Unpack<T>::load1(base + begin + (int64_t)nvec * EPV + e) : -INFINITY;
-  auto index_of = [&](int k) -> int {  // token id of the thread's k-th element
-    return k < kVecs * EPV ? (int)begin + (tid + (k / EPV) * kThreads) * EPV + k % EPV
-                           : (int)begin + nvec * EPV + (k - kVecs * EPV);
+  // The largest element of every vector: a round then looks at these, and only the thread that
+  // holds the winner looks into the vector it lies in.
+  constexpr int kGroups = kVecs + 1;
+  float top[kGroups];
+#pragma unroll
+  for (int u = 0; u < kGroups; ++u) {
+    top[u] = x[u * EPV];
+#pragma unroll
+    for (int e = 1; e < EPV; ++e) top[u] = fmaxf(top[u], x[u * EPV + e]);
+  }
+  auto largest = [&]() {  // NaN loses
+    float t = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < kGroups; ++u) t = fmaxf(t, top[u]);
+    return t;
   };
-
-  __shared__ float w_val[kThreads / 32];
-  __shared__ int w_idx[kThreads / 32];
-  __shared__ float w_sum[kThreads / 32];
-  // the thread's best remaining element; it is searched again only by the thread whose
-  // element has just been taken (every other thread's best is still its best)
-  float tv;
-  int ti;
-#define SPIFFY_DRAFT_RESCAN()                                                          \
-  do {                                                                                 \
-    tv = -INFINITY;                                                                    \
-    ti = 0x7fffffff;                                                                   \
-    _Pragma("unroll") for (int k = NE - 1; k >= 0; --k) /* descending: ties end on the lowest token */ \
-      if (x[k] >= tv && x[k] != -INFINITY) {                                           \
-        tv = x[k];                                                                     \
-        ti = index_of(k);                                                              \
-      }                                                                                \
-  } while (0)
-  SPIFFY_DRAFT_RESCAN();
+  __shared__ float w_max[kThreads / 32], w_sum[kThreads / 32];
+  __shared__ float w_val[kThreads / 32][kMaxK];
+  __shared__ int w_idx[kThreads / 32][kMaxK];
+  float tv = largest();
+  float wm = warp_max(tv);
+  if (lane == 0) w_max[warp] = wm;
+  __syncthreads();
+  float m = w_max[0];
+#pragma unroll
+  for (int w = 1; w < kThreads / 32; ++w) m = fmaxf(m, w_max[w]);
+  {  // sum of exp(x - m), before anything is knocked out
+    const float ml = (m == -INFINITY) ? 0.f : m * kLog2e;
+    float s = 0.f;
+#pragma unroll
+    for (int k = 0; k < NE; ++k) s += ex2(fmaf(x[k], kLog2e, -ml));
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) w_sum[warp] = s;
+  }
+  // the warp's K best, by itself
+  for (int r = 0; r < K; ++r) {
+    int mine = 0x7fffffff, at_u = -1, at_e = 0;
+    if (tv == wm && wm != -INFINITY) {
+#pragma unroll
+      for (int u = kGroups - 1; u >= 0; --u)  // descending: ties end on the lowest token
+        if (top[u] == wm) at_u = u;
+#pragma unroll
+      for (int u = 0; u < kGroups; ++u)
+        if (u == at_u) {
+#pragma unroll
+          for (int e = EPV - 1; e >= 0; --e)
+            if (x[u * EPV + e] == wm) at_e = e;
+        }
+      mine = at_u < kVecs ? (int)begin + (tid + at_u * kThreads) * EPV + at_e : (int)begin + nvec * EPV + at_e;
+    }
+    const int best = (int)__reduce_min_sync(0xffffffffu, (unsigned)mine);
+    if (lane == 0) { w_val[warp][r] = wm; w_idx[warp][r] = best; }
+    if (r + 1 < K) {
+      if (mine == best && at_u >= 0) {  // taken: knock it out
+#pragma unroll
+        for (int u = 0; u < kGroups; ++u)
+          if (u == at_u) {
+            float t = -INFINITY;
+#pragma unroll
+            for (int e = 0; e < EPV; ++e) {
+              if (e == at_e) x[u * EPV + e] = -INFINITY;
+              t = fmaxf(t, x[u * EPV + e]);
+            }
+            top[u] = t;
+          }
+        tv = largest();
+      }
+      wm = warp_max(tv);
+    }
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  // the K best of the four warps' lists: lane 4 w + t holds entry t of warp w
+  float v = -INFINITY;
+  int i = 0x7fffffff;
+  if (lane < kThreads / 32 * kMaxK && lane % kMaxK < K) {
+    v = w_val[lane / kMaxK][lane % kMaxK];
+    i = w_idx[lane / kMaxK][lane % kMaxK];
+  }
   TopPartial out;
-  out.s = 0.f;
+  out.m = m;
+  out.s = w_sum[0];
+#pragma unroll
+  for (int w = 1; w < kThreads / 32; ++w) out.s += w_sum[w];
 #pragma unroll
   for (int r = 0; r < kMaxK; ++r) {
-    float bv = -INFINITY;
-    int bi = 0x7fffffff;
-    if (r < K) {
-      // the best remaining element of the CTA: the best over the threads
-      bv = tv;
-      bi = ti;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const float v2 = __shfl_xor_sync(0xffffffffu, bv, off);
-        const int i2 = __shfl_xor_sync(0xffffffffu, bi, off);
-        if (ahead(v2, i2, bv, bi)) { bv = v2; bi = i2; }
-      }
-      __syncthreads();  // the previous round's reads of w_val / w_idx are done
-      if (lane == 0) { w_val[warp] = bv; w_idx[warp] = bi; }
-      __syncthreads();
-      bv = w_val[0];
-      bi = w_idx[0];
-#pragma unroll
-      for (int w = 1; w < kThreads / 32; ++w)
-        if (ahead(w_val[w], w_idx[w], bv, bi)) { bv = w_val[w]; bi = w_idx[w]; }
-      if (r == 0) {
-        // sum of exp(x - m) against the slice maximum, before anything is knocked out
-        const float ml = (bv == -INFINITY) ? 0.f : bv * kLog2e;
-        float s = 0.f;
-#pragma unroll
-        for (int k = 0; k < NE; ++k) s += ex2(fmaf(x[k], kLog2e, -ml));
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0) w_sum[warp] = s;
-        __syncthreads();
-        s = w_sum[0];
-        for (int w = 1; w < kThreads / 32; ++w) s += w_sum[w];
-        out.m = bv;
-        out.s = s;
-      }
-      if (bv != -INFINITY && ti == bi && r + 1 < K) {  // this thread's element was taken: knock it out, search again
-#pragma unroll
-        for (int k = 0; k < NE; ++k)
-          if (index_of(k) == bi) x[k] = -INFINITY;
-        SPIFFY_DRAFT_RESCAN();
-      }
-    }
-    out.val[r] = bv;
-    out.idx[r] = bv == -INFINITY ? 0x7fffffff : bi;
+    const float bv = warp_max(v);
+    const int bi = bv == -INFINITY ? 0x7fffffff
+                                   : (int)__reduce_min_sync(0xffffffffu, v == bv ? (unsigned)i : 0x7fffffffu);
+    out.val[r] = r < K ? bv : -INFINITY;
+    out.idx[r] = r < K ? bi : 0x7fffffff;
+    if (i == bi) v = -INFINITY;
   }
-#undef SPIFFY_DRAFT_RESCAN
   out.pad[0] = out.pad[1] = 0;
   if (tid == 0) partials[(int64_t)row * splits + split] = out;
 }
@@ -224,7 +253,8 @@ draft_build_kernel(BuildArgs g) {
   float* cand_p = reinterpret_cast<float*>(draft_smem);      // [L][kMaxK]
   int* cand_tok = reinterpret_cast<int*>(cand_p + L * kMaxK);  // [L][kMaxK]
   int* pos_of_rank = cand_tok + L * kMaxK;                   // [L]
-  float* local = reinterpret_cast<float*>(pos_of_rank + L);  // [D]
+  int* now = pos_of_rank + L;                                // [L] the current block
+  float* local = reinterpret_cast<float*>(now + L);          // [D]
   float* total = local + D;                                  // [D]
   int* keep = reinterpret_cast<int*>(total + D);             // [D] slot + 1 of a kept formula, else 0
   int* node_formula = keep + D;                              // [budget + 1] formula of each node, -1 for node 0 / padding
@@ -251,6 +281,18 @@ draft_build_kernel(BuildArgs g) {
       g.formula_off = f_off; g.child_off = c_off; g.formula_i = f_i; g.formula_j = f_j; g.child_idx = c_idx;
     }
   }
+  // Which formulas are strict subsets of which, for the parent lists: also known before the wait.
+  // Bit a of subsets[c]: a < c is one of c's.  Graphs of more formulas find it out when needed.
+  __shared__ unsigned subsets[kRelated][kRelated / 32];
+  const bool related = D <= kRelated;
+  if (related) {
+    for (int i = tid; i < kRelated * (kRelated / 32); i += kBuildThreads) (&subsets[0][0])[i] = 0u;
+    __syncthreads();
+    for (int i = tid; i < D * D; i += kBuildThreads) {
+      const int c = i / D, a = i - c * D;
+      if (a < c && strict_subset(g, a, c)) atomicOr(&subsets[c][a >> 5], 1u << (a & 31));
+    }
+  }
 #if __CUDA_ARCH__ >= 900
   cudaGridDependencySynchronize();  // the top-k kernel's partial results, and the caller's logits and state, are visible
 #endif
@@ -258,12 +300,19 @@ draft_build_kernel(BuildArgs g) {
 
   // 1. candidates c_ij and their probabilities: one warp per position
   for (int l = warp; l < L; l += kBuildThreads / 32) {
-    const bool masked = state[l] == g.mask_id;
-    if (!masked) {
-      if (lane < kMaxK) { cand_p[l * kMaxK + lane] = -1.f; cand_tok[l * kMaxK + lane] = state[l]; }
+    const TopPartial* p = g.partials + ((int64_t)b * L + l) * g.splits;
+    // read together with the token (one trip); those of an unmasked row were never written and are ignored
+    uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0, q2 = q0;
+    if (g.splits <= 32 && lane < g.splits) {
+      const uint4* q = reinterpret_cast<const uint4*>(p + lane);
+      q0 = __ldcg(q); q1 = __ldcg(q + 1); q2 = __ldcg(q + 2);
+    }
+    const int32_t token = state[l];
+    if (lane == 0) now[l] = token;
+    if (token != g.mask_id) {
+      if (lane < kMaxK) { cand_p[l * kMaxK + lane] = -1.f; cand_tok[l * kMaxK + lane] = token; }
       continue;
     }
-    const TopPartial* p = g.partials + ((int64_t)b * L + l) * g.splits;
     float m = -INFINITY, s = 0.f;
     float hv[kMaxK];
     int hi[kMaxK];
@@ -273,8 +322,6 @@ draft_build_kernel(BuildArgs g) {
       // one slice per lane, fetched whole in one trip: its maximum and sum, and its K
       // candidates, which the top-k kernel left sorted
       if (lane < g.splits) {
-        const uint4* q = reinterpret_cast<const uint4*>(p + lane);
-        const uint4 q0 = q[0], q1 = q[1], q2 = q[2];
         m = __uint_as_float(q0.x);
         s = __uint_as_float(q0.y);
         hv[0] = __uint_as_float(q0.z); hv[1] = __uint_as_float(q0.w);
@@ -339,15 +386,16 @@ draft_build_kernel(BuildArgs g) {
   }
   __syncthreads();
   // 2. token position ranks (Eq. token-position-sort): by maximum probability, ties to the lower position
-  for (int l = tid; l < L; l += kBuildThreads) {
+  for (int l = warp; l < L; l += kBuildThreads / 32) {  // a warp per position, its lanes over the others
     const float pl = cand_p[l * kMaxK];
     if (pl < 0.f) continue;  // unmasked
     int rank = 0;
-    for (int j = 0; j < L; ++j) {
-      const float pj = cand_p[j * kMaxK];
-      rank += (pj >= 0.f && (pj > pl || (pj == pl && j < l))) ? 1 : 0;
+    for (int j0 = 0; j0 < L; j0 += 32) {
+      const int j = j0 + lane;
+      const float pj = j < L ? cand_p[j * kMaxK] : -1.f;
+      rank += __popc(__ballot_sync(0xffffffffu, pj >= 0.f && (pj > pl || (pj == pl && j < l))));
     }
-    pos_of_rank[rank] = l;
+    if (lane == 0) pos_of_rank[rank] = l;
   }
   __syncthreads();
   // 3. local score of every formula: geometric mean of its candidates' probabilities
@@ -408,7 +456,7 @@ draft_build_kernel(BuildArgs g) {
   __syncthreads();
   // 6. blocks: the current block, then each kept draft = current block + its candidates
   int32_t* tokens = g.tokens + (int64_t)b * (g.budget + 1) * L;
-  for (int i = tid; i < (g.budget + 1) * L; i += kBuildThreads) tokens[i] = state[i % L];
+  for (int i = tid; i < (g.budget + 1) * L; i += kBuildThreads) tokens[i] = now[i % L];
   for (int n = tid; n < g.budget; n += kBuildThreads) g.kept[(int64_t)b * g.budget + n] = node_formula[n + 1];
   __syncthreads();
   for (int n = 1 + warp; n <= g.budget; n += kBuildThreads / 32) {
@@ -422,8 +470,9 @@ draft_build_kernel(BuildArgs g) {
   // 7. parent lists: every earlier kept node whose candidate set is a strict subset.
   // One warp per child, its lanes over the candidate parents.
   auto is_parent = [&](int a, int c) {
-    return a < c && (a == 0 || node_formula[a] >= 0) &&
-           strict_subset(g, a == 0 ? -1 : node_formula[a], node_formula[c]);
+    if (a >= c || (a > 0 && node_formula[a] < 0)) return false;
+    const int fa = a == 0 ? -1 : node_formula[a], fc = node_formula[c];
+    return related && fa >= 0 ? ((subsets[fc][fa >> 5] >> (fa & 31)) & 1u) != 0u : strict_subset(g, fa, fc);
   };
   for (int c = warp; c <= g.budget; c += kBuildThreads / 32) {
     int n = 0;
@@ -505,7 +554,7 @@ spiffy_status launch_draft(const spiffy_draft_desc& d, const void* logits, const
   g.state = state; g.formula_off = formula_off; g.formula_i = formula_i; g.formula_j = formula_j;
   g.child_off = child_off; g.child_idx = child_idx; g.tokens = tokens; g.kept = kept; g.score = score;
   g.parent_off = parent_off; g.parent_idx = parent_idx; g.dev_status = dev_status; g.fill_parents = fresh ? 1 : 0;
-  const size_t smem = (size_t)d.block_len * kMaxK * 8 + (size_t)d.block_len * 4 +
+  const size_t smem = (size_t)d.block_len * kMaxK * 8 + (size_t)d.block_len * 8 +
                       (size_t)d.n_formulas * 12 + (size_t)(d.budget + 1) * 8 + 16;
   e = launch_pdl(draft_build_kernel, dim3(d.batch), dim3(kBuildThreads), smem, stream, g);
   count_launch();
