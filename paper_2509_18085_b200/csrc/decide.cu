@@ -37,7 +37,7 @@ decide_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V,
   if (early_trigger) pdl_launch_dependents();
 #endif
   const int row = blockIdx.y;
-  clear.run(row);
+  if (blockIdx.x == 0 && threadIdx.x == kReduceThreads - 1) clear.run(row);
   if (__ldcg(block_tokens + row) == mask_id)  // already unmasked: never read
     reduce_slice(logits + (int64_t)row * row_stride, V, chunk, (int)blockIdx.x,
                  partials + (int64_t)row * splits + blockIdx.x);

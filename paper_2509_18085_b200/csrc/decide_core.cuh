@@ -30,19 +30,21 @@ struct __align__(16) Partial {
 };
 
 // Clears the status words of a call whose caller left them arbitrary
-// (SPIFFY_FRESH_STATUS); part of the call's first kernel, which sets no bit itself.
+// (SPIFFY_FRESH_STATUS); part of the call's first kernel, which sets no bit itself: the CTA
+// of row i, of which there are more than sequences, clears word i.
 struct StatusClear {
   int32_t* a;  // [B], null when there is nothing to clear
   int32_t* b;
-  int rows_per_seq;
+  int batch;   // 0: nothing to clear
+  // one thread per row calls it, and not the one whose chain the CTA waits for
   __device__ __forceinline__ void run(int row) const {
-    if (blockIdx.x != 0 || threadIdx.x != 0 || rows_per_seq == 0 || row % rows_per_seq != 0) return;
-    if (a) a[row / rows_per_seq] = 0;
-    if (b) b[row / rows_per_seq] = 0;
+    if (row >= batch) return;
+    if (a) a[row] = 0;
+    if (b) b[row] = 0;
   }
 };
 inline StatusClear status_clear(const spiffy_decide_desc& d, bool fresh, int32_t* a, int32_t* b) {
-  return fresh ? StatusClear{a, b, d.n_nodes * d.block_len} : StatusClear{nullptr, nullptr, 0};
+  return fresh ? StatusClear{a, b, d.batch} : StatusClear{nullptr, nullptr, 0};
 }
 
 // acc += {2^(x0 * log2e - ml), 2^(x1 * log2e - ml)}; k2 = {log2e, log2e}, nml2 = {-ml, -ml}
@@ -167,8 +169,8 @@ __device__ __forceinline__ void store16(void* p, uint64_t lo, uint64_t hi) {
 // found first and the exponentials are then taken against it directly.  All
 // threads of the CTA call it together; thread 0 stores the result.  `k` is
 // log2(e) for the plain softmax; the sampled decision passes log2(e) / T and
-// gets the sum of exp((x - maximum) / T).  `tag` goes into the result's spare word, in the
-// one 16-byte store that writes it: a reader that polls for the tag has the rest with it.
+// gets the sum of exp((x - maximum) / T).  `tag`, if not 0, goes into the result's spare word
+// in the one 16-byte access that writes it: a reader that polls for the tag has the rest with it.
 // `out` may be null: thread 0 has the result anyway.  `keep`, in shared memory, gets the slice's
 // vectors, number i at kept_at(i).
 __device__ __forceinline__ int kept_at(int i) { return i ^ ((i >> 3) & 7); }  // no bank conflicts at stride 8 either
@@ -256,7 +258,8 @@ __device__ __forceinline__ Partial reduce_slice(const T* __restrict__ base, int 
     s = warp_s[0];
     for (int w = 1; w < kReduceThreads / 32; ++w) s += warp_s[w];
     r = Partial{m, s, slice_idx, tag};
-    if (out)
+    if (out && tag == 0) *out = r;
+    if (out && tag != 0)
       store16(out, (uint64_t)__float_as_uint(m) | (uint64_t)__float_as_uint(s) << 32,
               (uint64_t)(uint32_t)slice_idx | (uint64_t)(uint32_t)tag << 32);
   }

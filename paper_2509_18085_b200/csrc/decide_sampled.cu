@@ -89,19 +89,21 @@ __device__ __forceinline__ void merge_t(float& m, float& s, float m2, float s2, 
 }
 
 // grid = (splits, B*N*L); one CTA reduces one vocabulary slice of one row and
-// the first CTA of a node clears the node's arrival counter for the select kernel.
+// the first CTA of row i clears node i's arrival counter for the select kernel.
 template <typename T>
 __global__ void __launch_bounds__(kReduceThreads, 8)
 decide_sampled_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V, int64_t chunk,
-                             int splits, int L, const int32_t* __restrict__ block_tokens, int mask_id,
+                             int splits, int nodes, const int32_t* __restrict__ block_tokens, int mask_id,
                              float k, Partial* __restrict__ partials, int* __restrict__ node_count,
                              StatusClear clear) {
 #if __CUDA_ARCH__ >= 900
   cudaGridDependencySynchronize();
 #endif
   const int row = blockIdx.y;
-  clear.run(row);
-  if (blockIdx.x == 0 && threadIdx.x == 0 && row % L == 0) node_count[row / L] = 0;
+  if (blockIdx.x == 0 && threadIdx.x == kReduceThreads - 1) {
+    if (row < nodes) node_count[row] = 0;
+    clear.run(row);
+  }
   if (block_tokens[row] != mask_id) return;  // already unmasked: never read
   reduce_slice(logits + (int64_t)row * row_stride, V, chunk, (int)blockIdx.x,
                partials + (int64_t)row * splits + blockIdx.x, k);
@@ -140,7 +142,7 @@ struct SliceChoice {
 // 8 t ... 8 t + 7 of the chosen slice, i.e. a contiguous run of entries.  kWhole: the row is one
 // slice, reduced here, and the rule is left to decide_sampled_rule_kernel.
 template <typename T, bool kWhole>
-__global__ void __launch_bounds__(kReduceThreads, kWhole ? 5 : 1)
+__global__ void __launch_bounds__(kReduceThreads, 5)  // 96 registers
 decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, int V, int64_t chunk,
                              int splits, int N, int L, const int32_t* __restrict__ block_tokens,
                              int mask_id, int rule, int top_s, float tau, float inv_t,
@@ -429,7 +431,7 @@ spiffy_status launch_decide_sampled(const spiffy_decide_desc& d, float temperatu
     cudaError_t r = cudaSuccess;
     if (!whole) {
       r = launch_pdl(decide_sampled_reduce_kernel<T>, dim3(splits, rows), dim3(kReduceThreads), (size_t)0, stream,
-                     typed, (int64_t)d.row_stride, (int)d.vocab, chunk, splits, (int)d.block_len, block_tokens,
+                     typed, (int64_t)d.row_stride, (int)d.vocab, chunk, splits, (int)(d.batch * d.n_nodes), block_tokens,
                      (int)d.mask_token_id, inv_t * kLog2e, partials, node_count, status_clear(d, fresh, dev_status, nullptr));
       count_launch();
       if (r != cudaSuccess) return r;

@@ -92,7 +92,7 @@ lmhead_gather_kernel(const uint4* __restrict__ h, int row_vecs, const int32_t* _
   pdl_launch_dependents();
   const int row = blockIdx.x, tid = threadIdx.x;
   const bool last = row + 1 == (int)gridDim.x;
-  if (clear.rows_per_seq > 0 && tid == 0 && row % clear.rows_per_seq == 0 && clear.a) clear.a[row / clear.rows_per_seq] = 0;
+  if (tid == kGatherThreads - 1) clear.run(row);
   const bool masked = tokens[row] == mask_id;
   if (!masked && !last) return;
   int before = 0;
