@@ -15,6 +15,7 @@ namespace spiffy {
 namespace {
 
 constexpr size_t kAlign = 256;
+constexpr size_t kDirectNodes = 8192;  // nodes up to which the walk keeps its links in shared memory
 size_t up(size_t n) { return (n + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
@@ -95,6 +96,14 @@ bool device_can_read(const void* host_ptr) {
   }
   return at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeManaged || at.type == cudaMemoryTypeDevice;
 }
+bool device_can_write(const void* host_ptr) {  // at the same address
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, host_ptr) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeHost && at.devicePointer == host_ptr;
+}
 
 }  // namespace
 }  // namespace spiffy
@@ -143,6 +152,8 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
   // the staging buffers are free once earlier work on the caller's stream is done
   ok = ok && cudaEventRecord(h->start, stream) == cudaSuccess;
   ok = ok && cudaStreamWaitEvent(h->stream, h->start, 0) == cudaSuccess;
+  // the status words are OR-ed into by the kernels: [attention | decision per sequence | walk per sequence]
+  ok = ok && cudaMemsetAsync(ws + l.status, 0, (1 + 2 * B) * 4, stream) == cudaSuccess;
   h2d(l.tokens, block_tokens, rows * 4, stream);  // the row-staging kernel below reads them
   h2d(l.q, q, l.qn, h->stream);
   h2d(l.kp, k_prefix, l.pn, h->stream);
@@ -166,31 +177,48 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
   ok = ok && cudaStreamWaitEvent(stream, h->done, 0) == cudaSuccess;
   if (!ok) return SPIFFY_ECUDA;
 
-  // the status words are OR-ed into by the kernels: [attention | decision per sequence | walk per sequence]
-  if (cudaMemsetAsync(ws + l.status, 0, (1 + 2 * B) * 4, stream) != cudaSuccess) return SPIFFY_ECUDA;
   int32_t* dev_status = reinterpret_cast<int32_t*>(ws + l.status);
-  st = spiffy_graph_attention(&s.attn, ws + l.q, s.attn.prefix_len ? ws + l.kp : nullptr,
-                              s.attn.prefix_len ? ws + l.vp : nullptr, ws + l.kb, ws + l.vb, ws + l.attn_out,
-                              dev_status, ws + l.attn_ws, l.decide_ws - l.attn_ws, cuda_stream);
+  // The verdict goes straight to the caller's arrays where the device can write them (a copy each
+  // otherwise, about 2 us): the walk writes each word once and, with its links in shared memory,
+  // reads none back.
+  struct Out {
+    int32_t* host;
+    size_t at, bytes;
+    bool direct;
+    int32_t* device(char* ws) const { return direct ? host : reinterpret_cast<int32_t*>(ws + at); }
+  } outs[4] = {{accepted_node, l.accepted, B * 4, false},
+               {n_accepted, l.n_accepted, B * 4, false},
+               {path, l.path, B * N * 4, false},
+               {next_block, l.next_block, B * L * 4, false}};
+  for (Out& o : outs) o.direct = N <= kDirectNodes && device_can_write(o.host);
+  auto attention = [&](int flags) {
+    spiffy_attn_desc a = s.attn;
+    a.kernel |= flags;
+    return spiffy_graph_attention(&a, ws + l.q, s.attn.prefix_len ? ws + l.kp : nullptr,
+                                  s.attn.prefix_len ? ws + l.vp : nullptr, ws + l.kb, ws + l.vb, ws + l.attn_out,
+                                  dev_status, ws + l.attn_ws, l.decide_ws - l.attn_ws, cuda_stream);
+  };
+  // On the tensor-core kernel the two run side by side, the attention second; else one after the other.
+  const bool second = attention_tc_supported(s.attn) &&
+                      ((s.attn.kernel & 0xff) == SPIFFY_ATTN_AUTO ||
+                       ((s.attn.kernel & 0xff) == SPIFFY_ATTN_TCGEN05 && s.attn.head_dim == 128));
+  if (!second) st = attention(0);
   if (st != SPIFFY_OK) return st;
+  if (second) s.decide.logits_dtype |= SPIFFY_INDEPENDENT_NEXT;
   st = spiffy_decide_walk(&s.decide, ws + l.logits, reinterpret_cast<const int32_t*>(ws + l.tokens),
                           reinterpret_cast<const int32_t*>(ws + l.poff),
                           reinterpret_cast<const int32_t*>(ws + l.pidx), s.parent_cap,
                           reinterpret_cast<float*>(ws + l.conf), reinterpret_cast<int32_t*>(ws + l.top_tok),
                           reinterpret_cast<uint64_t*>(ws + l.bits), reinterpret_cast<int32_t*>(ws + l.n_unmask),
-                          dev_status + 1, reinterpret_cast<int32_t*>(ws + l.accepted),
-                          reinterpret_cast<int32_t*>(ws + l.n_accepted), reinterpret_cast<int32_t*>(ws + l.path),
-                          reinterpret_cast<int32_t*>(ws + l.next_block), dev_status + 1 + B,
-                          ws + l.decide_ws, l.total - l.decide_ws, cuda_stream);
+                          dev_status + 1, outs[0].device(ws), outs[1].device(ws), outs[2].device(ws),
+                          outs[3].device(ws), dev_status + 1 + B, ws + l.decide_ws, l.total - l.decide_ws, cuda_stream);
+  if (st == SPIFFY_OK && second) st = attention(SPIFFY_ATTN_INDEPENDENT);
   if (st != SPIFFY_OK) return st;
-  // the verdict: four small arrays and the status words
   auto d2h = [&](void* dst, size_t at, size_t bytes) {
     ok = ok && cudaMemcpyAsync(dst, ws + at, bytes, cudaMemcpyDeviceToHost, stream) == cudaSuccess;
   };
-  d2h(accepted_node, l.accepted, B * 4);
-  d2h(n_accepted, l.n_accepted, B * 4);
-  d2h(path, l.path, B * N * 4);
-  d2h(next_block, l.next_block, B * L * 4);
+  for (const Out& o : outs)
+    if (!o.direct) d2h(o.host, o.at, o.bytes);
   d2h(status, l.status, (1 + 2 * B) * 4);
   ok = ok && cudaStreamSynchronize(stream) == cudaSuccess;
   return ok ? SPIFFY_OK : SPIFFY_ECUDA;
