@@ -3,10 +3,16 @@
 // tensors sit in HOST memory.  The call stages the inputs on the device, runs the
 // three kernels of the step and brings the verdict back; see include/spiffy.h.
 //
-// Staging.  Everything but the logits goes through the copy engine on a helper
-// stream of the library; meanwhile, on the caller's stream, one kernel pulls the
-// logits rows of still-masked positions (the only rows the decision reads)
-// straight out of the pinned host buffer.  Both meet before the first kernel.
+// The attention's inputs go through the copy engine on a helper stream of the
+// library, and the attention follows them there.  Meanwhile, on the caller's
+// stream, the decision reads the logits rows of still-masked positions, each once,
+// straight out of the pinned host buffer, and the parent lists likewise: its work
+// is hidden under the transfer.  Staging those rows first, by a kernel that copied
+// them, and running both halves after the last byte took 3 to 8 us more
+// (146 against 142 at 18 x 16 positions, 1155 against 1150 us at the LLaDA-8B shape,
+// where the bus is the bound).
+// Where the parent lists are not pinned, or too long for the walk to keep on chip,
+// that is still the way; logits that are not pinned are copied whole.
 #include <mutex>
 
 #include "common.cuh"
@@ -146,38 +152,56 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
   const size_t le = s.decide.logits_dtype == SPIFFY_BF16 ? 2 : 4;
   const size_t rows = B * N * L;
   bool ok = true;
+  const bool readable = device_can_read(logits) && rows <= 65535;
+  // the decision reads logits and parent lists where they are, the lists once
+  const bool in_place = readable && (2 * rows / B + 3 * N + 1 + s.parent_cap) * 4 <= 40 * 1024 &&
+                        (reinterpret_cast<uintptr_t>(logits) & 15) == 0 && device_can_write(logits) &&
+                        device_can_write(parent_off) && device_can_write(parent_idx);
   auto h2d = [&](size_t at, const void* src, size_t bytes, cudaStream_t on) {
     if (bytes) ok = ok && cudaMemcpyAsync(ws + at, src, bytes, cudaMemcpyHostToDevice, on) == cudaSuccess;
   };
+  // the status words are OR-ed into by the kernels: [attention | decision per sequence | walk per sequence]
+  ok = ok && cudaMemsetAsync(ws + l.status, 0, (1 + 2 * B) * 4, stream) == cudaSuccess;
   // the staging buffers are free once earlier work on the caller's stream is done
   ok = ok && cudaEventRecord(h->start, stream) == cudaSuccess;
   ok = ok && cudaStreamWaitEvent(h->stream, h->start, 0) == cudaSuccess;
-  // the status words are OR-ed into by the kernels: [attention | decision per sequence | walk per sequence]
-  ok = ok && cudaMemsetAsync(ws + l.status, 0, (1 + 2 * B) * 4, stream) == cudaSuccess;
-  h2d(l.tokens, block_tokens, rows * 4, stream);  // the row-staging kernel below reads them
+  h2d(l.tokens, block_tokens, rows * 4, stream);
   h2d(l.q, q, l.qn, h->stream);
   h2d(l.kp, k_prefix, l.pn, h->stream);
   h2d(l.vp, v_prefix, l.pn, h->stream);
   h2d(l.kb, k_block, l.bn, h->stream);
   h2d(l.vb, v_block, l.bn, h->stream);
-  h2d(l.poff, parent_off, B * (N + 1) * 4, h->stream);
-  h2d(l.pidx, parent_idx, B * (size_t)s.parent_cap * 4, h->stream);
+  int32_t* dev_status = reinterpret_cast<int32_t*>(ws + l.status);
+  auto attention = [&](int flags, cudaStream_t on) {
+    spiffy_attn_desc a = s.attn;
+    a.kernel |= flags;
+    return spiffy_graph_attention(&a, ws + l.q, s.attn.prefix_len ? ws + l.kp : nullptr,
+                                  s.attn.prefix_len ? ws + l.vp : nullptr, ws + l.kb, ws + l.vb, ws + l.attn_out,
+                                  dev_status, ws + l.attn_ws, l.decide_ws - l.attn_ws, on);
+  };
+  if (in_place) {
+    if (ok) st = attention(0, h->stream);
+    if (st != SPIFFY_OK) return st;
+  } else {
+    h2d(l.poff, parent_off, B * (N + 1) * 4, h->stream);
+    h2d(l.pidx, parent_idx, B * (size_t)s.parent_cap * 4, h->stream);
+  }
   ok = ok && cudaEventRecord(h->done, h->stream) == cudaSuccess;
   if (!ok) return SPIFFY_ECUDA;
-  // logits: only the rows of still-masked positions cross the bus
-  const size_t row_bytes = (size_t)s.decide.row_stride * le;
-  if (device_can_read(logits) && rows <= 65535) {
-    st = launch_stage_masked_rows(logits, ws + l.logits, (int64_t)row_bytes,
-                                  reinterpret_cast<const int32_t*>(ws + l.tokens), s.decide.mask_token_id,
-                                  (int64_t)rows, stream);
-    if (st != SPIFFY_OK) return st;
-  } else {  // pageable memory: the runtime stages it; all rows go
-    h2d(l.logits, logits, rows * row_bytes, stream);
+  if (!in_place) {
+    // logits: only the rows of still-masked positions cross the bus
+    const size_t row_bytes = (size_t)s.decide.row_stride * le;
+    if (readable) {
+      st = launch_stage_masked_rows(logits, ws + l.logits, (int64_t)row_bytes,
+                                    reinterpret_cast<const int32_t*>(ws + l.tokens), s.decide.mask_token_id,
+                                    (int64_t)rows, stream);
+      if (st != SPIFFY_OK) return st;
+    } else {  // pageable memory: the runtime stages it; all rows go
+      h2d(l.logits, logits, rows * row_bytes, stream);
+    }
+    ok = ok && cudaStreamWaitEvent(stream, h->done, 0) == cudaSuccess;
+    if (!ok) return SPIFFY_ECUDA;
   }
-  ok = ok && cudaStreamWaitEvent(stream, h->done, 0) == cudaSuccess;
-  if (!ok) return SPIFFY_ECUDA;
-
-  int32_t* dev_status = reinterpret_cast<int32_t*>(ws + l.status);
   // The verdict goes straight to the caller's arrays where the device can write them (a copy each
   // otherwise, about 2 us): the walk writes each word once and, with its links in shared memory,
   // reads none back.
@@ -191,29 +215,25 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
                {path, l.path, B * N * 4, false},
                {next_block, l.next_block, B * L * 4, false}};
   for (Out& o : outs) o.direct = N <= kDirectNodes && device_can_write(o.host);
-  auto attention = [&](int flags) {
-    spiffy_attn_desc a = s.attn;
-    a.kernel |= flags;
-    return spiffy_graph_attention(&a, ws + l.q, s.attn.prefix_len ? ws + l.kp : nullptr,
-                                  s.attn.prefix_len ? ws + l.vp : nullptr, ws + l.kb, ws + l.vb, ws + l.attn_out,
-                                  dev_status, ws + l.attn_ws, l.decide_ws - l.attn_ws, cuda_stream);
-  };
-  // On the tensor-core kernel the two run side by side, the attention second; else one after the other.
-  const bool second = attention_tc_supported(s.attn) &&
+  // Behind the staging the two run side by side on the tensor-core kernel, the attention second;
+  // else one after the other.
+  const bool second = !in_place && attention_tc_supported(s.attn) &&
                       ((s.attn.kernel & 0xff) == SPIFFY_ATTN_AUTO ||
                        ((s.attn.kernel & 0xff) == SPIFFY_ATTN_TCGEN05 && s.attn.head_dim == 128));
-  if (!second) st = attention(0);
+  if (!second && !in_place) st = attention(0, stream);
   if (st != SPIFFY_OK) return st;
   if (second) s.decide.logits_dtype |= SPIFFY_INDEPENDENT_NEXT;
-  st = spiffy_decide_walk(&s.decide, ws + l.logits, reinterpret_cast<const int32_t*>(ws + l.tokens),
-                          reinterpret_cast<const int32_t*>(ws + l.poff),
-                          reinterpret_cast<const int32_t*>(ws + l.pidx), s.parent_cap,
+  st = spiffy_decide_walk(&s.decide, in_place ? logits : ws + l.logits,
+                          reinterpret_cast<const int32_t*>(ws + l.tokens),
+                          in_place ? parent_off : reinterpret_cast<const int32_t*>(ws + l.poff),
+                          in_place ? parent_idx : reinterpret_cast<const int32_t*>(ws + l.pidx), s.parent_cap,
                           reinterpret_cast<float*>(ws + l.conf), reinterpret_cast<int32_t*>(ws + l.top_tok),
                           reinterpret_cast<uint64_t*>(ws + l.bits), reinterpret_cast<int32_t*>(ws + l.n_unmask),
                           dev_status + 1, outs[0].device(ws), outs[1].device(ws), outs[2].device(ws),
-                          outs[3].device(ws), dev_status + 1 + B, ws + l.decide_ws, l.total - l.decide_ws, cuda_stream);
-  if (st == SPIFFY_OK && second) st = attention(SPIFFY_ATTN_INDEPENDENT);
+                          outs[3].device(ws), dev_status + 1 + B, ws + l.decide_ws, l.total - l.decide_ws, stream);
+  if (st == SPIFFY_OK && second) st = attention(SPIFFY_ATTN_INDEPENDENT, stream);
   if (st != SPIFFY_OK) return st;
+  if (in_place) ok = ok && cudaStreamWaitEvent(stream, h->done, 0) == cudaSuccess;
   auto d2h = [&](void* dst, size_t at, size_t bytes) {
     ok = ok && cudaMemcpyAsync(dst, ws + at, bytes, cudaMemcpyDeviceToHost, stream) == cudaSuccess;
   };

@@ -44,3 +44,28 @@ def _results(s):
 
 def _fields(x):
     return [getattr(x, f.name) for f in dataclasses.fields(x)] if dataclasses.is_dataclass(x) else list(x)
+
+
+@pytest.mark.parametrize("pinned", ["all", "lists not", "logits not", "verdict not"])
+@pytest.mark.parametrize("N,L,Hq,Hkv,d,dtype", [(5, 8, 4, 4, 128, "bf16"), (40, 20, 8, 2, 64, "bf16"), (3, 5, 2, 2, 64, "f32")])
+def test_host_step_from_pinned_and_pageable_arrays(pinned, N, L, Hq, Hkv, d, dtype):
+    cfg = W.Config("t", 2, N, L, 70, Hq, Hkv, d, dtype, 1000, spiffy.RULE_THRESHOLD)
+    w = W.make(cfg, 5)
+    step = VerifyStep(cfg)
+    step.run(inputs_from_workload(w))
+    want = [t.cpu() for t in (step.walk.accepted_node, step.walk.n_accepted, step.walk.path, step.walk.next_block)]
+    host = inputs_from_workload(w, device="cpu", pin=True)
+    if pinned == "lists not":
+        host.parent_off, host.parent_idx = host.parent_off.clone(), host.parent_idx.clone()
+    if pinned == "logits not":
+        host.logits = host.logits.clone()
+    for i in range(3):
+        got = step.run_host(host)
+        if pinned == "verdict not" and i == 0:
+            step.host_verdict = tuple(torch.full_like(t, 77) for t in step.host_verdict)
+            continue
+        for a, b in zip(step.host_verdict, want):
+            assert torch.equal(a, b)
+        assert int(step.host_verdict[4].abs().sum()) == 0
+        for t in step.host_verdict:
+            t.fill_(77)
