@@ -379,10 +379,11 @@ def run_lmhead_part(args, cfg):
         stream.synchronize()
         sec = e0.elapsed_time(e1) * 1e-3 / reps
     peaks = measured_peaks()
-    flops = 2.0 * B * N * L * V * hidden
-    by = (V + B * N * L) * hidden * 2.0
+    masked = int((tokens == cfg.mask_id).sum().item())  # the rows the call computes
+    flops = 2.0 * masked * V * hidden
+    by = (V + masked) * hidden * 2.0
     print(json.dumps({"part": "lmhead", "config": f"config{args.config}-{cfg.name}", "us_per_call": sec * 1e6,
-                      "rows": B * N * L, "hidden": hidden, "vocab": V, "calls_timed": reps,
+                      "rows": B * N * L, "masked_rows": masked, "hidden": hidden, "vocab": V, "calls_timed": reps,
                       "tflops": flops / sec / 1e12, "frac_of_bf16_peak": flops / sec / 1e12 / peaks["bf16_tflops"],
                       "gbs": by / sec / 1e9, "frac_of_hbm": by / sec / 1e9 / peaks["hbm_gbs"],
                       "algorithmic_flops": flops, "algorithmic_bytes": by, "peaks": peaks["source"],
