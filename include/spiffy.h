@@ -500,6 +500,9 @@ spiffy_status spiffy_decide_walk_lazy(const spiffy_decide_desc* desc, const void
  *                    spiffy_verify_step_host_workspace(desc) bytes: staging copies
  *                    of every input, the attention output and the decision's
  *                    per-node results (which stay there), the kernels' scratch
+ * A descriptor that either component call would refuse is refused before anything
+ * is enqueued.  A call that fails later waits for what it has enqueued before it
+ * returns, so that no copy or kernel still uses the caller's arrays or workspace.
  * Calls sharing a workspace, or made from several threads on one device, must
  * not overlap (the helper stream is shared).
  */

@@ -37,11 +37,12 @@ spiffy_status check_attn_desc(const spiffy_attn_desc* d) {
   return SPIFFY_OK;
 }
 
-bool use_tc(const spiffy_attn_desc& d) {
-  if ((d.kernel & 0xff) == SPIFFY_ATTN_SIMT) return false;
-  // asked for by name, the tensor-core kernel is the one of head dimension 128
-  if ((d.kernel & 0xff) == SPIFFY_ATTN_TCGEN05 && d.head_dim != 128) return false;
-  return attention_tc_supported(d);
+// For a descriptor that is in order: is there a kernel for it?
+spiffy_status check_attn_route(const spiffy_attn_desc& d) {
+  if (attention_uses_tc(d)) return SPIFFY_OK;
+  if ((d.kernel & 0xff) == SPIFFY_ATTN_TCGEN05) return SPIFFY_EUNSUPPORTED;
+  if (d.block_len > 64) return SPIFFY_EUNSUPPORTED;  // the CUDA-core kernel keeps a block's rows in registers
+  return SPIFFY_OK;
 }
 
 spiffy_status check_decide_desc(const spiffy_decide_desc* d, bool need_vocab) {
@@ -88,6 +89,19 @@ spiffy_status check_draft_desc(const spiffy_draft_desc* d) {
 }
 
 }  // namespace
+
+bool attention_uses_tc(const spiffy_attn_desc& d) {
+  if ((d.kernel & 0xff) == SPIFFY_ATTN_SIMT) return false;
+  // asked for by name, the tensor-core kernel is the one of head dimension 128
+  if ((d.kernel & 0xff) == SPIFFY_ATTN_TCGEN05 && d.head_dim != 128) return false;
+  return attention_tc_supported(d);
+}
+
+spiffy_status check_attention(const spiffy_attn_desc& d) {
+  const spiffy_status st = check_attn_desc(&d);
+  return st != SPIFFY_OK ? st : check_attn_route(d);
+}
+
 }  // namespace spiffy
 
 using namespace spiffy;
@@ -116,12 +130,12 @@ spiffy_status spiffy_graph_attention(const spiffy_attn_desc* desc, const void* q
       !aligned16(k_prefix) || !aligned16(v_prefix))
     return SPIFFY_EINVAL;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  if (use_tc(d)) {
+  const spiffy_status route = check_attn_route(d);
+  if (route != SPIFFY_OK) return route;
+  if (attention_uses_tc(d)) {
     const AttnProblem a = {q, {k_prefix, v_prefix, d.prefix_len, 0}, {nullptr, nullptr, 0, 0}, k_block, v_block, out};
     return launch_attention_tc(d, a, dev_status, stream);
   }
-  if ((d.kernel & 0xff) == SPIFFY_ATTN_TCGEN05) return SPIFFY_EUNSUPPORTED;
-  if (d.block_len > 64) return SPIFFY_EUNSUPPORTED;  // the CUDA-core kernel keeps a block's rows in registers
   return launch_attention_simt(d, q, k_prefix, v_prefix, k_block, v_block, out, stream);
 }
 
@@ -138,7 +152,7 @@ spiffy_status check_full_sequence(const spiffy_attn_desc* desc, int32_t suffix_l
   if (st != SPIFFY_OK) return st;
   if (suffix_len < 0) return SPIFFY_EINVAL;
   if (suffix_len > 1024) return SPIFFY_EUNSUPPORTED;
-  if (!use_tc(*desc) || desc->head_dim != 128) return SPIFFY_EUNSUPPORTED;  // bf16, head dimension 128 only
+  if (!attention_uses_tc(*desc) || desc->head_dim != 128) return SPIFFY_EUNSUPPORTED;  // bf16, head dimension 128 only
   return SPIFFY_OK;
 }
 }  // namespace

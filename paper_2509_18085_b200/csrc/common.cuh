@@ -166,6 +166,10 @@ struct AttnProblem {
   void* out;
 };
 bool attention_tc_supported(const spiffy_attn_desc& d);
+// What spiffy_graph_attention makes of a descriptor: the status it would refuse it with, and,
+// for one it takes, whether that goes to the tensor-core kernel.
+spiffy_status check_attention(const spiffy_attn_desc& d);
+bool attention_uses_tc(const spiffy_attn_desc& d);
 spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const AttnProblem& a, int32_t* dev_status,
                                   cudaStream_t stream);
 // Two problems of the same batch, heads and head dimension (128) in one launch.

@@ -66,9 +66,9 @@ spiffy_status check(const spiffy_step_desc* s) {
       s->attn.block_len != s->decide.block_len || s->parent_cap < 1)
     return SPIFFY_EINVAL;
   if (s->attn.block_len > 64) return SPIFFY_EUNSUPPORTED;
-  // the component calls check the rest; their workspace queries return 0 for a bad descriptor
+  // all that the component calls would refuse: nothing is enqueued for a call that fails
   if (spiffy_unmask_decide_workspace(&s->decide) == 0) return SPIFFY_EINVAL;
-  return SPIFFY_OK;
+  return check_attention(s->attn);
 }
 
 // One helper stream and two events per device, created at the first call there.
@@ -179,15 +179,22 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
                                   s.attn.prefix_len ? ws + l.vp : nullptr, ws + l.kb, ws + l.vb, ws + l.attn_out,
                                   dev_status, ws + l.attn_ws, l.decide_ws - l.attn_ws, on);
   };
+  // From here on work is in flight on both streams, one of which the caller cannot see: whatever
+  // fails, the caller's arrays and workspace are at rest when it is told.
+  auto leave = [&](spiffy_status why) {
+    cudaStreamSynchronize(h->stream);
+    cudaStreamSynchronize(stream);
+    return why;
+  };
   if (in_place) {
     if (ok) st = attention(0, h->stream);
-    if (st != SPIFFY_OK) return st;
+    if (st != SPIFFY_OK) return leave(st);
   } else {
     h2d(l.poff, parent_off, B * (N + 1) * 4, h->stream);
     h2d(l.pidx, parent_idx, B * (size_t)s.parent_cap * 4, h->stream);
   }
   ok = ok && cudaEventRecord(h->done, h->stream) == cudaSuccess;
-  if (!ok) return SPIFFY_ECUDA;
+  if (!ok) return leave(SPIFFY_ECUDA);
   if (!in_place) {
     // logits: only the rows of still-masked positions cross the bus
     const size_t row_bytes = (size_t)s.decide.row_stride * le;
@@ -195,12 +202,12 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
       st = launch_stage_masked_rows(logits, ws + l.logits, (int64_t)row_bytes,
                                     reinterpret_cast<const int32_t*>(ws + l.tokens), s.decide.mask_token_id,
                                     (int64_t)rows, stream);
-      if (st != SPIFFY_OK) return st;
+      if (st != SPIFFY_OK) return leave(st);
     } else {  // pageable memory: the runtime stages it; all rows go
       h2d(l.logits, logits, rows * row_bytes, stream);
     }
     ok = ok && cudaStreamWaitEvent(stream, h->done, 0) == cudaSuccess;
-    if (!ok) return SPIFFY_ECUDA;
+    if (!ok) return leave(SPIFFY_ECUDA);
   }
   // The verdict goes straight to the caller's arrays where the device can write them (a copy each
   // otherwise, about 2 us): the walk writes each word once and, with its links in shared memory,
@@ -217,11 +224,9 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
   for (Out& o : outs) o.direct = N <= kDirectNodes && device_can_write(o.host);
   // Behind the staging the two run side by side on the tensor-core kernel, the attention second;
   // else one after the other.
-  const bool second = !in_place && attention_tc_supported(s.attn) &&
-                      ((s.attn.kernel & 0xff) == SPIFFY_ATTN_AUTO ||
-                       ((s.attn.kernel & 0xff) == SPIFFY_ATTN_TCGEN05 && s.attn.head_dim == 128));
+  const bool second = !in_place && attention_uses_tc(s.attn);
   if (!second && !in_place) st = attention(0, stream);
-  if (st != SPIFFY_OK) return st;
+  if (st != SPIFFY_OK) return leave(st);
   if (second) s.decide.logits_dtype |= SPIFFY_INDEPENDENT_NEXT;
   st = spiffy_decide_walk(&s.decide, in_place ? logits : ws + l.logits,
                           reinterpret_cast<const int32_t*>(ws + l.tokens),
@@ -232,7 +237,7 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
                           dev_status + 1, outs[0].device(ws), outs[1].device(ws), outs[2].device(ws),
                           outs[3].device(ws), dev_status + 1 + B, ws + l.decide_ws, l.total - l.decide_ws, stream);
   if (st == SPIFFY_OK && second) st = attention(SPIFFY_ATTN_INDEPENDENT, stream);
-  if (st != SPIFFY_OK) return st;
+  if (st != SPIFFY_OK) return leave(st);
   if (in_place) ok = ok && cudaStreamWaitEvent(stream, h->done, 0) == cudaSuccess;
   auto d2h = [&](void* dst, size_t at, size_t bytes) {
     ok = ok && cudaMemcpyAsync(dst, ws + at, bytes, cudaMemcpyDeviceToHost, stream) == cudaSuccess;
@@ -241,7 +246,7 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
     if (!o.direct) d2h(o.host, o.at, o.bytes);
   d2h(status, l.status, (1 + 2 * B) * 4);
   ok = ok && cudaStreamSynchronize(stream) == cudaSuccess;
-  return ok ? SPIFFY_OK : SPIFFY_ECUDA;
+  return ok ? SPIFFY_OK : leave(SPIFFY_ECUDA);
 }
 
 }  // extern "C"

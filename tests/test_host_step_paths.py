@@ -1,0 +1,91 @@
+"""The host code of the host-buffer step without a GPU: compiled against a runtime
+that logs what it is asked for (tests/host_runtime/runtime.cpp) and fails where told."""
+import ctypes
+import os
+import re
+import subprocess
+
+import pytest
+
+from paper_2509_18085_b200 import build as builder
+from paper_2509_18085_b200 import spiffy
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+UNITS = ["step_host", "decide", "walk", "stage", "api"]
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    """The library's host code with the stand-in runtime."""
+    out = tmp_path_factory.mktemp("host")
+    inc = ["-I", os.path.join(builder.ROOT, "include"), "-I", builder.CSRC]
+    cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    jobs = [subprocess.Popen([os.environ.get("NVCC", "nvcc"), "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17",
+                              "-Xcompiler", "-fPIC", "-c", os.path.join(builder.CSRC, u + ".cu"), "-o",
+                              str(out / (u + ".o"))] + inc) for u in UNITS]
+    assert [j.wait() for j in jobs] == [0] * len(jobs)
+    so = out / "host.so"
+    subprocess.run([os.environ.get("CXX", "g++"), "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-isystem", cuda] + inc +
+                   [os.path.join(HERE, "host_runtime", "runtime.cpp")] + [str(out / (u + ".o")) for u in UNITS] +
+                   ["-o", str(so)], check=True)
+    lib = ctypes.CDLL(str(so))
+    lib.fake_log.restype = ctypes.c_char_p
+    lib.fake_reset.argtypes = [ctypes.c_char_p, ctypes.c_size_t, ctypes.c_size_t]
+    lib.spiffy_verify_step_host_workspace.restype = ctypes.c_size_t
+    return lib
+
+
+STREAM = 7
+BASE, STEP = 1 << 32, 1 << 24  # the host arrays: never touched, only told apart
+NAMES = ["q", "k_prefix", "v_prefix", "k_block", "v_block", "logits", "block_tokens", "parent_off", "parent_idx",
+         "accepted_node", "n_accepted", "path", "next_block", "status"]
+
+
+def desc(N=4, L=8, d=128, dtype=spiffy.BF16, kernel=spiffy.ATTN_AUTO, cap=4, V=1024, Hq=4, Hkv=4):
+    return spiffy.StepDesc(spiffy.AttnDesc(1, N, L, 16, Hq, Hkv, d, dtype, 0.0, kernel),
+                           spiffy.DecideDesc(1, N, L, V, dtype, V, V - 1, spiffy.RULE_TOPS, 1, 0.9), cap)
+
+
+def step(lib, d, fail="", pinned=True, **moved):
+    """(status, log lines) of one call."""
+    lib.fake_reset(fail.encode(), BASE if pinned else 0, BASE + 100 * STEP if pinned else 0)
+    at = {n: BASE + i * STEP for i, n in enumerate(NAMES)}
+    at.update({n: at[n] + by for n, by in moved.items()})
+    st = lib.spiffy_verify_step_host(ctypes.byref(d), *(ctypes.c_void_p(at[n]) for n in NAMES),
+                                     ctypes.c_void_p(1 << 20), ctypes.c_size_t(1 << 40), ctypes.c_void_p(STREAM))
+    return st, lib.fake_log().decode().splitlines()
+
+
+def busy_streams(log):
+    """Streams that hold work nobody has waited for when the call returns."""
+    busy = set()
+    for line in log:
+        s = int(re.search(r" on (\d+)", line).group(1))
+        if line.startswith("sync"):
+            busy.discard(s)
+        elif line.startswith(("memcpy", "memset", "launch")) and not line.endswith("FAILED"):
+            busy.add(s)
+    return busy
+
+
+@pytest.mark.parametrize("bad", [dict(d=96), dict(kernel=spiffy.ATTN_TCGEN05, d=64),
+                                 dict(kernel=spiffy.ATTN_TCGEN05, dtype=spiffy.F32), dict(Hkv=3), dict(kernel=9)])
+@pytest.mark.parametrize("pinned", [True, False])
+def test_a_refused_step_enqueues_nothing(host, bad, pinned):
+    st, log = step(host, desc(**bad), pinned=pinned)
+    assert st in (spiffy.EINVAL, spiffy.EUNSUPPORTED)
+    assert log == []
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+@pytest.mark.parametrize("dtype", [spiffy.BF16, spiffy.F32])
+def test_nothing_is_in_flight_when_a_step_fails(host, dtype, pinned):
+    """Whatever call fails, the caller's arrays and workspace are at rest when it hears of it."""
+    st, log = step(host, desc(dtype=dtype), pinned=pinned)
+    assert st == spiffy.OK
+    kinds = {re.sub(r"( on \d+).*", r"\1", line) for line in log if not line.startswith("sync")}
+    assert any(k.startswith("launch attention") for k in kinds)
+    for kind in sorted(kinds):
+        st, log = step(host, desc(dtype=dtype), fail=kind, pinned=pinned)
+        assert st == spiffy.ECUDA, kind
+        assert busy_streams(log) == set(), (kind, log)
