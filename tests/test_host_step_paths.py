@@ -89,3 +89,16 @@ def test_nothing_is_in_flight_when_a_step_fails(host, dtype, pinned):
         st, log = step(host, desc(dtype=dtype), fail=kind, pinned=pinned)
         assert st == spiffy.ECUDA, kind
         assert busy_streams(log) == set(), (kind, log)
+
+
+@pytest.mark.parametrize("by", [2, 8])
+def test_kernels_read_pinned_logits_only_on_16_byte_boundaries(host, by):
+    """Elsewhere their vector loads would be misaligned: the runtime copies all rows."""
+    d = desc()
+    for pinned_lists in (True, False):  # would be read in place; would be staged by a kernel
+        moved = dict(logits=by) if pinned_lists else dict(logits=by, parent_off=100 * STEP)
+        st, log = step(host, d, **moved)
+        assert st == spiffy.OK
+        assert not any("stage_masked_rows" in line for line in log)
+        src = BASE + NAMES.index("logits") * STEP + by
+        assert any(line.startswith("memcpy") and f"from {src} bytes {4 * 8 * 1024 * 2}" in line for line in log)
