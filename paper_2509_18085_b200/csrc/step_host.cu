@@ -36,7 +36,7 @@ struct Layout {
 Layout layout_of(const spiffy_step_desc& s) {
   const spiffy_attn_desc& a = s.attn;
   const spiffy_decide_desc& d = s.decide;
-  const size_t e = a.dtype == SPIFFY_BF16 ? 2 : 4, le = (d.logits_dtype & ~SPIFFY_FRESH_STATUS) == SPIFFY_BF16 ? 2 : 4;
+  const size_t e = a.dtype == SPIFFY_BF16 ? 2 : 4, le = d.logits_dtype == SPIFFY_BF16 ? 2 : 4;
   const size_t B = a.batch, N = a.n_nodes, L = a.block_len;
   Layout l;
   l.qn = B * N * L * a.n_q_heads * a.head_dim * e;
@@ -58,6 +58,15 @@ Layout layout_of(const spiffy_step_desc& s) {
   l.decide_ws = take(spiffy_unmask_decide_workspace(&d));
   l.total = o;
   return l;
+}
+
+// The descriptor without the flags of the component calls: the step orders its own calls and
+// clears all its status words.
+spiffy_step_desc plain(const spiffy_step_desc& desc) {
+  spiffy_step_desc s = desc;
+  s.decide.logits_dtype &= ~(SPIFFY_FRESH_STATUS | SPIFFY_INDEPENDENT | SPIFFY_INDEPENDENT_NEXT);
+  s.attn.kernel &= ~(SPIFFY_ATTN_EARLY_DEPENDENTS | SPIFFY_ATTN_INDEPENDENT);
+  return s;
 }
 
 spiffy_status check(const spiffy_step_desc* s) {
@@ -120,7 +129,7 @@ extern "C" {
 
 size_t spiffy_verify_step_host_workspace(const spiffy_step_desc* desc) {
   if (check(desc) != SPIFFY_OK) return 0;
-  return layout_of(*desc).total;
+  return layout_of(plain(*desc)).total;
 }
 
 spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* q, const void* k_prefix,
@@ -132,8 +141,7 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
                                       size_t workspace_bytes, void* cuda_stream) {
   spiffy_status st = check(desc);
   if (st != SPIFFY_OK) return st;
-  spiffy_step_desc s = *desc;
-  s.decide.logits_dtype &= ~SPIFFY_FRESH_STATUS;  // the call clears all its status words
+  spiffy_step_desc s = plain(*desc);
   if (!q || !k_block || !v_block || !logits || !block_tokens || !parent_off || !parent_idx ||
       !accepted_node || !n_accepted || !path || !next_block || !status)
     return SPIFFY_EINVAL;

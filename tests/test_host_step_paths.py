@@ -102,3 +102,16 @@ def test_kernels_read_pinned_logits_only_on_16_byte_boundaries(host, by):
         assert not any("stage_masked_rows" in line for line in log)
         src = BASE + NAMES.index("logits") * STEP + by
         assert any(line.startswith("memcpy") and f"from {src} bytes {4 * 8 * 1024 * 2}" in line for line in log)
+
+
+@pytest.mark.parametrize("flags", [0x100, 0x200, 0x400, 0x700])
+@pytest.mark.parametrize("pinned", [True, False])
+def test_flags_of_the_component_calls_change_nothing(host, flags, pinned):
+    """Least of all the size of a logits element, which sizes the staging and its copies."""
+    want = step(host, desc(), pinned=pinned)
+    flagged = desc()
+    flagged.decide.logits_dtype |= flags
+    flagged.attn.kernel |= flags & 0x300
+    assert host.spiffy_verify_step_host_workspace(ctypes.byref(flagged)) == \
+        host.spiffy_verify_step_host_workspace(ctypes.byref(desc()))
+    assert step(host, flagged, pinned=pinned) == want
