@@ -81,6 +81,9 @@ spiffy_status launch_decide(const spiffy_decide_desc& d, const void* logits,
 size_t decide_workspace_bytes(const spiffy_decide_desc& d);
 int decide_splits(const spiffy_decide_desc& d, int64_t* chunk_elems);
 
+// Does the walk copy a sequence's graph to shared memory, reading every list once?  (The fused
+// tail does for all such sizes: at 512 rows its arrays take 2 KB more than the walk's, of 48 KB.)
+bool walk_stages_graph(const spiffy_decide_desc& d, int32_t parent_cap);
 spiffy_status launch_walk(const spiffy_decide_desc& d,
                           const int32_t* block_tokens,
                           const int32_t* parent_off, const int32_t* parent_idx,

@@ -163,8 +163,8 @@ spiffy_status spiffy_verify_step_host(const spiffy_step_desc* desc, const void* 
   // (by 16-byte loads: rows that do not start on such a boundary are copied by the runtime)
   const bool readable = device_can_read(logits) && rows <= 65535 && (reinterpret_cast<uintptr_t>(logits) & 15) == 0;
   // the decision reads logits and parent lists where they are, the lists once
-  const bool in_place = readable && (2 * rows / B + 3 * N + 1 + s.parent_cap) * 4 <= 40 * 1024 &&
-                        device_can_write(logits) && device_can_write(parent_off) && device_can_write(parent_idx);
+  const bool in_place = readable && walk_stages_graph(s.decide, s.parent_cap) && device_can_write(logits) &&
+                        device_can_write(parent_off) && device_can_write(parent_idx);
   auto h2d = [&](size_t at, const void* src, size_t bytes, cudaStream_t on) {
     if (bytes) ok = ok && cudaMemcpyAsync(ws + at, src, bytes, cudaMemcpyHostToDevice, on) == cudaSuccess;
   };

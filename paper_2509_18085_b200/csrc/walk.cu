@@ -75,7 +75,16 @@ accept_walk_kernel(int N, int L, const int32_t* __restrict__ block_tokens,
                n_accepted + b, lane);
 }
 
+size_t graph_bytes(const spiffy_decide_desc& d, int32_t parent_cap) {
+  return (size_t)d.n_nodes * 8 + ((size_t)2 * d.n_nodes * d.block_len + d.n_nodes + 1 + parent_cap) * 4;
+}
+size_t link_bytes(const spiffy_decide_desc& d) { return (size_t)d.n_nodes * 4; }
+
 }  // namespace
+
+bool walk_stages_graph(const spiffy_decide_desc& d, int32_t parent_cap) {
+  return graph_bytes(d, parent_cap) + link_bytes(d) <= 40 * 1024;
+}
 
 spiffy_status launch_walk(const spiffy_decide_desc& d,
                           const int32_t* block_tokens,
@@ -85,10 +94,8 @@ spiffy_status launch_walk(const spiffy_decide_desc& d,
                           int32_t* n_accepted, int32_t* path,
                           int32_t* next_block, int32_t* dev_status, bool fresh,
                           cudaStream_t stream) {
-  const size_t graph = (size_t)d.n_nodes * 8 +
-                       ((size_t)2 * d.n_nodes * d.block_len + d.n_nodes + 1 + parent_cap) * 4;
-  const size_t links = (size_t)d.n_nodes * 4;
-  const int stage_in_smem = graph + links <= 40 * 1024;
+  const size_t graph = graph_bytes(d, parent_cap), links = link_bytes(d);
+  const int stage_in_smem = walk_stages_graph(d, parent_cap);
   const int link_in_smem = stage_in_smem || links <= 40 * 1024;
   const size_t smem = (stage_in_smem ? graph : 0) + (link_in_smem ? links : 0);
   const cudaError_t e = launch_pdl(

@@ -115,3 +115,17 @@ def test_flags_of_the_component_calls_change_nothing(host, flags, pinned):
     assert host.spiffy_verify_step_host_workspace(ctypes.byref(flagged)) == \
         host.spiffy_verify_step_host_workspace(ctypes.byref(desc()))
     assert step(host, flagged, pinned=pinned) == want
+
+
+@pytest.mark.parametrize("N,L", [(200, 20), (16, 32)])  # separate walk; fused tail
+def test_lists_are_left_in_host_memory_only_where_they_are_read_once(host, N, L):
+    """Around the largest graph that the walk copies to shared memory: 40 KB."""
+    edge = 40 * 1024 // 4 - (2 * N * L + 4 * N + 1)
+    lists = str(BASE + NAMES.index("parent_off") * STEP)
+    for cap in (edge - 1, edge, edge + 1, edge + N, edge + N + 1):
+        st, log = step(host, desc(N=N, L=L, cap=cap))
+        assert st == spiffy.OK
+        (walk,) = [line for line in log if "accept_walk" in line or "decide_tail" in line]
+        in_place = f" lists {lists} " in walk
+        assert in_place == (cap <= edge), (cap - edge, walk)
+        assert not in_place or "decide_tail" in walk or walk.endswith("staged 1")
