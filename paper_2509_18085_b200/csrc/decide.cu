@@ -229,11 +229,13 @@ spiffy_status decide_only(const spiffy_decide_desc& d, const void* logits,
                           const int32_t* block_tokens, float* conf,
                           int32_t* top_tok, uint64_t* unmask_bits,
                           int32_t* n_unmask, int32_t* dev_status, void* ws, bool fresh, bool independent,
-                          cudaStream_t stream) {
+                          bool next, cudaStream_t stream) {
   int64_t chunk = 0;
   const int splits = decide_splits(d, &chunk);
   Partial* partials = static_cast<Partial*>(ws);
-  const spiffy_status st = launch_reduce(d, logits, block_tokens, partials, splits, chunk, 0, independent,
+  // `next`: an independent kernel comes after this call and takes the SMs the reduce leaves; the
+  // small kernels in between trigger as soon as they are resident, so it is the reduce that lets it in.
+  const spiffy_status st = launch_reduce(d, logits, block_tokens, partials, splits, chunk, next, independent,
                                          status_clear(d, fresh, dev_status, nullptr), stream);
   if (st != SPIFFY_OK) return st;
   // The finalize kernel's launch overlaps the tail of the reduce kernel; it
@@ -254,7 +256,7 @@ spiffy_status launch_decide(const spiffy_decide_desc& d, const void* logits, con
                             float* conf, int32_t* top_tok, uint64_t* unmask_bits, int32_t* n_unmask,
                             int32_t* dev_status, void* ws, bool fresh, cudaStream_t stream) {
   return decide_only(d, logits, block_tokens, conf, top_tok, unmask_bits, n_unmask, dev_status, ws, fresh, false,
-                     stream);
+                     false, stream);
 }
 
 // The finalize kernel alone, on partial results another kernel produced
@@ -289,7 +291,7 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
   const size_t smem = tail_smem_bytes(d, parent_cap);
   if ((int64_t)d.n_nodes * d.block_len > kTailRows || smem > 48 * 1024) {
     const spiffy_status st = decide_only(d, logits, block_tokens, conf, top_tok, unmask_bits,
-                                         n_unmask, decide_status, ws, fresh, independent, stream);
+                                         n_unmask, decide_status, ws, fresh, independent, next, stream);
     if (st != SPIFFY_OK) return st;
     return launch_walk(d, block_tokens, parent_off, parent_idx, parent_cap, top_tok, unmask_bits,
                        accepted_node, n_accepted, path, next_block, walk_status, fresh, stream);

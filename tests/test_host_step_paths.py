@@ -1,5 +1,6 @@
-"""The host code of the host-buffer step without a GPU: compiled against a runtime
-that logs what it is asked for (tests/host_runtime/runtime.cpp) and fails where told."""
+"""The host code of the host-buffer step and of the decision without a GPU: compiled
+against a runtime that logs what it is asked for (tests/host_runtime/runtime.cpp) and
+fails where told."""
 import ctypes
 import os
 import re
@@ -129,3 +130,23 @@ def test_lists_are_left_in_host_memory_only_where_they_are_read_once(host, N, L)
         in_place = f" lists {lists} " in walk
         assert in_place == (cap <= edge), (cap - edge, walk)
         assert not in_place or "decide_tail" in walk or walk.endswith("staged 1")
+
+
+@pytest.mark.parametrize("N,L,cap", [(4, 8, 4), (16, 32, 4), (54, 32, 4), (3, 8, 14000)])
+def test_an_independent_kernel_may_start_as_the_reduce_ends(host, N, L, cap):
+    """SPIFFY_INDEPENDENT_NEXT on both routes: every kernel of the call lets its dependents start ahead
+    of its own wait, so that what follows moves in behind the reduce.  (The fused tail does anyway
+    once it has waited, the small kernels of the other route at once.)"""
+    fused = N * L <= 512 and cap < 10000
+    d = spiffy.DecideDesc(1, N, L, 1024, spiffy.BF16, 1024, 1023, spiffy.RULE_TOPS, 1, 0.9)
+    p = ctypes.c_void_p(1 << 20)
+    for flags, early in ((0, "0"), (spiffy.INDEPENDENT_NEXT, "1")):
+        d.logits_dtype = spiffy.BF16 | flags
+        host.fake_reset(b"", 0, 0)
+        assert host.spiffy_decide_walk(ctypes.byref(d), p, p, p, p, cap, *[p] * 11, ctypes.c_size_t(1 << 40),
+                                       ctypes.c_void_p(STREAM)) == spiffy.OK
+        log = host.fake_log().decode().splitlines()
+        assert len(log) == (2 if fused else 3)
+        assert log[0].endswith(f" early {'1' if fused else early} independent 0")
+        if fused:  # the tail is resident while the reduce runs either way
+            assert log[1].endswith(f" early {early}")
