@@ -96,6 +96,16 @@ void* stream_of(PyObject* o) {
   return p;
 }
 
+// One call into the library, without the interpreter lock: a launch waits when the stream's queue is
+// full, and other Python threads have their own work.  All it needs has been read by now.
+template <typename F, typename... Args>
+int unlocked(F f, Args... args) {
+  PyThreadState* const held = PyEval_SaveThread();
+  const int status = f(args...);
+  PyEval_RestoreThread(held);
+  return status;
+}
+
 void check(int status, const char* where) {
   if (status == SPIFFY_OK) return;
   PyObject* e = PyObject_CallFunction(g_error_class, "is", status, where);
@@ -271,7 +281,7 @@ PyObject* graph_attention(PyObject* const* a) {
   void* op = device_ptr(output_like(a[5], q, "out", &out), "out", t);
   int32_t* status = (int32_t*)device_ptr(a[8], "dev_status", at::kInt);
   const Scratch ws(a[9], a[9] == Py_None ? spiffy_graph_attention_workspace(&d) : 0, q, false);
-  check(spiffy_graph_attention(&d, qp, kp, vp, kb, vb, op, status, ws.ptr, ws.bytes, stream_of(a[10])),
+  check(unlocked(spiffy_graph_attention, &d, qp, kp, vp, kb, vb, op, status, ws.ptr, ws.bytes, stream_of(a[10])),
         "spiffy_graph_attention");
   return out.release();
 }
@@ -295,8 +305,8 @@ PyObject* full_sequence_attention(PyObject* const* a) {
   void* osp = device_ptr(output_like(a[11], qs, "out_suffix", &os), "out_suffix", t);
   int32_t* status = (int32_t*)device_ptr(a[12], "dev_status", at::kInt);
   const Scratch ws(a[13], a[13] == Py_None ? spiffy_full_sequence_attention_workspace(&d, S) : 0, q, false);
-  check(spiffy_full_sequence_attention(&d, S, qp, qsp, kv[0], kv[1], kv[2], kv[3], kv[4], kv[5], onp, osp, status,
-                                       ws.ptr, ws.bytes, stream_of(a[14])),
+  check(unlocked(spiffy_full_sequence_attention, &d, S, qp, qsp, kv[0], kv[1], kv[2], kv[3], kv[4], kv[5], onp, osp,
+                 status, ws.ptr, ws.bytes, stream_of(a[14])),
         "spiffy_full_sequence_attention");
   PyObject* r = PyTuple_Pack(2, on.o, os.o);
   if (!r) throw PyError{};
@@ -355,8 +365,8 @@ PyObject* unmask_decide(PyObject* const* a) {
   Ref out(decision_for(a[6], &d, logits));
   const DecisionPtrs p(out.o, "dev_status");
   const Scratch ws(a[7], a[7] == Py_None ? spiffy_unmask_decide_workspace(&d) : 0, logits, true);
-  check(spiffy_unmask_decide(&d, lp, tp, p.conf, p.top_tok, p.bits, p.n_unmask, p.status, ws.ptr, ws.bytes,
-                             stream_of(a[8])),
+  check(unlocked(spiffy_unmask_decide, &d, lp, tp, p.conf, p.top_tok, p.bits, p.n_unmask, p.status, ws.ptr, ws.bytes,
+                 stream_of(a[8])),
         "spiffy_unmask_decide");
   return out.release();
 }
@@ -376,8 +386,8 @@ PyObject* unmask_decide_sampled(PyObject* const* a) {
   Ref out(decision_for(a[8], &d, logits));
   const DecisionPtrs p(out.o, "dev_status");
   const Scratch ws(a[9], a[9] == Py_None ? spiffy_unmask_decide_sampled_workspace(&d) : 0, logits, true);
-  check(spiffy_unmask_decide_sampled(&d, &s, lp, tp, p.conf, p.top_tok, p.bits, p.n_unmask, p.status, ws.ptr,
-                                     ws.bytes, stream_of(a[10])),
+  check(unlocked(spiffy_unmask_decide_sampled, &d, &s, lp, tp, p.conf, p.top_tok, p.bits, p.n_unmask, p.status, ws.ptr,
+                 ws.bytes, stream_of(a[10])),
         "spiffy_unmask_decide_sampled");
   return out.release();
 }
@@ -413,8 +423,8 @@ PyObject* lmhead_decide(PyObject* const* a) {
   Ref out(decision_for(a[7], &d, h));
   const DecisionPtrs p(out.o, "dev_status");
   const Scratch ws(a[8], a[8] == Py_None ? spiffy_lmhead_decide_workspace(&d, (int32_t)H) : 0, h, true);
-  check(spiffy_lmhead_decide(&d, (int32_t)H, hp, wp, tp, p.conf, p.top_tok, p.bits, p.n_unmask, p.status, ws.ptr,
-                             ws.bytes, stream_of(a[9])),
+  check(unlocked(spiffy_lmhead_decide, &d, (int32_t)H, hp, wp, tp, p.conf, p.top_tok, p.bits, p.n_unmask, p.status,
+                 ws.ptr, ws.bytes, stream_of(a[9])),
         "spiffy_lmhead_decide");
   return out.release();
 }
@@ -453,8 +463,8 @@ PyObject* accept_walk(PyObject* const* a) {
     out.o = new_walk(c, d.batch, d.n_nodes, d.block_len);
   }
   const WalkPtrs w(out.o, "dev_status");
-  check(spiffy_accept_walk(&d, tp, op, ip, cap, top, bits, w.accepted_node, w.n_accepted, w.path, w.next_block,
-                           w.status, stream_of(a[6])),
+  check(unlocked(spiffy_accept_walk, &d, tp, op, ip, cap, top, bits, w.accepted_node, w.n_accepted, w.path, w.next_block,
+                 w.status, stream_of(a[6])),
         "spiffy_accept_walk");
   return out.release();
 }
@@ -512,9 +522,9 @@ PyObject* decide_walk(PyObject* const* a) {
                       : lazy           ? spiffy_decide_walk_lazy_workspace(&d)
                                        : spiffy_unmask_decide_workspace(&d);
   const Scratch ws(a[10], need, logits, true);
-  check((lazy ? spiffy_decide_walk_lazy : spiffy_decide_walk)(
-            &d, lp, tp, op, ip, cap, p.conf, p.top_tok, p.bits, p.n_unmask, p.status, w.accepted_node, w.n_accepted,
-            w.path, w.next_block, w.status, ws.ptr, ws.bytes, stream_of(a[11])),
+  check(unlocked(lazy ? spiffy_decide_walk_lazy : spiffy_decide_walk, &d, lp, tp, op, ip, cap, p.conf, p.top_tok, p.bits,
+                 p.n_unmask, p.status, w.accepted_node, w.n_accepted, w.path, w.next_block, w.status, ws.ptr, ws.bytes,
+                 stream_of(a[11])),
         lazy ? "spiffy_decide_walk_lazy" : "spiffy_decide_walk");
   PyObject* r = PyTuple_Pack(2, dec.o, walk.o);
   if (!r) throw PyError{};
@@ -575,8 +585,8 @@ PyObject* draft_blocks(PyObject* const* a) {
   int32_t* pidx = (int32_t*)field_ptr(out.o, g_names.parent_idx, "parent_idx", at::kInt);
   int32_t* status = (int32_t*)field_ptr(out.o, g_names.dev_status, "dev_status", at::kInt);
   const Scratch ws(a[8], a[8] == Py_None ? spiffy_draft_blocks_workspace(&d) : 0, logits, true);
-  check(spiffy_draft_blocks(&d, logits.data_ptr(), sp, fo, fi, fj, co, ci, tokens, kept, score, poff, pidx, status,
-                            ws.ptr, ws.bytes, stream_of(a[9])),
+  check(unlocked(spiffy_draft_blocks, &d, logits.data_ptr(), sp, fo, fi, fj, co, ci, tokens, kept, score, poff, pidx,
+                 status, ws.ptr, ws.bytes, stream_of(a[9])),
         "spiffy_draft_blocks");
   return out.release();
 }
