@@ -10,10 +10,11 @@
 // walk are views of it), and outputs made here are not cleared by kernels of
 // their own: SPIFFY_FRESH_STATUS has the call's first kernel do it.
 #include <ATen/ATen.h>
-#include <c10/cuda/CUDAStream.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <initializer_list>
+#include <optional>
 #include <utility>
 #include <vector>
 
@@ -85,16 +86,33 @@ double as_float(PyObject* o) {
   return v;
 }
 
-// None: the current stream of the current device; else an object with a cuda_stream attribute.
-void* stream_of(PyObject* o) {
-  if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
-  PyObject* h = PyObject_GetAttrString(o, "cuda_stream");
-  if (!h) throw PyError{};
-  void* p = PyLong_AsVoidPtr(h);
-  Py_DECREF(h);
-  if (!p && PyErr_Occurred()) throw PyError{};
-  return p;
-}
+// The stream of a call.  None: the current stream of the current device; else an object with a
+// cuda_stream attribute, which is then the current stream for as long as the call's results and
+// scratch are allocated and cleared: the allocator hands memory out, and takes it back, in the order
+// of the stream that was current.
+class CallStream {
+ public:
+  CallStream(PyObject* o, const at::Tensor& like) {
+    if (o == Py_None) {
+      ptr_ = c10::cuda::getCurrentCUDAStream().stream();
+      return;
+    }
+    PyObject* h = PyObject_GetAttrString(o, "cuda_stream");
+    if (!h) throw PyError{};
+    ptr_ = static_cast<cudaStream_t>(PyLong_AsVoidPtr(h));
+    Py_DECREF(h);
+    if (!ptr_ && PyErr_Occurred()) throw PyError{};
+    if (!like.is_cuda()) return;  // refused further down
+    // cudaStreamLegacy is the default stream by another name
+    const cudaStream_t named = ptr_ == cudaStreamLegacy ? nullptr : ptr_;
+    guard_.emplace(c10::cuda::getStreamFromExternal(named, like.device().index()));
+  }
+  void* get() const { return ptr_; }
+
+ private:
+  cudaStream_t ptr_ = nullptr;
+  std::optional<c10::cuda::CUDAStreamGuard> guard_;
+};
 
 // One call into the library, without the interpreter lock: a launch waits when the stream's queue is
 // full, and other Python threads have their own work.  All it needs has been read by now.
@@ -116,8 +134,8 @@ void check(int status, const char* where) {
   throw PyError{};
 }
 
-// A call's scratch: the caller's, or allocated for the call (in stream order, so
-// that it may go back to the allocator when the call returns).
+// A call's scratch: the caller's, or allocated for the call (in the order of the
+// call's stream, so that it may go back to the allocator when the call returns).
 struct Scratch {
   at::Tensor own;
   void* ptr = nullptr;
@@ -277,11 +295,12 @@ PyObject* graph_attention(PyObject* const* a) {
   const void* vp = device_ptr(a[2], "v_prefix", t);
   const void* kb = device_ptr(a[3], "k_block", t);
   const void* vb = device_ptr(a[4], "v_block", t);
+  const CallStream stream(a[10], q);
   Ref out;
   void* op = device_ptr(output_like(a[5], q, "out", &out), "out", t);
   int32_t* status = (int32_t*)device_ptr(a[8], "dev_status", at::kInt);
   const Scratch ws(a[9], a[9] == Py_None ? spiffy_graph_attention_workspace(&d) : 0, q, false);
-  check(unlocked(spiffy_graph_attention, &d, qp, kp, vp, kb, vb, op, status, ws.ptr, ws.bytes, stream_of(a[10])),
+  check(unlocked(spiffy_graph_attention, &d, qp, kp, vp, kb, vb, op, status, ws.ptr, ws.bytes, stream.get()),
         "spiffy_graph_attention");
   return out.release();
 }
@@ -300,13 +319,14 @@ PyObject* full_sequence_attention(PyObject* const* a) {
   static const char* const names[] = {"k_prefix", "v_prefix", "k_suffix", "v_suffix", "k_block", "v_block"};
   const void* kv[6];
   for (int i = 0; i < 6; ++i) kv[i] = device_ptr(a[2 + i], names[i], t);
+  const CallStream stream(a[14], q);
   Ref on, os;
   void* onp = device_ptr(output_like(a[10], q, "out_nodes", &on), "out_nodes", t);
   void* osp = device_ptr(output_like(a[11], qs, "out_suffix", &os), "out_suffix", t);
   int32_t* status = (int32_t*)device_ptr(a[12], "dev_status", at::kInt);
   const Scratch ws(a[13], a[13] == Py_None ? spiffy_full_sequence_attention_workspace(&d, S) : 0, q, false);
   check(unlocked(spiffy_full_sequence_attention, &d, S, qp, qsp, kv[0], kv[1], kv[2], kv[3], kv[4], kv[5], onp, osp,
-                 status, ws.ptr, ws.bytes, stream_of(a[14])),
+                 status, ws.ptr, ws.bytes, stream.get()),
         "spiffy_full_sequence_attention");
   PyObject* r = PyTuple_Pack(2, on.o, os.o);
   if (!r) throw PyError{};
@@ -362,11 +382,12 @@ PyObject* unmask_decide(PyObject* const* a) {
   spiffy_decide_desc d = decide_desc(logits, tokens, a + 2);
   const void* lp = logits_ptr(logits);
   const int32_t* tp = (const int32_t*)device_ptr(tokens, "block_tokens", at::kInt);
+  const CallStream stream(a[8], logits);
   Ref out(decision_for(a[6], &d, logits));
   const DecisionPtrs p(out.o, "dev_status");
   const Scratch ws(a[7], a[7] == Py_None ? spiffy_unmask_decide_workspace(&d) : 0, logits, true);
   check(unlocked(spiffy_unmask_decide, &d, lp, tp, p.conf, p.top_tok, p.bits, p.n_unmask, p.status, ws.ptr, ws.bytes,
-                 stream_of(a[8])),
+                 stream.get()),
         "spiffy_unmask_decide");
   return out.release();
 }
@@ -383,11 +404,12 @@ PyObject* unmask_decide_sampled(PyObject* const* a) {
   if (PyErr_Occurred()) throw PyError{};
   const void* lp = logits_ptr(logits);
   const int32_t* tp = (const int32_t*)device_ptr(tokens, "block_tokens", at::kInt);
+  const CallStream stream(a[10], logits);
   Ref out(decision_for(a[8], &d, logits));
   const DecisionPtrs p(out.o, "dev_status");
   const Scratch ws(a[9], a[9] == Py_None ? spiffy_unmask_decide_sampled_workspace(&d) : 0, logits, true);
   check(unlocked(spiffy_unmask_decide_sampled, &d, &s, lp, tp, p.conf, p.top_tok, p.bits, p.n_unmask, p.status, ws.ptr,
-                 ws.bytes, stream_of(a[10])),
+                 ws.bytes, stream.get()),
         "spiffy_unmask_decide_sampled");
   return out.release();
 }
@@ -420,11 +442,12 @@ PyObject* lmhead_decide(PyObject* const* a) {
   const void* hp = device_ptr(h, "hidden_states", kAnyType);
   const void* wp = device_ptr(w, "weight", kAnyType);
   const int32_t* tp = (const int32_t*)device_ptr(tokens, "block_tokens", at::kInt);
+  const CallStream stream(a[9], h);
   Ref out(decision_for(a[7], &d, h));
   const DecisionPtrs p(out.o, "dev_status");
   const Scratch ws(a[8], a[8] == Py_None ? spiffy_lmhead_decide_workspace(&d, (int32_t)H) : 0, h, true);
   check(unlocked(spiffy_lmhead_decide, &d, (int32_t)H, hp, wp, tp, p.conf, p.top_tok, p.bits, p.n_unmask, p.status,
-                 ws.ptr, ws.bytes, stream_of(a[9])),
+                 ws.ptr, ws.bytes, stream.get()),
         "spiffy_lmhead_decide");
   return out.release();
 }
@@ -453,6 +476,7 @@ PyObject* accept_walk(PyObject* const* a) {
   const int32_t* ip = (const int32_t*)device_ptr(idx, "parent_idx", at::kInt);
   const int32_t* top = (const int32_t*)device_ptr(a[3], "top_tok", at::kInt);
   const uint64_t* bits = (const uint64_t*)device_ptr(a[4], "unmask_bits", at::kLong);
+  const CallStream stream(a[6], tokens);
   Ref out;
   if (a[5] != Py_None) {
     Py_INCREF(a[5]);
@@ -464,7 +488,7 @@ PyObject* accept_walk(PyObject* const* a) {
   }
   const WalkPtrs w(out.o, "dev_status");
   check(unlocked(spiffy_accept_walk, &d, tp, op, ip, cap, top, bits, w.accepted_node, w.n_accepted, w.path, w.next_block,
-                 w.status, stream_of(a[6])),
+                 w.status, stream.get()),
         "spiffy_accept_walk");
   return out.release();
 }
@@ -487,6 +511,7 @@ PyObject* decide_walk(PyObject* const* a) {
   const int32_t* tp = (const int32_t*)device_ptr(tokens, "block_tokens", at::kInt);
   const int32_t* op = (const int32_t*)device_ptr(off, "parent_off", at::kInt);
   const int32_t* ip = (const int32_t*)device_ptr(idx, "parent_idx", at::kInt);
+  const CallStream stream(a[11], logits);
   Ref dec, walk;
   if (a[8] == Py_None && a[9] == Py_None) {
     d.logits_dtype |= SPIFFY_FRESH_STATUS;
@@ -524,7 +549,7 @@ PyObject* decide_walk(PyObject* const* a) {
   const Scratch ws(a[10], need, logits, true);
   check(unlocked(lazy ? spiffy_decide_walk_lazy : spiffy_decide_walk, &d, lp, tp, op, ip, cap, p.conf, p.top_tok, p.bits,
                  p.n_unmask, p.status, w.accepted_node, w.n_accepted, w.path, w.next_block, w.status, ws.ptr, ws.bytes,
-                 stream_of(a[11])),
+                 stream.get()),
         lazy ? "spiffy_decide_walk_lazy" : "spiffy_decide_walk");
   PyObject* r = PyTuple_Pack(2, dec.o, walk.o);
   if (!r) throw PyError{};
@@ -563,6 +588,7 @@ PyObject* draft_blocks(PyObject* const* a) {
   const int32_t* fj = (const int32_t*)field_ptr(g, g_names.formula_j, "formula_j", at::kInt);
   const int32_t* co = (const int32_t*)field_ptr(g, g_names.child_off, "child_off", at::kInt);
   const int32_t* ci = (const int32_t*)field_ptr(g, g_names.child_idx, "child_idx", at::kInt);
+  const CallStream stream(a[9], logits);
   Ref out;
   if (a[7] != Py_None) {
     Py_INCREF(a[7]);
@@ -586,7 +612,7 @@ PyObject* draft_blocks(PyObject* const* a) {
   int32_t* status = (int32_t*)field_ptr(out.o, g_names.dev_status, "dev_status", at::kInt);
   const Scratch ws(a[8], a[8] == Py_None ? spiffy_draft_blocks_workspace(&d) : 0, logits, true);
   check(unlocked(spiffy_draft_blocks, &d, logits.data_ptr(), sp, fo, fi, fj, co, ci, tokens, kept, score, poff, pidx,
-                 status, ws.ptr, ws.bytes, stream_of(a[9])),
+                 status, ws.ptr, ws.bytes, stream.get()),
         "spiffy_draft_blocks");
   return out.release();
 }
