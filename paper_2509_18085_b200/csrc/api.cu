@@ -17,6 +17,18 @@ uint32_t mbar_poll_limit() { return g_mbar_polls.load(std::memory_order_relaxed)
 uint32_t flag_poll_limit() { return g_flag_polls.load(std::memory_order_relaxed); }
 int32_t lazy_extra_arrivals() { return g_lazy_extra.load(std::memory_order_relaxed); }
 
+int sm_count() {
+  static std::atomic<int> known[64];
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return 0;
+  int n = known[device].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
+    known[device].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
 namespace {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

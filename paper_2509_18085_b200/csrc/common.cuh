@@ -59,6 +59,9 @@ __device__ __forceinline__ void st_global(void* p, uint4 v) {
   asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
 }
 
+// Multiprocessors of the current device, 0 when it cannot be asked.  Safe with several threads.
+int sm_count();
+
 // Every launch of the library goes through this counter (spiffy_launch_count).
 void count_launch(int n = 1);
 

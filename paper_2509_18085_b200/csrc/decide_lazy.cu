@@ -331,19 +331,14 @@ size_t lazy_graph_bytes(const spiffy_decide_desc& d, int parent_cap) {
   return ((size_t)d.n_nodes * d.block_len + d.n_nodes + 1 + parent_cap) * 4;
 }
 
-// CTAs that can be resident at once on `device` (cooperative launch limit).
+// CTAs that can be resident at once on the current device (cooperative launch limit).
 template <typename T>
-int resident_ctas(int device, size_t smem) {
-  static int sm_count[64];
-  if (device < 0 || device >= 64) return 0;
-  if (sm_count[device] == 0 &&
-      cudaDeviceGetAttribute(&sm_count[device], cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
-    return 0;
+int resident_ctas(size_t smem) {
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decide_walk_lazy_kernel<T>,
                                                     kReduceThreads, smem) != cudaSuccess)
     return 0;
-  return per_sm * sm_count[device];
+  return per_sm * sm_count();
 }
 
 }  // namespace
@@ -362,15 +357,13 @@ spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc& d, const void* l
                                       int32_t* accepted_node, int32_t* n_accepted, int32_t* path,
                                       int32_t* next_block, int32_t* walk_status, void* ws,
                                       bool fresh, cudaStream_t stream) {
-  int device = 0;
-  if (cudaGetDevice(&device) != cudaSuccess) return SPIFFY_ECUDA;
   const bool bf16 = d.logits_dtype == SPIFFY_BF16;
   const size_t graph = lazy_graph_bytes(d, parent_cap);
   const int stage_graph = graph <= 16 * 1024;  // beyond that it would cost resident CTAs
   const size_t slices = (size_t)d.block_len * decide_splits(d, nullptr) * sizeof(Partial);
   const int stage_slices = slices <= 20 * 1024;
   const size_t smem = (stage_graph ? graph : 0) + (stage_slices ? slices : 0);
-  const int resident = bf16 ? resident_ctas<__nv_bfloat16>(device, smem) : resident_ctas<float>(device, smem);
+  const int resident = bf16 ? resident_ctas<__nv_bfloat16>(smem) : resident_ctas<float>(smem);
   if (resident <= 0) return SPIFFY_ECUDA;
   if (d.batch > resident) return SPIFFY_EUNSUPPORTED;  // one resident CTA per sequence runs its tail
   LazyParams p;

@@ -381,14 +381,7 @@ size_t list_bytes(const spiffy_decide_desc& d) { return up256(((size_t)d.batch *
 
 // One CTA per SM, or fewer for a vocabulary of fewer than 32 entries each.
 int lmhead_grid(const spiffy_decide_desc& d) {
-  static std::atomic<int> sms[64];
-  int device = 0;
-  if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return 0;
-  int n = sms[device].load(std::memory_order_relaxed);
-  if (n == 0) {
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-    sms[device].store(n, std::memory_order_relaxed);
-  }
+  const int n = sm_count();
   const int units = (d.vocab + kBox - 1) / kBox;
   return units < n ? units : n;
 }
