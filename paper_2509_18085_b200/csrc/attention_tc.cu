@@ -56,9 +56,15 @@
 // gets.
 //
 // Head dimension 64 halves every tile (one 64-column half instead of two) and the
-// products, not the exponentials: the softmax warps bound it.  3 sequences of 100
-// positions x 24 heads over 777 + 20 keys: 215 us on the CUDA cores, about 13 us
-// here.
+// products, not the exponentials.  The CUDA-core kernel, which this one stands in for
+// there, keeps P in fp32: here P enters the second product as two bf16 terms, its
+// rounding and what that left over (2^-17 of a value short of fp32, in the tensor
+// memory that the narrower O leaves), so that the result's error against float64 is
+// the CUDA cores' (0.166 % in the 2-norm, the rounding of the output, over 50 to 4096
+// keys; with one term 0.18 to 0.23 %).  The second term costs 4 to 9 % of a call of
+// few key tiles, 24 % of a long one (4 x 32 x 32 positions x 32 heads over 4096 keys:
+// 232 -> 288 us; CUDA cores 4596); 3 sequences of 100 positions x 24 heads over 777 +
+// 20 keys: 12.5 us, 11.6 with one term, 89 on the CUDA cores.
 //
 // Every wait is bounded; a wait that gives up raises SPIFFY_DEV_TIMEOUT in the
 // caller's status word and the CTA winds down without touching its output.
@@ -82,8 +88,10 @@ constexpr int kRegsIssue = 40, kRegsSoftmax = 232;
 static_assert(kRegsIssue + 2 * kRegsSoftmax <= 3 * 168, "within what the block was launched with");
 constexpr int kHalfBytes = BN * 128;           // one 64-column half of a tile: 128 rows x 128 B
 constexpr uint32_t kTmemCols = 512;
-// S: 128 columns; warpgroup w: P (bf16 pairs) at 128 + 64 w, O at 256 + w * head dim
-constexpr uint32_t kColS = 0, kColP = 128, kColO = 256;
+// S: 128 columns; warpgroup w: P (bf16 pairs) at 128 + 64 w, O at 256 + w * head dim, and at head
+// dimension 64, what the rounding of P left over at 384 + 64 w
+constexpr uint32_t kColS = 0, kColP = 128, kColO = 256, kColRest = 384;
+static_assert(kColRest + 2 * 64 <= kTmemCols && kColO + 2 * 64 <= kColRest, "tensor memory at head dimension 64");
 constexpr float kRescaleLog2 = 8.0f;
 
 // Shared memory: NQ Q tiles, a K ring of 3 stages and a V ring of 4 - NQ, seven tiles of
@@ -163,11 +171,12 @@ __device__ __forceinline__ float row_max(const uint32_t (&s)[BN]) {
 
 // p = 2^(s * k2 - m_use) for the flagged 32-column chunks among columns C0 .. C0 + 63 (zero
 // elsewhere), packed as bf16 pairs into pk; returns the sum of the p's (fp32, before rounding to
-// bf16).  The special-function unit takes 8 cycles per warp and exponential; everything else a pair
+// bf16).  kRest: rest gets p - bf16(p), rounded to bf16 in its turn, so that pk + rest is p to 2^-17.
+// The special-function unit takes 8 cycles per warp and exponential; everything else a pair
 // needs fits under its two.
-template <int C0>
+template <int C0, bool kRest>
 __device__ __forceinline__ float row_exps(const uint32_t (&s)[BN], uint32_t need, float k2, float m_use,
-                                          uint32_t (&pk)[32]) {
+                                          uint32_t (&pk)[32], uint32_t (&rest)[32]) {
   const uint64_t k22 = pack2(k2, k2), nm2 = pack2(-m_use, -m_use);
   uint64_t sum_a = pack2(0.f, 0.f), sum_b = pack2(0.f, 0.f);
 #pragma unroll
@@ -180,11 +189,16 @@ __device__ __forceinline__ float row_exps(const uint32_t (&s)[BN], uint32_t need
         unpack2(x2, x0, x1);
         const float p0 = ex2(x0), p1 = ex2(x1);
         if ((c >> 1) & 1) sum_b = add2(sum_b, pack2(p0, p1)); else sum_a = add2(sum_a, pack2(p0, p1));
-        pk[c >> 1] = pack_bf16(p0, p1);
+        const uint32_t w = pack_bf16(p0, p1);
+        pk[c >> 1] = w;
+        if (kRest) rest[c >> 1] = pack_bf16(p0 - __uint_as_float(w << 16), p1 - __uint_as_float(w & 0xffff0000u));
       }
     } else {
 #pragma unroll
-      for (int c = 16 * h; c < 16 * h + 16; ++c) pk[c] = 0u;
+      for (int c = 16 * h; c < 16 * h + 16; ++c) {
+        pk[c] = 0u;
+        if (kRest) rest[c] = 0u;
+      }
     }
   }
   float a0, a1;
@@ -228,6 +242,7 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
   using SM = Smem<NQ, HD>;
   constexpr int KS = SM::ks, VS = SM::vs, kTileBytes = SM::tile;
   constexpr int kHalves = HD / 64;    // 64-column halves of a tile
+  constexpr bool kRest = HD == 64;    // P in two bf16 terms
   constexpr int kLogNQ = NQ - 1;      // key tile of unit u = u >> kLogNQ
   uint8_t* sq = smem + SM::q;
   uint8_t* sk = smem + SM::k;
@@ -411,6 +426,9 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
           tc_fence_after_sync();
           umma_ts_k128(tmem + kColO + (uint32_t)(u & 1) * HD, tmem + kColP + (uint32_t)(u & 1) * 64u,
                        v_lo + (uint32_t)stage * (kTileBytes >> 4), hi, idesc, u >= 2 ? 1u : 0u);
+          if constexpr (kRest)
+            umma_ts_k128(tmem + kColO + (uint32_t)(u & 1) * HD, tmem + kColRest + (uint32_t)(u & 1) * 64u,
+                         v_lo + (uint32_t)stage * (kTileBytes >> 4), hi, idesc, 1u);
           umma_commit(pv_done + (u & 1));
           if (NQ == 1 || (u & 1)) {
             umma_commit(v_empty + stage);
@@ -436,6 +454,7 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
     bool ok = true;
     const uint32_t at_p = tmem_addr(tmem, lane_base, kColP + (uint32_t)wg * 64u);
     const uint32_t at_o = tmem_addr(tmem, lane_base, kColO + (uint32_t)wg * HD);
+    const uint32_t at_rest = tmem_addr(tmem, lane_base, kColRest + (uint32_t)wg * 64u);
     // the P V products of unit u (one of this warpgroup's) have completed
     auto wait_pv = [&](int u) -> bool {
       const bool yes = __all_sync(0xffffffffu, mbar_wait(pv_done + wg, (uint32_t)(u >> 1) & 1u, abort_flag, p.spin_limit));
@@ -507,14 +526,16 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
         }
       }
       const float m_use = (m_run == -INFINITY) ? 0.f : m_run;
-      uint32_t pk[32];
-      l_run += row_exps<0>(s, chunks, k2, m_use, pk);
+      uint32_t pk[32], rest[32];
+      l_run += row_exps<0, kRest>(s, chunks, k2, m_use, pk, rest);
       // the products that read this P buffer last (two units ago) are done
       ok = u < 2 || wait_pv(u - 2);
       if (!ok) break;
       tmem_st_x32(at_p, pk);
-      l_run += row_exps<64>(s, chunks, k2, m_use, pk);
+      if (kRest) tmem_st_x32(at_rest, rest);
+      l_run += row_exps<64, kRest>(s, chunks, k2, m_use, pk, rest);
       tmem_st_x32(at_p + 32u, pk);
+      if (kRest) tmem_st_x32(at_rest + 32u, rest);
       tmem_wait_st();
       tc_fence_before_sync();
       __syncwarp();  // every lane's P is in tensor memory: one arrival speaks for the warp

@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
     (1, 3, 7, 127, 16, 16), (1, 3, 7, 129, 16, 16),  # context one short of / one past a key tile
     (1, 8, 32, 512, 16, 16),                      # cluster pairs, odd number of key tiles
     (1, 8, 32, 640, 16, 16),                      # cluster pairs, even
-    (1, 9, 8, 1000, 3, 3),                        # many slices through the workspace
+    (1, 9, 8, 1000, 3, 3),                        # clusters of eight
     (3, 9, 32, 300, 32, 32),                      # two M-tiles per CTA, the second one partly beyond the rows
     (2, 4, 12, 129, 28, 4),                       # grouped heads: M-tiles of 126 rows
     (1, 2, 3, 20, 128, 1),                        # one position per M-tile
@@ -46,3 +46,36 @@ def test_reruns_are_bit_identical_and_the_kernel_is_the_tensor_core_one():
     finally:
         spiffy.set_wait_limits()
     assert int(status[0]) == spiffy.DEV_TIMEOUT
+
+
+@pytest.mark.parametrize("B,N,L,P,Hq,Hkv", [(3, 5, 20, 777, 24, 8), (1, 8, 32, 512, 16, 16), (2, 9, 32, 4096, 32, 32),
+                                            (1, 64, 4, 2048, 32, 8), (1, 3, 5, 50, 5, 5)])
+@pytest.mark.parametrize("spread", [1.0, 4.0])
+def test_no_less_precise_than_the_cuda_cores(B, N, L, P, Hq, Hkv, spread):
+    """Probabilities enter the second product in two bf16 terms, 2^-17 of their value short of fp32.  Both
+    kernels' error is then the rounding of the result to bf16 (2^-9 of a value at most, 0.17 % in the
+    2-norm): in quadrature the rest is 1e-5 of it.  One bf16 term would make the error a fifth larger."""
+    g = torch.Generator(device="cuda").manual_seed(P)
+    r = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    q, kp, vp, kb, vb = r(B, N, L, Hq, 64) * spread, r(B, P, Hkv, 64), r(B, P, Hkv, 64), r(B, N, L, Hkv, 64), r(B, N, L, Hkv, 64)
+    want = float64_attention(q, kp, vp, kb, vb)
+    err = {}
+    for kernel in (spiffy.ATTN_AUTO, spiffy.ATTN_SIMT):
+        out = spiffy.spiffy_graph_attention(q, kp, vp, kb, vb, kernel=kernel).double()
+        err[kernel] = float((out - want).norm() / want.norm())
+    print(err)
+    assert err[spiffy.ATTN_AUTO] <= 1.005 * err[spiffy.ATTN_SIMT]
+
+
+def float64_attention(q, kp, vp, kb, vb):
+    (B, N, L, Hq, d), Hkv = q.shape, kp.shape[2]
+    group = Hq // Hkv
+    up = lambda t: t.double().repeat_interleave(group, dim=-2)
+    out = torch.empty(q.shape, dtype=torch.float64, device=q.device)
+    for b in range(B):
+        kc, vc = up(kp[b]), up(vp[b])
+        for n in range(N):
+            k, v = torch.cat([kc, up(kb[b, n])]), torch.cat([vc, up(vb[b, n])])
+            p = torch.softmax(torch.einsum("lhd,khd->hlk", q[b, n].double(), k) / d ** 0.5, -1)
+            out[b, n] = torch.einsum("hlk,khd->lhd", p, v)
+    return out
