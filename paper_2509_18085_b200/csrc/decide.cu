@@ -22,28 +22,34 @@ namespace spiffy {
 namespace {
 
 // grid = (splits, B*N*L); one CTA reduces one vocabulary slice of one row.
-template <typename T>
+// kIndependent: the kernel before this one, which may still run, writes none of its inputs and has
+// let it start only when all others were complete (SPIFFY_INDEPENDENT).  A kernel of its own: the
+// token from L2 instead of L1, the wait at the end and the way to it cost the plain one 3 to 4 % of
+// the call, and the status words cleared ahead of the token's load, for which every CTA waits first,
+// another 1 to 2 % (256 rows x 126464 with 164 masked: 13.0 us with all that, 12.4 so; 512 rows x
+// 152064 with 348 masked: 24.6 and 23.4).
+template <typename T, bool kIndependent>
 __global__ void __launch_bounds__(kReduceThreads, 8)  // 64 registers: eight CTAs per SM
 decide_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V,
                      int64_t chunk, int splits,
                      const int32_t* __restrict__ block_tokens, int mask_id,
-                     Partial* __restrict__ partials, int early_trigger, int independent, StatusClear clear) {
+                     Partial* __restrict__ partials, int early_trigger, StatusClear clear) {
 #if __CUDA_ARCH__ >= 900
-  // Inputs written by earlier kernels are visible; the kernel before this one may write none of
-  // them and have let this one start only when all others were complete.
-  if (!independent) cudaGridDependencySynchronize();
+  if (!kIndependent) cudaGridDependencySynchronize();  // inputs written by earlier kernels are visible
   // The one-CTA-per-sequence tail kernel may take its SM while this grid still
   // runs (it waits there for this grid to finish): its launch latency is hidden.
   if (early_trigger) pdl_launch_dependents();
 #endif
   const int row = blockIdx.y;
-  if (blockIdx.x == 0 && threadIdx.x == kReduceThreads - 1) clear.run(row);
-  if (__ldcg(block_tokens + row) == mask_id)  // already unmasked: never read
+  const int32_t token = kIndependent ? __ldcg(block_tokens + row) : block_tokens[row];
+  if (blockIdx.x == 0 && threadIdx.x == kReduceThreads - 1 && row < clear.batch) clear.run(row);
+  if (!kIndependent && token != mask_id) return;  // already unmasked: never read
+  if (token == mask_id)
     reduce_slice(logits + (int64_t)row * row_stride, V, chunk, (int)blockIdx.x,
                  partials + (int64_t)row * splits + blockIdx.x);
 #if __CUDA_ARCH__ >= 900
   // This grid is complete, for all that wait for it, no sooner than the one before it.
-  if (independent && blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y) cudaGridDependencySynchronize();
+  if (kIndependent && blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y) cudaGridDependencySynchronize();
 #endif
 }
 
@@ -211,16 +217,16 @@ spiffy_status launch_reduce(const spiffy_decide_desc& d, const void* logits,
                             cudaStream_t stream) {
   const int rows = d.batch * d.n_nodes * d.block_len;
   const dim3 grid(splits, rows);
-  cudaError_t e;
-  if (d.logits_dtype == SPIFFY_BF16)
-    e = launch_pdl(decide_reduce_kernel<__nv_bfloat16>, grid, dim3(kReduceThreads), (size_t)0, stream,
-                   static_cast<const __nv_bfloat16*>(logits), (int64_t)d.row_stride, (int)d.vocab,
-                   chunk, splits, block_tokens, (int)d.mask_token_id, partials, early_trigger,
-                   (int)independent, clear);
-  else
-    e = launch_pdl(decide_reduce_kernel<float>, grid, dim3(kReduceThreads), (size_t)0, stream,
-                   static_cast<const float*>(logits), (int64_t)d.row_stride, (int)d.vocab, chunk,
-                   splits, block_tokens, (int)d.mask_token_id, partials, early_trigger, (int)independent, clear);
+  auto run = [&](auto* typed, auto plain, auto beside) {
+    return launch_pdl(independent ? beside : plain, grid, dim3(kReduceThreads), (size_t)0, stream, typed,
+                      (int64_t)d.row_stride, (int)d.vocab, chunk, splits, block_tokens, (int)d.mask_token_id,
+                      partials, early_trigger, clear);
+  };
+  const cudaError_t e = d.logits_dtype == SPIFFY_BF16
+                            ? run(static_cast<const __nv_bfloat16*>(logits), decide_reduce_kernel<__nv_bfloat16, false>,
+                                  decide_reduce_kernel<__nv_bfloat16, true>)
+                            : run(static_cast<const float*>(logits), decide_reduce_kernel<float, false>,
+                                  decide_reduce_kernel<float, true>);
   count_launch();
   return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
 }

@@ -36,9 +36,8 @@ struct StatusClear {
   int32_t* a;  // [B], null when there is nothing to clear
   int32_t* b;
   int batch;   // 0: nothing to clear
-  // one thread per row calls it, and not the one whose chain the CTA waits for
+  // one thread per row below `batch` calls it, and not the one whose chain the CTA waits for
   __device__ __forceinline__ void run(int row) const {
-    if (row >= batch) return;
     if (a) a[row] = 0;
     if (b) b[row] = 0;
   }

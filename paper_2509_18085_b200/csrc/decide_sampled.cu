@@ -100,11 +100,12 @@ decide_sampled_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, i
   cudaGridDependencySynchronize();
 #endif
   const int row = blockIdx.y;
-  if (blockIdx.x == 0 && threadIdx.x == kReduceThreads - 1) {
-    if (row < nodes) node_count[row] = 0;
-    clear.run(row);
+  const int32_t token = block_tokens[row];  // ahead of the clearing: every CTA waits for it first
+  if (blockIdx.x == 0 && threadIdx.x == kReduceThreads - 1 && row < nodes) {  // at least as many as sequences
+    node_count[row] = 0;
+    if (row < clear.batch) clear.run(row);
   }
-  if (block_tokens[row] != mask_id) return;  // already unmasked: never read
+  if (token != mask_id) return;  // already unmasked: never read
   reduce_slice(logits + (int64_t)row * row_stride, V, chunk, (int)blockIdx.x,
                partials + (int64_t)row * splits + blockIdx.x, k);
 }

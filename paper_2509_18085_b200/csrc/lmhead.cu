@@ -92,7 +92,7 @@ lmhead_gather_kernel(const uint4* __restrict__ h, int row_vecs, const int32_t* _
   pdl_launch_dependents();
   const int row = blockIdx.x, tid = threadIdx.x;
   const bool last = row + 1 == (int)gridDim.x;
-  if (tid == kGatherThreads - 1) clear.run(row);
+  if (tid == kGatherThreads - 1 && row < clear.batch) clear.run(row);
   const bool masked = tokens[row] == mask_id;
   if (!masked && !last) return;
   int before = 0;

@@ -70,7 +70,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
   auto i = [&](int k) { return std::to_string(*static_cast<int*>(args[k])); };
   auto p = [&](int k) { return num(*static_cast<void**>(args[k])); };
   std::string more;
-  if (name.find("decide_reduce_kernel") != std::string::npos) more = " early " + i(8) + " independent " + i(9);
+  if (name.find("decide_reduce_kernel") != std::string::npos) more = " early " + i(8);
   if (name.find("accept_walk_kernel") != std::string::npos) more = " lists " + p(3) + " staged " + i(13);
   if (name.find("decide_tail_kernel") != std::string::npos) more = " lists " + p(14) + " early " + i(22);
   return note("launch " + name + on(c->stream) + more);

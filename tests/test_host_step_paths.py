@@ -147,6 +147,6 @@ def test_an_independent_kernel_may_start_as_the_reduce_ends(host, N, L, cap):
                                        ctypes.c_void_p(STREAM)) == spiffy.OK
         log = host.fake_log().decode().splitlines()
         assert len(log) == (2 if fused else 3)
-        assert log[0].endswith(f" early {'1' if fused else early} independent 0")
+        assert log[0].endswith(f" early {'1' if fused else early}")
         if fused:  # the tail is resident while the reduce runs either way
             assert log[1].endswith(f" early {early}")
