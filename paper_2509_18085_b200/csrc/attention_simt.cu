@@ -316,7 +316,7 @@ struct Choice {
 Choice choose(const spiffy_attn_desc& d) {
   constexpr int kRows[3] = {64, 32, 16};
   constexpr float alone[3] = {9.6f, 6.4f, 3.4f}, shared[3] = {8.8f, 4.7f, 4.3f};
-  constexpr int kSms = 148;
+  const int sms = sm_count() > 0 ? sm_count() : 1;
   const int64_t rows = (int64_t)d.n_nodes * d.block_len * (d.n_q_heads / d.n_kv_heads);
   const int64_t bg = (int64_t)d.batch * d.n_kv_heads;
   const int tiles = (d.prefix_len + kKeys - 1) / kKeys + 1;  // at least
@@ -325,7 +325,7 @@ Choice choose(const spiffy_attn_desc& d) {
   for (int i = 0; i < 3; ++i) {
     const int64_t ctas = bg * ((rows + kRows[i] - 1) / kRows[i]);
     for (int s = 1; s <= kMaxCluster && s <= tiles; ++s) {
-      const int64_t per_sm = (ctas * s + kSms - 1) / kSms;
+      const int64_t per_sm = (ctas * s + sms - 1) / sms;
       const int per_slice = (tiles + s - 1) / s;
       if ((s & (s - 1)) != 0 && (s != tiles || per_sm > 1)) continue;
       const bool narrow = d.head_dim == 64;

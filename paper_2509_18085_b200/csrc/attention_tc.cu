@@ -62,8 +62,8 @@
 // memory that the narrower O leaves), so that the result's error against float64 is
 // the CUDA cores' (0.166 % in the 2-norm, the rounding of the output, over 50 to 4096
 // keys; with one term 0.18 to 0.23 %).  The second term costs 4 to 9 % of a call of
-// few key tiles, 24 % of a long one (4 x 32 x 32 positions x 32 heads over 4096 keys:
-// 232 -> 288 us; CUDA cores 4596); 3 sequences of 100 positions x 24 heads over 777 +
+// few key tiles, 20 % of a long one (4 x 32 x 32 positions x 32 heads over 4096 keys:
+// 232 -> 277 us; CUDA cores 4596); 3 sequences of 100 positions x 24 heads over 777 +
 // 20 keys: 12.5 us, 11.6 with one term, 89 on the CUDA cores.
 //
 // Every wait is bounded; a wait that gives up raises SPIFFY_DEV_TIMEOUT in the
@@ -803,22 +803,30 @@ int resident_clusters(int hd, int cs) {
 }
 
 // One or two M-tiles per CTA, and how many CTAs share the key tiles of an M-tile:
-// whatever a model of the kernel's time, fitted to measurements, finds cheapest.  A
-// round of CTAs (148, each holds its SM) takes 7 us plus 0.85 us per key tile with one
-// M-tile, 1.6 us with two; handing the partials around a cluster costs 2 us and a
-// little more in larger clusters, so that a second CTA pays from about six key tiles.
+// whatever a model of the kernel's time finds cheapest.  A round of CTAs (each holds its
+// SM) takes 7 us plus, per key tile, 0.85 us with one M-tile and 1.6 with two; at head
+// dimension 64, where the second product has two terms, 0.95 and 1.9.  Handing the
+// partials around a cluster costs about 2 us (1.5 with rows half as long), so that a second
+// CTA pays from about six key tiles.  The model is there to choose: of 35 shapes (1 to 1088
+// M-tiles, 2 to 33 key tiles), each timed with every plan it allows, it takes the fastest,
+// or one within 1.5 % of it, at both head dimensions.  Its times are low for long calls of
+// several rounds: 4 x 32 x 32 positions x 32 heads over 4096 keys, 239 us for two M-tiles a
+// CTA and 245 for one at head dimension 128, measured 264 and 274 back to back on the same
+// inputs; at 64, 279 and 269, measured 288 and 278.
 // `tiles` counts the M-tiles of all problems of the launch, `pairs` the CTAs that take two
 // of them, T is the key tiles of the longer problem.
 Plan make_plan(int64_t tiles, int64_t pairs, int T, int hd) {
-  constexpr int kSms = 148;
-  auto rounds = [](int64_t ctas) { return (float)((ctas + kSms - 1) / kSms); };
+  const int sms = sm_count();
+  const float one = hd == 128 ? 0.85f : 0.95f, two = hd == 128 ? 1.6f : 1.9f;
+  auto rounds = [&](int64_t ctas) { return (float)((ctas + sms - 1) / sms); };
   Plan pl = {2, 1};
-  float best = rounds(pairs) * (7.0f + 1.6f * (float)T);
+  if (sms <= 0) return pl;
+  float best = rounds(pairs) * (7.0f + two * (float)T);
   for (int cs = 1; cs <= 8 && cs <= T; cs *= 2) {
     // clusters only where all of them run at once
-    if (cs > 1 && (tiles * cs > kSms || tiles > resident_clusters(hd, cs))) continue;
-    const float exchange = cs == 1 ? 0.f : 1.9f + 0.07f * (float)cs;
-    const float cost = rounds(tiles * cs) * (7.0f + exchange + 0.85f * (float)((T + cs - 1) / cs));
+    if (cs > 1 && (tiles * cs > sms || tiles > resident_clusters(hd, cs))) continue;
+    const float exchange = cs == 1 ? 0.f : (hd == 128 ? 1.9f : 1.4f) + 0.07f * (float)cs;
+    const float cost = rounds(tiles * cs) * (7.0f + exchange + one * (float)((T + cs - 1) / cs));
     if (cost < best) {
       best = cost;
       pl = {1, cs};
