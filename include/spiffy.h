@@ -103,12 +103,17 @@ typedef enum { SPIFFY_RULE_TOPS = 0, SPIFFY_RULE_THRESHOLD = 1 } spiffy_rule;
 #define SPIFFY_FRESH_STATUS 0x100
 /* Flags, OR-ed into spiffy_decide_desc.logits_dtype of spiffy_decide_walk (other
  * calls ignore them), for a decision and an attention that take nothing from one
- * another and follow one another in a stream: they then run side by side, and
- * what follows in the stream still follows both.
+ * another and follow one another in a stream: the later one may start while the
+ * earlier one runs, and what follows in the stream still follows both.
  * SPIFFY_INDEPENDENT: the call before this one is an attention call on the
  * CUDA-core kernel and writes none of this call's inputs.
  * SPIFFY_INDEPENDENT_NEXT: the next call is an attention call with
- * SPIFFY_ATTN_INDEPENDENT. */
+ * SPIFFY_ATTN_INDEPENDENT.  It starts as the vocabulary reduce lets go of the
+ * multiprocessors (a tensor-core attention needs whole ones) and runs beside the
+ * rest of the decision: worth most where the call's end, the merge of the slices
+ * and the walk, is a good part of it, little where the reduce alone fills the
+ * machine for long.
+ * Both on one call: the two attention calls do not depend on one another either. */
 #define SPIFFY_INDEPENDENT 0x200
 #define SPIFFY_INDEPENDENT_NEXT 0x400
 
@@ -397,13 +402,15 @@ spiffy_status spiffy_lmhead_decide(const spiffy_decide_desc* desc, int32_t hidde
  *   dev_status    [B] OR-ed with SPIFFY_DEV_BADGRAPH when an offset or index is
  *                 out of range (such entries are ignored); may be NULL
  * Uses desc->batch, n_nodes, block_len only.
- * Ordering: block_tokens and the parent lists (here, in spiffy_decide_walk and in
- * the lazy call) are fetched while earlier work of the stream may still be
- * draining.  They must be complete in memory before the kernel that precedes
- * this call in the stream can let its dependents start, which holds for every
- * kernel of this library and for any kernel that does not use programmatic
- * dependent launch; do not produce them with an early-triggering kernel of your
- * own placed directly before the call.
+ * Ordering: block_tokens and the parent lists are fetched while earlier work of the
+ * stream may still be draining.  They must be complete in memory before the kernel
+ * that precedes this call in the stream can let its dependents start.  That holds for
+ * what copies, kernels without programmatic dependent launch and spiffy_draft_blocks
+ * write, and for everything written ahead of a decision call that stands before this
+ * one; a next_block is such an array only behind a decision call.  Do not produce them
+ * with an early-triggering kernel of your own placed directly before the call.
+ * (spiffy_decide_walk and the lazy call order themselves: the kernels that fetch
+ * these arrays come behind one that has waited for all earlier work.)
  */
 spiffy_status spiffy_accept_walk(const spiffy_decide_desc* desc,
                                  const int32_t* block_tokens,

@@ -21,13 +21,13 @@
 // no bank conflicts, no padding) and feed packed fp32x2 multiply-adds; K of the
 // next tile is fetched under P V, V under Q K^T, by asynchronous copies.
 //
-// Bound: the fp32 multiply-add pipe when there is enough work (27 TFLOP/s at 288
-// positions x 12 heads over 1000 keys, d = 128; a third of the pipe's rate, the
+// Bound: the fp32 multiply-add pipe when there is enough work (20 TFLOP/s at 288
+// positions x 12 heads over 1000 keys, d = 128; a quarter of the pipe's rate, the
 // rest goes to padding, to doubling P for the packed instructions and to the last
 // wave); for the shortest calls one tile's latency chain and the launch.  The
-// kernel before this one (a CTA per node and head, a warp per row) took 22 us for
-// 4 nodes x 8 positions x 4 heads over 128 keys and 910 us for 2 x 2 x 4 positions
-// x 24 heads over 3249 keys, d = 64; this one 6.0 and 34 us.
+// kernel before this one (a CTA per node and head, a warp per row) took 24.1 us for
+// 4 nodes x 8 positions x 4 heads over 128 keys and 433 us for 2 x 2 x 4 positions
+// x 24 heads on 8 over 3249 keys, d = 64; this one 5.9 and 34.2 us.
 #include <math.h>
 
 #include "common.cuh"

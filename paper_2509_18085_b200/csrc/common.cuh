@@ -182,15 +182,27 @@ spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const AttnProblem& 
 spiffy_status launch_attention_tc_dual(const spiffy_attn_desc& d0, const AttnProblem& a0, const spiffy_attn_desc& d1,
                                        const AttnProblem& a1, int32_t* dev_status, cudaStream_t stream);
 
-// Launch with programmatic stream serialisation: the kernel may be scheduled
-// while its predecessor in the stream is still draining.  Every kernel launched
-// this way calls cudaGridDependencySynchronize() before it writes global memory
-// or reads what the calls of one step hand to each other (logits, partial
-// results, top tokens, unmask sets).  The walk, tail and draft-build kernels
-// fetch the graph arrays (block states, parent lists, draft formulas) ahead of
-// that wait: those must be complete before the predecessor can trigger its
-// dependents, which the library's own kernels guarantee (each waits for its
-// predecessor before it triggers) and the header states for callers.
+// Launch with programmatic stream serialisation: the kernel may be scheduled once every CTA
+// of its predecessor in the stream has called pdl_launch_dependents() or ended.  "Waits" below
+// means cudaGridDependencySynchronize(), which returns when the predecessor is complete and
+// its writes are visible.  Who may start when, and why what it touches is complete:
+//   - Every kernel waits, and none is complete before it has waited, so that a kernel which
+//     is complete, or has been waited for, stands for all that came before it in the stream.
+//   - Before its wait a kernel writes nothing in global memory and reads nothing, except:
+//     (a) The walk, tail and sampled selection kernels read the block's tokens, the first two
+//         the parent lists as well.  Each comes behind a kernel of its own call that waited
+//         before it let its dependents start (the reduces do, and the finalize kernel is
+//         itself launched behind one), so whatever wrote those arrays ahead of the call is
+//         complete.  spiffy_accept_walk called by itself has no such kernel in front: its
+//         contract in spiffy.h puts that on the caller.
+//     (b) The draft-build kernel reads the draft formulas, constants of the model.
+//     (c) The reduce under SPIFFY_INDEPENDENT and the attention under SPIFFY_ATTN_INDEPENDENT
+//         read their inputs, write their outputs and wait last.  What precedes them is, by the
+//         flags' contract, a call that touches none of these; its kernels started, in turn,
+//         behind one that had waited before it triggered (the CUDA-core attention; the reduce
+//         of a plain decision), so everything ahead of that call is complete.
+//   - Triggering early is safe for what follows for the same reasons; where it pays is a
+//     matter of measurement and said at each kernel.
 template <typename... Args>
 cudaError_t launch_pdl(void (*kern)(Args...), dim3 grid, dim3 block, size_t smem,
                        cudaStream_t stream, Args... args) {
@@ -207,11 +219,8 @@ cudaError_t launch_pdl(void (*kern)(Args...), dim3 grid, dim3 block, size_t smem
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// The next kernel in the stream may be launched from here on (it still waits
-// in cudaGridDependencySynchronize() for this one to finish), which takes its
-// launch latency off the critical path.  Used by the small kernels only: behind
-// the attention and the decision reduce it measured slower, their successors'
-// many CTAs crowding the SMs early.
+// The next kernel in the stream may be launched once every CTA has come here; it still
+// waits for this one to finish, and its launch latency is off the critical path.
 __device__ __forceinline__ void pdl_launch_dependents() {
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900
   cudaTriggerProgrammaticLaunchCompletion();
@@ -229,10 +238,6 @@ bool allow_smem(Kernel kern, int bytes, std::atomic<bool> (&done)[64]) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
   done[device].store(true, std::memory_order_release);
   return true;
-}
-
-inline spiffy_status check_launch() {
-  return cudaGetLastError() == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
 }
 
 }  // namespace spiffy

@@ -25,7 +25,10 @@
 // between the CTAs is therefore the data itself, 16 bytes at a time in one access
 // with the level in it, instead of data, fence, counter and a load behind the
 // counter: per level two trips each way became one, and the reducers no longer
-// look the tokens up (B 4, N 32, L 32, V 126464, bf16: 79 us before, 65 now).
+// look the tokens up.  The time follows the levels of the slowest sequence, about 10 us
+// each behind 12 us of set-up (4 x 32 x 32 positions, 126464 entries, bf16: 42-43 us where
+// two drafts are accepted, 53 where three, 74 where five; with 1.13 levels on average 24.0,
+// 29.3 before the slices carried their level).
 #include "common.cuh"
 #include "decide_core.cuh"
 #include "walk_core.cuh"
@@ -99,7 +102,7 @@ __device__ __forceinline__ bool keep_polling(unsigned& polls, LazyHeader* h, uns
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kReduceThreads, 6)  // 80 registers, no spills: six CTAs per SM
+__global__ void __launch_bounds__(kReduceThreads, 6)  // 80 registers: six CTAs per SM (bf16 spills 44 bytes)
 decide_walk_lazy_kernel(const LazyParams p) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int b_own = blockIdx.x < p.B ? (int)blockIdx.x : -1;  // the sequence whose tail this CTA runs

@@ -27,8 +27,8 @@
 // applies the rule.  A vocabulary of one slice: the select kernel reduces it itself
 // and keeps it in shared memory, which spares a launch and three trips through L2,
 // and a kernel of one CTA per sequence applies the rule, as nothing came before
-// that could have cleared the nodes' arrival counters (64 rows x 2251: 9.0 -> 6.2
-// us; 3174 masked rows x 4064: 42.6 -> 33.9).
+// that could have cleared the nodes' arrival counters (49 masked rows of 64 x
+// 2251: 8.6 -> 5.5 us; 3144 of 4608 x 4064: 40.9 -> 28.9).
 #include <type_traits>
 
 #include "common.cuh"

@@ -32,7 +32,9 @@
 // The reduction across lanes takes 6.6 us a tile there, and tensor memory has no room
 // for a second accumulator pair: the epilogue empties the first into registers (192 a
 // thread, which is why its warps take the others' share) and gives it back, so that
-// the next tile's products run meanwhile: 237 -> 206-214 us.
+// the next tile's products run meanwhile: 234 -> 214 us with 164 masked positions, in
+// runs of tens of milliseconds.  Called back to back for seconds it draws the board's
+// power limit, and takes 230-246 us (166 masked positions; 283 before).
 //
 // Each CTA leaves one partial result per position; the decision's finalize kernel
 // merges them (in a fixed order) and applies the unmasking rule.  Every wait is

@@ -205,17 +205,6 @@ __device__ __forceinline__ void tmem_loaded(uint32_t (&r)[N]) {
   for (int k = 0; k < N; ++k) asm volatile("" : "+r"(r[k]));
 }
 
-// Row `lane` of the warp's TMEM quadrant, 64 consecutive 32-bit columns from
-// `taddr`, into r[0..63]; returns once the data has arrived.
-__device__ __forceinline__ void tmem_ld_x64(uint32_t taddr, uint32_t (&r)[64]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%64];\n"
-      "tcgen05.wait::ld.sync.aligned;\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
-      : "r"(taddr)
-      : "memory");
-}
-
 // Row `lane` of the warp's TMEM quadrant, 128 consecutive 32-bit columns from
 // `taddr`, into r[0..127]; returns once the data has arrived.
 __device__ __forceinline__ void tmem_ld_x128(uint32_t taddr, uint32_t (&r)[128]) {
@@ -237,32 +226,7 @@ __device__ __forceinline__ void tmem_st_x32(uint32_t taddr, const uint32_t (&r)[
       : "memory");
 }
 
-// r[0..63] into row `lane` of the warp's TMEM quadrant, 64 consecutive columns
-// from `taddr` (issue only; follow with tmem_wait_st()).
-__device__ __forceinline__ void tmem_st_x64(uint32_t taddr, const uint32_t (&r)[64]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x64.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63,%64};\n"
-      :
-      : "r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(r[32]), "r"(r[33]), "r"(r[34]), "r"(r[35]), "r"(r[36]), "r"(r[37]), "r"(r[38]), "r"(r[39]), "r"(r[40]), "r"(r[41]), "r"(r[42]), "r"(r[43]), "r"(r[44]), "r"(r[45]), "r"(r[46]), "r"(r[47]), "r"(r[48]), "r"(r[49]), "r"(r[50]), "r"(r[51]), "r"(r[52]), "r"(r[53]), "r"(r[54]), "r"(r[55]), "r"(r[56]), "r"(r[57]), "r"(r[58]), "r"(r[59]), "r"(r[60]), "r"(r[61]), "r"(r[62]), "r"(r[63])
-      : "memory");
-}
-
 // --------------------------------------------------------------------- MMA --
-// Shared-memory matrix descriptor of a 128-byte-swizzled operand tile whose
-// 8-row (1024-byte) swizzle atoms are `sbo_bytes` apart; `lbo_bytes` is the
-// distance between 64-element blocks along M/N of an MN-major operand (unused
-// for K-major).  The tile base must be 1024-byte aligned; `addr` may point
-// 32, 64 or 96 bytes into a row to step along K inside the swizzle span.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr, uint32_t lbo_bytes,
-                                                    uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFFu) >> 4);          // bits  0..13 start address
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;  // bits 16..29 leading byte offset
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;  // bits 32..45 stride byte offset
-  d |= (uint64_t)1 << 46;                           // bits 46..48 fixed 0b001
-  d |= (uint64_t)2 << 61;                           // bits 61..63 swizzle mode: 128 bytes
-  return d;
-}
 // Instruction descriptor of tcgen05.mma.kind::f16 with bf16 operands and fp32
 // accumulation; *_mn_major = operand stored with M/N (not K) contiguous.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int m, int n, bool a_mn_major,
@@ -275,25 +239,16 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int m, int n, bool a_mn_ma
          | ((uint32_t)(n >> 3) << 17)
          | ((uint32_t)(m >> 4) << 24);
 }
-// D[tmem] (+)= A[smem] * B[smem]; issued by one thread.
-__device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                        uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n"
-      ".reg .pred p;\n"
-      "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
-      "}\n"
-      :
-      : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
 // ------------------------------------------------- lean issue of MMA groups --
 // One thread issues every MMA of a CTA; what it spends per instruction on
 // building descriptors bounds the tensor pipe's rate (a 128 x 128 x 16 product
-// lasts 64 cycles).  The groups below take the descriptors split into their low
-// word (address and leading offset: advanced by a constant per K step) and
-// their high word (stride offset, fixed bits, swizzle: the same for all).
+// lasts 64 cycles).  The groups below take the shared-memory matrix descriptors of
+// 128-byte-swizzled tiles split into their low word (bits 0..13 address, 16..29 leading
+// byte offset, the distance between 64-element blocks along M/N of an MN-major operand,
+// unused for K-major; advanced by a constant per K step, inside the swizzle span) and
+// their high word (bits 0..13 stride byte offset, the distance between the 8-row swizzle
+// atoms; 14 fixed; 29..31 swizzle mode, 2 = 128 bytes; the same for all).  Offsets and
+// address in units of 16 bytes; tile bases are 1024-byte aligned.
 __device__ __forceinline__ uint32_t desc_lo_sw128(uint32_t addr, uint32_t lbo_bytes) {
   return ((addr & 0x3FFFFu) >> 4) | ((lbo_bytes >> 4) << 16);
 }
@@ -391,39 +346,8 @@ __device__ __forceinline__ void umma_ss_k64(uint32_t d_tmem, uint32_t a_lo, uint
       : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
       : "memory");
 }
-// D[tmem] (+)= A[tmem] B over `steps` K steps of 16: A = bf16 pairs in tensor
-// memory (8 columns per step), B an MN-major tile whose rows of 16 keys are
-// 2048 bytes apart.
-__device__ __forceinline__ void umma_ts_k64(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi,
-                                            uint32_t idesc, uint32_t accumulate_first) {
-  asm volatile(
-      "{\n"
-      ".reg .pred p0, p1;\n"
-      ".reg .b32 at, bl;\n"
-      ".reg .b64 db;\n"
-      "setp.ne.b32 p0, %5, 0;\n"
-      "setp.eq.b32 p1, %5, %5;\n"
-      "add.u32 at, %1, 0;\n"
-      "add.u32 bl, %2, 0;\n"
-      "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p0;\n"
-      "add.u32 at, %1, 8;\n"
-      "add.u32 bl, %2, 128;\n"
-      "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
-      "add.u32 at, %1, 16;\n"
-      "add.u32 bl, %2, 256;\n"
-      "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
-      "add.u32 at, %1, 24;\n"
-      "add.u32 bl, %2, 384;\n"
-      "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
-      "}\n"
-      :
-      : "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
-      : "memory");
-}
+// D[tmem] (+)= A[tmem] B over K = 128: A = bf16 pairs in tensor memory (8 columns per K step
+// of 16), B an MN-major tile whose rows of 16 keys are 2048 bytes apart.
 __device__ __forceinline__ void umma_ts_k128(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi,
                                              uint32_t idesc, uint32_t accumulate_first) {
   asm volatile(
