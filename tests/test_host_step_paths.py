@@ -7,9 +7,12 @@ import re
 import subprocess
 
 import pytest
+import torch
 
 from paper_2509_18085_b200 import build as builder
 from paper_2509_18085_b200 import spiffy
+from paper_2509_18085_b200 import workloads as W
+from paper_2509_18085_b200.step import VerifyStep, inputs_from_workload
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 UNITS = ["step_host", "decide", "walk", "stage", "api"]
@@ -150,3 +153,18 @@ def test_an_independent_kernel_may_start_as_the_reduce_ends(host, N, L, cap):
         assert log[0].endswith(f" early {'1' if fused else early}")
         if fused:  # the tail is resident while the reduce runs either way
             assert log[1].endswith(f" early {early}")
+
+
+def test_a_step_object_describes_each_input_anew(monkeypatch):
+    """The parent lists of one graph are longer than the next one's: a descriptor kept from the first
+    call would read past the end of the second call's arrays."""
+    seen = []
+    monkeypatch.setattr(torch.Tensor, "pin_memory", lambda t: t)
+    monkeypatch.setattr(spiffy, "spiffy_verify_step_host", lambda d, *a: seen.append((d.parent_cap, a[-1].numel())))
+    cfg = W.Config("t", 2, 4, 8, 16, 4, 4, 64, "bf16", 1000, spiffy.RULE_TOPS)
+    step, x = VerifyStep(cfg, device="cpu"), inputs_from_workload(W.make(cfg, 3), device="cpu")
+    for cap in (40, 4, 4000):
+        x.parent_idx = torch.zeros((2, cap), dtype=torch.int32)
+        step.run_host(x)
+    assert [cap for cap, _ in seen] == [40, 4, 4000]
+    assert seen[0][1] == seen[1][1] < seen[2][1]  # the workspace grows, and is otherwise kept
