@@ -97,6 +97,7 @@ class VerifyStep:
         self.attention_second = (cfg.dtype == "bf16" and attn_kernel != spiffy.ATTN_SIMT
                                  and cfg.n_q_heads <= 128 * cfg.n_kv_heads)
         self.host_ws = None
+        self.host_desc = self.host_sizes = None
         self.host_verdict = None
         self.lazy_ws = None
         self.sampled_ws = None
@@ -170,20 +171,25 @@ class VerifyStep:
         is in host memory when the call returns."""
         c = self.cfg
         B, N, L = c.batch, c.n_nodes, c.block_len
-        # of these inputs, every time: the length of the parent lists is theirs
-        desc = spiffy.step_desc(host.q, host.k_prefix, host.k_block, host.logits, host.block_tokens, host.parent_idx,
-                                c.mask_id, c.rule, c.top_s, c.threshold, kernel=self.attn_kernel)
-        need = spiffy.spiffy_verify_step_host_workspace(desc)
-        if self.host_ws is None or self.host_ws.numel() < need:
-            buf = torch.empty((need + 256,), dtype=torch.uint8, device=self.device)
-            off = (-buf.data_ptr()) % 256
-            self.host_ws = buf[off:off + need]
+        # described anew whenever a size differs (the parent lists' do from graph to graph); building the
+        # descriptor takes 6 us, which a call of small inputs, 100 us in all, would notice
+        sizes = (host.q.shape, None if host.k_prefix is None else host.k_prefix.shape, host.k_block.shape,
+                 host.logits.shape, host.block_tokens.shape, host.parent_idx.shape, host.q.dtype, host.logits.dtype)
+        if sizes != self.host_sizes:
+            desc = spiffy.step_desc(host.q, host.k_prefix, host.k_block, host.logits, host.block_tokens,
+                                    host.parent_idx, c.mask_id, c.rule, c.top_s, c.threshold, kernel=self.attn_kernel)
+            need = spiffy.spiffy_verify_step_host_workspace(desc)
+            if self.host_ws is None or self.host_ws.numel() < need:
+                buf = torch.empty((need + 256,), dtype=torch.uint8, device=self.device)
+                off = (-buf.data_ptr()) % 256
+                self.host_ws = buf[off:off + need]
+            self.host_desc, self.host_sizes = desc, sizes
         if self.host_verdict is None:
             pin = lambda *shape: torch.empty(shape, dtype=torch.int32).pin_memory()
             self.host_verdict = (pin(B), pin(B), pin(B, N), pin(B, L), pin(1 + 2 * B))
         kp = host.k_prefix if c.prefix_len else None
         vp = host.v_prefix if c.prefix_len else None
-        return spiffy.spiffy_verify_step_host(desc, host.q, kp, vp, host.k_block, host.v_block,
+        return spiffy.spiffy_verify_step_host(self.host_desc, host.q, kp, vp, host.k_block, host.v_block,
                                               host.logits, host.block_tokens, host.parent_off, host.parent_idx,
                                               *self.host_verdict, self.host_ws)
 
