@@ -262,6 +262,7 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
   uint64_t* xchg_full = xchg_ready + 1;  // cluster: the others' partials have arrived here
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + SM::tmem);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SM::abort_flag);
+  volatile int* invited = abort_flag + 1;  // cluster: the others have been told that they may send
   int* rows = reinterpret_cast<int*>(smem + SM::rows);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -326,7 +327,7 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
       const bool four = bar >= s_free && bar < pv_done;
       if (bar < bars + SM::n_bars) mbar_init(bar, four ? 4u : bar == xchg_ready ? (uint32_t)max(cs - 1, 1) : 1u);
     }
-    if (lane == 0) *abort_flag = 0;
+    if (lane == 0) *abort_flag = *invited = 0;
     mbar_fence_init();
     __syncwarp();
   }
@@ -476,8 +477,10 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
       }
       tc_fence_after_sync();
       // the last scores have been formed: the Q tile and the K ring are free for the others' partials
-      if (cs > 1 && u == U - 1 && quad == 0 && lane < cs && lane != rank)
-        mbar_arrive_remote(map_to_cta(smem_u32(xchg_ready), (uint32_t)lane));
+      if (cs > 1 && u == U - 1 && quad == 0 && lane < cs) {
+        if (lane != rank) mbar_arrive_remote(map_to_cta(smem_u32(xchg_ready), (uint32_t)lane));
+        else *invited = 1;
+      }
       uint32_t s[BN];
       tmem_ld_x128(tmem_addr(tmem, lane_base, kColS), s);
       tc_fence_before_sync();
@@ -664,6 +667,9 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
           }
         }
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait_cluster(xchg_full, 0, abort_flag, p.spin_limit));
+        // winding down: nobody sends before all have been told that they may; where this CTA has done
+        // so, what may be on its way here lands before its shared memory goes
+        if (!ok && warp == 4 && *invited) mbar_wait_quiet(xchg_full, 0);
         cluster_arrive();  // phase 2: what this CTA was sent has landed
         if (ok && tid < R) {
           float m = -INFINITY, l = 0.f;
