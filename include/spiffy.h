@@ -623,7 +623,9 @@ spiffy_status spiffy_draft_blocks(const spiffy_draft_desc* desc, const void* log
  * run out without hanging or faulting anything:
  *   mbarrier_polls       polls per mbarrier wait; 0 = give up without waiting
  *                        (the kernel then issues no copy it does not wait for
- *                        and no tensor-core product); < 0 restores the default
+ *                        and no tensor-core product); 1 to 16383 count as 16384, so
+ *                        that products already issued end before a wait gives up;
+ *                        < 0 restores the default
  *   flag_polls           polls (about 100 ns apart) per wait of the lazy call;
  *                        < 0 restores the default
  *   lazy_extra_arrivals  other than 0: sequence 0 of the lazy call waits for

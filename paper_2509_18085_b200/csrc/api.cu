@@ -443,8 +443,12 @@ const char* spiffy_status_string(spiffy_status status) {
 }
 
 void spiffy_set_wait_limits(int64_t mbarrier_polls, int64_t flag_polls, int32_t lazy_extra_arrivals) {
-  g_mbar_polls.store(mbarrier_polls < 0 ? (1u << 20) : (uint32_t)(mbarrier_polls > (1 << 20) ? (1 << 20) : mbarrier_polls),
-                     std::memory_order_relaxed);
+  // A limit between none and a few thousand polls could run out while tensor-core products that were
+  // issued are still being executed, and the block would give its memory back under them.
+  constexpr int64_t kMost = 1 << 20, kLeast = 1 << 14;
+  int64_t polls = mbarrier_polls < 0 || mbarrier_polls > kMost ? kMost : mbarrier_polls;
+  if (polls > 0 && polls < kLeast) polls = kLeast;
+  g_mbar_polls.store((uint32_t)polls, std::memory_order_relaxed);
   g_flag_polls.store(flag_polls < 0 ? (1u << 21) : (uint32_t)(flag_polls > (1 << 21) ? (1 << 21) : flag_polls),
                      std::memory_order_relaxed);
   g_lazy_extra.store(lazy_extra_arrivals < 0 ? 0 : lazy_extra_arrivals, std::memory_order_relaxed);

@@ -168,3 +168,14 @@ def test_a_step_object_describes_each_input_anew(monkeypatch):
         step.run_host(x)
     assert [cap for cap, _ in seen] == [40, 4, 4000]
     assert seen[0][1] == seen[1][1] < seen[2][1]  # the workspace grows, and is otherwise kept
+
+
+def test_poll_limits_leave_time_for_products_in_flight(host):
+    """None at all, or at least 16384 polls: far more than a group of tensor-core products takes."""
+    limit = getattr(host, "_ZN6spiffy15mbar_poll_limitEv")
+    limit.restype = ctypes.c_uint32
+    set_limits = host.spiffy_set_wait_limits
+    set_limits.argtypes = [ctypes.c_int64, ctypes.c_int64, ctypes.c_int32]
+    for asked, got in ((0, 0), (1, 1 << 14), (3000, 1 << 14), (1 << 14, 1 << 14), (100000, 100000), (1 << 40, 1 << 20), (-1, 1 << 20)):
+        set_limits(asked, -1, 0)
+        assert limit() == got
