@@ -66,7 +66,7 @@ def test_configs(index, n_nodes, kernel):
     dict(batch=2, n_nodes=4, block_len=12, prefix_len=129, n_q_heads=6, n_kv_heads=2, head_dim=128),
     # 26 nodes of 5 positions under one M-tile: their block keys need two key tiles
     dict(batch=1, n_nodes=30, block_len=5, prefix_len=70, n_q_heads=2, n_kv_heads=2, head_dim=128),
-    # enough M-tiles for the two-tiles-per-CTA variant; an odd tile count leaves one CTA half empty
+    # more M-tiles than fit one round of CTAs; two of them per CTA in the second shape
     dict(batch=3, n_nodes=9, block_len=32, prefix_len=300, n_q_heads=32, n_kv_heads=32, head_dim=128),
     dict(batch=10, n_nodes=6, block_len=16, prefix_len=130, n_q_heads=32, n_kv_heads=16, head_dim=128),
 ])
@@ -81,16 +81,17 @@ def test_odd_shapes(shape, dtype, kernel):
 
 
 @pytest.mark.parametrize("prefix_len,n_nodes,block_len", [
-    (384, 8, 32),   # 3 context tiles + 1 block tile: even, the two CTAs of a pair each finish half the columns
-    (512, 8, 32),   # 5 key tiles: odd, one CTA of the pair has a tile more
+    (384, 8, 32),   # 3 context tiles + 1 block tile: one for each CTA of a cluster of four
+    (512, 8, 32),   # 5 key tiles: one CTA has a tile more
     (640, 8, 32),   # 6
     (300, 4, 32),   # 4, ragged context tile, one M-tile per head
     (400, 6, 48),   # nodes of 48 positions: M-tiles with one and with two block-key tiles (odd and even in one launch)
     (257, 3, 7),    # 4 tiles, a nearly empty M-tile
 ])
 def test_cluster_pairs_with_even_and_odd_tile_counts(prefix_len, n_nodes, block_len):
-    """Few M-tiles (at most 74): the key tiles of each M-tile are split over the
-    two CTAs of a cluster, which merge through each other's shared memory."""
+    """Few M-tiles: the key tiles of each M-tile are split over the CTAs of a
+    cluster, four of them (nodes of 48 positions: one CTA for all), which merge
+    through each other's shared memory."""
     cfg = W.Config("pairs", dtype="bf16", vocab=16, rule=0, batch=1, n_nodes=n_nodes, block_len=block_len,
                    prefix_len=prefix_len, n_q_heads=16, n_kv_heads=16, head_dim=128)
     w = W.make(cfg, 31 + prefix_len, decision=False)

@@ -21,8 +21,9 @@ pytestmark = pytest.mark.gpu
     (1, 6, 32, 2562, 8, 1), (1, 2, 32, 1746, 28, 4),          # clusters of 8
     (1, 4, 32, 900, 30, 30),      # clusters of 4
     (1, 7, 32, 777, 32, 32),      # clusters of 2
-    (2, 9, 32, 500, 40, 40),      # two M-tiles per CTA, an odd number of M-tiles
-    (4, 32, 32, 140, 16, 8)])
+    (2, 9, 32, 500, 40, 40),      # two rounds of CTAs
+    (4, 32, 32, 140, 16, 8),      # two M-tiles per CTA
+    (2, 9, 32, 300, 35, 35)])     # ... an odd number of them: the last CTA's second one is empty
 def test_parity(B, N, L, P, Hq, Hkv):
     cfg = W.Config("splits", B, N, L, P, Hq, Hkv, 128, "bf16", 16, 0)
     w = W.make(cfg, 11 + P, decision=False)

@@ -201,8 +201,8 @@ def test_lazy_chain_evaluation_equals_the_eager_call_on_the_path(B, N, L, V):
                                            (7, 12, 64, 9000, "f32"), (40, 5, 32, 20000, "bf16")])
 def test_lazy_call_with_more_items_than_resident_thread_blocks(B, N, L, V, dtype):
     """B * L * slices exceeds what the device holds at once (six thread blocks
-    per SM): every block then takes several (position, slice) items per level,
-    each waiting on another sequence's epoch."""
+    per SM): every reducing block then takes several slices of its sequence, or
+    of several sequences, per level."""
     per_slice = 8192 if dtype == "bf16" else 4096
     items = B * L * -(-V // per_slice)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
