@@ -206,7 +206,7 @@ __device__ __forceinline__ float row_exps(const uint32_t (&s)[BN], uint32_t need
   return a0 + a1;
 }
 
-// Bounded wait that ignores the abort flag (used while winding down).
+// Bounded wait that ignores the abort flag: for what must not be in flight when the block ends.
 __device__ __forceinline__ void mbar_wait_quiet(uint64_t* bar, uint32_t parity) {
   for (uint32_t i = 0; i < kSpinLimit; ++i)
     if (mbar_try_wait(bar, parity)) return;
@@ -370,20 +370,18 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
       // ------------------------------------------------------------ producer --
       if (lane == 0) {
         // the rest of both rings, in the order the products need them: K(j+1) before V(j)
-      int jk = 1, jv = 0;
-      while (prod_ok && (jk < T || jv < T)) {
-        const bool is_k = jk < T && jk <= jv + 1;
-        produce(is_k, is_k ? jk : jv);
-        if (is_k) ++jk; else ++jv;
-      }
-      if (!prod_ok) {
-          // winding down: let the copies already in flight land before exit
-          mbar_wait_quiet(q_full, 0);
-          for (int j = max(0, issued_k - KS); j < issued_k; ++j)
-            mbar_wait_quiet(k_full + j % KS, (uint32_t)(j / KS) & 1u);
-          for (int j = max(0, issued_v - VS); j < issued_v; ++j)
-            mbar_wait_quiet(v_full + j % VS, (uint32_t)(j / VS) & 1u);
+        int jk = 1, jv = 0;
+        while (prod_ok && (jk < T || jv < T)) {
+          const bool is_k = jk < T && jk <= jv + 1;
+          produce(is_k, is_k ? jk : jv);
+          if (is_k) ++jk; else ++jv;
         }
+        // Whoever gives up, and when: no copy is in flight into shared memory whose block has ended.
+        mbar_wait_quiet(q_full, 0);
+        for (int j = max(0, issued_k - KS); j < issued_k; ++j)
+          mbar_wait_quiet(k_full + j % KS, (uint32_t)(j / KS) & 1u);
+        for (int j = max(0, issued_v - VS); j < issued_v; ++j)
+          mbar_wait_quiet(v_full + j % VS, (uint32_t)(j / VS) & 1u);
       }
     } else if (warp == 1) {
       // ------------------------------------------------ issuer of S = Q K^T --

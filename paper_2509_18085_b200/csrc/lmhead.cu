@@ -255,12 +255,11 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
           }
         }
       }
-      if (!ok) {  // winding down: let the copies already in flight land before exit
-        for (int q = 0; q < kMaxStages; ++q)
-          if ((used >> q) & 1u)
-            for (uint32_t s = 0; s < kSpinLimit; ++s)
-              if (mbar_try_wait(full + q, q < stage ? phase : phase ^ 1u)) break;
-      }
+      // Whoever gives up, and when: no copy is in flight into shared memory whose block has ended.
+      for (int q = 0; q < kMaxStages; ++q)
+        if ((used >> q) & 1u)
+          for (uint32_t s = 0; s < kSpinLimit; ++s)
+            if (mbar_try_wait(full + q, q < stage ? phase : phase ^ 1u)) break;
     } else if (warp == 1 && lane == 0) {
       // -------------------------------------------------------- MMA issuer --
       constexpr uint32_t hi = desc_hi_sw128(1024);
