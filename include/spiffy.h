@@ -171,7 +171,7 @@ size_t spiffy_graph_attention_workspace(const spiffy_attn_desc* desc);
  * NULL.  Accumulation is fp32; the result is rounded once to desc->dtype.  The
  * softmax weights are fp32 on the CUDA-core kernel; on the tensor-core kernel they
  * enter the second product as bf16 at head_dim 128 and as the sum of two bf16 terms
- * (16 bits of mantissa) at head_dim 64.
+ * (16 bits) at head_dim 64.
  */
 spiffy_status spiffy_graph_attention(const spiffy_attn_desc* desc,
                                      const void* q, const void* k_prefix,

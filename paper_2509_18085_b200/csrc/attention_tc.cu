@@ -58,13 +58,12 @@
 // Head dimension 64 halves every tile (one 64-column half instead of two) and the
 // products, not the exponentials.  The CUDA-core kernel, which this one stands in for
 // there, keeps P in fp32: here P enters the second product as two bf16 terms, its
-// rounding and what that left over (2^-17 of a value short of fp32, in the tensor
-// memory that the narrower O leaves), so that the result's error against float64 is
-// the CUDA cores' (0.166 % in the 2-norm, the rounding of the output, over 50 to 4096
-// keys; with one term 0.18 to 0.23 %).  The second term costs 4 to 9 % of a call of
-// few key tiles, 20 % of a long one (4 x 32 x 32 positions x 32 heads over 4096 keys:
-// 232 -> 277 us; CUDA cores 4596); 3 sequences of 100 positions x 24 heads over 777 +
-// 20 keys: 12.5 us, 11.6 with one term, 89 on the CUDA cores.
+// upper half and what that leaves (to 2^-16 of a value, in the tensor memory that the
+// narrower O leaves), so that the result's error against float64 is the CUDA cores'
+// (0.166 % in the 2-norm, the rounding of the output, over 50 to 4096 keys; with one
+// term 0.18 to 0.23 %).  The second term costs 5 to 20 % (4 x 32 x 32 positions x 32
+// heads over 4096 keys: 232 -> 262 us; CUDA cores 4596); 3 sequences of 100 positions x
+// 24 heads over 777 + 20 keys: 12.4 us, 11.6 with one term, 89 on the CUDA cores.
 //
 // Every wait is bounded; a wait that gives up raises SPIFFY_DEV_TIMEOUT in the
 // caller's status word and the CTA winds down without touching its output.
@@ -89,7 +88,7 @@ static_assert(kRegsIssue + 2 * kRegsSoftmax <= 3 * 168, "within what the block w
 constexpr int kHalfBytes = BN * 128;           // one 64-column half of a tile: 128 rows x 128 B
 constexpr uint32_t kTmemCols = 512;
 // S: 128 columns; warpgroup w: P (bf16 pairs) at 128 + 64 w, O at 256 + w * head dim, and at head
-// dimension 64, what the rounding of P left over at 384 + 64 w
+// dimension 64, P's second term at 384 + 64 w
 constexpr uint32_t kColS = 0, kColP = 128, kColO = 256, kColRest = 384;
 static_assert(kColRest + 2 * 64 <= kTmemCols && kColO + 2 * 64 <= kColRest, "tensor memory at head dimension 64");
 constexpr float kRescaleLog2 = 8.0f;
@@ -171,7 +170,8 @@ __device__ __forceinline__ float row_max(const uint32_t (&s)[BN]) {
 
 // p = 2^(s * k2 - m_use) for the flagged 32-column chunks among columns C0 .. C0 + 63 (zero
 // elsewhere), packed as bf16 pairs into pk; returns the sum of the p's (fp32, before rounding to
-// bf16).  kRest: rest gets p - bf16(p), rounded to bf16 in its turn, so that pk + rest is p to 2^-17.
+// bf16).  kRest: pk holds the upper 16 bits of p and rest what they leave of it, rounded to bf16, so
+// that pk + rest is p to 2^-16.
 // The special-function unit takes 8 cycles per warp and exponential; everything else a pair
 // needs fits under its two.
 template <int C0, bool kRest>
@@ -189,9 +189,16 @@ __device__ __forceinline__ float row_exps(const uint32_t (&s)[BN], uint32_t need
         unpack2(x2, x0, x1);
         const float p0 = ex2(x0), p1 = ex2(x1);
         if ((c >> 1) & 1) sum_b = add2(sum_b, pack2(p0, p1)); else sum_a = add2(sum_a, pack2(p0, p1));
-        const uint32_t w = pack_bf16(p0, p1);
-        pk[c >> 1] = w;
-        if (kRest) rest[c >> 1] = pack_bf16(p0 - __uint_as_float(w << 16), p1 - __uint_as_float(w & 0xffff0000u));
+        if constexpr (kRest) {  // cut off instead of rounded: a byte permutation, no conversion
+          const uint32_t w0 = __float_as_uint(p0), w1 = __float_as_uint(p1);
+          pk[c >> 1] = __byte_perm(w0, w1, 0x7632);
+          float r0, r1;
+          unpack2(fma2(pack2(__uint_as_float(w0 & 0xffff0000u), __uint_as_float(w1 & 0xffff0000u)), pack2(-1.f, -1.f),
+                       pack2(p0, p1)), r0, r1);
+          rest[c >> 1] = pack_bf16(r0, r1);
+        } else {
+          pk[c >> 1] = pack_bf16(p0, p1);
+        }
       }
     } else {
 #pragma unroll
@@ -813,10 +820,10 @@ int resident_clusters(int hd, int cs) {
 // partials around a cluster costs about 2 us (1.5 with rows half as long), so that a second
 // CTA pays from about six key tiles.  The model is there to choose: of 35 shapes (1 to 1088
 // M-tiles, 2 to 33 key tiles), each timed with every plan it allows, it takes the fastest,
-// or one within 1.5 % of it, at both head dimensions.  Its times are low for long calls of
-// several rounds: 4 x 32 x 32 positions x 32 heads over 4096 keys, 239 us for two M-tiles a
-// CTA and 245 for one at head dimension 128, measured 264 and 274 back to back on the same
-// inputs; at 64, 279 and 269, measured 288 and 278.
+// or one within 2 % of it, at both head dimensions.  The times themselves are 10 % low for
+// long calls of several rounds at 128: 4 x 32 x 32 positions x 32 heads over 4096 keys, 239 us
+// for two M-tiles a CTA and 245 for one, measured 265 and 273 back to back on the same
+// inputs; at 64, 279 and 268, measured 276 and 263.
 // `tiles` counts the M-tiles of all problems of the launch, `pairs` the CTAs that take two
 // of them, T is the key tiles of the longer problem.
 Plan make_plan(int64_t tiles, int64_t pairs, int T, int hd) {
