@@ -67,19 +67,11 @@
 //
 // Every wait is bounded; a wait that gives up raises SPIFFY_DEV_TIMEOUT in the
 // caller's status word and the CTA winds down without touching its output.
-#include <math.h>
-
-#include "common.cuh"
-#include "sm100_ptx.cuh"
-#include "tma_map.cuh"
+#include "attention_tc.cuh"
 
 namespace spiffy {
 namespace {
 
-using namespace sm100;
-
-constexpr int BM = 128;       // rows of an M-tile (TMEM lanes)
-constexpr int BN = 128;       // keys per key tile
 constexpr int kThreads = 384;  // a warpgroup with the producer and the MMA warp, two softmax warpgroups
 // Registers per thread: 168 at launch (65536 / 384 in steps of 8); the softmax warps, which hold
 // 128 scores each with two M-tiles, take over what the first warpgroup does not need.
@@ -91,8 +83,6 @@ constexpr uint32_t kTmemCols = 512;
 // dimension 64, P's second term at 384 + 64 w
 constexpr uint32_t kColS = 0, kColP = 128, kColO = 256, kColRest = 384;
 static_assert(kColRest + 2 * 64 <= kTmemCols && kColO + 2 * 64 <= kColRest, "tensor memory at head dimension 64");
-constexpr float kRescaleLog2 = 8.0f;
-
 // Shared memory: NQ Q tiles, a K ring of 3 stages and a V ring of 4 - NQ, seven tiles of
 // 32 KB in all; at head dimension 64 fourteen of 16 KB.  (The same amount for all: two
 // CTAs must not share an SM, each holds all of its tensor memory until it exits.)
@@ -114,46 +104,6 @@ constexpr int most(int a, int b) { return a > b ? a : b; }
 constexpr int kSmemBytes = most(most(Smem<1, 64>::total, Smem<2, 64>::total), most(Smem<1, 128>::total, Smem<2, 128>::total)) +
                            1024;  // slack for 1024-byte alignment
 static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
-
-struct Params {
-  int B, N, L, Hq, Hkv, group;
-  int P, P2;    // context keys: first and second segment
-  int TNL;      // (node, position) pairs per M-tile
-  int NL;       // N * L
-  int TP1, TP;  // context key tiles: of the first segment, of both
-  int cs;       // CTAs of a cluster that share an M-tile's key tiles
-  float scale_log2;
-  __nv_bfloat16* out;
-  int32_t* status;
-  uint32_t spin_limit;  // polls of one mbarrier wait
-  int early_trigger;    // let the next kernel of the stream begin its set-up while this one runs
-  int independent;      // the kernel before this one writes none of its inputs: waited for at the end
-};
-
-// The operands of one attention problem: Q, two context segments, block keys.
-struct Maps {
-  CUtensorMap q, kp, vp, kp2, vp2, kb, vb;
-};
-// One launch runs one problem, or two side by side (the nodes and the trailing rows of a
-// full-sequence model): the CTAs from x_split on along grid.x work on the second.
-template <int NP>
-struct Problems {
-  Maps maps[NP];
-  Params p[NP];
-  int x_split;
-};
-
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
 
 // The maximum of one thread's scores of a row (raw bits, -inf where masked).
 __device__ __forceinline__ float row_max(const uint32_t (&s)[BN]) {
@@ -211,28 +161,6 @@ __device__ __forceinline__ float row_exps(const uint32_t (&s)[BN], uint32_t need
   float a0, a1;
   unpack2(add2(sum_a, sum_b), a0, a1);
   return a0 + a1;
-}
-
-// Bounded wait that ignores the abort flag: for what must not be in flight when the block ends.
-__device__ __forceinline__ void mbar_wait_quiet(uint64_t* bar, uint32_t parity) {
-  for (uint32_t i = 0; i < kSpinLimit; ++i)
-    if (mbar_try_wait(bar, parity)) return;
-}
-
-// Row r of an M-tile sees the columns [lo, hi) of key tile t (tile-relative).
-struct Window {
-  int lo, hi;
-};
-__device__ __forceinline__ Window visible_window(const Params& p, int t, int kb_start, int node) {
-  Window w;
-  if (t < p.TP) {  // context: every row sees every key that exists
-    w.lo = 0;
-    w.hi = t < p.TP1 ? min(BN, p.P - t * BN) : min(BN, p.P2 - (t - p.TP1) * BN);
-  } else {  // block keys: the row's own node only
-    w.lo = node * p.L - (kb_start + (t - p.TP) * BN);
-    w.hi = w.lo + p.L;
-  }
-  return w;
 }
 
 // NQ = 1: the CTA owns one M-tile; unit u is key tile u.
@@ -301,10 +229,18 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
   // Producer (lane 0 of warp 0): tile j of the K or V ring.
   int issued_k = 0, issued_v = 0;
   bool prod_ok = true;
+  // (Counted along: a division by a number the compiler does not know takes some 200 cycles.)
+  int stage_k = 0, stage_v = 0;
+  uint32_t round_k = 0, round_v = 0;
   auto produce = [&](bool is_k, int j) {
-    const int depth = is_k ? KS : VS;
-    const int stage = j % depth;
-    const uint32_t round = (uint32_t)(j / depth);
+    int& next = is_k ? stage_k : stage_v;
+    uint32_t& round_next = is_k ? round_k : round_v;
+    const int stage = next;
+    const uint32_t round = round_next;
+    if (++next == (is_k ? KS : VS)) {
+      next = 0;
+      ++round_next;
+    }
     if (round > 0 && !mbar_wait((is_k ? k_empty : v_empty) + stage, (round & 1u) ^ 1u, abort_flag, p.spin_limit)) {
       prod_ok = false;
       return;
@@ -318,8 +254,7 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
     const int key0 = seg == 0 ? t * BN : seg == 1 ? (t - p.TP1) * BN : kb_start + (t - p.TP) * BN;
     uint8_t* dst = (is_k ? sk : sv) + stage * kTileBytes;
     mbar_arrive_expect_tx(full, kTileBytes);
-    tma_load_4d(dst, m, full, 0, g, key0, b);
-    if constexpr (kHalves == 2) tma_load_4d(dst + kHalfBytes, m, full, 64, g, key0, b);
+    tma_load_5d(dst, m, full, 0, g, key0, 0, b);
     if (is_k) issued_k = j + 1; else issued_v = j + 1;
   };
 
@@ -345,10 +280,9 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
     mbar_arrive_expect_tx(q_full, (uint32_t)(NQ * kHalves) * rows_box * 128u);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {  // an M-tile beyond the last one reads as zeros
-      tma_load_4d(sq + q * kTileBytes, &maps.q, q_full, 0, g * p.group, nl0 + q * p.TNL, b);
-      if constexpr (kHalves == 2)
-        tma_load_4d(sq + q * kTileBytes + kHalfBytes, &maps.q, q_full, 64, g * p.group,
-                    nl0 + q * p.TNL, b);
+#pragma unroll
+      for (int h = 0; h < kHalves; ++h)  // with fewer than 128 rows in the box the halves lie further apart than it is long
+        tma_load_5d(sq + q * kTileBytes + h * kHalfBytes, &maps.q, q_full, 0, g * p.group, nl0 + q * p.TNL, h, b);
     }
     produce(true, 0);
   }
@@ -756,10 +690,10 @@ struct Shape {
   int group, TNL, NL, MT, TP1, TP;
   int T;  // key tiles of an M-tile, at least
 };
-Shape shape_of(const spiffy_attn_desc& d, const AttnContext& ctx, const AttnContext& ctx2) {
+Shape shape_of(const spiffy_attn_desc& d, const AttnContext& ctx, const AttnContext& ctx2, bool pair) {
   Shape s;
   s.group = d.n_q_heads / d.n_kv_heads;
-  s.TNL = BM / s.group;
+  s.TNL = pair ? 2 * (BM / 2 / s.group) : BM / s.group;
   s.NL = d.n_nodes * d.block_len;
   s.MT = (s.NL + s.TNL - 1) / s.TNL;
   s.TP1 = (ctx.len + BN - 1) / BN;
@@ -769,8 +703,9 @@ Shape shape_of(const spiffy_attn_desc& d, const AttnContext& ctx, const AttnCont
 }
 
 struct Plan {
-  int nq;  // M-tiles per CTA
-  int cs;  // CTAs of a cluster that share an M-tile's key tiles (nq = 1)
+  int nq;     // M-tiles per CTA
+  int cs;     // CTAs of a cluster that share an M-tile's key tiles (nq = 1)
+  bool pair;  // a pair of CTAs per M-tile instead (attention_pair.cu)
 };
 
 template <int NP>
@@ -824,15 +759,26 @@ int resident_clusters(int hd, int cs) {
 // long calls of several rounds at 128: 4 x 32 x 32 positions x 32 heads over 4096 keys, 239 us
 // for two M-tiles a CTA and 245 for one, measured 265 and 273 back to back on the same
 // inputs; at 64, 279 and 268, measured 276 and 263.
-// `tiles` counts the M-tiles of all problems of the launch, `pairs` the CTAs that take two
-// of them, T is the key tiles of the longer problem.
-Plan make_plan(int64_t tiles, int64_t pairs, int T, int hd) {
+// A pair of CTAs per M-tile (head dimension 128, at most 64 query heads on a key/value head) takes 5.3 us and
+// 0.44 per key tile, a round: 8 x 32 positions x 32 heads over 512 + 32 keys 7.5 us (one CTA a tile 10.3),
+// 64 x 4 x 32 heads on 8 over 2048 12.8 (clusters of two 17.0).  One round only pays: 2 x 11 x 24 x 16
+// heads over 450 13.9 (11.3), and with more key tiles than some 20 clusters of eight are sooner done.
+// `tiles` counts the M-tiles of all problems of the launch, `doubles` the CTAs that take two
+// of them, `pair_tiles` the pairs (0: not possible); T is the key tiles of the longer problem.
+Plan make_plan(int64_t tiles, int64_t doubles, int64_t pair_tiles, int T, int hd) {
   const int sms = sm_count();
   const float one = hd == 128 ? 0.85f : 0.95f, two = hd == 128 ? 1.6f : 1.9f;
   auto rounds = [&](int64_t ctas) { return (float)((ctas + sms - 1) / sms); };
-  Plan pl = {2, 1};
+  Plan pl = {2, 1, false};
   if (sms <= 0) return pl;
-  float best = rounds(pairs) * (7.0f + two * (float)T);
+  float best = rounds(doubles) * (7.0f + two * (float)T);
+  if (pair_tiles > 0) {
+    const float cost = rounds(2 * pair_tiles) * (5.3f + 0.44f * (float)T);
+    if (cost < best) {
+      best = cost;
+      pl = {1, 1, true};
+    }
+  }
   for (int cs = 1; cs <= 8 && cs <= T; cs *= 2) {
     // clusters only where all of them run at once
     if (cs > 1 && (tiles * cs > sms || tiles > resident_clusters(hd, cs))) continue;
@@ -840,35 +786,38 @@ Plan make_plan(int64_t tiles, int64_t pairs, int T, int hd) {
     const float cost = rounds(tiles * cs) * (7.0f + exchange + one * (float)((T + cs - 1) / cs));
     if (cost < best) {
       best = cost;
-      pl = {1, cs};
+      pl = {1, cs, false};
     }
   }
   return pl;
 }
 
-bool make_problem(const spiffy_attn_desc& d, const Shape& sh, const AttnProblem& a, Maps* m, Params* p, int cs,
+bool make_problem(const spiffy_attn_desc& d, const Shape& sh, const AttnProblem& a, Maps* m, Params* p, const Plan& pl,
                   int32_t* dev_status) {
-  const int hd = d.head_dim;
-  bool ok = make_map(&m->q, a.q, d.n_q_heads, sh.NL, d.batch, sh.group, sh.TNL, 0, hd);
-  ok = ok && make_map(&m->kb, a.kb, d.n_kv_heads, sh.NL, d.batch, 1, BN, 0, hd);
-  ok = ok && make_map(&m->vb, a.vb, d.n_kv_heads, sh.NL, d.batch, 1, BN, 0, hd);
+  const int halves = d.head_dim / 64;
+  const int ctas = pl.pair ? 2 : 1;  // of a pair, each reads half of the rows, of the keys of K and of the columns of V
+  const int64_t bs = a.ctx.batch_stride_rows, bs2 = a.ctx2.batch_stride_rows;
+  auto keys = [&](CUtensorMap* map, const void* base, int64_t rows, int64_t stride, bool is_v) {
+    return make_tile_map(map, base, d.n_kv_heads, rows, d.batch, 1, is_v ? BN : BN / ctas, is_v ? halves / ctas : halves,
+                         stride, halves);
+  };
+  bool ok = make_tile_map(&m->q, a.q, d.n_q_heads, sh.NL, d.batch, sh.group, sh.TNL / ctas, 1, 0, halves);
+  ok = ok && keys(&m->kb, a.kb, sh.NL, 0, false) && keys(&m->vb, a.vb, sh.NL, 0, true);
   if (a.ctx.len > 0) {
-    ok = ok && make_map(&m->kp, a.ctx.k, d.n_kv_heads, a.ctx.len, d.batch, 1, BN, a.ctx.batch_stride_rows, hd);
-    ok = ok && make_map(&m->vp, a.ctx.v, d.n_kv_heads, a.ctx.len, d.batch, 1, BN, a.ctx.batch_stride_rows, hd);
+    ok = ok && keys(&m->kp, a.ctx.k, a.ctx.len, bs, false) && keys(&m->vp, a.ctx.v, a.ctx.len, bs, true);
   } else {  // never dereferenced: the segment has no tile
     m->kp = m->kb;
     m->vp = m->vb;
   }
   if (a.ctx2.len > 0) {
-    ok = ok && make_map(&m->kp2, a.ctx2.k, d.n_kv_heads, a.ctx2.len, d.batch, 1, BN, a.ctx2.batch_stride_rows, hd);
-    ok = ok && make_map(&m->vp2, a.ctx2.v, d.n_kv_heads, a.ctx2.len, d.batch, 1, BN, a.ctx2.batch_stride_rows, hd);
+    ok = ok && keys(&m->kp2, a.ctx2.k, a.ctx2.len, bs2, false) && keys(&m->vp2, a.ctx2.v, a.ctx2.len, bs2, true);
   } else {
     m->kp2 = m->kb;
     m->vp2 = m->vb;
   }
   p->B = d.batch; p->N = d.n_nodes; p->L = d.block_len; p->P = a.ctx.len; p->P2 = a.ctx2.len;
   p->Hq = d.n_q_heads; p->Hkv = d.n_kv_heads; p->group = sh.group;
-  p->TNL = sh.TNL; p->NL = sh.NL; p->TP1 = sh.TP1; p->TP = sh.TP; p->cs = cs;
+  p->TNL = sh.TNL; p->NL = sh.NL; p->TP1 = sh.TP1; p->TP = sh.TP; p->cs = pl.cs;
   const float scale = d.scale != 0.f ? d.scale : 1.0f / sqrtf((float)d.head_dim);
   p->scale_log2 = scale * kLog2e;
   p->out = static_cast<__nv_bfloat16*>(a.out);
@@ -892,23 +841,30 @@ spiffy_status launch(const spiffy_attn_desc* const (&d)[NP], const AttnProblem* 
     if (!allow_smem(kernel_of<1>(hd, 1), kSmemBytes, allowed)) return SPIFFY_ECUDA;
   }
   const int64_t bg = (int64_t)d[0]->batch * d[0]->n_kv_heads;
-  Shape sh[NP];
-  int64_t tiles = 0, pairs = 0;
+  Shape sh[NP], by_pairs[NP];
+  int64_t tiles = 0, doubles = 0, pair_tiles = 0;
+  const bool pairs_can = hd == 128 && d[0]->n_q_heads / d[0]->n_kv_heads <= BM / 2;
   int T = 0;
   for (int i = 0; i < NP; ++i) {
-    sh[i] = shape_of(*d[i], a[i]->ctx, a[i]->ctx2);
+    sh[i] = shape_of(*d[i], a[i]->ctx, a[i]->ctx2, false);
     tiles += bg * sh[i].MT;
-    pairs += bg * ((sh[i].MT + 1) / 2);
+    doubles += bg * ((sh[i].MT + 1) / 2);
+    if (pairs_can) {
+      by_pairs[i] = shape_of(*d[i], a[i]->ctx, a[i]->ctx2, true);
+      pair_tiles += bg * by_pairs[i].MT;
+    }
     T = sh[i].T > T ? sh[i].T : T;
   }
-  const Plan pl = make_plan(tiles, pairs, T, hd);
+  const Plan pl = make_plan(tiles, doubles, pair_tiles, T, hd);
   Problems<NP> pr;
   int x = 0;
   for (int i = 0; i < NP; ++i) {
-    if (!make_problem(*d[i], sh[i], *a[i], &pr.maps[i], &pr.p[i], pl.cs, dev_status)) return SPIFFY_ECUDA;
+    if (pl.pair) sh[i] = by_pairs[i];
+    if (!make_problem(*d[i], sh[i], *a[i], &pr.maps[i], &pr.p[i], pl, dev_status)) return SPIFFY_ECUDA;
     if (i == 1) pr.x_split = x;
-    x += (sh[i].MT + pl.nq - 1) / pl.nq;
+    x += pl.pair ? 2 * sh[i].MT : (sh[i].MT + pl.nq - 1) / pl.nq;
   }
+  if (pl.pair) return launch_attention_pair<NP>(pr, x, stream);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)x, (unsigned)bg, (unsigned)pl.cs);
   cfg.blockDim = dim3(kThreads);

@@ -45,12 +45,25 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// The same by one lane of a converged warp.
+__device__ __forceinline__ void mbar_arrive_expect_tx_one(uint64_t* bar, uint32_t bytes) {
+  asm volatile(
+      "{\n"
+      ".reg .pred one;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "@one mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+      "}\n" ::"r"(smem_u32(bar)),
+      "r"(bytes)
+      : "memory");
+}
+
 // Bounded wait: gives up after `limit` polls (kSpinLimit unless the host lowered
 // it) or as soon as another thread of the CTA has given up (*abort != 0); the
 // first to give up raises *abort.  A limit of 0 gives up without polling.
 constexpr uint32_t kSpinLimit = 1u << 20;
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
                                           uint32_t limit) {
+#pragma unroll 1
   for (uint32_t i = 0; i < limit; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((i & 15u) == 15u && *abort) return false;
@@ -76,6 +89,16 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* m
         "r"(c1), "r"(c2), "r"(c3)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_5d(void* smem_dst, const CUtensorMap* m, uint64_t* bar,
+                                            int c0, int c1, int c2, int c3, int c4) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
+      :
+      : "r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(c0),
+        "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+      : "memory");
+}
 // Generic-proxy writes to shared memory become visible to the async proxy
 // (TMA stores, tensor-core operand reads).
 __device__ __forceinline__ void fence_proxy_async_smem() {
@@ -94,6 +117,9 @@ __device__ __forceinline__ void cluster_arrive() {
 __device__ __forceinline__ void cluster_arrive_relaxed() {
   asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
 }
+// What this thread has written, in its own CTA or another, is ordered before what follows for
+// every thread of the cluster.
+__device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
@@ -102,6 +128,16 @@ __device__ __forceinline__ void cluster_wait() {
 // shared memory, before the arrival.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+// The same without that order at cluster scope, which takes 500 cycles and more: for arrivals that hand
+// over nothing that the other CTA's threads read.  _relaxed: nothing in memory at all (tensor memory, behind
+// tcgen05.fence).  _own: shared memory of the arriving CTA, written behind fence.proxy.async and read by
+// that CTA's tensor core alone.
+__device__ __forceinline__ void mbar_arrive_remote_relaxed(uint32_t addr) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_remote_own(uint32_t addr) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 // `bytes` (a multiple of 16) from this CTA's shared memory into another CTA's
 // without waiting for them: the destination CTA's mbarrier `bar` (same CTA as
@@ -129,6 +165,7 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
 }
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort,
                                                   uint32_t limit) {
+#pragma unroll 1
   for (uint32_t i = 0; i < limit; ++i) {
     if (mbar_try_wait_cluster(bar, parity)) return true;
     if ((i & 15u) == 15u && *abort) return false;
@@ -223,6 +260,15 @@ __device__ __forceinline__ void tmem_st_x32(uint32_t taddr, const uint32_t (&r)[
       "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};\n"
       :
       : "r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+
+// The same for 16 columns.
+__device__ __forceinline__ void tmem_st_x16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"
+      :
+      : "r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
 
@@ -401,6 +447,180 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                    smem_u32(bar))
                : "memory");
+}
+
+// ------------------------------------------------------- a pair of CTAs --
+// cta_group::2: the two CTAs of a cluster work on one product, issued by one thread of the
+// even-ranked one.  With M = 128 each CTA holds 64 rows of A and of D and half of the rows of B (of
+// its columns when it is MN-major) at the same offsets of its shared and tensor memory; D has, in
+// each CTA, row r in lane r for the first half of the N columns and in lane 64 + r for the second.
+// Allocated and freed by one warp of each.  What one thread issues is called by its whole warp,
+// converged, and issued by an elected lane: operands that the compiler knows to be the same for all
+// lanes need no trip into uniform registers (a 128 x 128 x 16 product then takes 32 cycles; 45 where
+// one lane runs on its own).
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* smem_result, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_result)), "r"(ncols)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+// A tile load into this CTA whose bytes count on a barrier of either CTA of the pair (`bar` from
+// map_to_cta).
+__device__ __forceinline__ void tma_load_5d_pair(void* smem_dst, const CUtensorMap* m, uint32_t bar, int c0, int c1,
+                                                 int c2, int c3, int c4) {
+  asm volatile(
+      "{\n"
+      ".reg .pred one;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "@one cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 "
+      "[%0], [%1, {%3, %4, %5, %6, %7}], [%2];\n"
+      "}\n"
+      :
+      : "r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+      : "memory");
+}
+// One arrival on the mbarrier at this offset of both CTAs, or of the issuing one, when every
+// product issued so far by this thread has completed.
+__device__ __forceinline__ void umma_commit_both(uint64_t* bar) {
+  asm volatile(
+      "{\n"
+      ".reg .pred one;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "@one tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n"
+      "}\n" ::"r"(smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "{\n"
+      ".reg .pred one;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "@one tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+      "}\n" ::"r"(smem_u32(bar))
+      : "memory");
+}
+__device__ __forceinline__ void st_cta(uint32_t addr, uint32_t v) {  // addr from map_to_cta
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_cta(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+// D (+)= A B^T over K = 128: A and B K-major, each CTA's 64 rows as two 64-element halves 8 KB apart.
+__device__ __forceinline__ void umma_pair_kk_k128(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                                uint32_t accumulate_first) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p0, p1, one;\n"
+      ".reg .b32 al, bl;\n"
+      ".reg .b64 da, db;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "setp.ne.b32 p0, %5, 0;\n"
+      "setp.eq.b32 p1, %5, %5;\n"
+      "add.u32 al, %1, 0;\n"
+      "add.u32 bl, %2, 0;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p0;\n"
+      "add.u32 al, %1, 2;\n"
+      "add.u32 bl, %2, 2;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 4;\n"
+      "add.u32 bl, %2, 4;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 6;\n"
+      "add.u32 bl, %2, 6;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 512;\n"
+      "add.u32 bl, %2, 512;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 514;\n"
+      "add.u32 bl, %2, 514;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 516;\n"
+      "add.u32 bl, %2, 516;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 518;\n"
+      "add.u32 bl, %2, 518;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "}\n"
+      :
+      : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
+      : "memory");
+}
+// D (+)= A B over K = 128: A as above, B MN-major, each CTA's 64 columns in one block of 128 rows.
+__device__ __forceinline__ void umma_pair_kn_k128(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                                uint32_t accumulate_first) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p0, p1, one;\n"
+      ".reg .b32 al, bl;\n"
+      ".reg .b64 da, db;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "setp.ne.b32 p0, %5, 0;\n"
+      "setp.eq.b32 p1, %5, %5;\n"
+      "add.u32 al, %1, 0;\n"
+      "add.u32 bl, %2, 0;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p0;\n"
+      "add.u32 al, %1, 2;\n"
+      "add.u32 bl, %2, 128;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 4;\n"
+      "add.u32 bl, %2, 256;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 6;\n"
+      "add.u32 bl, %2, 384;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 512;\n"
+      "add.u32 bl, %2, 512;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 514;\n"
+      "add.u32 bl, %2, 640;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 516;\n"
+      "add.u32 bl, %2, 768;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "add.u32 al, %1, 518;\n"
+      "add.u32 bl, %2, 896;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %3};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p1;\n"
+      "}\n"
+      :
+      : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
+      : "memory");
 }
 
 }  // namespace sm100
