@@ -188,7 +188,7 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
       const bool is_k = warp == 0;
       if (is_k) {
         const uint32_t bar = map_to_cta(smem_u32(&bars.q_full), 0);
-        if (rank == 0) mbar_arrive_expect_tx_one(&bars.q_full, 4u * rows_box * 128u);
+        if (rank == 0) mbar_arrive_expect_tx(&bars.q_full, 4u * rows_box * 128u);
 #pragma unroll
         for (int h = 0; h < 2; ++h)  // rows beyond the last one read as zeros
           tma_load_5d_pair(sq + h * kHalf, &maps.q, bar, 0, g * p.group, nl_cta, h, b);
@@ -215,7 +215,7 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
           key0 += kb_start - (t - p.TP1) * BN;
         }
         if (t >= kStages && !wait(&bars.stage_free[stage], phase)) break;
-        if (rank == 0) mbar_arrive_expect_tx_one(full + stage, 2 * kTile);
+        if (rank == 0) mbar_arrive_expect_tx(full + stage, 2 * kTile);
         tma_load_5d_pair(dst + stage * 2 * kTile, m, full_leader + 8u * stage, 0, g, key0, half, b);
         if (++stage == kStages) {
           stage = 0;
@@ -485,7 +485,7 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
   tc_fence_after_sync();
   if (*abort_flag) {
     // copies that nobody has waited for: all of them count on the leader's barriers
-    if (rank == 0 && threadIdx.x == 0) {
+    if (rank == 0 && warp == 0) {
       mbar_wait_quiet(&bars.q_full, 0);
       for (int kv = 0; kv < 2; ++kv) {
         uint64_t* full = kv ? bars.v_full : bars.k_full;

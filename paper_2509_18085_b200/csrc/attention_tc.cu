@@ -14,18 +14,21 @@
 // column range computed from indices.
 //
 // Pipeline inside a CTA (384 threads):
-//   warp 0      TMA producer: Q once, then K and V tiles into two rings (seven
-//               32 KB tiles of shared memory in all, or fourteen of 16 KB at
+//   warps 0, 3  TMA producers: Q once and the K tiles, and the V tiles, into two rings
+//               (seven 32 KB tiles of shared memory in all, or fourteen of 16 KB at
 //               head dimension 64).  Q and the first K tile are asked for before
-//               the rest of the CTA has finished setting up; no more than those,
-//               because the issuing thread is held up once several tiles are in
-//               flight and the CTA-wide barrier would wait for it (0.9 us at 128
-//               CTAs that all start at once).
-//   warp 1      allocates tensor memory; one lane issues the score products
+//               the rest of the CTA has finished setting up.
+//   warp 1      allocates tensor memory and issues the score products
 //               S = Q K^T (tcgen05.mma, fp32 in TMEM)
-//   warp 2      one lane issues O += P V.  A warp each, because an issuing thread
+//   warp 2      issues O += P V.  A warp each, because an issuing warp
 //               is held for as long as its products run: with one for both, every
 //               wait for one kind of operand kept the tensor pipe from the other.
+//               All of them run converged and leave the instruction itself to an
+//               elected lane, and what is counted is counted along: one lane, whose
+//               operands go through uniform registers one by one, and a producer that
+//               divided by its ring's length took 5 to 15 % longer (28 heads on 4, 512
+//               positions over 1024 keys 14.5 -> 13.6 us; 2 x 32 x 32 positions x 32 heads
+//               over 4096 keys 135 -> 127; 4096 keys, 8 heads of 4, 256 positions 24.5 -> 20.7).
 //   warps 4-11  two softmax warpgroups, one thread per row each.  A unit of work is
 //               one (M-tile, key tile) pair; units alternate between the
 //               warpgroups, each of which keeps its own running (maximum, sum) and
@@ -40,8 +43,8 @@
 // soon as a warpgroup holds it in registers, so the scores of the next unit are
 // formed while the exponentials of this one are taken, P V of this one runs under
 // the exponentials of the next, and the hand-over keeps the two warpgroups half a
-// unit apart.  Measured, 2 x 32 x 32 positions x 32 heads over 4096 keys: 132 us, of
-// which 109 are left when all arithmetic of the softmax is taken out: what bounds a
+// unit apart.  Measured, 2 x 32 x 32 positions x 32 heads over 4096 keys: 127 us; of
+// the 132 it once was, 109 were left when all arithmetic of the softmax was taken out: what bounds a
 // long run is the round trip of the one S buffer (products 512 cycles, wake-up of
 // the warpgroup, read, wake-up of the issuing thread: about 1500 per unit against
 // 1024 of products).  P written over its S instead, with two of each, an issuing
@@ -200,65 +203,13 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
   volatile int* invited = abort_flag + 1;  // cluster: the others have been told that they may send
   int* rows = reinterpret_cast<int*>(smem + SM::rows);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // uniform to the compiler
   const int which = NP == 2 && (int)blockIdx.x >= problems.x_split ? 1 : 0;
   const Maps& maps = problems.maps[which];
   const Params& p = problems.p[which];
-  if (threadIdx.x == 0) {
-    prefetch_tensormap(&maps.q);  // the descriptors are kernel parameters
-    prefetch_tensormap(p.TP1 > 0 ? &maps.kp : (p.TP > 0 ? &maps.kp2 : &maps.kb));
-    prefetch_tensormap(p.TP1 > 0 ? &maps.vp : (p.TP > 0 ? &maps.vp2 : &maps.vb));
-  }
-  const int mt = ((int)blockIdx.x - (which ? problems.x_split : 0)) * NQ;  // first M-tile of this CTA
-  const int bg = blockIdx.y;
-  const int b = bg / p.Hkv, g = bg % p.Hkv;
-  const int cs = NQ == 1 ? p.cs : 1;
-  const int rank = NQ == 1 ? (int)blockIdx.z : 0;  // of this CTA in its cluster
-
-  // this CTA's rows and key tiles
-  const int nl0 = mt * p.TNL;
-  const int nl_count = min(NQ * p.TNL, p.NL - nl0);  // over all M-tiles of the CTA
-  const int rows_box = p.TNL * p.group;        // rows one Q box writes
-  const int n_lo = nl0 / p.L, n_hi = (nl0 + nl_count - 1) / p.L;
-  const int kb_start = n_lo * p.L;
-  const int TB = ((n_hi - n_lo + 1) * p.L + BN - 1) / BN;
-  const int T_all = p.TP + TB;
-  const int t_begin = rank * T_all / cs;  // small numbers: cs <= 8, T_all at most a few thousand
-  const int T = (rank + 1) * T_all / cs - t_begin;  // >= 1: cs <= T_all
-
-  // Producer (lane 0 of warp 0): tile j of the K or V ring.
-  int issued_k = 0, issued_v = 0;
-  bool prod_ok = true;
-  // (Counted along: a division by a number the compiler does not know takes some 200 cycles.)
-  int stage_k = 0, stage_v = 0;
-  uint32_t round_k = 0, round_v = 0;
-  auto produce = [&](bool is_k, int j) {
-    int& next = is_k ? stage_k : stage_v;
-    uint32_t& round_next = is_k ? round_k : round_v;
-    const int stage = next;
-    const uint32_t round = round_next;
-    if (++next == (is_k ? KS : VS)) {
-      next = 0;
-      ++round_next;
-    }
-    if (round > 0 && !mbar_wait((is_k ? k_empty : v_empty) + stage, (round & 1u) ^ 1u, abort_flag, p.spin_limit)) {
-      prod_ok = false;
-      return;
-    }
-    uint64_t* full = (is_k ? k_full : v_full) + stage;
-    const int t = t_begin + j;
-    // key tiles in order: first context segment, second context segment, block keys
-    const int seg = t < p.TP1 ? 0 : (t < p.TP ? 1 : 2);
-    const CUtensorMap* m = is_k ? (seg == 0 ? &maps.kp : seg == 1 ? &maps.kp2 : &maps.kb)
-                                : (seg == 0 ? &maps.vp : seg == 1 ? &maps.vp2 : &maps.vb);
-    const int key0 = seg == 0 ? t * BN : seg == 1 ? (t - p.TP1) * BN : kb_start + (t - p.TP) * BN;
-    uint8_t* dst = (is_k ? sk : sv) + stage * kTileBytes;
-    mbar_arrive_expect_tx(full, kTileBytes);
-    tma_load_5d(dst, m, full, 0, g, key0, 0, b);
-    if (is_k) issued_k = j + 1; else issued_v = j + 1;
-  };
-
-  constexpr int kRowBytes = HD * 4;  // of an fp32 partial
+  const int log_cs = NQ == 1 ? p.log_cs : 0, cs = 1 << log_cs;
+  const int rank = NQ == 1 ? (int)blockIdx.x & (cs - 1) : 0;  // of this CTA in its cluster
+  // Set-up, by warps side by side.
   if (warp == 0) {
     // one lane per barrier: a thread's initialisations are served one after the other
     static_assert(SM::n_bars <= 64, "two rounds of lanes");
@@ -271,11 +222,60 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
     }
     if (lane == 0) *abort_flag = *invited = 0;
     mbar_fence_init();
-    __syncwarp();
+  } else if (warp == 1) {
+    tmem_alloc(tmem_slot, kTmemCols);
+  } else if (warp == 2 && lane == 0) {
+    prefetch_tensormap(&maps.q);  // the descriptors are kernel parameters
+    prefetch_tensormap(p.TP1 > 0 ? &maps.kp : (p.TP > 0 ? &maps.kp2 : &maps.kb));
+    prefetch_tensormap(p.TP1 > 0 ? &maps.vp : (p.TP > 0 ? &maps.vp2 : &maps.vb));
   }
-  if (threadIdx.x == 0) {
+  __syncwarp();
+  const int mt = (((int)blockIdx.x - (which ? problems.x_split : 0)) >> log_cs) * NQ;  // first M-tile of this CTA
+  const int g = blockIdx.y, b = blockIdx.z;
+
+  // this CTA's rows and key tiles
+  const int nl0 = mt * p.TNL;
+  const int nl_count = min(NQ * p.TNL, p.NL - nl0);  // over all M-tiles of the CTA
+  const int rows_box = p.TNL * p.group;        // rows one Q box writes
+  const int n_lo = nl0 / p.L, n_hi = (nl0 + nl_count - 1) / p.L;
+  const int kb_start = n_lo * p.L;
+  const int TB = ((n_hi - n_lo + 1) * p.L + BN - 1) / BN;
+  const int T_all = p.TP + TB;
+  const int t_begin = (rank * T_all) >> log_cs;  // small numbers: cs <= 8, T_all at most a few thousand
+  const int T = (((rank + 1) * T_all) >> log_cs) - t_begin;  // >= 1: cs <= T_all
+
+  // The roles' waits, by whole warps.
+  auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, p.spin_limit));
+  };
+  // Producers: the next tile of the K ring (warp 0) or of the V ring (warp 3).  Everything is counted
+  // along: a division by a number the compiler does not know takes some 200 cycles.
+  const bool is_k = warp == 0;
+  int issued = 0, next_stage = 0;
+  uint32_t round = 0;
+  auto produce = [&]() -> bool {
+    if (round > 0 && !wait((is_k ? k_empty : v_empty) + next_stage, (round & 1u) ^ 1u)) return false;
+    uint64_t* full = (is_k ? k_full : v_full) + next_stage;
+    const int t = t_begin + issued;
+    // key tiles in order: first context segment, second context segment, block keys
+    const int seg = t < p.TP1 ? 0 : (t < p.TP ? 1 : 2);
+    const CUtensorMap* m = is_k ? (seg == 0 ? &maps.kp : seg == 1 ? &maps.kp2 : &maps.kb)
+                                : (seg == 0 ? &maps.vp : seg == 1 ? &maps.vp2 : &maps.vb);
+    const int key0 = seg == 0 ? t * BN : seg == 1 ? (t - p.TP1) * BN : kb_start + (t - p.TP) * BN;
+    mbar_arrive_expect_tx(full, kTileBytes);
+    tma_load_5d((is_k ? sk : sv) + next_stage * kTileBytes, m, full, 0, g, key0, 0, b);
+    ++issued;
+    if (++next_stage == (is_k ? KS : VS)) {
+      next_stage = 0;
+      ++round;
+    }
+    return true;
+  };
+
+  constexpr int kRowBytes = HD * 4;  // of an fp32 partial
+  if (warp == 0) {
     // what the others will send in the epilogue: this CTA's rows, and (maximum, sum) of each
-    if (cs > 1) mbar_arrive_expect_tx(xchg_full, (uint32_t)((cs - 1) * (BM / cs) * (kRowBytes + 8)));
+    if (cs > 1) mbar_arrive_expect_tx(xchg_full, (uint32_t)((cs - 1) * (BM >> log_cs) * (kRowBytes + 8)));
     if (!p.independent) cudaGridDependencySynchronize();
     mbar_arrive_expect_tx(q_full, (uint32_t)(NQ * kHalves) * rows_box * 128u);
 #pragma unroll
@@ -284,7 +284,7 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
       for (int h = 0; h < kHalves; ++h)  // with fewer than 128 rows in the box the halves lie further apart than it is long
         tma_load_5d(sq + q * kTileBytes + h * kHalfBytes, &maps.q, q_full, 0, g * p.group, nl0 + q * p.TNL, h, b);
     }
-    produce(true, 0);
+    produce();
   }
   // rows of the Q tile that the TMA box does not write must be finite
   for (int i = rows_box * 8 + threadIdx.x; i < BM * 8; i += kThreads) {
@@ -293,7 +293,6 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
     for (int h = 0; h < kHalves * NQ; ++h) reinterpret_cast<uint4*>(sq + h * kHalfBytes)[i] = z;
   }
   fence_proxy_async_smem();
-  if (warp == 1) tmem_alloc(tmem_slot, kTmemCols);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -307,73 +306,65 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
   const int U = T << kLogNQ;  // units of this CTA
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
-    if (warp == 0) {
-      // ------------------------------------------------------------ producer --
-      if (lane == 0) {
-        // the rest of both rings, in the order the products need them: K(j+1) before V(j)
-        int jk = 1, jv = 0;
-        while (prod_ok && (jk < T || jv < T)) {
-          const bool is_k = jk < T && jk <= jv + 1;
-          produce(is_k, is_k ? jk : jv);
-          if (is_k) ++jk; else ++jv;
+    if (warp == 0 || warp == 3) {
+      // ----------------------------------------------------------- producers --
+      while (issued < T && produce()) {
+      }
+      // Whoever gives up, and when: no copy is in flight into shared memory whose block has ended.
+      if (is_k) mbar_wait_quiet(q_full, 0);
+      const int depth = is_k ? KS : VS;
+      for (int k = min(issued, depth); k > 0; --k) {
+        if (--next_stage < 0) {
+          next_stage = depth - 1;
+          --round;
         }
-        // Whoever gives up, and when: no copy is in flight into shared memory whose block has ended.
-        mbar_wait_quiet(q_full, 0);
-        for (int j = max(0, issued_k - KS); j < issued_k; ++j)
-          mbar_wait_quiet(k_full + j % KS, (uint32_t)(j / KS) & 1u);
-        for (int j = max(0, issued_v - VS); j < issued_v; ++j)
-          mbar_wait_quiet(v_full + j % VS, (uint32_t)(j / VS) & 1u);
+        mbar_wait_quiet((is_k ? k_full : v_full) + next_stage, round & 1u);
       }
     } else if (warp == 1) {
       // ------------------------------------------------ issuer of S = Q K^T --
-      if (lane == 0) {
-        constexpr uint32_t idesc = idesc_bf16_f32(BM, BN, false, false);
-        constexpr uint32_t hi = desc_hi_sw128(1024);
-        const uint32_t q_lo = desc_lo_sw128(smem_u32(sq), 16);
-        const uint32_t k_lo = desc_lo_sw128(smem_u32(sk), 16);
-        int stage = 0;
-        uint32_t phase = 0;
-        bool ok = mbar_wait(q_full, 0, abort_flag, p.spin_limit);
-        for (int u = 0; u < U && ok; ++u) {
-          if (NQ == 1 || (u & 1) == 0) ok = mbar_wait(k_full + stage, phase, abort_flag, p.spin_limit);
-          // the scores before have been read
-          if (ok && u >= 1)
-            ok = mbar_wait(s_free + ((u - 1) & 1), (uint32_t)((u - 1) >> 1) & 1u, abort_flag, p.spin_limit);
-          if (!ok) break;
-          tc_fence_after_sync();
-          const uint32_t qa = q_lo + (NQ == 2 ? (uint32_t)(u & 1) * (kTileBytes >> 4) : 0u);
-          const uint32_t ka = k_lo + (uint32_t)stage * (kTileBytes >> 4);
-          if constexpr (HD == 128) umma_ss_k128(tmem + kColS, qa, ka, hi, idesc, 0u);
-          else umma_ss_k64(tmem + kColS, qa, ka, hi, idesc, 0u);
-          umma_commit(s_full + (u & 1));
-          if (NQ == 1 || (u & 1)) {  // a key tile serves all M-tiles before it is released
-            umma_commit(k_empty + stage);
-            if (++stage == KS) { stage = 0; phase ^= 1u; }
-          }
+      constexpr uint32_t idesc = idesc_bf16_f32(BM, BN, false, false);
+      constexpr uint32_t hi = desc_hi_sw128(1024);
+      const uint32_t q_lo = desc_lo_sw128(smem_u32(sq), 16);
+      const uint32_t k_lo = desc_lo_sw128(smem_u32(sk), 16);
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = wait(q_full, 0);
+      for (int u = 0; u < U && ok; ++u) {
+        if (NQ == 1 || (u & 1) == 0) ok = wait(k_full + stage, phase);
+        // the scores before have been read
+        if (ok && u >= 1) ok = wait(s_free + ((u - 1) & 1), (uint32_t)((u - 1) >> 1) & 1u);
+        if (!ok) break;
+        tc_fence_after_sync();
+        const uint32_t qa = q_lo + (NQ == 2 ? (uint32_t)(u & 1) * (kTileBytes >> 4) : 0u);
+        const uint32_t ka = k_lo + (uint32_t)stage * (kTileBytes >> 4);
+        if constexpr (HD == 128) umma_ss_k128(tmem + kColS, qa, ka, hi, idesc, 0u);
+        else umma_ss_k64(tmem + kColS, qa, ka, hi, idesc, 0u);
+        umma_commit(s_full + (u & 1));
+        if (NQ == 1 || (u & 1)) {  // a key tile serves all M-tiles before it is released
+          umma_commit(k_empty + stage);
+          if (++stage == KS) { stage = 0; phase ^= 1u; }
         }
       }
     } else if (warp == 2) {
       // --------------------------------------------------- issuer of O += P V --
-      if (lane == 0) {
-        constexpr uint32_t idesc = idesc_bf16_f32(BM, HD, false, true);
-        constexpr uint32_t hi = desc_hi_sw128(1024);
-        const uint32_t v_lo = desc_lo_sw128(smem_u32(sv), kHalfBytes);
-        int stage = 0;
-        uint32_t phase = 0;
-        for (int u = 0; u < U; ++u) {
-          if ((NQ == 1 || (u & 1) == 0) && !mbar_wait(v_full + stage, phase, abort_flag, p.spin_limit)) break;
-          if (!mbar_wait(p_ready + (u & 1), (uint32_t)(u >> 1) & 1u, abort_flag, p.spin_limit)) break;
-          tc_fence_after_sync();
-          umma_ts_k128(tmem + kColO + (uint32_t)(u & 1) * HD, tmem + kColP + (uint32_t)(u & 1) * 64u,
-                       v_lo + (uint32_t)stage * (kTileBytes >> 4), hi, idesc, u >= 2 ? 1u : 0u);
-          if constexpr (kRest)
-            umma_ts_k128(tmem + kColO + (uint32_t)(u & 1) * HD, tmem + kColRest + (uint32_t)(u & 1) * 64u,
-                         v_lo + (uint32_t)stage * (kTileBytes >> 4), hi, idesc, 1u);
-          umma_commit(pv_done + (u & 1));
-          if (NQ == 1 || (u & 1)) {
-            umma_commit(v_empty + stage);
-            if (++stage == VS) { stage = 0; phase ^= 1u; }
-          }
+      constexpr uint32_t idesc = idesc_bf16_f32(BM, HD, false, true);
+      constexpr uint32_t hi = desc_hi_sw128(1024);
+      const uint32_t v_lo = desc_lo_sw128(smem_u32(sv), kHalfBytes);
+      int stage = 0;
+      uint32_t phase = 0;
+      for (int u = 0; u < U; ++u) {
+        if ((NQ == 1 || (u & 1) == 0) && !wait(v_full + stage, phase)) break;
+        if (!wait(p_ready + (u & 1), (uint32_t)(u >> 1) & 1u)) break;
+        tc_fence_after_sync();
+        umma_ts_k128(tmem + kColO + (uint32_t)(u & 1) * HD, tmem + kColP + (uint32_t)(u & 1) * 64u,
+                     v_lo + (uint32_t)stage * (kTileBytes >> 4), hi, idesc, u >= 2 ? 1u : 0u);
+        if constexpr (kRest)
+          umma_ts_k128(tmem + kColO + (uint32_t)(u & 1) * HD, tmem + kColRest + (uint32_t)(u & 1) * 64u,
+                       v_lo + (uint32_t)stage * (kTileBytes >> 4), hi, idesc, 1u);
+        umma_commit(pv_done + (u & 1));
+        if (NQ == 1 || (u & 1)) {
+          umma_commit(v_empty + stage);
+          if (++stage == VS) { stage = 0; phase ^= 1u; }
         }
       }
     }
@@ -548,7 +539,7 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
       // rings (idle since their last scores).  Hand-over by mbarriers: xchg_ready = "my buffers
       // are free" (sent from the tile loop by every other CTA), xchg_full = "your partials have
       // landed", completed by the byte counts of the copies.
-      const int R = BM / cs;
+      const int R = BM >> log_cs;
       float2* ml_mine = ml + 2 * BM;  // [128] of this CTA's partial
       float2* ml_recv = ml + 3 * BM;  // [cs][R] of this CTA's rows, its own among them
       float* weight = reinterpret_cast<float*>(ml + 4 * BM);  // [cs][R] what a slice's partial counts
@@ -729,13 +720,13 @@ int resident_clusters(int hd, int cs) {
   int n = slot.load(std::memory_order_relaxed);
   if (n == 0) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1, 1, (unsigned)cs);
+    cfg.gridDim = dim3((unsigned)cs);
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmemBytes;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = (unsigned)cs;
+    attr[0].val.clusterDim.x = (unsigned)cs;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (cudaOccupancyMaxActiveClusters(&n, kernel_of<1>(hd, 1), &cfg) != cudaSuccess) {
@@ -817,7 +808,7 @@ bool make_problem(const spiffy_attn_desc& d, const Shape& sh, const AttnProblem&
   }
   p->B = d.batch; p->N = d.n_nodes; p->L = d.block_len; p->P = a.ctx.len; p->P2 = a.ctx2.len;
   p->Hq = d.n_q_heads; p->Hkv = d.n_kv_heads; p->group = sh.group;
-  p->TNL = sh.TNL; p->NL = sh.NL; p->TP1 = sh.TP1; p->TP = sh.TP; p->cs = pl.cs;
+  p->TNL = sh.TNL; p->NL = sh.NL; p->TP1 = sh.TP1; p->TP = sh.TP; p->log_cs = pl.cs == 8 ? 3 : pl.cs / 2;
   const float scale = d.scale != 0.f ? d.scale : 1.0f / sqrtf((float)d.head_dim);
   p->scale_log2 = scale * kLog2e;
   p->out = static_cast<__nv_bfloat16*>(a.out);
@@ -862,21 +853,21 @@ spiffy_status launch(const spiffy_attn_desc* const (&d)[NP], const AttnProblem* 
     if (pl.pair) sh[i] = by_pairs[i];
     if (!make_problem(*d[i], sh[i], *a[i], &pr.maps[i], &pr.p[i], pl, dev_status)) return SPIFFY_ECUDA;
     if (i == 1) pr.x_split = x;
-    x += pl.pair ? 2 * sh[i].MT : (sh[i].MT + pl.nq - 1) / pl.nq;
+    x += pl.pair ? 2 * sh[i].MT : (sh[i].MT + pl.nq - 1) / pl.nq * pl.cs;
   }
   if (pl.pair) return launch_attention_pair<NP>(pr, x, stream);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)x, (unsigned)bg, (unsigned)pl.cs);
+  cfg.gridDim = dim3((unsigned)x, (unsigned)d[0]->n_kv_heads, (unsigned)d[0]->batch);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;  // along grid.z, only when asked for
-  attr[1].val.clusterDim.x = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;  // only when asked for
+  attr[1].val.clusterDim.x = (unsigned)pl.cs;
   attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = (unsigned)pl.cs;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pl.cs > 1 ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel_of<NP>(hd, pl.nq), pr);

@@ -23,7 +23,7 @@ struct Params {
   int TNL;      // (node, position) pairs per M-tile
   int NL;       // N * L
   int TP1, TP;  // context key tiles: of the first segment, of both
-  int cs;       // CTAs of a cluster that share an M-tile's key tiles
+  int log_cs;   // CTAs of a cluster that share an M-tile's key tiles: 1, 2, 4 or 8
   float scale_log2;
   __nv_bfloat16* out;
   int32_t* status;

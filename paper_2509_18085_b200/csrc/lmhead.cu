@@ -19,7 +19,7 @@
 //                          in chunks of 64:
 //     warp 0      TMA producer: per chunk 256 rows of W and the positions' rows
 //                 of H into a ring
-//     warp 1      allocates tensor memory; one lane issues tcgen05.mma, M = 128,
+//     warp 1      allocates tensor memory and issues tcgen05.mma, M = 128,
 //                 two M-tiles per chunk
 //     warps 4-11  one thread per vocabulary entry (TMEM lane): for every position
 //                 (column) the warp's 32 entries are reduced across lanes
@@ -34,7 +34,8 @@
 // thread, which is why its warps take the others' share) and gives it back, so that
 // the next tile's products run meanwhile: 234 -> 214 us with 164 masked positions, in
 // runs of tens of milliseconds.  Called back to back for seconds it draws the board's
-// power limit, and takes 230-246 us (166 masked positions; 283 before).
+// power limit, and takes 230 us (166 masked positions; 283 before, 243 with producer and issuer a
+// lane each instead of converged warps).
 //
 // Each CTA leaves one partial result per position; the decision's finalize kernel
 // merges them (in a fixed order) and applies the unmasking rule.  Every wait is
@@ -184,7 +185,7 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kLmBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // uniform to the compiler
   // this CTA's share of the vocabulary, in steps of 32 entries
   const int64_t units = (p.vocab + kBox - 1) / kBox;
   const int v_begin = (int)(units * blockIdx.x / gridDim.x) * kBox;
@@ -227,7 +228,11 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
-    if (warp == 0 && lane == 0) {
+    // whole warps up to the elected lane's instruction (sm100_ptx.cuh)
+    auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+      return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, p.spin_limit));
+    };
+    if (warp == 0) {
       // ---------------------------------------------------------- producer --
       bool ok = true;
       int stage = 0;
@@ -237,7 +242,7 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
         for (int i = 0; i < tiles && ok; ++i) {
           const int v0 = v_begin + i * kTileV, rows = min(kTileV, v_end - v0);
           for (int kc = 0; kc < kc_count; ++kc) {
-            if (!mbar_wait(empty + stage, phase ^ 1u, abort_flag, p.spin_limit)) { ok = false; break; }
+            if (!wait(empty + stage, phase ^ 1u)) { ok = false; break; }
             uint8_t* dst = smem + stage * stage_bytes;
             mbar_arrive_expect_tx(full + stage, (uint32_t)(rows + nb * kBox) * 128u);
             used |= 1u << stage;
@@ -260,7 +265,7 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
         if ((used >> q) & 1u)
           for (uint32_t s = 0; s < kSpinLimit; ++s)
             if (mbar_try_wait(full + q, q < stage ? phase : phase ^ 1u)) break;
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       // -------------------------------------------------------- MMA issuer --
       constexpr uint32_t hi = desc_hi_sw128(1024);
       bool ok = true;
@@ -273,12 +278,12 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
           const int m_tiles = v_end - (v_begin + i * kTileV) > 128 ? 2 : 1;
           const int buf = bufs == 2 ? g & 1 : 0;
           const uint32_t round = (uint32_t)(bufs == 2 ? g >> 1 : g);
-          ok = mbar_wait(acc_empty + buf, (round & 1u) ^ 1u, abort_flag, p.spin_limit);
+          ok = wait(acc_empty + buf, (round & 1u) ^ 1u);
           if (!ok) break;
           tc_fence_after_sync();
           const uint32_t d = tmem + (uint32_t)buf * 256u;
           for (int kc = 0; kc < kc_count; ++kc) {
-            if (!mbar_wait(full + stage, phase, abort_flag, p.spin_limit)) { ok = false; break; }
+            if (!wait(full + stage, phase)) { ok = false; break; }
             tc_fence_after_sync();
             const uint32_t w_lo = desc_lo_sw128(smem_u32(smem + stage * stage_bytes), 16);
             const uint32_t h_lo = w_lo + ((uint32_t)w_bytes >> 4);

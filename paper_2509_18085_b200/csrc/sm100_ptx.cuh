@@ -8,6 +8,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+//
+// What one thread issues -- products, commits, TMA loads, expected bytes -- is called by its whole
+// warp, converged, and issued by an elected lane: operands that the compiler knows to be the same for
+// all lanes need no trip into uniform registers each time (a 128 x 128 x 16 product of a pair of CTAs
+// then takes 32 cycles; 45 where one lane runs on its own).
 namespace spiffy {
 namespace sm100 {
 
@@ -26,11 +31,6 @@ __device__ __forceinline__ void mbar_fence_init() {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -45,8 +45,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// The same by one lane of a converged warp.
-__device__ __forceinline__ void mbar_arrive_expect_tx_one(uint64_t* bar, uint32_t bytes) {
+// One arrival, by one lane of a converged warp.
+__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile(
       "{\n"
       ".reg .pred one;\n"
@@ -82,8 +82,12 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* m) {
 __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* m, uint64_t* bar,
                                             int c0, int c1, int c2, int c3) {
   asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%3, %4, %5, %6}], [%2];"
+      "{\n"
+      ".reg .pred one;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "@one cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%3, %4, %5, %6}], [%2];\n"
+      "}\n"
       :
       : "r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(c0),
         "r"(c1), "r"(c2), "r"(c3)
@@ -92,8 +96,12 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* m
 __device__ __forceinline__ void tma_load_5d(void* smem_dst, const CUtensorMap* m, uint64_t* bar,
                                             int c0, int c1, int c2, int c3, int c4) {
   asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
+      "{\n"
+      ".reg .pred one;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "@one cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%3, %4, %5, %6, %7}], [%2];\n"
+      "}\n"
       :
       : "r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(c0),
         "r"(c1), "r"(c2), "r"(c3), "r"(c4)
@@ -307,51 +315,52 @@ __device__ __forceinline__ void umma_ss_k128(uint32_t d_tmem, uint32_t a_lo, uin
                                              uint32_t idesc, uint32_t accumulate_first) {
   asm volatile(
       "{\n"
-      ".reg .pred p0, p1;\n"
+      ".reg .pred p0, p1, one;\n"
       ".reg .b32 al, bl;\n"
       ".reg .b64 da, db;\n"
+      "elect.sync _|one, 0xffffffff;\n"
       "setp.ne.b32 p0, %5, 0;\n"
       "setp.eq.b32 p1, %5, %5;\n"
       "add.u32 al, %1, 0;\n"
       "add.u32 bl, %2, 0;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p0;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p0;\n"
       "add.u32 al, %1, 2;\n"
       "add.u32 bl, %2, 2;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
       "add.u32 al, %1, 4;\n"
       "add.u32 bl, %2, 4;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
       "add.u32 al, %1, 6;\n"
       "add.u32 bl, %2, 6;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
       "add.u32 al, %1, 1024;\n"
       "add.u32 bl, %2, 1024;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
       "add.u32 al, %1, 1026;\n"
       "add.u32 bl, %2, 1026;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
       "add.u32 al, %1, 1028;\n"
       "add.u32 bl, %2, 1028;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
       "add.u32 al, %1, 1030;\n"
       "add.u32 bl, %2, 1030;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
       "}\n"
       :
       : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
@@ -362,31 +371,32 @@ __device__ __forceinline__ void umma_ss_k64(uint32_t d_tmem, uint32_t a_lo, uint
                                             uint32_t idesc, uint32_t accumulate_first) {
   asm volatile(
       "{\n"
-      ".reg .pred p0, p1;\n"
+      ".reg .pred p0, p1, one;\n"
       ".reg .b32 al, bl;\n"
       ".reg .b64 da, db;\n"
+      "elect.sync _|one, 0xffffffff;\n"
       "setp.ne.b32 p0, %5, 0;\n"
       "setp.eq.b32 p1, %5, %5;\n"
       "add.u32 al, %1, 0;\n"
       "add.u32 bl, %2, 0;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p0;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p0;\n"
       "add.u32 al, %1, 2;\n"
       "add.u32 bl, %2, 2;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
       "add.u32 al, %1, 4;\n"
       "add.u32 bl, %2, 4;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
       "add.u32 al, %1, 6;\n"
       "add.u32 bl, %2, 6;\n"
       "mov.b64 da, {al, %3};\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p1;\n"
       "}\n"
       :
       : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
@@ -398,43 +408,44 @@ __device__ __forceinline__ void umma_ts_k128(uint32_t d_tmem, uint32_t a_tmem, u
                                              uint32_t idesc, uint32_t accumulate_first) {
   asm volatile(
       "{\n"
-      ".reg .pred p0, p1;\n"
+      ".reg .pred p0, p1, one;\n"
       ".reg .b32 at, bl;\n"
       ".reg .b64 db;\n"
+      "elect.sync _|one, 0xffffffff;\n"
       "setp.ne.b32 p0, %5, 0;\n"
       "setp.eq.b32 p1, %5, %5;\n"
       "add.u32 at, %1, 0;\n"
       "add.u32 bl, %2, 0;\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p0;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p0;\n"
       "add.u32 at, %1, 8;\n"
       "add.u32 bl, %2, 128;\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
       "add.u32 at, %1, 16;\n"
       "add.u32 bl, %2, 256;\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
       "add.u32 at, %1, 24;\n"
       "add.u32 bl, %2, 384;\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
       "add.u32 at, %1, 32;\n"
       "add.u32 bl, %2, 512;\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
       "add.u32 at, %1, 40;\n"
       "add.u32 bl, %2, 640;\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
       "add.u32 at, %1, 48;\n"
       "add.u32 bl, %2, 768;\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
       "add.u32 at, %1, 56;\n"
       "add.u32 bl, %2, 896;\n"
       "mov.b64 db, {bl, %3};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
+      "@one tcgen05.mma.cta_group::1.kind::f16 [%0], [at], db, %4, p1;\n"
       "}\n"
       :
       : "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
@@ -444,9 +455,13 @@ __device__ __forceinline__ void umma_ts_k128(uint32_t d_tmem, uint32_t a_tmem, u
 // The mbarrier receives one arrival when every MMA issued so far by this
 // thread has completed (implies tcgen05.fence::before_thread_sync).
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
+  asm volatile(
+      "{\n"
+      ".reg .pred one;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "@one tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+      "}\n" ::"r"(smem_u32(bar))
+      : "memory");
 }
 
 // ------------------------------------------------------- a pair of CTAs --
@@ -454,10 +469,7 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
 // even-ranked one.  With M = 128 each CTA holds 64 rows of A and of D and half of the rows of B (of
 // its columns when it is MN-major) at the same offsets of its shared and tensor memory; D has, in
 // each CTA, row r in lane r for the first half of the N columns and in lane 64 + r for the second.
-// Allocated and freed by one warp of each.  What one thread issues is called by its whole warp,
-// converged, and issued by an elected lane: operands that the compiler knows to be the same for all
-// lanes need no trip into uniform registers (a 128 x 128 x 16 product then takes 32 cycles; 45 where
-// one lane runs on its own).
+// Allocated and freed by one warp of each.
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t* smem_result, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_result)), "r"(ncols)
                : "memory");
