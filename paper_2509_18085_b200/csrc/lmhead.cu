@@ -33,9 +33,10 @@
 // for a second accumulator pair: the epilogue empties the first into registers (192 a
 // thread, which is why its warps take the others' share) and gives it back, so that
 // the next tile's products run meanwhile: 234 -> 214 us with 164 masked positions, in
-// runs of tens of milliseconds.  Called back to back for seconds it draws the board's
-// power limit, and takes 230 us (166 masked positions; 283 before, 243 with producer and issuer a
-// lane each instead of converged warps).
+// runs of tens of milliseconds.  With the producer and the issuer as converged warps, and two or three
+// TMA instructions a chunk where there were eight, 193 us in such runs (209 before on that board), and
+// 210 us called back to back for seconds, which draws the board's power limit (228 before).  A ring of
+// its own for the weights, four chunks deep beside three of H, with a producer each: 222.
 //
 // Each CTA leaves one partial result per position; the decision's finalize kernel
 // merges them (in a fixed order) and applies the unmasking rule.  Every wait is
@@ -58,7 +59,8 @@ constexpr int kPass = 256;              // positions per pass
 // Up to this many positions are taken as they are, masked or not: they cost less time as columns
 // (their part of what an SM takes in stays below the weights' third) than the launch that packs.
 constexpr int kDirectRows = 128;
-constexpr int kBox = 32;                // rows of H per TMA box (and of W in a tile that is not whole)
+constexpr int kBox = 32;                // rows of W and H are loaded in boxes of 32, 64, 128 or 256
+constexpr int kBoxSizes = 4;
 constexpr int kTileV = 256;             // vocabulary entries per tile: two M-tiles
 constexpr int kRing = 200 * 1024;
 constexpr int kMaxStages = 12;          // at least three: 64 KB per stage at 256 positions
@@ -85,6 +87,10 @@ struct LmParams {
   int n_status;
   int clear_status;      // the status words arrive with arbitrary contents (without a list only)
   uint32_t spin_limit;   // polls of one mbarrier wait
+};
+
+struct LmMaps {
+  CUtensorMap w[kBoxSizes], h[kBoxSizes];  // [i]: boxes of 32 << i rows, 64 columns
 };
 
 // grid = rows.  Block r copies row r, if its position is masked, behind the masked rows before it.
@@ -172,8 +178,7 @@ __device__ __forceinline__ void add_columns(ColumnState& state, int ew, int at, 
 }
 
 __global__ void __launch_bounds__(kLmThreads, 1)
-lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w,
-                     const __grid_constant__ CUtensorMap tm_w32, const LmParams p) {
+lmhead_reduce_kernel(const __grid_constant__ LmMaps maps, const LmParams p) {
   extern __shared__ uint8_t lm_smem_raw[];
   uint8_t* smem = lm_smem_raw + ((0u - smem_u32(lm_smem_raw)) & 1023u);
   ColumnState& state = *reinterpret_cast<ColumnState*>(smem + kRing);
@@ -194,9 +199,7 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
   const int kc_count = p.hidden / 64;
 
   if (threadIdx.x == 0) {
-    prefetch_tensormap(&tm_h);
-    prefetch_tensormap(&tm_w);
-    prefetch_tensormap(&tm_w32);
+    prefetch_tensormap(&maps.w[kBoxSizes - 1]);
     for (int i = 0; i < kMaxStages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(acc_full + i, 1); mbar_init(acc_empty + i, 8); }  // the epilogue warps
     *abort_flag = 0;
@@ -246,16 +249,19 @@ lmhead_reduce_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_cons
             uint8_t* dst = smem + stage * stage_bytes;
             mbar_arrive_expect_tx(full + stage, (uint32_t)(rows + nb * kBox) * 128u);
             used |= 1u << stage;
-            const int c0 = (kc & 1) * 64, head = kc >> 1;
-            if (rows == kTileV) {
-              tma_load_4d(dst, &tm_w, full + stage, c0, head, v0, 0);
-              tma_load_4d(dst + 128 * 128, &tm_w, full + stage, c0, head, v0 + 128, 0);
-            } else {
-              for (int q = 0; q < rows / kBox; ++q)
-                tma_load_4d(dst + q * kBox * 128, &tm_w32, full + stage, c0, head, v0 + q * kBox, 0);
-            }
-            for (int q = 0; q < nb; ++q)
-              tma_load_4d(dst + w_bytes + q * kBox * 128, &tm_h, full + stage, c0, head, pass * kPass + q * kBox, 0);
+            // as few instructions as the rows' number has binary digits: each takes its warp some 200 cycles
+            auto load = [&](const CUtensorMap* m, uint8_t* to, int row, int n) {
+#pragma unroll
+              for (int s = kBoxSizes - 1; s >= 0; --s) {
+                if (n < (kBox << s)) continue;
+                tma_load_4d(to, m + s, full + stage, (kc & 1) * 64, kc >> 1, row, 0);
+                to += kBox * 128 << s;
+                row += kBox << s;
+                n -= kBox << s;
+              }
+            };
+            load(maps.w, dst, v0, rows);
+            load(maps.h, dst + w_bytes, pass * kPass, nb * kBox);
             if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
         }
@@ -407,12 +413,12 @@ spiffy_status launch_lmhead_decide(const spiffy_decide_desc& d, int hidden, cons
   char* at = static_cast<char*>(ws);
   int* list = reinterpret_cast<int*>(at + partial_bytes(d, grid));
   uint4* packed = reinterpret_cast<uint4*>(at + partial_bytes(d, grid) + list_bytes(d));
-  CUtensorMap tm_h, tm_w, tm_w32;
+  LmMaps maps;
   const bool pack = rows > kDirectRows;
-  if (!make_map(&tm_h, pack ? static_cast<const void*>(packed) : hstates, hidden / 128, rows, 1, 1, kBox) ||
-      !make_map(&tm_w, weight, hidden / 128, d.vocab, 1, 1, 128) ||
-      !make_map(&tm_w32, weight, hidden / 128, d.vocab, 1, 1, kBox))
-    return SPIFFY_ECUDA;
+  for (int i = 0; i < kBoxSizes; ++i)
+    if (!make_map(&maps.w[i], weight, hidden / 128, d.vocab, 1, 1, kBox << i) ||
+        !make_map(&maps.h[i], pack ? static_cast<const void*>(packed) : hstates, hidden / 128, rows, 1, 1, kBox << i))
+      return SPIFFY_ECUDA;
   static std::atomic<bool> smem_allowed[64];
   if (!allow_smem(lmhead_reduce_kernel, kLmSmem, smem_allowed)) return SPIFFY_ECUDA;
   cudaError_t e = cudaSuccess;
@@ -433,7 +439,7 @@ spiffy_status launch_lmhead_decide(const spiffy_decide_desc& d, int hidden, cons
   p.status = dev_status;
   p.n_status = d.batch;
   p.spin_limit = mbar_poll_limit();
-  e = launch_pdl(lmhead_reduce_kernel, dim3(grid), dim3(kLmThreads), (size_t)kLmSmem, stream, tm_h, tm_w, tm_w32, p);
+  e = launch_pdl(lmhead_reduce_kernel, dim3(grid), dim3(kLmThreads), (size_t)kLmSmem, stream, maps, p);
   count_launch();
   if (e != cudaSuccess) return SPIFFY_ECUDA;
   return launch_decide_finalize(d, ws, grid, block_tokens, conf, top_tok, unmask_bits, n_unmask, dev_status,
