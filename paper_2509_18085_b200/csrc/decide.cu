@@ -28,8 +28,16 @@ namespace {
 // the call, and the status words cleared ahead of the token's load, for which every CTA waits first,
 // another 1 to 2 % (256 rows x 126464 with 164 masked: 13.0 us with all that, 12.4 so; 512 rows x
 // 152064 with 348 masked: 24.6 and 23.4).
+// What bounds it beside the bytes is instructions issued, and CTAs in flight to cover one another's
+// chains: the search for the maximum's index by the threads that hold it alone, their vote through one
+// atomic, a maximum by one instruction a warp, and with the registers that saves nine CTAs per SM
+// (56 registers; eight before, with 64): 4096 rows x 126464 with 2596 masked 121 -> 108.5 us (6.05
+// TB/s), 512 x 152064 with 322 masked 27.3 -> 25.3 with the walk, 256 x 126464 with 142 13.8 -> 13.1.
+// Tried and dropped: ten CTAs (113.6), slices in shared memory by asynchronous copies with ten or
+// twelve CTAs (120), runs of slices per CTA, the next one's loads under this one's end (111 to 120, and
+// 3 us more at 256 rows) or in a second set of registers (150).
 template <typename T, bool kIndependent>
-__global__ void __launch_bounds__(kReduceThreads, 8)  // 64 registers: eight CTAs per SM
+__global__ void __launch_bounds__(kReduceThreads, 9)  // 56 registers: nine CTAs per SM
 decide_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V,
                      int64_t chunk, int splits,
                      const int32_t* __restrict__ block_tokens, int mask_id,

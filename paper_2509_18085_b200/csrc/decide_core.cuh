@@ -160,6 +160,13 @@ __device__ __forceinline__ void store16(void* p, uint64_t lo, uint64_t hi) {
                : "memory");
 }
 
+// The maximum over the warp's lanes; NaNs lose, as in fmaxf.
+__device__ __forceinline__ float warp_max(float x) {
+  float m;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+  return m;
+}
+
 // One CTA of kReduceThreads threads reduces one vocabulary slice
 // [split * chunk, min(V, (split + 1) * chunk)) of the logits row at `base` to
 // (maximum, sum of exp(x - maximum), lowest index attaining the maximum).  A
@@ -204,8 +211,8 @@ __device__ __forceinline__ Partial reduce_slice(const T* __restrict__ base, int 
   float m = Elem<T>::gmax(v);
 #pragma unroll
   for (int e = 0; e < EPV; ++e) m = fmaxf(m, tail[e]);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+  const float mine = m;
+  m = warp_max(m);
   __shared__ float warp_m[kReduceThreads / 32], warp_s[kReduceThreads / 32];
   __shared__ int slice_idx;
   if (lane == 0) warp_m[warp] = m;
@@ -214,17 +221,23 @@ __device__ __forceinline__ Partial reduce_slice(const T* __restrict__ base, int 
   m = warp_m[0];
 #pragma unroll
   for (int w = 1; w < kReduceThreads / 32; ++w) m = fmaxf(m, warp_m[w]);
-  // 3. sum of exp(x - m) and the lowest index that attains m
+  // 3. the lowest index that attains m: only the threads whose own maximum it is search for it
+  if (mine == m && m != -INFINITY) {
+    int idx = 0x7fffffff;
+#pragma unroll
+    for (int e = EPV - 1; e >= 0; --e)
+      if (e < ntail && tail[e] == m) idx = (int)begin + nvec * EPV + e;  // thread 0 alone has a tail
+#pragma unroll
+    for (int u = kUnroll - 1; u >= 0; --u)
+      if (Elem<T>::holds(v[u], m)) idx = (int)begin + (tid + u * kReduceThreads) * EPV + Elem<T>::first_equal(v[u], m);
+    atomicMin(&slice_idx, idx);
+  }
+  // 4. sum of exp(x - m)
   const float ml = (m == -INFINITY) ? 0.f : m * k;  // an all -inf slice sums to 0
   const uint64_t k2 = pack2(k, k), nml2 = pack2(-ml, -ml);
   uint64_t acc = pack2(0.f, 0.f);
-  int idx = 0x7fffffff;
 #pragma unroll
-  for (int u = kUnroll - 1; u >= 0; --u) {
-    acc = Elem<T>::sum_terms(v[u], k2, nml2, acc);
-    if (Elem<T>::holds(v[u], m))  // rare: only the vectors that hold the slice maximum are searched
-      idx = (int)begin + (tid + u * kReduceThreads) * EPV + Elem<T>::first_equal(v[u], m);
-  }
+  for (int u = kUnroll - 1; u >= 0; --u) acc = Elem<T>::sum_terms(v[u], k2, nml2, acc);
   float s;
   {
     float s0, s1;
@@ -232,25 +245,13 @@ __device__ __forceinline__ Partial reduce_slice(const T* __restrict__ base, int 
     s = s0 + s1;
   }
   if (ntail > 0 && tid == 0) {
-    int tidx = 0x7fffffff;
 #pragma unroll
-    for (int e = EPV - 1; e >= 0; --e) {
-      s += ex2(fmaf(tail[e], k, -ml));  // -inf beyond the tail: adds 0
-      if (e < ntail && tail[e] == m) tidx = (int)begin + nvec * EPV + e;
-    }
-    idx = min(idx, tidx);
+    for (int e = EPV - 1; e >= 0; --e) s += ex2(fmaf(tail[e], k, -ml));  // -inf beyond the tail: adds 0
   }
-  if (m == -INFINITY) idx = 0x7fffffff;
   // fixed order: lanes (butterfly), then warps
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    s += __shfl_xor_sync(0xffffffffu, s, off);
-    idx = min(idx, __shfl_xor_sync(0xffffffffu, idx, off));
-  }
-  if (lane == 0) {
-    warp_s[warp] = s;
-    if (idx != 0x7fffffff) atomicMin(&slice_idx, idx);
-  }
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if (lane == 0) warp_s[warp] = s;
   __syncthreads();
   Partial r = {m, s, 0, tag};
   if (tid == 0) {

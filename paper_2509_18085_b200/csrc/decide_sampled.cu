@@ -91,7 +91,7 @@ __device__ __forceinline__ void merge_t(float& m, float& s, float m2, float s2, 
 // grid = (splits, B*N*L); one CTA reduces one vocabulary slice of one row and
 // the first CTA of row i clears node i's arrival counter for the select kernel.
 template <typename T>
-__global__ void __launch_bounds__(kReduceThreads, 8)
+__global__ void __launch_bounds__(kReduceThreads, 9)
 decide_sampled_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V, int64_t chunk,
                              int splits, int nodes, const int32_t* __restrict__ block_tokens, int mask_id,
                              float k, Partial* __restrict__ partials, int* __restrict__ node_count,
