@@ -111,6 +111,8 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // uniform to the compiler
   const int rank = (int)(blockIdx.x & 1);  // x_split is even
+  const int unit = ((int)blockIdx.x - (which ? problems.x_split : 0)) >> 1;
+  if (no_such_tile<NP>(p, unit)) return;  // both CTAs
   // Set-up, by warps side by side: what comes before the first copy is on the path of a call whose
   // CTAs find no room beside the call before.
   if (warp == 1) {
@@ -140,9 +142,8 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
   cluster_arrive_relaxed();  // this warp's part is done: both CTAs' barriers and tensor memory exist when all are here
 
   // the pair's rows and key tiles
-  const int mt = ((int)blockIdx.x - (which ? problems.x_split : 0)) >> 1;
-  const int g = blockIdx.y, b = blockIdx.z;
-  const int nl0 = mt * p.TNL;
+  const Place place = place_of<NP>(p, unit);
+  const int nl0 = place.mt * p.TNL, g = place.g, b = place.b;
   const int nl_count = min(p.TNL, p.NL - nl0);
   const int tnl = p.TNL >> 1;          // of this CTA
   const int nl_cta = nl0 + rank * tnl;
@@ -509,16 +510,15 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
 }  // namespace
 
 template <int NP>
-spiffy_status launch_attention_pair(const Problems<NP>& pr, int ctas_x, cudaStream_t stream) {
+spiffy_status launch_attention_pair(const Problems<NP>& pr, dim3 grid, cudaStream_t stream) {
   static std::atomic<bool> allowed[64];
   if (!allow_smem(graph_attention_pair_kernel<NP>, kSmemBytes, allowed)) return SPIFFY_ECUDA;
   const cudaError_t e =
-      launch_pdl(graph_attention_pair_kernel<NP>, dim3((unsigned)ctas_x, (unsigned)pr.p[0].Hkv, (unsigned)pr.p[0].B),
-                 dim3(kThreads), (size_t)kSmemBytes, stream, pr);
+      launch_pdl(graph_attention_pair_kernel<NP>, grid, dim3(kThreads), (size_t)kSmemBytes, stream, pr);
   count_launch();
   return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
 }
-template spiffy_status launch_attention_pair<1>(const Problems<1>&, int, cudaStream_t);
-template spiffy_status launch_attention_pair<2>(const Problems<2>&, int, cudaStream_t);
+template spiffy_status launch_attention_pair<1>(const Problems<1>&, dim3, cudaStream_t);
+template spiffy_status launch_attention_pair<2>(const Problems<2>&, dim3, cudaStream_t);
 
 }  // namespace spiffy

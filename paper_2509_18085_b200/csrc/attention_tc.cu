@@ -54,7 +54,7 @@
 // loops that are not the inner ones stay rolled (a kernel of 87 KB instead of 60
 // cost 2 us of 19 at 9 units).
 // With few CTAs the key tiles of an M-tile are split over the 2, 4 or 8 CTAs of a
-// cluster (grid.z).  Each finishes its share of the rows: it sends its partial of
+// cluster.  Each finishes its share of the rows: it sends its partial of
 // the others' rows into their shared memory, one bulk copy each, and merges what it
 // gets.
 //
@@ -209,6 +209,8 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
   const Params& p = problems.p[which];
   const int log_cs = NQ == 1 ? p.log_cs : 0, cs = 1 << log_cs;
   const int rank = NQ == 1 ? (int)blockIdx.x & (cs - 1) : 0;  // of this CTA in its cluster
+  const int unit = (((int)blockIdx.x - (which ? problems.x_split : 0)) >> log_cs) * NQ;  // the first of this CTA's M-tiles
+  if (no_such_tile<NP>(p, unit)) return;
   // Set-up, by warps side by side.
   if (warp == 0) {
     // one lane per barrier: a thread's initialisations are served one after the other
@@ -230,11 +232,9 @@ graph_attention_tc_kernel(const __grid_constant__ Problems<NP> problems) {
     prefetch_tensormap(p.TP1 > 0 ? &maps.vp : (p.TP > 0 ? &maps.vp2 : &maps.vb));
   }
   __syncwarp();
-  const int mt = (((int)blockIdx.x - (which ? problems.x_split : 0)) >> log_cs) * NQ;  // first M-tile of this CTA
-  const int g = blockIdx.y, b = blockIdx.z;
-
   // this CTA's rows and key tiles
-  const int nl0 = mt * p.TNL;
+  const Place place = place_of<NP>(p, unit);
+  const int nl0 = place.mt * p.TNL, g = place.g, b = place.b;
   const int nl_count = min(NQ * p.TNL, p.NL - nl0);  // over all M-tiles of the CTA
   const int rows_box = p.TNL * p.group;        // rows one Q box writes
   const int n_lo = nl0 / p.L, n_hi = (nl0 + nl_count - 1) / p.L;
@@ -697,6 +697,10 @@ struct Plan {
   int nq;     // M-tiles per CTA
   int cs;     // CTAs of a cluster that share an M-tile's key tiles (nq = 1)
   bool pair;  // a pair of CTAs per M-tile instead (attention_pair.cu)
+  // nq = 2: rounds that are full; what is left goes into a second launch, with one M-tile per CTA or
+  // pair.  0: one launch.
+  int full_rounds;
+  bool rest_by_pairs;
 };
 
 template <int NP>
@@ -741,44 +745,54 @@ int resident_clusters(int hd, int cs) {
 
 // One or two M-tiles per CTA, and how many CTAs share the key tiles of an M-tile:
 // whatever a model of the kernel's time finds cheapest.  A round of CTAs (each holds its
-// SM) takes 7 us plus, per key tile, 0.85 us with one M-tile and 1.6 with two; at head
-// dimension 64, where the second product has two terms, 0.95 and 1.9.  Handing the
+// SM) takes 6.6 us plus 0.88 per key tile with one M-tile, 8 us plus 1.75 with two; at head
+// dimension 64, where the second product has two terms, 4.9 and 0.93, 6 and 1.8.  Handing the
 // partials around a cluster costs about 2 us (1.5 with rows half as long), so that a second
-// CTA pays from about six key tiles.  The model is there to choose: of 35 shapes (1 to 1088
-// M-tiles, 2 to 33 key tiles), each timed with every plan it allows, it takes the fastest,
-// or one within 2 % of it, at both head dimensions.  The times themselves are 10 % low for
-// long calls of several rounds at 128: 4 x 32 x 32 positions x 32 heads over 4096 keys, 239 us
-// for two M-tiles a CTA and 245 for one, measured 265 and 273 back to back on the same
-// inputs; at 64, 279 and 268, measured 276 and 263.
-// A pair of CTAs per M-tile (head dimension 128, at most 64 query heads on a key/value head) takes 5.3 us and
-// 0.44 per key tile, a round: 8 x 32 positions x 32 heads over 512 + 32 keys 7.5 us (one CTA a tile 10.3),
-// 64 x 4 x 32 heads on 8 over 2048 12.8 (clusters of two 17.0).  One round only pays: 2 x 11 x 24 x 16
-// heads over 450 13.9 (11.3), and with more key tiles than some 20 clusters of eight are sooner done.
+// CTA pays from about six key tiles.  (16 x 32 positions x 32 heads, one M-tile: 11.0, 21.8 and 36.0 us
+// over 512, 2048 and 4096 keys; 32 x 32 positions, two: 16.6, 37.3 and 68.2.)
+// A pair of CTAs per M-tile (head dimension 128, at most 64 query heads on a key/value head) takes 5 us and
+// 0.46 per key tile, a round: 8 x 32 positions x 32 heads over 512 + 32 keys 7.3 us (one CTA a tile 9.7),
+// 64 x 4 x 32 heads on 8 over 2048 12.8 (clusters of two 15.6).  One round only pays: 2 x 11 x 24 x 16
+// heads over 450 13.9 (10.3), and with more key tiles than some 20 clusters of eight are sooner done.
+// A call of several rounds whose last one half fills the SMs or less does that one in half the time by a
+// second launch, with one M-tile per CTA or pair: 4 x 32 x 32 positions x 32 heads over 4096 keys, three
+// rounds and 136 M-tiles instead of four rounds, 253 -> 243 us (289 -> 278 under the power limit, which
+// gives an idle SM's share to the others); 2 x 44 x 32 positions x 32 heads on 16 over 1000 62.9 -> 57.5.
 // `tiles` counts the M-tiles of all problems of the launch, `doubles` the CTAs that take two
 // of them, `pair_tiles` the pairs (0: not possible); T is the key tiles of the longer problem.
-Plan make_plan(int64_t tiles, int64_t doubles, int64_t pair_tiles, int T, int hd) {
+// `may_split`: the call may be two launches; `same_tiles`: a pair's M-tiles are one CTA's.
+Plan make_plan(int64_t tiles, int64_t doubles, int64_t pair_tiles, int T, int hd, bool may_split, bool same_tiles) {
   const int sms = sm_count();
-  const float one = hd == 128 ? 0.85f : 0.95f, two = hd == 128 ? 1.6f : 1.9f;
+  const float one0 = hd == 128 ? 6.6f : 4.9f, one = hd == 128 ? 0.88f : 0.93f;
+  const float two0 = hd == 128 ? 8.0f : 6.0f, two = hd == 128 ? 1.75f : 1.8f;
+  const float pair = 5.0f + 0.46f * (float)T;
   auto rounds = [&](int64_t ctas) { return (float)((ctas + sms - 1) / sms); };
-  Plan pl = {2, 1, false};
+  Plan pl = {2, 1, false, 0, false};
   if (sms <= 0) return pl;
-  float best = rounds(doubles) * (7.0f + two * (float)T);
+  float best = rounds(doubles) * (two0 + two * (float)T);
   if (pair_tiles > 0) {
-    const float cost = rounds(2 * pair_tiles) * (5.3f + 0.44f * (float)T);
+    const float cost = rounds(2 * pair_tiles) * pair;
     if (cost < best) {
       best = cost;
-      pl = {1, 1, true};
+      pl = {1, 1, true, 0, false};
     }
   }
   for (int cs = 1; cs <= 8 && cs <= T; cs *= 2) {
     // clusters only where all of them run at once
     if (cs > 1 && (tiles * cs > sms || tiles > resident_clusters(hd, cs))) continue;
     const float exchange = cs == 1 ? 0.f : (hd == 128 ? 1.9f : 1.4f) + 0.07f * (float)cs;
-    const float cost = rounds(tiles * cs) * (7.0f + exchange + one * (float)((T + cs - 1) / cs));
+    const float cost = rounds(tiles * cs) * (one0 + exchange + one * (float)((T + cs - 1) / cs));
     if (cost < best) {
       best = cost;
-      pl = {1, cs, false};
+      pl = {1, cs, false, 0, false};
     }
+  }
+  // A last round that half fills the SMs or less is done in half the time with one M-tile per CTA.
+  const int64_t full = doubles / sms, left = doubles - full * sms;
+  if (may_split && full > 0 && left > 0 && 2 * left <= sms) {
+    const bool by_pairs = pair_tiles > 0 && same_tiles && 4 * left <= sms;
+    const float rest = by_pairs ? pair : one0 + one * (float)T;
+    if ((float)full * (two0 + two * (float)T) + rest < best) pl = {2, 1, false, (int)full, by_pairs};
   }
   return pl;
 }
@@ -819,6 +833,45 @@ bool make_problem(const spiffy_attn_desc& d, const Shape& sh, const AttnProblem&
   return ok;
 }
 
+// One launch: of the whole call (grid.x = 0: as many CTAs as it takes), or of `grid.x` CTAs from
+// M-tile `first` on.  `flags` come on top of the caller's.
+template <int NP>
+spiffy_status launch_part(const spiffy_attn_desc* const (&d)[NP], const AttnProblem* const (&a)[NP], const Shape (&sh)[NP],
+                          const Plan& pl, dim3 grid, int first, int slots, int flags, int32_t* dev_status,
+                          cudaStream_t stream) {
+  Problems<NP> pr;
+  unsigned x = 0;
+  for (int i = 0; i < NP; ++i) {
+    Params& p = pr.p[i];
+    if (!make_problem(*d[i], sh[i], *a[i], &pr.maps[i], &p, pl, dev_status)) return SPIFFY_ECUDA;
+    p.first = first;
+    p.slots = slots;
+    if (flags & SPIFFY_ATTN_EARLY_DEPENDENTS) p.early_trigger = 1;
+    if (flags & SPIFFY_ATTN_INDEPENDENT) p.independent = 1;
+    if (i == 1) pr.x_split = (int)x;
+    x += pl.pair ? 2 * sh[i].MT : (sh[i].MT + pl.nq - 1) / pl.nq * pl.cs;
+  }
+  if (grid.x == 0) grid.x = x;
+  if (pl.pair) return launch_attention_pair<NP>(pr, grid, stream);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;  // only when asked for
+  attr[1].val.clusterDim.x = (unsigned)pl.cs;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pl.cs > 1 ? 2 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel_of<NP>(d[0]->head_dim, pl.nq), pr);
+  count_launch();
+  return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
+}
+
 template <int NP>
 spiffy_status launch(const spiffy_attn_desc* const (&d)[NP], const AttnProblem* const (&a)[NP], int32_t* dev_status,
                      cudaStream_t stream) {
@@ -846,33 +899,20 @@ spiffy_status launch(const spiffy_attn_desc* const (&d)[NP], const AttnProblem* 
     }
     T = sh[i].T > T ? sh[i].T : T;
   }
-  const Plan pl = make_plan(tiles, doubles, pair_tiles, T, hd);
-  Problems<NP> pr;
-  int x = 0;
-  for (int i = 0; i < NP; ++i) {
-    if (pl.pair) sh[i] = by_pairs[i];
-    if (!make_problem(*d[i], sh[i], *a[i], &pr.maps[i], &pr.p[i], pl, dev_status)) return SPIFFY_ECUDA;
-    if (i == 1) pr.x_split = x;
-    x += pl.pair ? 2 * sh[i].MT : (sh[i].MT + pl.nq - 1) / pl.nq * pl.cs;
-  }
-  if (pl.pair) return launch_attention_pair<NP>(pr, x, stream);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)x, (unsigned)d[0]->n_kv_heads, (unsigned)d[0]->batch);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;  // only when asked for
-  attr[1].val.clusterDim.x = (unsigned)pl.cs;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pl.cs > 1 ? 2 : 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel_of<NP>(hd, pl.nq), pr);
-  count_launch();
-  return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
+  const bool split = NP == 1 && bg * (sh[0].MT + 1) < (1 << 30);
+  const Plan pl = make_plan(tiles, doubles, pair_tiles, T, hd, split, by_pairs[0].TNL == sh[0].TNL);
+  const dim3 grid(0, (unsigned)d[0]->n_kv_heads, (unsigned)d[0]->batch);
+  if (pl.full_rounds == 0) return launch_part(d, a, pl.pair ? by_pairs : sh, pl, grid, 0, 0, 0, dev_status, stream);
+  // Full rounds first, which let the rest begin as they end; the rest reads nothing of theirs, and is
+  // complete no sooner.
+  const int slots = (sh[0].MT + 1) / 2 * 2, first = pl.full_rounds * sm_count() * 2;
+  const int rest = (int)bg * slots - first;
+  const spiffy_status st = launch_part(d, a, sh, pl, dim3((unsigned)first / 2), 0, slots, SPIFFY_ATTN_EARLY_DEPENDENTS,
+                                       dev_status, stream);
+  if (st != SPIFFY_OK) return st;
+  const Plan one = {1, 1, pl.rest_by_pairs, 0, false};
+  return launch_part(d, a, one.pair ? by_pairs : sh, one, dim3((unsigned)(one.pair ? 2 * rest : rest)), first, slots,
+                     SPIFFY_ATTN_INDEPENDENT, dev_status, stream);
 }
 
 }  // namespace

@@ -24,6 +24,10 @@ struct Params {
   int NL;       // N * L
   int TP1, TP;  // context key tiles: of the first segment, of both
   int log_cs;   // CTAs of a cluster that share an M-tile's key tiles: 1, 2, 4 or 8
+  // A launch that takes a part of the call only, in one row of CTAs: its first M-tile, counted over all
+  // (sequence, key/value head) pairs at `slots` each (the M-tiles of one, rounded up to even); 0: the
+  // grid's y and z are key/value head and sequence.
+  int first, slots;
   float scale_log2;
   __nv_bfloat16* out;
   int32_t* status;
@@ -44,6 +48,22 @@ struct Problems {
   Params p[NP];
   int x_split;
 };
+
+// Which M-tile, head and sequence: `unit` is the M-tile among those of the CTA's row of the grid.
+struct Place {
+  int mt, g, b;
+};
+// (Two problems are one launch always: spared the look, 2 % of a short call.)
+template <int NP>
+__device__ __forceinline__ Place place_of(const Params& p, int unit) {
+  if (NP == 2 || p.slots == 0) return {unit, (int)blockIdx.y, (int)blockIdx.z};
+  const int at = p.first + unit, bg = at / p.slots;
+  return {at - bg * p.slots, bg % p.Hkv, bg / p.Hkv};
+}
+template <int NP>
+__device__ __forceinline__ bool no_such_tile(const Params& p, int unit) {
+  return NP == 1 && p.slots != 0 && (p.first + unit) % p.slots * p.TNL >= p.NL;
+}
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   uint32_t r;
@@ -80,8 +100,8 @@ __device__ __forceinline__ Window visible_window(const Params& p, int t, int kb_
   return w;
 }
 
-// attention_pair.cu: `ctas_x` CTAs per key/value head and sequence.
+// attention_pair.cu: `grid` CTAs, two neighbouring ones to an M-tile.
 template <int NP>
-spiffy_status launch_attention_pair(const Problems<NP>& pr, int ctas_x, cudaStream_t stream);
+spiffy_status launch_attention_pair(const Problems<NP>& pr, dim3 grid, cudaStream_t stream);
 
 }  // namespace spiffy

@@ -46,3 +46,18 @@ def test_late_maximum_in_another_slice():
     got = G.gpu_attention(w, spiffy.ATTN_TCGEN05)
     want = oracle.graph_attention(w.q, w.k_prefix, w.v_prefix, w.k_block, w.v_block)
     assert np.all(np.isfinite(got)) and np.max(np.abs(got - want)) <= G.TOL["bf16"]
+
+
+@pytest.mark.parametrize("B,N,L,P,Hq,Hkv", [
+    (5, 8, 25, 100, 64, 64),    # 320 CTAs of two M-tiles: 24 of them, beyond two rounds, by pairs of blocks
+    (4, 7, 20, 40, 89, 89),     # 356: 60 of them with one M-tile per block
+    (2, 10, 30, 50, 90, 90),    # ... three M-tiles a head: every fourth block of the second launch has none
+    (3, 5, 60, 20, 330, 110)])  # groups of three query heads
+def test_last_round_in_a_launch_of_its_own(B, N, L, P, Hq, Hkv):
+    cfg = W.Config("splits", B, N, L, P, Hq, Hkv, 128, "bf16", 16, 0)
+    w = W.make(cfg, 17 + P, decision=False)
+    got = G.gpu_attention(w, spiffy.ATTN_TCGEN05)
+    want = oracle.graph_attention(w.q, w.k_prefix, w.v_prefix, w.k_block, w.v_block)
+    assert np.max(np.abs(got - want)) <= G.TOL["bf16"]
+    assert np.sqrt(np.mean((got - want) ** 2)) < 4e-3
+    assert np.array_equal(got, G.gpu_attention(w, spiffy.ATTN_TCGEN05))
