@@ -1,4 +1,4 @@
-// Packed draft-graph attention by pairs of CTAs: bf16, head dimension 128, calls whose key
+// Packed draft-graph attention by pairs of CTAs: bf16, head dimension 128 or 64, calls whose key
 // tiles need no splitting over more CTAs.  The mathematics, the order of the key tiles and the
 // mask are those of attention_tc.cu; what differs is who holds what.
 //
@@ -18,6 +18,8 @@
 // P goes through shared memory (an A operand of this shape would have to be in tensor memory
 // twice), over the K tile that its scores came from, which nobody reads any more.  A stage of
 // the ring is therefore K and V together, free again when P V is done.
+// At head dimension 64 P is two terms (attention_tc.cu says why), four times a K tile, and has a
+// place of its own for each warpgroup; a CTA's half of V is 32 columns, rows of 64 bytes.
 //
 //   warp 0, 3   TMA producers of Q and K, and of V (both CTAs; bytes count on the leader's barriers)
 //   warp 1      tensor memory; the leader's issues S = Q K^T
@@ -32,7 +34,8 @@
 // warpgroups and barriers' arrivals across the pair with release semantics at cluster scope (500
 // cycles and more each); 9.5 without; 9.1 four warpgroups; 8.1 issuing warps converged instead of one
 // lane; 7.5 set-up side by side by warps, no division in the producers' loops.  The kernel
-// of attention_tc.cu takes 10.3.  Per further key tile 0.44 us (0.85 there).  Tried and dropped: two
+// of attention_tc.cu took 10.3 then (9.7 now).  Per further key tile 0.45 us (0.88 there).  At head
+// dimension 64 7.1 us (9.3 there) and 0.69 (0.93).  Tried and dropped: two
 // CTAs of two warpgroups on an SM (10.6), references other than the maximum (nothing to exchange at
 // the first tile, 0.5 us; but the largest weight is then no longer exact, and the error 4 % larger).
 //
@@ -48,13 +51,21 @@ constexpr int kThreads = 128 * (1 + NW), kSoftmax = 128 * NW;
 // 96 registers a thread at launch; the softmax warps take over what the others do not need.
 constexpr int kRegsIssue = 32, kRegsSoftmax = 104;
 static_assert(kRegsIssue + NW * kRegsSoftmax <= (1 + NW) * 96, "within what the block was launched with");
-constexpr int HD = 128;
-constexpr int kRows = 64;              // of a CTA
-constexpr int kTile = kRows * HD * 2;  // a CTA's share of Q, K, V or P
-constexpr int kHalf = kTile / 2;       // 64 rows of 128 bytes
-constexpr int kStages = 6;
-// Tensor memory: warpgroup w has its scores at 64 w and its accumulator at 256 + 64 w.
+constexpr int kRows = 64;           // of a CTA
+constexpr int kHalf = kRows * 128;  // 64 rows of 128 bytes
+constexpr int kMaxStages = 6;
+// Tensor memory: warpgroup w has its scores at 64 w and its accumulator at 256 + (head dimension / 2) w.
 constexpr uint32_t kTmemCols = 512, kColS = 0, kColO = 64 * NW;
+// Shared memory: Q | P of each warpgroup, where it does not go over K | the ring, stage s: K at 2 s, V at
+// 2 s + 1 | Tail.
+template <int HD>
+struct Smem {
+  static constexpr int tile = kRows * HD * 2;               // a CTA's share of Q, K or V
+  static constexpr int p = HD == 64 ? 4 * kHalf : 0;        // two terms of 128 keys
+  static constexpr int stages = HD == 64 ? 5 : kMaxStages;
+  static constexpr int ring = tile + NW * p;
+  static constexpr int tail = ring + 2 * stages * tile;
+};
 
 struct Bars {
   uint64_t q_full;
@@ -63,8 +74,8 @@ struct Bars {
   uint64_t s_free[NW];      // ... and read (leader)
   uint64_t p_ready[NW];     // P written (leader)
   uint64_t pv_done[NW];     // ... and used (both)
-  uint64_t k_full[kStages], v_full[kStages];  // both CTAs' halves have landed (leader)
-  uint64_t stage_free[kStages];               // (both)
+  uint64_t k_full[kMaxStages], v_full[kMaxStages];  // both CTAs' halves have landed (leader)
+  uint64_t stage_free[kMaxStages];               // (both)
 };
 struct Tail {  // behind the tiles in shared memory
   Bars bars;
@@ -75,8 +86,10 @@ struct Tail {  // behind the tiles in shared memory
   int abort_flag;
   int issued_k, issued_v;         // by this CTA's producers
 };
-constexpr int kSmemBytes = (1 + 2 * kStages) * kTile + (int)sizeof(Tail);
-static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
+template <int HD>
+constexpr int kSmemBytes = Smem<HD>::tail + (int)sizeof(Tail);
+// (two CTAs must not share an SM: each holds all of its tensor memory until it exits)
+static_assert(kSmemBytes<64> <= 227 * 1024 && kSmemBytes<128> <= 227 * 1024 && kSmemBytes<64> > 114 * 1024, "one CTA");
 
 // Is `mine` true for any thread of the two warps that meet at this barrier?
 __device__ __forceinline__ bool any_of_two_warps(int barrier, bool mine) {
@@ -96,16 +109,20 @@ __device__ __forceinline__ bool any_of_two_warps(int barrier, bool mine) {
 constexpr int kBarSoftmax = 1, kBarProducers = 2, kBarTwoWarps = 3;  // 3 .. 10
 constexpr int kHeadStart = 2;  // K tiles that are asked for before the first V tile
 
-template <int NP>
+template <int HD, int NP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const int which = NP == 2 && (int)blockIdx.x >= problems.x_split ? 1 : 0;
   const Maps& maps = problems.maps[which];
   const Params& p = problems.p[which];
+  using SM = Smem<HD>;
+  constexpr int kTile = SM::tile, kStages = SM::stages, kHalves = HD / 64;
+  constexpr bool kRest = HD == 64;  // P in two bf16 terms, as in attention_tc.cu
+  constexpr int kColsO = HD / 2;    // columns of an accumulator: half of the head dimension
   uint8_t* sq = smem;
-  uint8_t* ring = smem + kTile;  // stage s: K, later P, at 2 s; V at 2 s + 1
-  Tail& tail = *reinterpret_cast<Tail*>(ring + kStages * 2 * kTile);
+  uint8_t* ring = smem + SM::ring;
+  Tail& tail = *reinterpret_cast<Tail*>(smem + SM::tail);
   Bars& bars = tail.bars;
   volatile int* abort_flag = &tail.abort_flag;
 
@@ -154,8 +171,8 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
   // rows of the Q tile that the TMA box does not write must be finite
   for (int i = rows_box * 8 + threadIdx.x; i < kRows * 8; i += kThreads) {
     const uint4 z = make_uint4(0, 0, 0, 0);
-    reinterpret_cast<uint4*>(sq)[i] = z;
-    reinterpret_cast<uint4*>(sq + kHalf)[i] = z;
+#pragma unroll
+    for (int h = 0; h < kHalves; ++h) reinterpret_cast<uint4*>(sq + h * kHalf)[i] = z;
   }
   fence_proxy_async_smem();
   __syncthreads();
@@ -189,9 +206,9 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
       const bool is_k = warp == 0;
       if (is_k) {
         const uint32_t bar = map_to_cta(smem_u32(&bars.q_full), 0);
-        if (rank == 0) mbar_arrive_expect_tx(&bars.q_full, 4u * rows_box * 128u);
+        if (rank == 0) mbar_arrive_expect_tx(&bars.q_full, 2u * kHalves * rows_box * 128u);
 #pragma unroll
-        for (int h = 0; h < 2; ++h)  // rows beyond the last one read as zeros
+        for (int h = 0; h < kHalves; ++h)  // rows beyond the last one read as zeros
           tma_load_5d_pair(sq + h * kHalf, &maps.q, bar, 0, g * p.group, nl_cta, h, b);
       }
       // Key tiles in order: first context segment, second context segment, block keys.  Everything is
@@ -241,8 +258,9 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
         if (ok && t >= NW) ok = wait(&bars.s_free[t % NW], (uint32_t)(t / NW - 1) & 1u);
         if (!ok) break;
         tc_fence_after_sync();
-        umma_pair_kk_k128(tmem + kColS + (uint32_t)(t % NW) * 64u, q_lo, k_lo + (uint32_t)stage * (2 * kTile >> 4), hi,
-                          idesc, 0u);
+        const uint32_t d = tmem + kColS + (uint32_t)(t % NW) * 64u, k_at = k_lo + (uint32_t)stage * (2 * kTile >> 4);
+        if constexpr (HD == 128) umma_pair_kk_k128(d, q_lo, k_at, hi, idesc, 0u);
+        else umma_pair_kk_k64(d, q_lo, k_at, hi, hi, idesc, 0u);
         umma_commit_both(&bars.s_full[t % NW]);
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
@@ -252,7 +270,7 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
       // --------------------------------------------------- issuer of O += P V --
       constexpr uint32_t idesc = idesc_bf16_f32(BM, HD, false, true);
       constexpr uint32_t hi = desc_hi_sw128(1024);
-      const uint32_t p_lo = desc_lo_sw128(smem_u32(ring), 16);
+      const uint32_t p_lo = desc_lo_sw128(smem_u32(kRest ? smem + kTile : ring), 16);
       const uint32_t v_lo = desc_lo_sw128(smem_u32(ring + kTile), kHalf);
       int stage = 0;
       uint32_t phase = 0;
@@ -260,8 +278,15 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
         if (!wait(&bars.v_full[stage], phase)) break;
         if (!wait(&bars.p_ready[t % NW], (uint32_t)(t / NW) & 1u)) break;
         tc_fence_after_sync();
-        umma_pair_kn_k128(tmem + kColO + (uint32_t)(t % NW) * 64u, p_lo + (uint32_t)stage * (2 * kTile >> 4),
-                          v_lo + (uint32_t)stage * (2 * kTile >> 4), hi, idesc, t >= NW ? 1u : 0u);
+        const uint32_t d = tmem + kColO + (uint32_t)(t % NW) * kColsO, v_at = v_lo + (uint32_t)stage * (2 * kTile >> 4);
+        if constexpr (kRest) {
+          constexpr uint32_t v_hi = desc_hi_sw64(512);
+          const uint32_t p_at = p_lo + (uint32_t)(t % NW) * (SM::p >> 4);
+          umma_pair_kn32_k128(d, p_at, v_at, hi, v_hi, idesc, t >= NW ? 1u : 0u);
+          umma_pair_kn32_k128(d, p_at + (SM::p / 2 >> 4), v_at, hi, v_hi, idesc, 1u);
+        } else {
+          umma_pair_kn_k128(d, p_lo + (uint32_t)stage * (2 * kTile >> 4), v_at, hi, idesc, t >= NW ? 1u : 0u);
+        }
         umma_commit_both(&bars.pv_done[t % NW]);
         if (t + kStages < T) umma_commit_both(&bars.stage_free[stage]);
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
@@ -288,7 +313,7 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
     int turn = 0;
     bool ok = true;
     const uint32_t at_s = tmem_addr(tmem, lane_base, kColS + (uint32_t)wg * 64u);
-    const uint32_t at_o = tmem_addr(tmem, lane_base, kColO + (uint32_t)wg * 64u);
+    const uint32_t at_o = tmem_addr(tmem, lane_base, kColO + (uint32_t)wg * kColsO);
     const uint32_t s_free = map_to_cta(smem_u32(&bars.s_free[wg]), 0), p_ready = map_to_cta(smem_u32(&bars.p_ready[wg]), 0);
     // the P V products of key tile t (one of this warpgroup's) have completed
     auto wait_pv = [&](int t) -> bool {
@@ -342,7 +367,8 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
         }
         mx = fmaxf(m0, m1) * k2;
       }
-      uint8_t* p_row = ring + 2 * stage * kTile + half * kHalf + row * 128;  // where K was, read for the last time
+      // over K, read for the last time, or where the products that read it last are done
+      uint8_t* p_row = (kRest ? smem + kTile + wg * SM::p : ring + 2 * stage * kTile) + half * kHalf + row * 128;
       stage += NW;
       if (stage >= kStages) stage -= kStages;
       // The two halves of a row agree on its maximum (by turns in two places, so that nobody writes
@@ -365,7 +391,7 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
         }
         if (t >= NW) {  // the accumulator holds earlier tiles, whose products are done
 #pragma unroll 1
-          for (uint32_t c0 = 0; c0 < 64; c0 += 16) {
+          for (uint32_t c0 = 0; c0 < kColsO; c0 += 16) {
             uint32_t o[16];
             tmem_ld_async(at_o + c0, o);
             tmem_wait_ld();
@@ -383,25 +409,42 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
       uint64_t sum_a = pack2(0.f, 0.f), sum_b = pack2(0.f, 0.f);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        uint32_t pk[16];
+        auto store = [&](int c, const uint32_t (&pk)[4], const uint32_t (&rest)[4]) {
+          uint8_t* at = p_row + (((4 * h + c / 8) ^ (row & 7)) << 4);
+          *reinterpret_cast<uint4*>(at) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+          if constexpr (kRest) *reinterpret_cast<uint4*>(at + SM::p / 2) = make_uint4(rest[0], rest[1], rest[2], rest[3]);
+        };
         if ((chunks >> h) & 1u) {
 #pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            const uint64_t x2 = fma2(pack2(__uint_as_float(s[h][c]), __uint_as_float(s[h][c + 1])), k22, nm2);
-            float x0, x1;
-            unpack2(x2, x0, x1);
-            const float p0 = ex2(x0), p1 = ex2(x1);
-            if ((c >> 1) & 1) sum_b = add2(sum_b, pack2(p0, p1)); else sum_a = add2(sum_a, pack2(p0, p1));
-            pk[c >> 1] = pack_bf16(p0, p1);
+          for (int c = 0; c < 32; c += 8) {
+            uint32_t pk[4], rest[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const uint64_t x2 =
+                  fma2(pack2(__uint_as_float(s[h][c + 2 * e]), __uint_as_float(s[h][c + 2 * e + 1])), k22, nm2);
+              float x0, x1;
+              unpack2(x2, x0, x1);
+              const float p0 = ex2(x0), p1 = ex2(x1);
+              if (e & 1) sum_b = add2(sum_b, pack2(p0, p1)); else sum_a = add2(sum_a, pack2(p0, p1));
+              if constexpr (kRest) {  // cut off instead of rounded: a byte permutation, no conversion
+                const uint32_t w0 = __float_as_uint(p0), w1 = __float_as_uint(p1);
+                pk[e] = __byte_perm(w0, w1, 0x7632);
+                float r0, r1;
+                unpack2(fma2(pack2(__uint_as_float(w0 & 0xffff0000u), __uint_as_float(w1 & 0xffff0000u)), pack2(-1.f, -1.f),
+                             pack2(p0, p1)), r0, r1);
+                rest[e] = pack_bf16(r0, r1);
+              } else {
+                pk[e] = pack_bf16(p0, p1);
+                rest[e] = 0u;
+              }
+            }
+            store(c, pk, rest);
           }
         } else {
+          const uint32_t zero[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-          for (int c = 0; c < 16; ++c) pk[c] = 0u;
+          for (int c = 0; c < 32; c += 8) store(c, zero, zero);
         }
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          *reinterpret_cast<uint4*>(p_row + (((4 * h + c) ^ (row & 7)) << 4)) =
-              make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
       }
       float a0, a1;
       unpack2(add2(sum_a, sum_b), a0, a1);
@@ -419,11 +462,11 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
     tc_fence_before_sync();
     asm volatile("bar.sync %0, %1;" ::"n"(kBarSoftmax), "n"(kSoftmax) : "memory");  // all of them, whatever `ok` says
     tc_fence_after_sync();
-    constexpr int kCols = 64 / NW;
+    constexpr int kCols = kColsO / NW;
     uint32_t o[NW][kCols];
     if (ok) {
 #pragma unroll
-      for (int w = 0; w < NW; ++w) tmem_ld_async(tmem_addr(tmem, lane_base, kColO + 64u * w + (uint32_t)(wg * kCols)), o[w]);
+      for (int w = 0; w < NW; ++w) tmem_ld_async(tmem_addr(tmem, lane_base, kColO + (uint32_t)(kColsO * w + wg * kCols)), o[w]);
       tmem_wait_ld();
 #pragma unroll
       for (int w = 0; w < NW; ++w) tmem_loaded(o[w]);
@@ -464,17 +507,18 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
           }
           pk[e] = pack_bf16(x, y);
         }
-        *reinterpret_cast<uint4*>(out_row + (((half * 8 + (wg * kCols + c) / 8) ^ (row & 7)) << 4)) =
+        *reinterpret_cast<uint4*>(out_row + (((half * (kColsO / 8) + (wg * kCols + c) / 8) ^ (row & 7)) << 4)) =
             make_uint4(pk[0], pk[1], pk[2], pk[3]);
       }
     }
     asm volatile("bar.sync %0, %1;" ::"n"(kBarSoftmax), "n"(kSoftmax) : "memory");
     if (!*abort_flag) {
-      const int tid = (int)threadIdx.x - 128, row0 = tid / 16, chunk = tid % 16;
+      constexpr int kChunks = HD / 8, kStep = kSoftmax / kChunks;  // 16-byte chunks of a row, rows per pass
+      const int tid = (int)threadIdx.x - 128, row0 = tid / kChunks, chunk = tid % kChunks;
       __nv_bfloat16* out = p.out + (((int64_t)b * p.NL + nl_cta) * p.Hq + (int64_t)g * p.group) * HD + chunk * 8;
 #pragma unroll
-      for (int k = 0; k < kRows / (kSoftmax / 16); ++k) {
-        const int r = row0 + (kSoftmax / 16) * k, at = tail.rows[r];
+      for (int k = 0; k < kRows / kStep; ++k) {
+        const int r = row0 + kStep * k, at = tail.rows[r];
         const uint4 w = *reinterpret_cast<const uint4*>(sq + r * (HD * 2) + ((chunk ^ (r & 7)) << 4));
         if (at >= 0) st_global(out + at, w);
       }
@@ -510,15 +554,19 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
 }  // namespace
 
 template <int NP>
-spiffy_status launch_attention_pair(const Problems<NP>& pr, dim3 grid, cudaStream_t stream) {
-  static std::atomic<bool> allowed[64];
-  if (!allow_smem(graph_attention_pair_kernel<NP>, kSmemBytes, allowed)) return SPIFFY_ECUDA;
-  const cudaError_t e =
-      launch_pdl(graph_attention_pair_kernel<NP>, grid, dim3(kThreads), (size_t)kSmemBytes, stream, pr);
-  count_launch();
-  return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
+spiffy_status launch_attention_pair(const Problems<NP>& pr, int head_dim, dim3 grid, cudaStream_t stream) {
+  static std::atomic<bool> allowed[2][64];
+  auto run = [&](auto kernel, int smem, std::atomic<bool>(&done)[64]) {
+    if (!allow_smem(kernel, smem, done)) return SPIFFY_ECUDA;
+    const cudaError_t e = launch_pdl(kernel, grid, dim3(kThreads), (size_t)smem, stream, pr);
+    count_launch();
+    return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
+  };
+  if constexpr (NP == 1)  // the full-sequence call takes head dimension 128 only
+    if (head_dim == 64) return run(graph_attention_pair_kernel<64, NP>, kSmemBytes<64>, allowed[0]);
+  return run(graph_attention_pair_kernel<128, NP>, kSmemBytes<128>, allowed[1]);
 }
-template spiffy_status launch_attention_pair<1>(const Problems<1>&, dim3, cudaStream_t);
-template spiffy_status launch_attention_pair<2>(const Problems<2>&, dim3, cudaStream_t);
+template spiffy_status launch_attention_pair<1>(const Problems<1>&, int, dim3, cudaStream_t);
+template spiffy_status launch_attention_pair<2>(const Problems<2>&, int, dim3, cudaStream_t);
 
 }  // namespace spiffy

@@ -65,8 +65,7 @@
 // narrower O leaves), so that the result's error against float64 is the CUDA cores'
 // (0.166 % in the 2-norm, the rounding of the output, over 50 to 4096 keys; with one
 // term 0.18 to 0.23 %).  The second term costs 5 to 20 % (4 x 32 x 32 positions x 32
-// heads over 4096 keys: 232 -> 262 us; CUDA cores 4596); 3 sequences of 100 positions x
-// 24 heads over 777 + 20 keys: 12.4 us, 11.6 with one term, 89 on the CUDA cores.
+// heads over 4096 keys: 232 -> 262 us when it came; CUDA cores 4596).
 //
 // Every wait is bounded; a wait that gives up raises SPIFFY_DEV_TIMEOUT in the
 // caller's status word and the CTA winds down without touching its output.
@@ -750,10 +749,11 @@ int resident_clusters(int hd, int cs) {
 // partials around a cluster costs about 2 us (1.5 with rows half as long), so that a second
 // CTA pays from about six key tiles.  (16 x 32 positions x 32 heads, one M-tile: 11.0, 21.8 and 36.0 us
 // over 512, 2048 and 4096 keys; 32 x 32 positions, two: 16.6, 37.3 and 68.2.)
-// A pair of CTAs per M-tile (head dimension 128, at most 64 query heads on a key/value head) takes 5 us and
-// 0.46 per key tile, a round: 8 x 32 positions x 32 heads over 512 + 32 keys 7.3 us (one CTA a tile 9.7),
-// 64 x 4 x 32 heads on 8 over 2048 12.8 (clusters of two 15.6).  One round only pays: 2 x 11 x 24 x 16
-// heads over 450 13.9 (10.3), and with more key tiles than some 20 clusters of eight are sooner done.
+// A pair of CTAs per M-tile (at most 64 query heads on a key/value head) takes 5 us and 0.45 per key tile, at
+// head dimension 64 3.7 and 0.69, a round: 8 x 32 positions x 32 heads over 512 + 32 keys 7.3 and 7.1 us (one
+// CTA a tile 9.7 and 9.3), 64 x 4 x 32 heads on 8 over 2048 12.4 (clusters of two 15.6), 3 x 100 positions x
+// 24 heads of 64 on 8 over 777 9.2 (10.4).  One round only pays: 2 x 11 x 24 x 16 heads over 450 13.9 (10.3),
+// and with more key tiles than some 20 (8) clusters of eight are sooner done.
 // A call of several rounds whose last one half fills the SMs or less does that one in half the time by a
 // second launch, with one M-tile per CTA or pair: 4 x 32 x 32 positions x 32 heads over 4096 keys, three
 // rounds and 136 M-tiles instead of four rounds, 253 -> 243 us (289 -> 278 under the power limit, which
@@ -765,7 +765,7 @@ Plan make_plan(int64_t tiles, int64_t doubles, int64_t pair_tiles, int T, int hd
   const int sms = sm_count();
   const float one0 = hd == 128 ? 6.6f : 4.9f, one = hd == 128 ? 0.88f : 0.93f;
   const float two0 = hd == 128 ? 8.0f : 6.0f, two = hd == 128 ? 1.75f : 1.8f;
-  const float pair = 5.0f + 0.46f * (float)T;
+  const float pair = hd == 128 ? 5.0f + 0.45f * (float)T : 3.7f + 0.69f * (float)T;
   auto rounds = [&](int64_t ctas) { return (float)((ctas + sms - 1) / sms); };
   Plan pl = {2, 1, false, 0, false};
   if (sms <= 0) return pl;
@@ -803,8 +803,9 @@ bool make_problem(const spiffy_attn_desc& d, const Shape& sh, const AttnProblem&
   const int ctas = pl.pair ? 2 : 1;  // of a pair, each reads half of the rows, of the keys of K and of the columns of V
   const int64_t bs = a.ctx.batch_stride_rows, bs2 = a.ctx2.batch_stride_rows;
   auto keys = [&](CUtensorMap* map, const void* base, int64_t rows, int64_t stride, bool is_v) {
-    return make_tile_map(map, base, d.n_kv_heads, rows, d.batch, 1, is_v ? BN : BN / ctas, is_v ? halves / ctas : halves,
-                         stride, halves);
+    if (is_v && pl.pair)
+      return make_tile_map(map, base, d.n_kv_heads, rows, d.batch, 1, BN, 1, stride, 2, d.head_dim / 2);
+    return make_tile_map(map, base, d.n_kv_heads, rows, d.batch, 1, BN / ctas, halves, stride, halves);
   };
   bool ok = make_tile_map(&m->q, a.q, d.n_q_heads, sh.NL, d.batch, sh.group, sh.TNL / ctas, 1, 0, halves);
   ok = ok && keys(&m->kb, a.kb, sh.NL, 0, false) && keys(&m->vb, a.vb, sh.NL, 0, true);
@@ -852,7 +853,7 @@ spiffy_status launch_part(const spiffy_attn_desc* const (&d)[NP], const AttnProb
     x += pl.pair ? 2 * sh[i].MT : (sh[i].MT + pl.nq - 1) / pl.nq * pl.cs;
   }
   if (grid.x == 0) grid.x = x;
-  if (pl.pair) return launch_attention_pair<NP>(pr, grid, stream);
+  if (pl.pair) return launch_attention_pair<NP>(pr, d[0]->head_dim, grid, stream);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(kThreads);
@@ -887,7 +888,7 @@ spiffy_status launch(const spiffy_attn_desc* const (&d)[NP], const AttnProblem* 
   const int64_t bg = (int64_t)d[0]->batch * d[0]->n_kv_heads;
   Shape sh[NP], by_pairs[NP];
   int64_t tiles = 0, doubles = 0, pair_tiles = 0;
-  const bool pairs_can = hd == 128 && d[0]->n_q_heads / d[0]->n_kv_heads <= BM / 2;
+  const bool pairs_can = d[0]->n_q_heads / d[0]->n_kv_heads <= BM / 2;
   int T = 0;
   for (int i = 0; i < NP; ++i) {
     sh[i] = shape_of(*d[i], a[i]->ctx, a[i]->ctx2, false);

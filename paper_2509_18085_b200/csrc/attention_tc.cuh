@@ -102,6 +102,6 @@ __device__ __forceinline__ Window visible_window(const Params& p, int t, int kb_
 
 // attention_pair.cu: `grid` CTAs, two neighbouring ones to an M-tile.
 template <int NP>
-spiffy_status launch_attention_pair(const Problems<NP>& pr, dim3 grid, cudaStream_t stream);
+spiffy_status launch_attention_pair(const Problems<NP>& pr, int head_dim, dim3 grid, cudaStream_t stream);
 
 }  // namespace spiffy

@@ -226,7 +226,7 @@ __device__ __forceinline__ void tmem_ld_x32(uint32_t taddr, uint32_t (&r)[32]) {
       : "memory");
 }
 
-// The same for 32 or 16 columns, issue only: the registers may be used after
+// The same for 32, 16 or 8 columns, issue only: the registers may be used after
 // tmem_wait_ld() on the same arrays.
 __device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -241,6 +241,12 @@ __device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&r)[16])
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
+}
+__device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // Nothing that uses r moves ahead of this point.
@@ -308,6 +314,9 @@ __device__ __forceinline__ uint32_t desc_lo_sw128(uint32_t addr, uint32_t lbo_by
 }
 __host__ __device__ constexpr uint32_t desc_hi_sw128(uint32_t sbo_bytes) {
   return ((sbo_bytes >> 4) & 0x3FFFu) | (1u << 14) | (2u << 29);
+}
+__host__ __device__ constexpr uint32_t desc_hi_sw64(uint32_t sbo_bytes) {  // rows of 64 bytes
+  return ((sbo_bytes >> 4) & 0x3FFFu) | (1u << 14) | (4u << 29);
 }
 // D[tmem] (+)= A B^T over K = 128: A and B K-major tiles of 128-byte-swizzled
 // rows, stored as two 64-element halves 16 KB apart (eight K steps of 16).
@@ -632,6 +641,100 @@ __device__ __forceinline__ void umma_pair_kn_k128(uint32_t d_tmem, uint32_t a_lo
       "}\n"
       :
       : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate_first)
+      : "memory");
+}
+
+// The same over K = 64: one half each.
+__device__ __forceinline__ void umma_pair_kk_k64(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t a_hi, uint32_t b_hi,
+                                                uint32_t idesc, uint32_t accumulate_first) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p0, p1, one;\n"
+      ".reg .b32 al, bl;\n"
+      ".reg .b64 da, db;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "setp.ne.b32 p0, %6, 0;\n"
+      "setp.eq.b32 p1, %6, %6;\n"
+      "add.u32 al, %1, 0;\n"
+      "add.u32 bl, %2, 0;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p0;\n"
+      "add.u32 al, %1, 2;\n"
+      "add.u32 bl, %2, 2;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p1;\n"
+      "add.u32 al, %1, 4;\n"
+      "add.u32 bl, %2, 4;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p1;\n"
+      "add.u32 al, %1, 6;\n"
+      "add.u32 bl, %2, 6;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p1;\n"
+      "}\n"
+      :
+      : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(a_hi), "r"(b_hi), "r"(idesc), "r"(accumulate_first)
+      : "memory");
+}
+// D (+)= A B over K = 128: A as above, B MN-major with 32 columns in each CTA, 128 rows of 64 bytes, swizzled
+// within those.
+__device__ __forceinline__ void umma_pair_kn32_k128(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t a_hi, uint32_t b_hi,
+                                                uint32_t idesc, uint32_t accumulate_first) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p0, p1, one;\n"
+      ".reg .b32 al, bl;\n"
+      ".reg .b64 da, db;\n"
+      "elect.sync _|one, 0xffffffff;\n"
+      "setp.ne.b32 p0, %6, 0;\n"
+      "setp.eq.b32 p1, %6, %6;\n"
+      "add.u32 al, %1, 0;\n"
+      "add.u32 bl, %2, 0;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p0;\n"
+      "add.u32 al, %1, 2;\n"
+      "add.u32 bl, %2, 64;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p1;\n"
+      "add.u32 al, %1, 4;\n"
+      "add.u32 bl, %2, 128;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p1;\n"
+      "add.u32 al, %1, 6;\n"
+      "add.u32 bl, %2, 192;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p1;\n"
+      "add.u32 al, %1, 512;\n"
+      "add.u32 bl, %2, 256;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p1;\n"
+      "add.u32 al, %1, 514;\n"
+      "add.u32 bl, %2, 320;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p1;\n"
+      "add.u32 al, %1, 516;\n"
+      "add.u32 bl, %2, 384;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p1;\n"
+      "add.u32 al, %1, 518;\n"
+      "add.u32 bl, %2, 448;\n"
+      "mov.b64 da, {al, %3};\n"
+      "mov.b64 db, {bl, %4};\n"
+      "@one tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p1;\n"
+      "}\n"
+      :
+      : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(a_hi), "r"(b_hi), "r"(idesc), "r"(accumulate_first)
       : "memory");
 }
 

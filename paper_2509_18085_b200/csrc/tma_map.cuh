@@ -48,20 +48,20 @@ bool make_map(CUtensorMap* m, const void* base, int heads, int64_t rows, int out
 // Tensor [outer][rows][heads][64 * halves] of bf16 as a 5-D TMA tensor {64 elements, head, row, half,
 // outer}; box = 64 x box_heads x box_rows x box_halves x 1.  The half of a head row comes behind the
 // rows, so that one instruction brings a tile's halves as they lie in shared memory, one 64-element
-// swizzled block behind the other: an instruction takes its thread some 400 cycles to issue, whatever
+// swizzled block behind the other (`block`: or 32-element ones): an instruction takes its thread some 400 cycles to issue, whatever
 // its size.
 bool make_tile_map(CUtensorMap* m, const void* base, int heads, int64_t rows, int outer, int box_heads, int box_rows,
-                   int box_halves, int64_t outer_stride_rows, int halves) {
+                   int box_halves, int64_t outer_stride_rows, int halves, int block = 64) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
   if (outer_stride_rows <= 0) outer_stride_rows = rows;
-  const cuuint64_t row_bytes = (cuuint64_t)halves * 128;
-  const cuuint64_t dims[5] = {64, (cuuint64_t)heads, (cuuint64_t)rows, (cuuint64_t)halves, (cuuint64_t)outer};
-  const cuuint64_t strides[4] = {row_bytes, heads * row_bytes, 128, (cuuint64_t)outer_stride_rows * heads * row_bytes};
-  const cuuint32_t box[5] = {64, (cuuint32_t)box_heads, (cuuint32_t)box_rows, (cuuint32_t)box_halves, 1};
+  const cuuint64_t row_bytes = (cuuint64_t)halves * block * 2;
+  const cuuint64_t dims[5] = {(cuuint64_t)block, (cuuint64_t)heads, (cuuint64_t)rows, (cuuint64_t)halves, (cuuint64_t)outer};
+  const cuuint64_t strides[4] = {row_bytes, heads * row_bytes, (cuuint64_t)block * 2, (cuuint64_t)outer_stride_rows * heads * row_bytes};
+  const cuuint32_t box[5] = {(cuuint32_t)block, (cuuint32_t)box_heads, (cuuint32_t)box_rows, (cuuint32_t)box_halves, 1};
   const cuuint32_t es[5] = {1, 1, 1, 1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, es,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, block == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

@@ -16,13 +16,15 @@ def check(cfg, seed, scale=None):
     w = W.make(cfg, seed, decision=False)
     if scale:
         scale(w)
-    got = G.gpu_attention(w, spiffy.ATTN_TCGEN05)
+    kernel = spiffy.ATTN_TCGEN05 if cfg.head_dim == 128 else spiffy.ATTN_AUTO
+    got = G.gpu_attention(w, kernel)
     want = oracle.graph_attention(w.q, w.k_prefix, w.v_prefix, w.k_block, w.v_block)
     assert np.max(np.abs(got - want)) <= G.TOL["bf16"]
     assert np.sqrt(np.mean((got - want) ** 2)) < 4e-3
-    assert np.array_equal(got, G.gpu_attention(w, spiffy.ATTN_TCGEN05))
+    assert np.array_equal(got, G.gpu_attention(w, kernel))
 
 
+@pytest.mark.parametrize("d", [128, 64])
 @pytest.mark.parametrize("B,N,L,P,Hq,Hkv", [
     (1, 1, 4, 0, 1, 1),            # one key tile: three warpgroups without any, the second block without rows
     (1, 2, 32, 0, 2, 2), (1, 2, 33, 60, 2, 2),   # 64 rows, and two more in the second block
@@ -33,12 +35,13 @@ def check(cfg, seed, scale=None):
     (1, 3, 5, 190, 64, 1), (1, 7, 3, 300, 66, 2),   # one position a block; groups of 33
     (1, 1, 200, 65, 2, 1),         # block keys over two key tiles
     (3, 4, 9, 449, 10, 2), (1, 9, 16, 1, 24, 8), (4, 2, 31, 127, 12, 4)])
-def test_parity(B, N, L, P, Hq, Hkv):
-    check(W.Config("pair", B, N, L, P, Hq, Hkv, 128, "bf16", 16, 0), 100 + P)
+def test_parity(B, N, L, P, Hq, Hkv, d):
+    check(W.Config("pair", B, N, L, P, Hq, Hkv, d, "bf16", 16, 0), 100 + P)
 
 
+@pytest.mark.parametrize("d", [128, 64])
 @pytest.mark.parametrize("factor", [3.0, 40.0])
-def test_maxima_that_grow_from_tile_to_tile(factor):
+def test_maxima_that_grow_from_tile_to_tile(factor, d):
     """Accumulators are rescaled, in some rows by the other half's maximum alone."""
     def scale(w):
         w.q *= factor / 3.0
@@ -46,7 +49,7 @@ def test_maxima_that_grow_from_tile_to_tile(factor):
         w.k_prefix[:, ::7] *= 2.0
         for a in ("q", "k_prefix"):
             setattr(w, a, W.round_to(getattr(w, a), "bf16"))
-    check(W.Config("pair", 1, 4, 20, 128 * 9 + 5, 6, 3, 128, "bf16", 16, 0), 3, scale)
+    check(W.Config("pair", 1, 4, 20, 128 * 9 + 5, 6, 3, d, "bf16", 16, 0), 3, scale)
 
 
 def test_two_problems_in_one_launch():
