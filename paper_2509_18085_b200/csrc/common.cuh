@@ -7,6 +7,7 @@
 
 #include <atomic>
 
+#include "fast_div.cuh"
 #include "spiffy.h"
 
 namespace spiffy {

@@ -52,6 +52,7 @@ struct LazyParams {
   const void* logits;
   int64_t row_stride, chunk;
   int B, N, L, V, splits, mask_id, rule, top_s;
+  FastDiv by_splits;
   float tau;
   const int32_t* block_tokens;
   const int32_t* parent_off;
@@ -199,8 +200,9 @@ decide_walk_lazy_kernel(const LazyParams p) {
       const int stride = many ? (reducers - b + p.B - 1) / p.B : 1;
       for (int i = many ? r / p.B : 0; i < items; i += stride) {
         uint64_t left = w.masked;
-        for (int k = i / p.splits; k > 0; --k) left &= left - 1;
-        const int l = __ffsll((long long)left) - 1, split = i % p.splits;
+        const int nth = p.by_splits.div(i), split = i - nth * p.splits;
+        for (int k = nth; k > 0; --k) left &= left - 1;
+        const int l = __ffsll((long long)left) - 1;
         const int64_t row = ((int64_t)b * N + w.node) * L + l;
         reduce_slice(static_cast<const T*>(p.logits) + row * p.row_stride, p.V, p.chunk, split,
                      p.partials + ((int64_t)b * L + l) * p.splits + split, kLog2e, level + 1);
@@ -224,7 +226,7 @@ decide_walk_lazy_kernel(const LazyParams p) {
         const int tag = b == 0 && p.lost_slices != 0 ? -1 : level + 1;
         unsigned polls = 0;
         for (int i = tid; i < L * p.splits && ok_wait; i += kReduceThreads) {
-          if (state[i / p.splits] != p.mask_id) continue;
+          if (state[p.by_splits.div(i)] != p.mask_id) continue;
           LazyWord w;  // 16 bytes, the tag last
           while ((int)((w = load_word(reinterpret_cast<const LazyWord*>(from + i))).masked >> 32) != tag)
             if (!(ok_wait = keep_polling(polls, p.header, p.wait_spins))) break;
@@ -373,6 +375,7 @@ spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc& d, const void* l
   p.logits = logits;
   p.row_stride = d.row_stride;
   p.splits = decide_splits(d, &p.chunk);
+  p.by_splits = FastDiv::by(p.splits);
   p.B = d.batch;
   p.N = d.n_nodes;
   p.L = d.block_len;
