@@ -89,9 +89,9 @@ class VerifyStep:
         # A step's attention and decision take nothing from one another and run side by side.  The
         # tensor-core kernel's CTAs hold whole SMs: they come second and move in as the reduce kernel
         # lets go, the decision's tail runs beside them (16 nodes x 32 positions x 28 heads, 156 MB of
-        # logits: 44 -> 35 us; attention first: 45).  Where both fill the machine for long there is
-        # little to overlap (4 x 32 x 32 positions, 32 heads over 4096 keys, 645 MB of logits: 431 us,
-        # of which the attention alone takes 305 and the decision 130).  The CUDA-core kernel's come
+        # logits: 44 -> 35 us when it came, 31.5 now; attention first: 45).  Where both fill the machine for
+        # long there is little to overlap (4 x 32 x 32 positions, 32 heads over 4096 keys, 645 MB of logits:
+        # 382 to 400 us, of which the attention alone takes 243 to 278 and the decision 108).  The CUDA-core kernel's come
         # several to an SM and would crowd the first ones that are free: there the decision comes second
         # (8 positions x 24 heads over 3249 keys: 38 -> 34 us; attention second: 42).
         self.attention_second = (cfg.dtype == "bf16" and attn_kernel != spiffy.ATTN_SIMT
