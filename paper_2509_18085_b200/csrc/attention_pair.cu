@@ -179,6 +179,8 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
   cluster_wait();
   tc_fence_after_sync();
   const uint32_t tmem = tail.tmem;
+  // Ahead of the wait, so that what follows a call of few CTAs sets itself up beside it: no kernel that reads
+  // without waiting itself comes directly behind this one (launch_pdl, common.cuh).
   if (p.early_trigger) pdl_launch_dependents();
   // everything above is on-chip set-up; global memory is touched from here on, behind a wait in each role
 

@@ -201,7 +201,9 @@ spiffy_status launch_attention_tc_dual(const spiffy_attn_desc& d0, const AttnPro
 //         read their inputs, write their outputs and wait last.  What precedes them is, by the
 //         flags' contract, a call that touches none of these; its kernels started, in turn,
 //         behind one that had waited before it triggered (the CUDA-core attention; the reduce
-//         of a plain decision), so everything ahead of that call is complete.
+//         of a plain decision), so everything ahead of that call is complete.  The second launch
+//         of an attention in two does the same behind the first, which touches other rows of the
+//         output and has waited before it triggered, or is itself under the flag.
 //   - Triggering early is safe for what follows for the same reasons; where it pays is a
 //     matter of measurement and said at each kernel.
 template <typename... Args>
