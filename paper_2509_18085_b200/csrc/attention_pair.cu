@@ -33,9 +33,11 @@
 // before, last P 4700 later, merge and output 2000.  What it took to get there: 12.8 us with two
 // warpgroups and barriers' arrivals across the pair with release semantics at cluster scope (500
 // cycles and more each); 9.5 without; 9.1 four warpgroups; 8.1 issuing warps converged instead of one
-// lane; 7.5 set-up side by side by warps, no division in the producers' loops.  The kernel
+// lane; 7.2 set-up side by side by warps, no division in the producers' loops; 7.3 with arrivals and waits
+// across the pair at cluster scope again, but the order they give confined to shared memory (fences with
+// sync_restrict; unconfined 7.5, and 14.1 instead of 12.5 over 17 key tiles).  The kernel
 // of attention_tc.cu took 10.3 then (9.7 now).  Per further key tile 0.45 us (0.88 there).  At head
-// dimension 64 7.1 us (9.3 there) and 0.69 (0.93).  Tried and dropped: two
+// dimension 64 7.2 us (9.3 there) and 0.69 (0.93).  Tried and dropped: two
 // CTAs of two warpgroups on an SM (10.6), references other than the maximum (nothing to exchange at
 // the first tile, 0.5 us; but the largest weight is then no longer exact, and the error 4 % larger).
 //
@@ -200,7 +202,7 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
     // whole warps up to the elected lane's instruction (sm100_ptx.cuh)
     auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
-      return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, p.spin_limit));
+      return __all_sync(0xffffffffu, mbar_wait_pair(bar, parity, abort_flag, p.spin_limit));
     };
     if (!p.independent) cudaGridDependencySynchronize();
     if (warp == 0 || warp == 3) {
@@ -320,7 +322,7 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
     // the P V products of key tile t (one of this warpgroup's) have completed
     auto wait_pv = [&](int t) -> bool {
       const bool yes =
-          __all_sync(0xffffffffu, mbar_wait(&bars.pv_done[wg], (uint32_t)(t / NW) & 1u, abort_flag, p.spin_limit));
+          __all_sync(0xffffffffu, mbar_wait_pair(&bars.pv_done[wg], (uint32_t)(t / NW) & 1u, abort_flag, p.spin_limit));
       tc_fence_after_sync();
       return yes;
     };
@@ -331,7 +333,7 @@ graph_attention_pair_kernel(const __grid_constant__ Problems<NP> problems) {
       // Wait outcomes are made warp-uniform: the TMEM accesses below are warp-collective.  A warp that
       // has given up still meets the other one of its rows, so that both leave together.
       bool good =
-          __all_sync(0xffffffffu, ok && mbar_wait(&bars.s_full[wg], (uint32_t)(t / NW) & 1u, abort_flag, p.spin_limit));
+          __all_sync(0xffffffffu, ok && mbar_wait_pair(&bars.s_full[wg], (uint32_t)(t / NW) & 1u, abort_flag, p.spin_limit));
       uint32_t s[2][32];
       uint32_t chunks = 3u;  // 32-column chunks that no row of the warp sees cost nothing but zeros in P
       float mx = -INFINITY;

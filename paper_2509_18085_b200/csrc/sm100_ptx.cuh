@@ -137,15 +137,16 @@ __device__ __forceinline__ void cluster_wait() {
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
-// The same without that order at cluster scope, which takes 500 cycles and more: for arrivals that hand
-// over nothing that the other CTA's threads read.  _relaxed: nothing in memory at all (tensor memory, behind
-// tcgen05.fence).  _own: shared memory of the arriving CTA, written behind fence.proxy.async and read by
-// that CTA's tensor core alone.
+// The same without that order, which takes 500 cycles and more, for memory of every kind.  _relaxed: hands
+// over nothing in memory at all (tensor memory, behind tcgen05.fence).  _own: what was written in the arriving
+// CTA's own shared memory alone (by this thread, or by others of the CTA that it has met); whoever waits
+// with mbar_wait_pair sees it.
 __device__ __forceinline__ void mbar_arrive_remote_relaxed(uint32_t addr) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_remote_own(uint32_t addr) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+  asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+  mbar_arrive_remote_relaxed(addr);
 }
 // `bytes` (a multiple of 16) from this CTA's shared memory into another CTA's
 // without waiting for them: the destination CTA's mbarrier `bar` (same CTA as
@@ -176,6 +177,31 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
 #pragma unroll 1
   for (uint32_t i = 0; i < limit; ++i) {
     if (mbar_try_wait_cluster(bar, parity)) return true;
+    if ((i & 15u) == 15u && *abort) return false;
+  }
+  *abort = 1;
+  return false;
+}
+// mbar_wait for barriers that count what both CTAs of a pair do (their threads' arrivals, their copies' bytes,
+// products that read both): also orders what mbar_arrive_remote_own handed over, or the copies brought
+// into either CTA's shared memory, before what follows.
+__device__ __forceinline__ bool mbar_wait_pair(uint64_t* bar, uint32_t parity, volatile int* abort, uint32_t limit) {
+#pragma unroll 1
+  for (uint32_t i = 0; i < limit; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) {
+      asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory");
+      return true;
+    }
     if ((i & 15u) == 15u && *abort) return false;
   }
   *abort = 1;
