@@ -428,9 +428,12 @@ spiffy_status spiffy_accept_walk(const spiffy_decide_desc* desc,
  * layouts, outputs (bit for bit) and status codes; decide_status and
  * walk_status are the dev_status arrays of the two calls (either may be NULL).
  * When a sequence's graph is small (N * L <= 512 and its arrays fit the
- * default shared memory of one CTA) the merge of the vocabulary slices, the
- * unmasking rule and the walk run in one kernel per sequence, one launch
- * fewer than the two separate calls; otherwise this is the two calls.
+ * default shared memory of one CTA) and so is what there is to merge (at most
+ * 4096 partial results, N * L times the vocabulary slices of 8192 bf16 or 4096
+ * fp32 entries a row comes in; any number under SPIFFY_INDEPENDENT_NEXT), the
+ * merge of the slices, the unmasking rule and the walk run in one kernel per
+ * sequence, one launch fewer than the two separate calls; otherwise this is the
+ * two calls.
  * Workspace: spiffy_unmask_decide_workspace(desc).
  */
 spiffy_status spiffy_decide_walk(const spiffy_decide_desc* desc, const void* logits,

@@ -296,12 +296,19 @@ spiffy_status launch_decide_finalize(const spiffy_decide_desc& d, const void* pa
 
 // Decision and walk in one call.  Small graphs (at most kTailRows rows per sequence, arrays within the
 // default shared-memory limit) take the fused tail: two launches instead of three.  Larger ones keep
-// one finalize CTA per node, which spreads the merging over more SMs, and so do those whose partial
-// results are more than one SM takes in as fast (kTailPartials, 96 KB): 512 rows x 19 slices, 322
-// masked, 25.3 us with the tail and 22.7 without; 256 x 16 13.1 and 14.0.  Where an attention follows
-// beside the decision (`next`) the merging runs under it, on one SM instead of many that the
-// attention waits for (16 x 32 positions x 28 heads 31.6 us, 31.8 without the tail).
-constexpr int kTailRows = 512, kTailPartials = 6144;
+// one finalize CTA per node, which spreads the merging over more SMs, and so do those with more partial
+// results than one SM merges as fast, whatever part of them is of rows still masked.  Tail and kernels,
+// us, with 5, 40 and 95 % of the rows masked:
+//   512 rows x  4 slices  7.7  9.0    9.2 10.3   11.0 12.1
+//   512 x  8, 4096 in all 8.7  9.2   11.3 12.1   16.4 16.5     256 x 16  8.2  8.2   11.8 11.8   15.9 15.9
+//   512 x  9              9.2  9.2   13.3 12.8   18.1 17.7     256 x 19  9.5  9.0   13.2 12.5   18.5 17.8
+//   512 x 19             14.4 13.1   21.5 18.8   31.4 29.0     4 x 512 x 19  30.6 28.0  51.7 49.2  99.3 96.4
+// Beside a CUDA-core attention (`independent`; 512 rows of fp32, 40 % masked) the line lies there too:
+// x 8 25.1 and 26.1, x 10 26.6 and 26.2, x 31 37.9 and 33.7; where the attention is by far the longer
+// one (170 us) 1 us either way.  Where an attention follows beside the decision (`next`) the merging
+// runs under it, on one SM instead of many that the attention waits for: the tail, whatever there is to
+// merge (16 x 32 positions x 28 heads, x 19: 21.5 and 21.5, 27.0 and 27.7, 36.9 and 37.3).
+constexpr int kTailRows = 512, kTailPartials = 4096;
 spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits,
                                  const int32_t* block_tokens, float* conf, int32_t* top_tok,
                                  uint64_t* unmask_bits, int32_t* n_unmask,
@@ -312,16 +319,15 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
                                  bool fresh, bool independent, bool next, cudaStream_t stream) {
   const size_t smem = tail_smem_bytes(d, parent_cap);
   const int64_t rows_of_one = (int64_t)d.n_nodes * d.block_len;
-  const int splits_of_row = decide_splits(d, nullptr);
-  if (rows_of_one > kTailRows || smem > 48 * 1024 || (!next && rows_of_one * splits_of_row > kTailPartials)) {
+  int64_t chunk = 0;
+  const int splits = decide_splits(d, &chunk);
+  if (rows_of_one > kTailRows || smem > 48 * 1024 || (!next && rows_of_one * splits > kTailPartials)) {
     const spiffy_status st = decide_only(d, logits, block_tokens, conf, top_tok, unmask_bits,
                                          n_unmask, decide_status, ws, fresh, independent, next, stream);
     if (st != SPIFFY_OK) return st;
     return launch_walk(d, block_tokens, parent_off, parent_idx, parent_cap, top_tok, unmask_bits,
                        accepted_node, n_accepted, path, next_block, walk_status, fresh, stream);
   }
-  int64_t chunk = 0;
-  const int splits = decide_splits(d, &chunk);
   Partial* partials = static_cast<Partial*>(ws);
   const spiffy_status st = launch_reduce(d, logits, block_tokens, partials, splits, chunk, 1, independent,
                                          status_clear(d, fresh, decide_status, walk_status), stream);

@@ -256,8 +256,9 @@ def test_lazy_call_in_a_cuda_graph():
     assert int(walk0.n_accepted.max()) >= 2
 
 
-@pytest.mark.parametrize("N,L,V", [(16, 32, 12 * 4096), (16, 32, 12 * 4096 + 4), (8, 64, 70000)])
+@pytest.mark.parametrize("N,L,V", [(16, 32, 8 * 4096), (16, 32, 8 * 4096 + 4),
+                                   (16, 32, 12 * 4096), (16, 32, 12 * 4096 + 4), (8, 64, 70000)])
 def test_one_call_equals_two_calls_around_the_tails_partial_results(N, L, V):
-    """Rows x slices on both sides of what the fused tail takes (512 x 12), and beyond."""
+    """Rows x slices on both sides of what the fused tail takes (512 x 8), and beyond."""
     logits, tokens, off, idx, mask = random_case(71, 1, N, L, V)
     both(logits, tokens, off, idx, mask, spiffy.RULE_TOPS)

@@ -37,6 +37,27 @@ def test_same_bits_as_one_after_the_other(B, N, L, P, Hq, Hkv, d, V, dtype):
                 assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("N,V,dtype", [(16, 4000, "bf16"), (16, 70000, "bf16"), (17, 4000, "bf16"),
+                                       (16, 4000, "f32"), (16, 40000, "f32"), (17, 4000, "f32")])
+def test_late_in_a_block(N, V, dtype):
+    """Most rows unmasked, the last one among them: the blocks of the reduce that end at once, and the one that
+    waits for the kernel before, on both routes of the decision."""
+    cfg = W.Config("t", 1, N, 32, 300, 8, 4, 64, dtype, V, spiffy.RULE_THRESHOLD)
+    step, apart = VerifyStep(cfg), VerifyStep(cfg)
+    x = inputs_from_workload(W.make(cfg, 4))
+    for masked in (0, 3, 40):
+        x.block_tokens.fill_(7)
+        at = torch.randperm(N * 31, generator=torch.Generator().manual_seed(masked))[:masked].cuda()
+        x.block_tokens[0, at // 31, at % 31] = cfg.mask_id  # the last position of every node stays
+        apart.attention(x)
+        apart.decide_accept(x)
+        want = _results(apart)
+        for _ in range(5):
+            step.run(x)
+            for a, b in zip(_results(step), want):
+                assert torch.equal(a, b)
+
+
 def _results(s):
     out = [s.attn_out, s.attn_status] + list(_fields(s.decision)) + list(_fields(s.walk))
     return [t.clone().view(torch.uint8) for t in out]

@@ -155,6 +155,25 @@ def test_an_independent_kernel_may_start_as_the_reduce_ends(host, N, L, cap):
             assert log[1].endswith(f" early {early}")
 
 
+@pytest.mark.parametrize("flags", [0, spiffy.INDEPENDENT, spiffy.INDEPENDENT_NEXT])
+@pytest.mark.parametrize("N,L,V,dtype", [
+    (16, 32, 8 * 8192, spiffy.BF16), (16, 32, 8 * 8192 + 8, spiffy.BF16),        # 512 rows of 8 slices, of 9
+    (8, 32, 16 * 8192, spiffy.BF16), (8, 32, 16 * 8192 + 8, spiffy.BF16),
+    (3, 13, 105 * 4096, spiffy.F32), (3, 13, 105 * 4096 + 4, spiffy.F32),        # 39 rows of 105, of 106
+    (9, 57, 1000, spiffy.BF16), (16, 32, 1000, spiffy.BF16)])                    # 513 rows, and 512, of one
+def test_fused_tail_up_to_4096_partial_results(host, N, L, V, dtype, flags):
+    """Beyond, the kernels apart, unless an attention comes next and the merging runs beside it."""
+    slices = -(-V // (8192 if dtype == spiffy.BF16 else 4096))
+    fused = N * L <= 512 and (N * L * slices <= 4096 or flags == spiffy.INDEPENDENT_NEXT)
+    d = spiffy.DecideDesc(1, N, L, V, dtype | flags, V, V - 1, spiffy.RULE_TOPS, 1, 0.9)
+    p = ctypes.c_void_p(1 << 20)
+    host.fake_reset(b"", 0, 0)
+    assert host.spiffy_decide_walk(ctypes.byref(d), p, p, p, p, 4, *[p] * 11, ctypes.c_size_t(1 << 40),
+                                   ctypes.c_void_p(STREAM)) == spiffy.OK
+    kernels = [re.search("(decide_reduce|decide_tail|decide_finalize|accept_walk)_kernel", line).group(1) for line in host.fake_log().decode().splitlines()]
+    assert kernels == (["decide_reduce", "decide_tail"] if fused else ["decide_reduce", "decide_finalize", "accept_walk"])
+
+
 def test_a_step_object_describes_each_input_anew(monkeypatch):
     """The parent lists of one graph are longer than the next one's: a descriptor kept from the first
     call would read past the end of the second call's arrays."""
