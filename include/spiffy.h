@@ -132,7 +132,10 @@ typedef enum { SPIFFY_RULE_TOPS = 0, SPIFFY_RULE_THRESHOLD = 1 } spiffy_rule;
 #define SPIFFY_ATTN_EARLY_DEPENDENTS 0x100
 /* Flag, OR-ed into spiffy_attn_desc.kernel: the call before this one in the stream
  * is spiffy_decide_walk with SPIFFY_INDEPENDENT_NEXT, and none of this call's
- * inputs or outputs is touched by it.  Tensor-core kernel only. */
+ * inputs or outputs is touched by it.  Tensor-core kernel only.  (A shape that
+ * would fill every multiprocessor may take another of the tensor-core kernels
+ * than without the flag, since the decision's end holds some of them; its
+ * results then differ by their rounding.) */
 #define SPIFFY_ATTN_INDEPENDENT 0x200
 
 /* ------------------------------------------------------------------------- */

@@ -761,40 +761,57 @@ int resident_clusters(int hd, int cs) {
 // `tiles` counts the M-tiles of all problems of the launch, `doubles` the CTAs that take two
 // of them, `pair_tiles` the pairs (0: not possible); T is the key tiles of the longer problem.
 // `may_split`: the call may be two launches; `same_tiles`: a pair's M-tiles are one CTA's.
-Plan make_plan(int64_t tiles, int64_t doubles, int64_t pair_tiles, int T, int hd, bool may_split, bool same_tiles) {
+// `held`: SMs that the end of a decision beside this call holds as its CTAs move in, one a sequence.  A call
+// whose one round needs them as well ends 3 to 4 us later, and plans of fewer CTAs are another 2 us sooner
+// done beside a decision than their costs say (kLate in all).  2 x 32 positions x 74 heads, 74 pairs, with a
+// decision of 32000 entries: over 100 keys 11.8 us (73 heads 8.7), with one M-tile per CTA 9.2; over 512
+// 13.8 and 12.6; over 1000 18.0 and 17.9, where the line is.  8 x 32 x 74 heads, 148 CTAs of one M-tile: over 100
+// keys 16.4, two M-tiles per CTA 13.9; over 512 19.7 and 20.2, left at one.  Measured for one, two and four
+// sequences, at head dimension 64, and with a graph too large for the fused tail (146 x 32 x 2 heads 27.2 -> 22.3).
+Plan make_plan(int64_t tiles, int64_t doubles, int64_t pair_tiles, int T, int hd, bool may_split, bool same_tiles,
+               int held) {
   const int sms = sm_count();
   const float one0 = hd == 128 ? 6.6f : 4.9f, one = hd == 128 ? 0.88f : 0.93f;
   const float two0 = hd == 128 ? 8.0f : 6.0f, two = hd == 128 ? 1.75f : 1.8f;
   const float pair = hd == 128 ? 5.0f + 0.45f * (float)T : 3.7f + 0.69f * (float)T;
+  const float kLate = hd == 128 ? 5.5f : 4.0f;
   auto rounds = [&](int64_t ctas) { return (float)((ctas + sms - 1) / sms); };
-  Plan pl = {2, 1, false, 0, false};
-  if (sms <= 0) return pl;
-  float best = rounds(doubles) * (two0 + two * (float)T);
-  if (pair_tiles > 0) {
-    const float cost = rounds(2 * pair_tiles) * pair;
-    if (cost < best) {
-      best = cost;
-      pl = {1, 1, true, 0, false};
+  if (sms <= 0) return {2, 1, false, 0, false};
+  struct Choice {
+    Plan plan;
+    int64_t ctas;
+    float cost;
+  };
+  // The cheapest plan of at most `most` CTAs.
+  auto cheapest = [&](int64_t most) {
+    Choice c = {{2, 1, false, 0, false}, 0, INFINITY};
+    auto consider = [&](const Plan& pl, int64_t ctas, float a_round) {
+      const float cost = rounds(ctas) * a_round;
+      if (ctas <= most && cost < c.cost) c = {pl, ctas, cost};
+    };
+    consider({2, 1, false, 0, false}, doubles, two0 + two * (float)T);
+    if (pair_tiles > 0) consider({1, 1, true, 0, false}, 2 * pair_tiles, pair);
+    for (int cs = 1; cs <= 8 && cs <= T; cs *= 2) {
+      // clusters only where all of them run at once
+      if (cs > 1 && (tiles * cs > sms || tiles > resident_clusters(hd, cs))) continue;
+      const float exchange = cs == 1 ? 0.f : (hd == 128 ? 1.9f : 1.4f) + 0.07f * (float)cs;
+      consider({1, cs, false, 0, false}, tiles * cs, one0 + exchange + one * (float)((T + cs - 1) / cs));
     }
-  }
-  for (int cs = 1; cs <= 8 && cs <= T; cs *= 2) {
-    // clusters only where all of them run at once
-    if (cs > 1 && (tiles * cs > sms || tiles > resident_clusters(hd, cs))) continue;
-    const float exchange = cs == 1 ? 0.f : (hd == 128 ? 1.9f : 1.4f) + 0.07f * (float)cs;
-    const float cost = rounds(tiles * cs) * (one0 + exchange + one * (float)((T + cs - 1) / cs));
-    if (cost < best) {
-      best = cost;
-      pl = {1, cs, false, 0, false};
-    }
+    return c;
+  };
+  Choice best = cheapest(INT64_MAX);
+  if (best.ctas <= sms && best.ctas > sms - held) {
+    const Choice fewer = cheapest(sms - held);
+    if (fewer.cost < best.cost + kLate) best = fewer;
   }
   // A last round that half fills the SMs or less is done in half the time with one M-tile per CTA.
   const int64_t full = doubles / sms, left = doubles - full * sms;
   if (may_split && full > 0 && left > 0 && 2 * left <= sms) {
     const bool by_pairs = pair_tiles > 0 && same_tiles && 4 * left <= sms;
     const float rest = by_pairs ? pair : one0 + one * (float)T;
-    if ((float)full * (two0 + two * (float)T) + rest < best) pl = {2, 1, false, (int)full, by_pairs};
+    if ((float)full * (two0 + two * (float)T) + rest < best.cost) best.plan = {2, 1, false, (int)full, by_pairs};
   }
-  return pl;
+  return best.plan;
 }
 
 bool make_problem(const spiffy_attn_desc& d, const Shape& sh, const AttnProblem& a, Maps* m, Params* p, const Plan& pl,
@@ -901,7 +918,8 @@ spiffy_status launch(const spiffy_attn_desc* const (&d)[NP], const AttnProblem* 
     T = sh[i].T > T ? sh[i].T : T;
   }
   const bool split = NP == 1 && bg * (sh[0].MT + 1) < (1 << 30);
-  const Plan pl = make_plan(tiles, doubles, pair_tiles, T, hd, split, by_pairs[0].TNL == sh[0].TNL);
+  const int held = (d[0]->kernel & SPIFFY_ATTN_INDEPENDENT) ? d[0]->batch : 0;
+  const Plan pl = make_plan(tiles, doubles, pair_tiles, T, hd, split, by_pairs[0].TNL == sh[0].TNL, held);
   const dim3 grid(0, (unsigned)d[0]->n_kv_heads, (unsigned)d[0]->batch);
   if (pl.full_rounds == 0) return launch_part(d, a, pl.pair ? by_pairs : sh, pl, grid, 0, 0, 0, dev_status, stream);
   // Full rounds first, which let the rest begin as they end; the rest reads nothing of theirs, and is

@@ -1,6 +1,8 @@
 // A stand-in for the CUDA runtime and for the attention kernels' launchers, so that
 // the library's host code can run where there is no GPU: every call is written to a
-// log, any of them can be made to fail, nothing is copied and no kernel runs.
+// log, any of them can be made to fail, nothing is copied and no kernel runs.  With REAL_ATTENTION the
+// launcher of the tensor-core kernels is the library's own, on a device of 148 multiprocessors.
+#include <cuda.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -63,6 +65,20 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* at, const void* p) {
   at->devicePointer = at->hostPointer = const_cast<void*>(p);
   return cudaSuccess;
 }
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+// as a B200 answers for thread blocks that hold a multiprocessor each
+cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t* c) {
+  const unsigned size = c->attrs[0].val.clusterDim.x;
+  *n = size == 2 ? 74 : size == 4 ? 33 : 15;
+  return cudaSuccess;
+}
+static CUresult encode_tiled(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                             const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill) { return CUDA_SUCCESS; }
+cudaError_t cudaGetDriverEntryPoint(const char*, void** f, unsigned long long, cudaDriverEntryPointQueryResult*) {
+  *f = reinterpret_cast<void*>(encode_tiled);
+  return cudaSuccess;
+}
 cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void**, size_t, cudaStream_t s) { return note("launch " + g_kernels[f] + on(s)); }
 // The arguments that decide what a kernel may read and when, by position.
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
@@ -73,11 +89,21 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
   if (name.find("decide_reduce_kernel") != std::string::npos) more = " early " + i(8);
   if (name.find("accept_walk_kernel") != std::string::npos) more = " lists " + p(3) + " staged " + i(13);
   if (name.find("decide_tail_kernel") != std::string::npos) more = " lists " + p(14) + " early " + i(22);
+  if (name.find("graph_attention") != std::string::npos) {
+    unsigned cluster = 1;
+    for (unsigned k = 0; k < c->numAttrs; ++k)
+      if (c->attrs[k].id == cudaLaunchAttributeClusterDimension) cluster = c->attrs[k].val.clusterDim.x;
+    more = " blocks " + std::to_string((long)c->gridDim.x * c->gridDim.y * c->gridDim.z) + " cluster " + std::to_string(cluster);
+  }
   return note("launch " + name + on(c->stream) + more);
 }
 }  // extern "C"
 
 namespace spiffy {
+#ifdef REAL_ATTENTION
+spiffy_status launch_attention_simt(const spiffy_attn_desc&, const void*, const void*, const void*, const void*,
+                                    const void*, void*, cudaStream_t) { return SPIFFY_ECUDA; }
+#else
 bool attention_tc_supported(const spiffy_attn_desc& d) { return d.dtype == SPIFFY_BF16; }
 spiffy_status launch_attention_tc(const spiffy_attn_desc& d, const AttnProblem&, int32_t*, cudaStream_t s) {
   return note("launch attention" + on(s) + " independent " + std::to_string((d.kernel & SPIFFY_ATTN_INDEPENDENT) != 0)) ==
@@ -87,9 +113,10 @@ spiffy_status launch_attention_simt(const spiffy_attn_desc& d, const void*, cons
                                     const void*, void*, cudaStream_t s) {
   return launch_attention_tc(d, AttnProblem{}, nullptr, s);
 }
-// calls that no test here makes
 spiffy_status launch_attention_tc_dual(const spiffy_attn_desc&, const AttnProblem&, const spiffy_attn_desc&,
                                        const AttnProblem&, int32_t*, cudaStream_t) { return SPIFFY_ECUDA; }
+#endif
+// calls that no test here makes
 size_t decide_lazy_workspace_bytes(const spiffy_decide_desc&) { return 0; }
 spiffy_status launch_decide_walk_lazy(const spiffy_decide_desc&, const void*, const int32_t*, float*, int32_t*, uint64_t*,
                                       int32_t*, int32_t*, const int32_t*, const int32_t*, int32_t, int32_t*, int32_t*,
