@@ -81,17 +81,21 @@ def test_odd_shapes(shape, dtype, kernel):
 
 
 @pytest.mark.parametrize("prefix_len,n_nodes,block_len", [
-    (384, 8, 32),   # 3 context tiles + 1 block tile: one for each CTA of a cluster of four
-    (512, 8, 32),   # 5 key tiles: one CTA has a tile more
+    # pairs of CTAs to an M-tile
+    (384, 8, 32),   # 3 context tiles + 1 block tile: one for each warpgroup
+    (512, 8, 32),   # 5 key tiles: one warpgroup has a tile more
     (640, 8, 32),   # 6
     (300, 4, 32),   # 4, ragged context tile, one M-tile per head
     (400, 6, 48),   # nodes of 48 positions: M-tiles with one and with two block-key tiles (odd and even in one launch)
     (257, 3, 7),    # 4 tiles, a nearly empty M-tile
+    # longer: the key tiles of each M-tile are split over the CTAs of a cluster of four
+    (2700, 8, 32),  # 23 key tiles: three CTAs have a tile more
+    (2944, 4, 32),  # 24
+    (2600, 3, 7),   # ragged context tile, a nearly empty M-tile
 ])
 def test_cluster_pairs_with_even_and_odd_tile_counts(prefix_len, n_nodes, block_len):
-    """Few M-tiles: the key tiles of each M-tile are split over the CTAs of a
-    cluster, four of them (nodes of 48 positions: one CTA for all), which merge
-    through each other's shared memory."""
+    """Few M-tiles: each is worked on by a cluster of CTAs, two that share all of
+    its key tiles, or four that split them and merge through each other's shared memory."""
     cfg = W.Config("pairs", dtype="bf16", vocab=16, rule=0, batch=1, n_nodes=n_nodes, block_len=block_len,
                    prefix_len=prefix_len, n_q_heads=16, n_kv_heads=16, head_dim=128)
     w = W.make(cfg, 31 + prefix_len, decision=False)

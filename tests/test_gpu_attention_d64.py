@@ -1,5 +1,6 @@
 """Head dimension 64 in bf16 on the tensor cores (what SPIFFY_ATTN_AUTO takes),
-at the edges of its tiles and on each of its routes."""
+at the edges of its tiles.  (Every one
+of its routes: test_gpu_attention_routes.py.)"""
 import numpy as np
 import pytest
 import torch
@@ -15,12 +16,12 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("B,N,L,P,Hq,Hkv", [
     (1, 1, 1, 1, 1, 1), (1, 2, 5, 0, 2, 1),       # the smallest; block keys only
     (1, 3, 7, 127, 16, 16), (1, 3, 7, 129, 16, 16),  # context one short of / one past a key tile
-    (1, 8, 32, 512, 16, 16),                      # clusters of four, odd number of key tiles
-    (1, 8, 32, 640, 16, 16),                      # clusters of four, even
+    (1, 8, 32, 512, 16, 16),                      # pairs of CTAs (as all above), as many key tiles as stages of the ring
+    (1, 8, 32, 640, 16, 16),                      # ... one more
     (1, 9, 8, 1000, 3, 3),                        # clusters of eight
-    (3, 9, 32, 300, 32, 32),                      # two rounds of CTAs
+    (3, 9, 32, 300, 32, 32),                      # one M-tile per CTA, two rounds of CTAs
     (2, 9, 32, 300, 35, 35),                      # two M-tiles per CTA, the last one beyond the rows
-    (1, 7, 32, 777, 32, 32),                      # clusters of two
+    (1, 7, 32, 777, 32, 32),                      # 64 pairs
     (2, 4, 12, 129, 28, 4),                       # grouped heads: M-tiles of 126 rows
     (1, 2, 3, 20, 128, 1),                        # one position per M-tile
     (1, 1, 64, 2000, 4, 2)])

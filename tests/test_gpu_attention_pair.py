@@ -30,8 +30,10 @@ def check(cfg, seed, scale=None):
     (1, 2, 32, 0, 2, 2), (1, 2, 33, 60, 2, 2),   # 64 rows, and two more in the second block
     (1, 4, 32, 128 * 3, 3, 3),     # as many key tiles as warpgroups
     (1, 5, 32, 128 * 3 + 1, 3, 3),  # one more; the last pair has one block's rows
-    (2, 4, 32, 128 * 5, 3, 3), (2, 4, 32, 128 * 6, 3, 3),  # as many as the ring has stages, one more
-    (1, 3, 17, 128 * 12 - 3, 28, 4),  # the ring several times round, groups of 7: 63 rows of 64
+    # as many as the ring has stages, one more (at head dimension 64 that many already, then a cluster)
+    (2, 4, 32, 128 * 5, 3, 3), (2, 4, 32, 128 * 6, 3, 3),
+    (1, 3, 17, 128 * 12 - 3, 28, 4),  # long enough for a cluster of eight instead
+    (1, 9, 34, 128 * 12 - 3, 28, 4),  # the ring several times round, groups of 7: 63 rows of 64
     (1, 3, 5, 190, 64, 1), (1, 7, 3, 300, 66, 2),   # one position a block; groups of 33
     (1, 1, 200, 65, 2, 1),         # block keys over two key tiles
     (3, 4, 9, 449, 10, 2), (1, 9, 16, 1, 24, 8), (4, 2, 31, 127, 12, 4)])
@@ -42,7 +44,8 @@ def test_parity(B, N, L, P, Hq, Hkv, d):
 @pytest.mark.parametrize("d", [128, 64])
 @pytest.mark.parametrize("factor", [3.0, 40.0])
 def test_maxima_that_grow_from_tile_to_tile(factor, d):
-    """Accumulators are rescaled, in some rows by the other half's maximum alone."""
+    """Accumulators are rescaled, in some rows by the other half's maximum alone.  (Head dimension 64: this
+    shape goes to a cluster of eight; the pair's is in test_gpu_attention_routes.py.)"""
     def scale(w):
         w.q *= factor / 3.0
         w.k_prefix *= (1.0 + np.arange(w.k_prefix.shape[1]) // 100 * 0.5)[None, :, None, None].astype(w.k_prefix.dtype)

@@ -71,13 +71,13 @@ def same(a, b):
 ATTENTION_SHAPES = [
     # fp32: CUDA-core kernel
     (dict(batch=2, n_nodes=3, block_len=5, prefix_len=127, n_q_heads=6, n_kv_heads=2, head_dim=64), "f32"),
-    # tensor-core kernel: clusters of four twice, of eight, two rounds of single CTAs, one round
+    # tensor-core kernels: pairs of CTAs three times, two rounds of single CTAs, pairs
     (dict(batch=1, n_nodes=3, block_len=7, prefix_len=257, n_q_heads=16, n_kv_heads=16, head_dim=128), "bf16"),
     (dict(batch=1, n_nodes=8, block_len=32, prefix_len=512, n_q_heads=16, n_kv_heads=16, head_dim=128), "bf16"),
     (dict(batch=1, n_nodes=9, block_len=8, prefix_len=1000, n_q_heads=3, n_kv_heads=3, head_dim=128), "bf16"),
     (dict(batch=3, n_nodes=9, block_len=32, prefix_len=300, n_q_heads=32, n_kv_heads=32, head_dim=128), "bf16"),
     (dict(batch=2, n_nodes=4, block_len=12, prefix_len=129, n_q_heads=6, n_kv_heads=2, head_dim=128), "bf16"),
-    # two M-tiles per CTA, the last one empty; clusters of two; and the same at head dimension 64
+    # two M-tiles per CTA, the last one empty; pairs; head dimension 64: two M-tiles per CTA, a cluster of eight
     (dict(batch=2, n_nodes=9, block_len=32, prefix_len=300, n_q_heads=35, n_kv_heads=35, head_dim=128), "bf16"),
     (dict(batch=1, n_nodes=7, block_len=32, prefix_len=777, n_q_heads=32, n_kv_heads=32, head_dim=128), "bf16"),
     (dict(batch=2, n_nodes=9, block_len=32, prefix_len=300, n_q_heads=35, n_kv_heads=35, head_dim=64), "bf16"),

@@ -19,6 +19,8 @@ pytestmark = pytest.mark.gpu
     (3, 24, 4, 764, 24, 8, 128, 4000, "bf16"),  # one nearly full round of clusters
     (1, 54, 32, 300, 28, 4, 64, 4072, "bf16"),  # more than 512 rows: finalize and walk kernels
     (2, 16, 32, 2000, 32, 32, 128, 8192, "bf16"),  # several rounds
+    # a call of two launches, the second by pairs and by one M-tile per block; beside the fused tail and not
+    (5, 8, 32, 256, 32, 32, 128, 1000, "bf16"), (1, 18, 60, 100, 150, 50, 128, 1000, "bf16"),
     (2, 3, 32, 500, 5, 5, 128, 2864, "f32"),
 ])
 def test_same_bits_as_one_after_the_other(B, N, L, P, Hq, Hkv, d, V, dtype):

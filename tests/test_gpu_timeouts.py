@@ -47,10 +47,10 @@ def test_lazy_call_gives_up_on_an_arrival_that_never_comes(limits):
 @pytest.mark.parametrize("index,n_nodes,over", [(5, 8, {}), (5, 64, {}), (2, None, {}), (3, None, {}),
                                                 (2, None, dict(batch=5, prefix_len=256))])
 def test_attention_gives_up_when_its_mbarrier_waits_may_not_poll(limits, index, n_nodes, over):
-    """The routes of the tensor-core kernel: key tiles split over a cluster of
-    eight (5 with 8 nodes) or two (5 with 64), one M-tile per thread block over all
-    key tiles (2, 3), two M-tiles per block (2 with a batch of five).  With no poll allowed every role of the kernel gives up at its first
-    wait, before any tensor-core product is issued."""
+    """Key tiles split over a cluster of eight (5 with 8 nodes), pairs of thread blocks (5 with 64, 2), one
+    M-tile per block (3), two launches, of two M-tiles per block and of pairs (2 with a batch of five).
+    With no poll allowed every role of the kernel gives up at its first wait, before any tensor-core
+    product is issued.  (All routes: test_gpu_attention_routes.py.)"""
     cfg = W.config(index, n_nodes, **over)
     w = W.make(cfg, W.seed_for(index, 0), decision=False)
     dt = torch.bfloat16
