@@ -449,14 +449,26 @@ def kernel_sources_digest(files):
     return h.hexdigest()[:16]
 
 
+def ncu_record(key):
+    with open(os.path.join(ROOT, "profiles", "ncu_traffic.json")) as f:
+        return json.load(f)[key]
+
+
+def attention_kernels(key, per_call):
+    """The kernels of a tensor-core attention call, by the names under which the capture of `key` saw them;
+    the library chooses by the shape."""
+    try:
+        return ncu_record(key)["kernel"]
+    except (OSError, KeyError, ValueError):
+        return "graph_attention_pair_kernel or graph_attention_tc_kernel" + (", two launches" if per_call > 1 else "")
+
+
 def ncu_traffic(key):
     """DRAM bytes per launch of a kernel as ncu counted them (profiles/ncu_traffic.json, written
     next to the summary the figure comes from).  None when there is no record or the kernel's
     sources have changed since the capture."""
-    path = os.path.join(ROOT, "profiles", "ncu_traffic.json")
     try:
-        with open(path) as f:
-            rec = json.load(f)[key]
+        rec = ncu_record(key)
         if rec["sources_sha256_16"] != kernel_sources_digest(rec["sources"]):
             return None, f"stale: {rec['sources']} changed since the capture in {rec['summary']}"
         return float(rec["dram_bytes_per_launch"]), f"ncu dram read+write bytes per launch, {rec['summary']}"
@@ -734,9 +746,11 @@ def main():
     t_hbm = attn_bytes / (peaks["hbm_gbs"] * 1e9)
     attn_bound = "tensor" if t_tensor > t_hbm else "hbm"
     attn_tc = attn_flops / t_attn / 1e12
-    tr_attn, tr_attn_note = ncu_traffic("graph_attention_tc_kernel@config%d" % args.config)
+    attn_key = "graph_attention@config%d" % args.config
+    tr_attn, tr_attn_note = ncu_traffic(attn_key)
     attention_roof = {
-        "kernel": "graph_attention_tc_kernel" + (" (+ graph_attention_combine_kernel)" if k_attn > 1 else ""),
+        "kernel": attention_kernels(attn_key, k_attn) if cfg.dtype == "bf16" and args.attn_kernel != "simt"
+        else "graph_attention_simt_kernel",
         "timed_as": f"the spiffy_graph_attention call alone ({k_attn:g} kernel(s) per call), graph replay over "
                     f"{N_SETS} L2-cold input sets, CUDA events on the launching stream",
         "bound": attn_bound,

@@ -103,7 +103,7 @@ __device__ __forceinline__ bool keep_polling(unsigned& polls, LazyHeader* h, uns
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kReduceThreads, 6)  // 80 registers: six CTAs per SM (bf16 spills 44 bytes)
+__global__ void __launch_bounds__(kReduceThreads, 6)  // at most 80 registers (bf16 79): six CTAs per SM
 decide_walk_lazy_kernel(const LazyParams p) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int b_own = blockIdx.x < p.B ? (int)blockIdx.x : -1;  // the sequence whose tail this CTA runs

@@ -249,7 +249,7 @@ lmhead_reduce_kernel(const __grid_constant__ LmMaps maps, const LmParams p) {
             uint8_t* dst = smem + stage * stage_bytes;
             mbar_arrive_expect_tx(full + stage, (uint32_t)(rows + nb * kBox) * 128u);
             used |= 1u << stage;
-            // as few instructions as the rows' number has binary digits: each takes its warp some 200 cycles
+            // as few instructions as the rows' number has binary digits: each takes its warp 85 to 105 cycles, some 200 among others
             auto load = [&](const CUtensorMap* m, uint8_t* to, int row, int n) {
 #pragma unroll
               for (int s = kBoxSizes - 1; s >= 0; --s) {
