@@ -55,7 +55,8 @@ decide_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V,
   // The one-CTA-per-sequence tail kernel may take its SM while this grid still runs (it waits there for
   // this grid to finish): its launch latency is hidden.  A CTA that has nothing to read says the same by
   // ending; triggering first costs the grid 0.5 ns for each of them, much of the call where few rows are
-  // still masked (one in twenty of 512 rows x 152064, 9728 CTAs: 18.0 us, 14.4 so; of 4 x 512 rows 49.2 and 30.6).
+  // still masked (one in twenty of 256 rows x 126464: 9.7 us, 8.2 so; of 512 x 152064, 9728 CTAs, beside an
+  // attention of 28 heads 25.6 and 21.5).
   if (early_trigger && (token == mask_id || waits)) pdl_launch_dependents();
 #endif
   if (token == mask_id)

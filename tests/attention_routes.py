@@ -4,6 +4,7 @@ import ctypes
 import functools
 import os
 import re
+import shutil
 import subprocess
 import tempfile
 
@@ -29,6 +30,7 @@ def _library():
                     "-isystem", cuda] + inc + [os.path.join(HERE, "host_runtime", "runtime.cpp")] + list(obj.values()) +
                    ["-o", so], check=True)
     lib = ctypes.CDLL(so)
+    shutil.rmtree(out)
     lib.fake_log.restype = ctypes.c_char_p
     lib.fake_reset.argtypes = [ctypes.c_char_p, ctypes.c_size_t, ctypes.c_size_t]
     return lib
