@@ -451,8 +451,11 @@ spiffy_status spiffy_decide_walk(const spiffy_decide_desc* desc, const void* log
 /*
  * Lazy chain evaluation of steps 1-5 of Algorithm 1: the decision is computed
  * only for the nodes the walk reaches (the true block, then each accepted
- * draft), level by level inside one kernel, instead of for all N nodes.  Only
- * 1 + n_accepted of the N nodes' logits are read.  The paper has no
+ * draft), level by level, instead of for all N nodes.  Of the N nodes' logits
+ * those on the path are read, and those of nodes that were likely to come next
+ * when their turn was worked out; what the latter hold has no part in any
+ * result.  All logits must be readable and complete, as for
+ * spiffy_decide_walk.  The paper has no
  * counterpart; it evaluates every draft's distribution (Sec. 4.3).
  *
  * Same arguments and layouts as spiffy_decide_walk.  On return
@@ -464,18 +467,15 @@ spiffy_status spiffy_decide_walk(const spiffy_decide_desc* desc, const void* log
  *   - walk_status reports a malformed parent list only if the walk scanned it;
  *     SPIFFY_DEV_TIMEOUT in both status words when a bounded wait between the
  *     levels ran out (results are then unspecified).
- * There is no grid-wide barrier: per sequence, the thread blocks that reduce
- * the current node's rows tag their results with the level, the block that owns
- * the sequence waits for those tags, decides, and publishes the next node with
- * its level, for which the reducers wait; sequences never wait for one
- * another.  A level still costs two such round trips through memory, so the
+ * Two kernels, no grid-wide barrier: the first reduces the true blocks' rows;
+ * in the second, per sequence, one thread block decides and publishes the next
+ * node while others reduce the current one's rows and then those of the first
+ * node that lists it as a parent.  Sequences never wait for one another.  The
  * call pays off when one node's share of the logits is large (long
- * vocabularies, batches) and loses to spiffy_decide_walk on a single short
- * graph.  SPIFFY_EUNSUPPORTED when the batch exceeds the number of thread blocks
- * the device holds at once.
+ * vocabularies, batches) or the graph has many nodes.  SPIFFY_EUNSUPPORTED when
+ * the batch exceeds the number of thread blocks the device holds at once.
  * Workspace: spiffy_decide_walk_lazy_workspace(desc); contents on entry
- * arbitrary (the call zeroes the few bytes it needs with a memset on the
- * stream).
+ * arbitrary (the call clears what it needs on the stream).
  */
 size_t spiffy_decide_walk_lazy_workspace(const spiffy_decide_desc* desc);
 spiffy_status spiffy_decide_walk_lazy(const spiffy_decide_desc* desc, const void* logits,

@@ -196,6 +196,8 @@ spiffy_status launch_attention_tc_dual(const spiffy_attn_desc& d0, const AttnPro
 //         itself launched behind one), so whatever wrote those arrays ahead of the call is
 //         complete.  spiffy_accept_walk called by itself has no such kernel in front: its
 //         contract in spiffy.h puts that on the caller.
+//         The lazy call's walk kernel reads all inputs of its call, logits included: it comes behind
+//         the root kernel, which waited.
 //     (b) The draft-build kernel reads the draft formulas, constants of the model.
 //     (c) The reduce under SPIFFY_INDEPENDENT and the attention under SPIFFY_ATTN_INDEPENDENT
 //         read their inputs, write their outputs and wait last.  What precedes them is, by the

@@ -10,6 +10,8 @@
 #pragma once
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace spiffy {
@@ -266,17 +268,42 @@ __device__ __forceinline__ Partial reduce_slice(const T* __restrict__ base, int 
   return r;
 }
 
+// Sixteen bytes that another CTA may be writing, in one access.
+__device__ __forceinline__ int4 load16(const void* p) {
+  uint64_t a, b;
+  asm volatile("{\n.reg .b128 t;\nld.relaxed.gpu.global.b128 t, [%2];\nmov.b128 {%0, %1}, t;\n}"
+               : "=l"(a), "=l"(b)
+               : "l"(p)
+               : "memory");
+  return make_int4((int)(uint32_t)a, (int)(uint32_t)(a >> 32), (int)(uint32_t)b, (int)(uint32_t)(b >> 32));
+}
+
+// How finalize_row comes by a row's slices.  Complete: they are all there, written by an earlier kernel.
+// They are read at L2, as this CTA may have been resident while that kernel wrote them.
+struct CompleteSlices {
+  static constexpr bool kWaits = false;
+};
+// They are being written: a slice is there when its spare word is `tag`.  At most `polls` looks at a batch
+// of slices; `missing` when they ran out, and the row's results mean nothing.
+struct TaggedSlices {
+  static constexpr bool kWaits = true;
+  int tag;
+  unsigned polls;
+  bool missing = false;
+};
+
 // kLanes (8, 4, 2 or 1) neighbouring lanes merge the slices of one row and lane
 // 0 of the group gets the row's confidence and top token (Algorithm 1, steps
 // 1-2).  The order is fixed and the same for every kLanes: eight accumulators
 // (accumulator j takes slices j, j + 8, ...) are combined by the butterfly
 // 4, 2, 1 with the lower index first; a lane holds the accumulators j = sub,
 // sub + kLanes, ... and does the butterfly steps that stay inside it locally.
-// Returns false on lane 0 when the row is masked and not usable.  kShared: the slices are in
-// shared memory.
-template <int kLanes, bool kShared = false>
+// Returns false on lane 0 when the row is masked and not usable.
+template <int kLanes, class Source = CompleteSlices>
 __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int splits, int sub,
-                                             int32_t state, int mask_id, float& conf, int32_t& tok) {
+                                             int32_t state, int mask_id, float& conf, int32_t& tok,
+                                             Source&& from = Source{}) {
+  constexpr bool kWaits = std::remove_reference_t<Source>::kWaits;
   constexpr int kAcc = 8 / kLanes;
   float m[kAcc], s[kAcc];
   int idx[kAcc];
@@ -292,15 +319,30 @@ __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int 
   constexpr int kBatch = kAcc > 4 ? kAcc : 4;
   for (int t0 = 0; sub + kLanes * t0 < splits; t0 += kBatch) {
     Partial q[kBatch];
+    auto fetch = [&]() {
+      bool all = true;
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int k = sub + kLanes * (t0 + u);
-      q[u] = Partial{-INFINITY, 0.f, 0x7fffffff, 0};
-      if (k < splits && state == mask_id) {  // read at L2: another grid wrote these while this CTA may already have been resident; the slices of an unmasked row were never written
-        const int4* at = reinterpret_cast<const int4*>(p + k);
-        const int4 w = kShared ? *at : __ldcg(at);
-        q[u] = Partial{__int_as_float(w.x), __int_as_float(w.y), w.z, w.w};
+      for (int u = 0; u < kBatch; ++u) {
+        const int k = sub + kLanes * (t0 + u);
+        q[u] = Partial{-INFINITY, 0.f, 0x7fffffff, 0};
+        if (k < splits && state == mask_id) {  // the slices of an unmasked row were never written
+          const int4 w = kWaits ? load16(p + k) : __ldcg(reinterpret_cast<const int4*>(p + k));
+          q[u] = Partial{__int_as_float(w.x), __int_as_float(w.y), w.z, w.w};
+        }
       }
+      if constexpr (kWaits) {
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u)
+          if (sub + kLanes * (t0 + u) < splits && state == mask_id) all &= q[u].pad == from.tag;
+      }
+      return all;
+    };
+    if constexpr (kWaits) {
+      unsigned polls = from.polls;
+      while (!from.missing && !fetch())
+        if (polls-- == 0) from.missing = true;
+    } else {
+      fetch();
     }
 #pragma unroll
     for (int u = 0; u < kBatch; ++u)

@@ -218,6 +218,38 @@ def test_lazy_call_with_more_items_than_resident_thread_blocks(B, N, L, V, dtype
     assert hops > B  # deep walks: several levels per sequence
 
 
+@pytest.mark.parametrize("B,N,L,V,pad", [(2, 64, 16, 600, 0), (2, 65, 16, 600, 0), (1, 120, 4, 100, 0),  # children: table or lists
+                                         (2, 20, 32, 500, 20000),  # lists too long for shared memory
+                                         (500, 3, 4, 52, 0), (888, 2, 4, 52, 0)])  # more sequences than reducing blocks, none
+def test_lazy_call_at_the_edges_of_its_roles(B, N, L, V, pad):
+    logits, tokens, off, idx, mask = random_case(B * 7 + N, B, N, L, V, p_accept=0.9)
+    if pad:
+        idx = np.concatenate([idx, np.full((B, pad), 3, idx.dtype)], axis=1)
+    hops = 0
+    for rule, S in ((spiffy.RULE_TOPS, 1), (spiffy.RULE_TOPS, 2), (spiffy.RULE_THRESHOLD, 1)):
+        _, lwalk, _ = lazy_vs_eager(logits, tokens, off, idx, mask, rule, S, 0.5)
+        assert int(lwalk.dev_status.sum()) == 0
+        hops += int(lwalk.n_accepted.sum())
+    assert hops > 0
+
+
+def test_lazy_call_reports_malformed_lists_it_scanned():
+    """A bad offset or entry anywhere behind the true block: the eager call's status, the walk of the good lists."""
+    for spoil in ("entry", "offset"):
+        logits, tokens, off, idx, mask = random_case(5, 3, 12, 16, 300, p_accept=0.9)
+        if spoil == "entry":
+            idx[1, off[1, 8]] = 11  # node 8 lists a later node
+        else:
+            off[1, 9] = -4
+        lg, tk, of, ix = (G.to_dev(a) for a in (logits, tokens, off, idx))
+        _, want = spiffy.spiffy_decide_walk(lg, tk, of, ix, mask, spiffy.RULE_TOPS)
+        _, got = spiffy.spiffy_decide_walk(lg, tk, of, ix, mask, spiffy.RULE_TOPS, lazy=True)
+        torch.cuda.synchronize()
+        assert want.dev_status.tolist() == [0, spiffy.DEV_BADGRAPH, 0]
+        for f in ("dev_status", "accepted_node", "n_accepted", "path", "next_block"):
+            assert torch.equal(getattr(want, f), getattr(got, f)), (spoil, f)
+
+
 def test_lazy_chain_evaluation_at_the_benchmark_shapes():
     for index, cases in ((2, 2), (3, 1)):
         cfg = W.config(index)
