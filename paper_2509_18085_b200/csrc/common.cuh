@@ -198,7 +198,8 @@ spiffy_status launch_attention_tc_dual(const spiffy_attn_desc& d0, const AttnPro
 //         contract in spiffy.h puts that on the caller.
 //         The lazy call's walk kernel reads all inputs of its call, logits included: it comes behind
 //         the root kernel, which waited.
-//     (b) The draft-build kernel reads the draft formulas, constants of the model.
+//     (b) The draft-build kernel reads the draft formulas, constants of the model, and the block, as the
+//         top-k kernel in front of it waited before it let it start.
 //     (c) The reduce under SPIFFY_INDEPENDENT and the attention under SPIFFY_ATTN_INDEPENDENT
 //         read their inputs, write their outputs and wait last.  What precedes them is, by the
 //         flags' contract, a call that touches none of these; its kernels started, in turn,

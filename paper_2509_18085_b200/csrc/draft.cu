@@ -14,6 +14,8 @@
 //                       lists.
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace spiffy {
@@ -24,6 +26,7 @@ constexpr int kVecs = 8;       // 128-bit vectors per thread
 constexpr int kMaxK = 4;       // vocabulary ranks
 constexpr int kBuildThreads = 1024;  // a warp per block position
 constexpr int kRelated = 64;         // formulas whose subset relation fits its table
+constexpr int kFormulaBytes = 4096;  // shared memory for what is known about so many
 constexpr int kGraphInts = 6144;     // shared-memory copy of the draft graph (24 KB)
 
 struct __align__(16) TopPartial {
@@ -244,75 +247,131 @@ __device__ bool strict_subset(const BuildArgs& g, int a, int c) {
   return true;
 }
 
-// grid = B sequences, 1024 threads; dynamic shared memory, see the carve-up below.
+// grid = B sequences, a warp per block position (at most kBuildThreads); dynamic shared memory, see
+// build_smem_bytes.
+//
+// A chain of small steps in one CTA: what bounds it is how many dependent accesses it is long and how many
+// instructions it meets for the first time (some five cycles each), not how much it does.  All that does not
+// depend on the logits is worked out ahead of the wait: the graph copied to shared memory, each formula as a
+// set of bits, which formulas contain which, the block's masked positions.  Behind the wait a warp merges each
+// position's slices and takes its logarithms, a second step sorts the positions, and one warp, a formula a
+// lane, does the rest without another barrier, in loops that are not unrolled.  32 positions x 16 slices, ten
+// formulas: 4600 cycles to the wait and 14200 behind it with 1024 threads at eight barriers, formulas looked up
+// through generic pointers pair by pair, logarithms inside the chains and merges by shuffles; 4500 and 7900
+// now (the call 13.0 -> 9.8 us).  The whole chain gone through once beforehand, to have its instructions at
+// hand, takes longer than the top-k kernel leaves time for (22 us).
 __global__ void __launch_bounds__(kBuildThreads)
 draft_build_kernel(BuildArgs g) {
   const int b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int threads = blockDim.x, warps = threads >> 5;
   const int L = g.L, K = g.K, D = g.D;
-  extern __shared__ __align__(8) unsigned char draft_smem[];
-  float* cand_p = reinterpret_cast<float*>(draft_smem);      // [L][kMaxK]
-  int* cand_tok = reinterpret_cast<int*>(cand_p + L * kMaxK);  // [L][kMaxK]
-  int* pos_of_rank = cand_tok + L * kMaxK;                   // [L]
-  int* now = pos_of_rank + L;                                // [L] the current block
-  float* local = reinterpret_cast<float*>(now + L);          // [D]
-  float* total = local + D;                                  // [D]
-  int* keep = reinterpret_cast<int*>(total + D);             // [D] slot + 1 of a kept formula, else 0
-  int* node_formula = keep + D;                              // [budget + 1] formula of each node, -1 for node 0 / padding
-  int* n_parents = node_formula + g.budget + 1;              // [budget + 1]
-  __shared__ int n_masked;
-  const int32_t* state = g.state + (int64_t)b * L;
-  if (tid == 0) n_masked = 0;
-  // The formulas are walked several times with dependent reads: when the graph
-  // fits, copy it to shared memory and walk it there.  The draft graph is a
-  // constant of the model (calibrated offline), not the product of earlier work on
-  // the stream, so it is fetched before the wait on that work.
+  extern __shared__ __align__(16) unsigned char draft_smem[];
+  // of graphs of up to kRelated formulas
+  struct Formulas {
+    uint64_t sets[kRelated][kMaxK];           // bit i of word j: a formula has candidate (i, j)
+    unsigned subsets[kRelated][kRelated / 32];  // bit a of row c: formula a < c is a strict subset of c
+    int ranks_needed[kRelated];               // position ranks a formula asks for; INT_MAX: never built
+    float log[kRelated + 1];                  // ln of a local score
+    float local[kRelated + 1];                // the last one stands for children that do not exist: never built
+    alignas(16) float total[kRelated];
+  };
+  static_assert(sizeof(Formulas) <= kFormulaBytes, "dynamic shared memory");
+  Formulas& fs = *reinterpret_cast<Formulas*>(draft_smem);
+  // of larger ones
+  float* local = reinterpret_cast<float*>(draft_smem);  // [D]
+  float* total = local + D;                             // [D]
+  int* keep = reinterpret_cast<int*>(total + D);        // [D] whether a formula is kept
+  int* node_formula = keep + D;                         // [budget + 1] formula of each node, -1 for node 0 / padding
+  int* n_parents = node_formula + g.budget + 1;         // [budget + 1]
+  __shared__ int now[64];                          // the current block
+  __shared__ float top_p[64];                      // largest probability of a position, -1 of an unmasked one
+  __shared__ float by_rank_log[64 * kMaxK];        // by position rank and vocabulary rank: ln of a candidate's
+  __shared__ int by_rank_tok[64 * kMaxK];          // probability (-inf: none), its token
+  __shared__ int pos_of_rank[64];
   __shared__ int32_t graph_smem[kGraphInts];
-  {
-    const int npairs = g.formula_off[D], nkids = g.child_off[D];
-    if (2 * (D + 1) + 2 * npairs + nkids <= kGraphInts) {
-      int32_t* f_off = graph_smem;
-      int32_t* c_off = f_off + D + 1;
-      int32_t* f_i = c_off + D + 1;
-      int32_t* f_j = f_i + npairs;
-      int32_t* c_idx = f_j + npairs;
-      for (int i = tid; i <= D; i += kBuildThreads) { f_off[i] = g.formula_off[i]; c_off[i] = g.child_off[i]; }
-      for (int i = tid; i < npairs; i += kBuildThreads) { f_i[i] = g.formula_i[i]; f_j[i] = g.formula_j[i]; }
-      for (int i = tid; i < nkids; i += kBuildThreads) c_idx[i] = g.child_idx[i];
-      g.formula_off = f_off; g.child_off = c_off; g.formula_i = f_i; g.formula_j = f_j; g.child_idx = c_idx;
-    }
+  const int32_t* state = g.state + (int64_t)b * L;
+  // The draft graph is a constant of the model (calibrated offline), not the product of earlier work on the
+  // stream; and the top-k kernel waited before it let this one start, so that the state is complete.
+  // All loads that depend on nothing go out first.
+  const int npairs = g.formula_off[D], nkids = g.child_off[D];
+  const int f_mine = tid <= D ? g.formula_off[tid] : 0, c_mine = tid <= D ? g.child_off[tid] : 0;
+  const int32_t t0 = lane < L ? state[lane] : ~g.mask_id, t1 = lane + 32 < L ? state[lane + 32] : ~g.mask_id;
+  for (int l = tid; l < 64; l += threads) pos_of_rank[l] = 0;  // ranks that rows without a distribution leave out
+  for (int i = tid; i < 64 * kMaxK; i += threads) {
+    by_rank_log[i] = -INFINITY;
+    by_rank_tok[i] = 0;
   }
-  // Which formulas are strict subsets of which, for the parent lists: also known before the wait.
-  // Bit a of subsets[c]: a < c is one of c's.  Graphs of more formulas find it out when needed.
-  __shared__ unsigned subsets[kRelated][kRelated / 32];
-  const bool related = D <= kRelated;
-  if (related) {
-    for (int i = tid; i < kRelated * (kRelated / 32); i += kBuildThreads) (&subsets[0][0])[i] = 0u;
-    __syncthreads();
-    for (int i = tid; i < D * D; i += kBuildThreads) {
-      const int c = i / D, a = i - c * D;
-      if (a < c && strict_subset(g, a, c)) atomicOr(&subsets[c][a >> 5], 1u << (a & 31));
+  const bool staged = 2 * (D + 1) + 2 * npairs + nkids <= kGraphInts, one_warp = staged && D <= kRelated;
+  int32_t* const f_off = graph_smem;
+  int32_t* const c_off = f_off + D + 1;
+  int32_t* const f_i = c_off + D + 1;
+  int32_t* const f_j = f_i + npairs;
+  int32_t* const c_idx = f_j + npairs;
+  if (staged) {
+    if (tid <= D) { f_off[tid] = f_mine; c_off[tid] = c_mine; }
+    for (int i = tid + threads; i <= D; i += threads) { f_off[i] = g.formula_off[i]; c_off[i] = g.child_off[i]; }
+    for (int i = tid; i < npairs; i += threads) { f_i[i] = g.formula_i[i]; f_j[i] = g.formula_j[i]; }
+    for (int i = tid; i < nkids; i += threads) {
+      const int x = g.child_idx[i];
+      c_idx[i] = one_warp && (x < 0 || x >= D) ? kRelated : x;
     }
+    g.formula_off = f_off; g.child_off = c_off; g.formula_i = f_i; g.formula_j = f_j; g.child_idx = c_idx;
+  }
+  const uint64_t masked_bits = (uint64_t)__ballot_sync(0xffffffffu, t0 == g.mask_id) |
+                               (uint64_t)__ballot_sync(0xffffffffu, t1 == g.mask_id) << 32;
+  const int masked = __popcll(masked_bits);
+  if (warp == 0) {
+    now[lane] = t0;
+    now[lane + 32] = t1;
+  }
+  __syncthreads();
+  if (one_warp) {
+    if (tid == 0) fs.local[kRelated] = -INFINITY;
+    if (tid < kRelated) fs.total[tid] = -INFINITY;
+    for (int q = tid; q < D; q += threads) {
+      uint64_t set[kMaxK] = {};
+      const int e0 = f_off[q], e1 = f_off[q + 1];
+      int need = e1 > e0 ? 0 : 0x7fffffff;
+#pragma unroll 1
+      for (int e = e0; e < e1; ++e) {
+        const int i = f_i[e], j = f_j[e];
+        const bool exists = i >= 0 && i < 64 && j >= 0 && j < K;
+        need = exists ? max(need, i + 1) : 0x7fffffff;
+#pragma unroll
+        for (int t = 0; t < kMaxK; ++t)
+          if (exists && t == j) set[t] |= 1ull << i;
+      }
+#pragma unroll
+      for (int t = 0; t < kMaxK; ++t) fs.sets[q][t] = set[t];
+      fs.ranks_needed[q] = need;
+    }
+    __syncthreads();
+    for (int w = warp; w < D * (kRelated / 32); w += warps) {  // a warp per word, its lanes over the smaller formulas
+      const int c = w / (kRelated / 32), a = w % (kRelated / 32) * 32 + lane;
+      bool sub = a < c && f_off[a + 1] - f_off[a] < f_off[c + 1] - f_off[c];
+      if (sub) {
+#pragma unroll
+        for (int t = 0; t < kMaxK; ++t) sub &= (fs.sets[a][t] & ~fs.sets[c][t]) == 0ull;
+      }
+      const unsigned word = __ballot_sync(0xffffffffu, sub);
+      if (lane == 0) fs.subsets[c][w % (kRelated / 32)] = word;
+    }
+    __syncthreads();
   }
 #if __CUDA_ARCH__ >= 900
-  cudaGridDependencySynchronize();  // the top-k kernel's partial results, and the caller's logits and state, are visible
+  cudaGridDependencySynchronize();  // the top-k kernel's partial results are visible, the outputs free
 #endif
-  __syncthreads();
+  int32_t* tokens = g.tokens + (int64_t)b * (g.budget + 1) * L;
 
   // 1. candidates c_ij and their probabilities: one warp per position
-  for (int l = warp; l < L; l += kBuildThreads / 32) {
+  float cand_log[2] = {};  // lane r: that of vocabulary rank r, of the warp's first and second position
+  int cand_tok[2] = {};
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int l = warp + h * warps;  // two rounds are enough for 64 positions, as there are min(L, 32) warps
+    if (l >= L) break;
     const TopPartial* p = g.partials + ((int64_t)b * L + l) * g.splits;
-    // read together with the token (one trip); those of an unmasked row were never written and are ignored
-    uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0, q2 = q0;
-    if (g.splits <= 32 && lane < g.splits) {
-      const uint4* q = reinterpret_cast<const uint4*>(p + lane);
-      q0 = __ldcg(q); q1 = __ldcg(q + 1); q2 = __ldcg(q + 2);
-    }
-    const int32_t token = state[l];
-    if (lane == 0) now[l] = token;
-    if (token != g.mask_id) {
-      if (lane < kMaxK) { cand_p[l * kMaxK + lane] = -1.f; cand_tok[l * kMaxK + lane] = token; }
-      continue;
-    }
+    const bool is_masked = (masked_bits >> l & 1ull) != 0ull;
     float m = -INFINITY, s = 0.f;
     float hv[kMaxK];
     int hi[kMaxK];
@@ -321,27 +380,26 @@ draft_build_kernel(BuildArgs g) {
     if (g.splits <= 32) {
       // one slice per lane, fetched whole in one trip: its maximum and sum, and its K
       // candidates, which the top-k kernel left sorted
-      if (lane < g.splits) {
+      if (is_masked && lane < g.splits) {
+        const uint4* q = reinterpret_cast<const uint4*>(p + lane);
+        const uint4 q0 = __ldcg(q), q1 = __ldcg(q + 1), q2 = __ldcg(q + 2);
         m = __uint_as_float(q0.x);
         s = __uint_as_float(q0.y);
         hv[0] = __uint_as_float(q0.z); hv[1] = __uint_as_float(q0.w);
         hv[2] = __uint_as_float(q1.x); hv[3] = __uint_as_float(q1.y);
         hi[0] = (int)q1.z; hi[1] = (int)q1.w; hi[2] = (int)q2.x; hi[3] = (int)q2.y;
-#pragma unroll
-        for (int t = 0; t < kMaxK; ++t)
-          if (t >= K || hv[t] == -INFINITY) { hv[t] = -INFINITY; hi[t] = 0x7fffffff; }
       }
-    } else {
+    } else if (is_masked) {
       // maximum and sum over the slices, fixed order
       for (int k = lane; k < g.splits; k += 32) {
-        const float m2 = p[k].m, s2 = p[k].s, M = fmaxf(m, m2);
+        const float m2 = __ldcg(&p[k].m), s2 = __ldcg(&p[k].s), M = fmaxf(m, m2);
         s = s * ((m == M) ? 1.f : ex2((m - M) * kLog2e)) + s2 * ((m2 == M) ? 1.f : ex2((m2 - M) * kLog2e));
         m = M;
       }
       // every lane sorts the candidates it reads (each is read once)
       for (int c = lane; c < g.splits * K; c += 32) {
-        float v = p[c / K].val[c % K];
-        int i = p[c / K].idx[c % K];
+        float v = __ldcg(&p[c / K].val[c % K]);
+        int i = __ldcg(&p[c / K].idx[c % K]);
         if (v == -INFINITY) continue;
 #pragma unroll
         for (int t = 0; t < kMaxK; ++t)  // insertion into the sorted list
@@ -351,157 +409,256 @@ draft_build_kernel(BuildArgs g) {
           }
       }
     }
+    // every draft starts as the current block
+    for (int n = lane; n <= g.budget; n += 32) tokens[n * L + l] = now[l];
+    float p_top = -1.f;
+    if (is_masked) {
+      const float M = warp_max(m);
+      s *= m == M ? 1.f : ex2((m - M) * kLog2e);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const float m2 = __shfl_xor_sync(0xffffffffu, m, off), s2 = __shfl_xor_sync(0xffffffffu, s, off);
-      const float M = fmaxf(m, m2);
-      s = s * ((m == M) ? 1.f : ex2((m - M) * kLog2e)) + s2 * ((m2 == M) ? 1.f : ex2((m2 - M) * kLog2e));
-      m = M;
+      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+      // the K best of the slices' candidates (value desc, id asc): K rounds pick the best
+      // head over the lanes and pop it; lane r keeps the best of round r
+      float mine = -INFINITY;
+      int mine_tok = 0x7fffffff;
+#pragma unroll 1
+      for (int r = 0; r < K; ++r) {
+        const float bv = warp_max(hv[0]);
+        const int bi = (int)__reduce_min_sync(0xffffffffu, hv[0] == bv ? (unsigned)hi[0] : 0x7fffffffu);
+        if (hi[0] == bi) {  // this lane's head won, if there is any: pop it
+#pragma unroll
+          for (int t = 0; t + 1 < kMaxK; ++t) { hv[t] = hv[t + 1]; hi[t] = hi[t + 1]; }
+          hv[kMaxK - 1] = -INFINITY;
+          hi[kMaxK - 1] = 0x7fffffff;
+        }
+        if (lane == r) {
+          mine = bv;
+          mine_tok = bi;
+        }
+      }
+      p_top = mine == -INFINITY ? 0.f : ex2((mine - M) * kLog2e) / s;
+      cand_tok[h] = mine_tok;
+      cand_log[h] = p_top > 0.f ? logf(fmaxf(p_top, 1e-45f)) : -INFINITY;
+      if (lane == 0 && (!(fabsf(M) < INFINITY) || !(s > 0.f) || !(s < INFINITY)) && g.dev_status)
+        atomicOr(g.dev_status + b, SPIFFY_DEV_NONFINITE);
     }
-    if (lane == 0 && (!(fabsf(m) < INFINITY) || !(s > 0.f) || !(s < INFINITY)) && g.dev_status)
-      atomicOr(g.dev_status + b, SPIFFY_DEV_NONFINITE);
-    // the K best of the slices' candidates (value desc, id asc): K rounds pick the best
-    // head over the lanes and pop it
-    for (int r = 0; r < K; ++r) {
-      float bv = hv[0];
-      int bi = hi[0];
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const float v2 = __shfl_xor_sync(0xffffffffu, bv, off);
-        const int i2 = __shfl_xor_sync(0xffffffffu, bi, off);
-        if (ahead(v2, i2, bv, bi)) { bv = v2; bi = i2; }
-      }
-      if (hi[0] == bi && bv != -INFINITY) {  // this lane's head won: pop it
-#pragma unroll
-        for (int t = 0; t + 1 < kMaxK; ++t) { hv[t] = hv[t + 1]; hi[t] = hi[t + 1]; }
-        hv[kMaxK - 1] = -INFINITY;
-        hi[kMaxK - 1] = 0x7fffffff;
-      }
-      if (lane == 0) {
-        cand_tok[l * kMaxK + r] = bi;
-        cand_p[l * kMaxK + r] = bv == -INFINITY ? 0.f : ex2((bv - m) * kLog2e) / s;
-      }
-    }
-    if (lane == 0) atomicAdd(&n_masked, 1);
+    if (lane == 0) top_p[l] = p_top;
   }
   __syncthreads();
   // 2. token position ranks (Eq. token-position-sort): by maximum probability, ties to the lower position
-  for (int l = warp; l < L; l += kBuildThreads / 32) {  // a warp per position, its lanes over the others
-    const float pl = cand_p[l * kMaxK];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int l = warp + h * warps;
+    if (l >= L) break;
+    const float pl = top_p[l];
     if (pl < 0.f) continue;  // unmasked
     int rank = 0;
-    for (int j0 = 0; j0 < L; j0 += 32) {
+#pragma unroll
+    for (int j0 = 0; j0 < 64; j0 += 32) {
+      if (j0 >= L) break;
       const int j = j0 + lane;
-      const float pj = j < L ? cand_p[j * kMaxK] : -1.f;
+      const float pj = j < L ? top_p[j] : -1.f;
       rank += __popc(__ballot_sync(0xffffffffu, pj >= 0.f && (pj > pl || (pj == pl && j < l))));
     }
     if (lane == 0) pos_of_rank[rank] = l;
+    if (lane < K) {
+      by_rank_log[rank * kMaxK + lane] = cand_log[h];
+      by_rank_tok[rank * kMaxK + lane] = cand_tok[h];
+    }
   }
   __syncthreads();
-  // 3. local score of every formula: geometric mean of its candidates' probabilities
-  for (int q = tid; q < D; q += kBuildThreads) {
+  int32_t* out_off = g.parent_off + (int64_t)b * (g.budget + 2);
+  int32_t* out_idx = g.parent_idx + (int64_t)b * g.parent_cap;
+  int32_t* out_kept = g.kept + (int64_t)b * g.budget;
+
+  if (one_warp) {
+    // Two warps with the same numbers: what follows from them is written by one or the other.
+    if (warp > 1) return;
+    const bool lists = warp == 0, drafts = warp == 1 || warps == 1;
+#pragma unroll 1
+    for (int q = lane; q < D; q += 32) {  // 3. local scores: geometric means of the candidates' probabilities
+      const int e0 = f_off[q], e1 = f_off[q + 1];
+      float x = -INFINITY, lg = -INFINITY;
+      if (fs.ranks_needed[q] <= masked) {
+        float logsum = 0.f;
+#pragma unroll 2
+        for (int e = e0; e < e1; ++e) logsum += by_rank_log[f_i[e] * kMaxK + f_j[e]];
+        x = expf(logsum / (float)(e1 - e0));  // 0 where a candidate has no probability
+        lg = x > 0.f ? logf(fmaxf(x, 1e-45f)) : -INFINITY;
+      }
+      fs.local[q] = x;
+      fs.log[q] = lg;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int q = lane; q < D; q += 32) {  // 4. score = GM(local, GM(children's)); without buildable children local
+      float x = fs.local[q];
+      if (x != -INFINITY) {
+        float logsum = 0.f;
+        int n = 0;
+        const int e1 = c_off[q + 1];
+#pragma unroll 2
+        for (int e = c_off[q]; e < e1; ++e) {
+          const int y = c_idx[e];
+          if (fs.local[y] == -INFINITY) continue;
+          logsum += fs.log[y];
+          ++n;
+        }
+        if (n > 0) x = sqrtf(x * expf(logsum / (float)n));
+      }
+      fs.total[q] = x;
+      if (lists) g.score[(int64_t)b * D + q] = x;
+    }
+    __syncwarp();
+    uint64_t keep_bits = 0;  // 5. the D* best (score desc, formula index asc) keep their formula order
+#pragma unroll 1
+    for (int q = lane; q < D + lane; q += 32) {  // all lanes
+      const float mine = q < D ? fs.total[q] : -INFINITY;
+      int rank = 0;
+#pragma unroll 1
+      for (int x = 0; x < D; x += 4) {  // behind the last one -inf
+        const float4 t = *reinterpret_cast<const float4*>(fs.total + x);
+        rank += ((t.x > mine) | ((t.x == mine) & (x < q))) + ((t.y > mine) | ((t.y == mine) & (x + 1 < q))) +
+                ((t.z > mine) | ((t.z == mine) & (x + 2 < q))) + ((t.w > mine) | ((t.w == mine) & (x + 3 < q)));
+      }
+      keep_bits |= (uint64_t)__ballot_sync(0xffffffffu, mine != -INFINITY && rank < g.budget) << (q - lane);
+    }
+    // 6., 7. kept drafts' tokens, and parent lists: every earlier kept node whose candidate set is a
+    // strict subset, the current block (node 0, the empty set) among them
+    int base = 0;
+#pragma unroll 1
+    for (int q = lane; q < D + lane; q += 32) {
+      const uint64_t before = keep_bits & ((1ull << q) - 1ull);
+      const int node = 1 + __popcll(before);
+      // (scores that are no numbers have no order, and more of them than the budget may have been kept)
+      const bool kept = (keep_bits >> q & 1ull) != 0ull && node <= g.budget;
+      if (kept && drafts) {
+        out_kept[node - 1] = q;
+        const int e1 = f_off[q + 1];
+#pragma unroll 1
+        for (int e = f_off[q]; e < e1; ++e) tokens[node * L + pos_of_rank[f_i[e]]] = by_rank_tok[f_i[e] * kMaxK + f_j[e]];
+      }
+      if (!lists) continue;
+      uint64_t parents = kept ? ((uint64_t)fs.subsets[q][0] | (uint64_t)fs.subsets[q][1] << 32) & before : 0ull;
+      const int count = kept ? 1 + __popcll(parents) : 0;
+      int upto = count;
+#pragma unroll 1
+      for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, upto, off);
+        if (lane >= off) upto += y;
+      }
+      int at = base + upto - count;
+      base += __shfl_sync(0xffffffffu, upto, 31);
+      if (kept) {
+        out_off[node] = min(at, g.parent_cap);
+        if (at < g.parent_cap) out_idx[at] = 0;
+#pragma unroll 1
+        for (; parents; parents &= parents - 1) {
+          ++at;
+          if (at < g.parent_cap) out_idx[at] = 1 + __popcll(keep_bits & ((parents & (0ull - parents)) - 1ull));
+        }
+      }
+    }
+    const int nodes = min(__popcll(keep_bits), g.budget);
+    if (drafts)
+      for (int n = nodes + lane; n < g.budget; n += 32) out_kept[n] = -1;
+    if (lists) {
+      if (lane == 0) {
+        out_off[0] = 0;
+        if (base > g.parent_cap && g.dev_status) atomicOr(g.dev_status + b, SPIFFY_DEV_BADGRAPH);
+      }
+      for (int n = nodes + lane; n <= g.budget; n += 32) out_off[n + 1] = min(base, g.parent_cap);
+      if (g.fill_parents)
+        for (int i = base + lane; i < g.parent_cap; i += 32) out_idx[i] = 0;
+    }
+    return;
+  }
+
+  // Larger graphs: the same steps, by all threads.
+  for (int q = tid; q < D; q += threads) {
     const int e0 = g.formula_off[q], e1 = g.formula_off[q + 1];
     bool ok = e1 > e0;
     float logsum = 0.f;
-    bool zero = false;
     for (int e = e0; e < e1 && ok; ++e) {
       const int i = g.formula_i[e], j = g.formula_j[e];
-      if (i < 0 || i >= n_masked || j < 0 || j >= K) { ok = false; break; }
-      const float pr = cand_p[pos_of_rank[i] * kMaxK + j];
-      zero |= !(pr > 0.f);
-      logsum += logf(fmaxf(pr, 1e-45f));
+      if (i < 0 || i >= masked || j < 0 || j >= K) { ok = false; break; }
+      logsum += by_rank_log[i * kMaxK + j];
     }
-    local[q] = !ok ? -INFINITY : (zero ? 0.f : expf(logsum / (float)(e1 - e0)));
+    local[q] = !ok ? -INFINITY : expf(logsum / (float)(e1 - e0));
   }
   __syncthreads();
-  // 4. score = GM(local, GM(children's local scores)); a draft without buildable children keeps its local score
-  for (int q = tid; q < D; q += kBuildThreads) {
+  for (int q = tid; q < D; q += threads) {
     float sc = local[q];
     if (sc != -INFINITY) {
       float logsum = 0.f;
       int n = 0;
-      bool zero = false;
       for (int e = g.child_off[q]; e < g.child_off[q + 1]; ++e) {
         const int x = g.child_idx[e];
         if (x < 0 || x >= D || local[x] == -INFINITY) continue;
-        zero |= !(local[x] > 0.f);
-        logsum += logf(fmaxf(local[x], 1e-45f));
+        logsum += local[x] > 0.f ? logf(fmaxf(local[x], 1e-45f)) : -INFINITY;
         ++n;
       }
-      if (n > 0) {
-        const float child = zero ? 0.f : expf(logsum / (float)n);
-        sc = sqrtf(sc * child);
-      }
+      if (n > 0) sc = sqrtf(sc * expf(logsum / (float)n));
     }
     total[q] = sc;
     g.score[(int64_t)b * D + q] = sc;
   }
   __syncthreads();
-  // 5. the D* best (score desc, formula index asc) keep their formula order
-  for (int q = tid; q < D; q += kBuildThreads) {
+  for (int q = tid; q < D; q += threads) {
     int rank = 0;
     const float sq = total[q];
-    for (int x = 0; x < D; ++x)
-      rank += (total[x] != -INFINITY && (total[x] > sq || (total[x] == sq && x < q))) ? 1 : 0;
+    for (int x = 0; x < D; ++x) rank += (total[x] > sq || (total[x] == sq && x < q)) ? 1 : 0;
     keep[q] = (sq != -INFINITY && rank < g.budget) ? 1 : 0;
   }
-  for (int n = tid; n <= g.budget; n += kBuildThreads) node_formula[n] = -1;
+  for (int n = tid; n <= g.budget; n += threads) node_formula[n] = -1;
   __syncthreads();
-  for (int q = tid; q < D; q += kBuildThreads) {
+  for (int q = tid; q < D; q += threads) {
     if (!keep[q]) continue;
     int slot = 0;
     for (int x = 0; x < q; ++x) slot += keep[x];
-    node_formula[slot + 1] = q;
+    if (slot < g.budget) node_formula[slot + 1] = q;
   }
   __syncthreads();
-  // 6. blocks: the current block, then each kept draft = current block + its candidates
-  int32_t* tokens = g.tokens + (int64_t)b * (g.budget + 1) * L;
-  for (int i = tid; i < (g.budget + 1) * L; i += kBuildThreads) tokens[i] = now[i % L];
-  for (int n = tid; n < g.budget; n += kBuildThreads) g.kept[(int64_t)b * g.budget + n] = node_formula[n + 1];
-  __syncthreads();
-  for (int n = 1 + warp; n <= g.budget; n += kBuildThreads / 32) {
+  for (int n = tid; n < g.budget; n += threads) out_kept[n] = node_formula[n + 1];
+  for (int n = 1 + tid; n <= g.budget; n += threads) {
     const int q = node_formula[n];
     if (q < 0) continue;
-    for (int e = g.formula_off[q] + lane; e < g.formula_off[q + 1]; e += 32) {
-      const int l = pos_of_rank[g.formula_i[e]];
-      tokens[n * L + l] = cand_tok[l * kMaxK + g.formula_j[e]];
+    for (int e = g.formula_off[q]; e < g.formula_off[q + 1]; ++e) {
+      const int i = g.formula_i[e];
+      tokens[n * L + pos_of_rank[i]] = by_rank_tok[i * kMaxK + g.formula_j[e]];
     }
   }
-  // 7. parent lists: every earlier kept node whose candidate set is a strict subset.
-  // One warp per child, its lanes over the candidate parents.
+  // parent lists: one warp per child, its lanes over the candidate parents
   auto is_parent = [&](int a, int c) {
     if (a >= c || (a > 0 && node_formula[a] < 0)) return false;
-    const int fa = a == 0 ? -1 : node_formula[a], fc = node_formula[c];
-    return related && fa >= 0 ? ((subsets[fc][fa >> 5] >> (fa & 31)) & 1u) != 0u : strict_subset(g, fa, fc);
+    return strict_subset(g, a == 0 ? -1 : node_formula[a], node_formula[c]);
   };
-  for (int c = warp; c <= g.budget; c += kBuildThreads / 32) {
+  for (int c = warp; c <= g.budget; c += warps) {
     int n = 0;
     if (c > 0 && node_formula[c] >= 0)
       for (int a0 = 0; a0 < c; a0 += 32) n += __popc(__ballot_sync(0xffffffffu, is_parent(a0 + lane, c)));
     if (lane == 0) n_parents[c] = n;
   }
   __syncthreads();
-  for (int c = warp; c <= g.budget; c += kBuildThreads / 32) {
+  for (int c = warp; c <= g.budget; c += warps) {
     int start = 0;
     for (int x = lane; x < c; x += 32) start += n_parents[x];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) start += __shfl_xor_sync(0xffffffffu, start, off);
-    int32_t* off = g.parent_off + (int64_t)b * (g.budget + 2);
-    int32_t* idx = g.parent_idx + (int64_t)b * g.parent_cap;
     if (lane == 0) {
-      off[c] = min(start, g.parent_cap);
-      if (c == g.budget) off[c + 1] = min(start + n_parents[c], g.parent_cap);
+      out_off[c] = min(start, g.parent_cap);
+      if (c == g.budget) out_off[c + 1] = min(start + n_parents[c], g.parent_cap);
       if (start + n_parents[c] > g.parent_cap && g.dev_status) atomicOr(g.dev_status + b, SPIFFY_DEV_BADGRAPH);
     }
     if (g.fill_parents && c == g.budget)
-      for (int i = start + n_parents[c] + lane; i < g.parent_cap; i += 32) idx[i] = 0;
+      for (int i = start + n_parents[c] + lane; i < g.parent_cap; i += 32) out_idx[i] = 0;
     if (c > 0 && node_formula[c] >= 0) {
       int w = start;
       for (int a0 = 0; a0 < c; a0 += 32) {
         const bool par = is_parent(a0 + lane, c);
         const unsigned mask = __ballot_sync(0xffffffffu, par);
         const int at = w + __popc(mask & ((1u << lane) - 1u));
-        if (par && at < g.parent_cap) idx[at] = a0 + lane;
+        if (par && at < g.parent_cap) out_idx[at] = a0 + lane;
         w += __popc(mask);
       }
     }
@@ -516,6 +673,11 @@ int64_t draft_chunk(const spiffy_draft_desc& d, int* splits) {
   chunk = (chunk + epv - 1) / epv * epv;
   *splits = (int)n;
   return chunk;
+}
+
+size_t build_smem_bytes(const spiffy_draft_desc& d) {
+  return std::max(d.n_formulas <= kRelated ? (size_t)kFormulaBytes : (size_t)0,
+                  (size_t)d.n_formulas * 12 + (size_t)(d.budget + 1) * 8);  // a graph of few formulas may be too long to stage
 }
 
 }  // namespace
@@ -554,9 +716,8 @@ spiffy_status launch_draft(const spiffy_draft_desc& d, const void* logits, const
   g.state = state; g.formula_off = formula_off; g.formula_i = formula_i; g.formula_j = formula_j;
   g.child_off = child_off; g.child_idx = child_idx; g.tokens = tokens; g.kept = kept; g.score = score;
   g.parent_off = parent_off; g.parent_idx = parent_idx; g.dev_status = dev_status; g.fill_parents = fresh ? 1 : 0;
-  const size_t smem = (size_t)d.block_len * kMaxK * 8 + (size_t)d.block_len * 8 +
-                      (size_t)d.n_formulas * 12 + (size_t)(d.budget + 1) * 8 + 16;
-  e = launch_pdl(draft_build_kernel, dim3(d.batch), dim3(kBuildThreads), smem, stream, g);
+  e = launch_pdl(draft_build_kernel, dim3(d.batch), dim3(32 * std::min<int>(d.block_len, kBuildThreads / 32)),
+                 build_smem_bytes(d), stream, g);
   count_launch();
   return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
 }

@@ -130,3 +130,26 @@ def test_more_than_32_vocabulary_slices():
     got, want = run_both(logits, state, V - 1, 10, 3, torch.float32)
     assert assert_parity(got, want) == B
     assert int(want.parent_off[0, -1]) > 10
+
+
+@pytest.mark.parametrize("D,L,budget,top_k", [(1, 1, 1, 1), (31, 33, 31, 2), (33, 64, 20, 4), (64, 32, 64, 3),
+                                              (65, 32, 40, 3), (200, 40, 200, 4)])
+def test_graphs_at_the_edges_of_the_build_kernel(D, L, budget, top_k):
+    """Formulas by one warp (up to 64, in halves of 32) and by all threads, positions in one and two rounds of warps."""
+    r = np.random.default_rng(D)
+    B, V = 2, 300
+    logits = (r.standard_normal((B, L, V)) * 3).astype(np.float32)
+    state = np.where(r.random((B, L)) < 0.2, 7, V - 1).astype(np.int32)
+    state[0, 0] = V - 1
+    ranks = min(L, 9)
+    seen, formulas = set(), []
+    while len(formulas) < D:  # sizes ascending, so that subsets come first
+        n = 1 + len(formulas) * 6 // D
+        f = tuple(sorted((int(i), int(r.integers(top_k))) for i in r.choice(ranks, min(n, ranks), replace=False)))
+        if f not in seen:
+            seen.add(f)
+            formulas.append(list(f))
+    children = [[int(c) for c in r.integers(0, D, int(r.integers(0, 7)))] for _ in range(D)]
+    got, want = run_both(logits, state, V - 1, budget, top_k, torch.float32, formulas, children)
+    assert assert_parity(got, want, 2e-5) >= 1
+    assert budget < 3 or int(want.parent_off[0, -1]) > budget
