@@ -111,14 +111,22 @@ decide_finalize_kernel(const Partial* __restrict__ partials, int splits, int N,
 }
 
 // Decision tail and acceptance walk of one sequence in one CTA (Algorithm 1,
-// steps 1-5 after the vocabulary reduce): eight threads per row merge the
-// slices, one warp per node applies the rule, warp 0 walks the draft graph with
-// every array it needs already in shared memory.  The graph (states, parent
-// lists) does not depend on the reduce kernel and is fetched before the wait on
-// it.  grid = B, kTailThreads threads, dynamic shared memory tail_smem_bytes().
+// steps 1-5 after the vocabulary reduce): up to eight threads per row merge the
+// slices, then one warp per node applies the rule and looks for the child that
+// equals the node's next state, and warp 0 walks.  The graph (states, parent
+// lists) does not depend on the reduce kernel; ahead of the wait it is copied to
+// shared memory and, for up to kTableNodes nodes, made a table of children with
+// hashes of the states, which saves a step of its own for the links.
+// grid = B, kTailThreads threads, dynamic shared memory tail_smem_bytes().
+// Bound: a chain of short steps.  Behind the wait, 3 x 100 rows x 7 slices, two positions a node: 2640 cycles
+// for the merge, 1640 for the rule, 1020 for links and 1010 for the chase when the rule ranked positions one
+// by one and links were a step of their own with an exchange through atomics; 2040, 2110 for rule and links,
+// 770 now (the decision behind an attention of that shape 18.3 -> 17.6 us, 4 x 8 rows of one slice 9.1 -> 8.6).
+// 48 registers: with 56 and more, fewer reduce CTAs stay on the SM that the tail moves in on, and it comes
+// later (16 x 32 rows x 19 slices with an attention beside them 30.9 us, 30.8 so, 31.0 with 64).
 constexpr int kTailThreads = 1024;
 template <int kLanes>  // threads per row: all N * L rows are merged in one pass when kLanes * N * L <= 1024
-__global__ void __launch_bounds__(kTailThreads)
+__global__ void __launch_bounds__(kTailThreads + 256, 1)  // 48 registers
 decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int L,
                    const int32_t* __restrict__ block_tokens, int mask_id, int rule, int top_s,
                    float tau, float* __restrict__ conf_out, int32_t* __restrict__ tok_out,
@@ -129,6 +137,9 @@ decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int 
                    int32_t* __restrict__ n_accepted, int32_t* __restrict__ path,
                    int32_t* __restrict__ next_block, int32_t* __restrict__ walk_status, int early_trigger) {
   extern __shared__ __align__(8) unsigned char tail_smem[];
+#if __CUDA_ARCH__ >= 900
+  if (early_trigger) pdl_launch_dependents();  // an independent kernel comes next, and takes the SMs the reduce leaves
+#endif
   const int b = blockIdx.x;
   const int rows = N * L;
   uint64_t* s_bits = reinterpret_cast<uint64_t*>(tail_smem);
@@ -138,8 +149,13 @@ decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int 
   int32_t* s_off = reinterpret_cast<int32_t*>(s_conf + rows);
   int32_t* s_idx = s_off + (N + 1);
   int* s_link = s_idx + parent_cap;
-  const int32_t* state = block_tokens + (int64_t)b * rows;
+  __shared__ uint32_t s_kids[kTableNodes][2];
+  __shared__ uint32_t s_hash[kTableNodes];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool table = N <= kTableNodes;
+  bool good = true;  // no malformed offset or entry met
   {
+    const int32_t* state = block_tokens + (int64_t)b * rows;
     auto copy4 = [](void* dst, const void* src) {
       asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
                        (uint32_t)__cvta_generic_to_shared(dst)),
@@ -152,9 +168,20 @@ decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int 
     for (int i = threadIdx.x; i <= N; i += kTailThreads) copy4(s_off + i, off + i);
     for (int i = threadIdx.x; i < parent_cap; i += kTailThreads) copy4(s_idx + i, idx + i);
     for (int i = threadIdx.x; i < N; i += kTailThreads) s_link[i] = kNoLink;
+    if (threadIdx.x < 2 * kTableNodes) (&s_kids[0][0])[threadIdx.x] = 0u;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  if (table) {
+#pragma unroll 1
+    for (int n = warp; n < N; n += kTailThreads / 32) {
+      const int32_t mine[2] = {lane < L ? s_state[n * L + lane] : 0, lane + 32 < L ? s_state[n * L + lane + 32] : 0};
+      const uint32_t hash = hash_of(mine, lane);
+      if (lane == 0) s_hash[n] = hash;
+      if (n > 0) good &= enter_parents(s_kids, s_off, s_idx, parent_cap, n, lane);
+    }
   }
 #if __CUDA_ARCH__ >= 900
-  if (early_trigger) pdl_launch_dependents();  // an independent kernel comes next, and takes the SMs the reduce leaves
   cudaGridDependencySynchronize();  // the reduce kernel's partials are visible
   pdl_launch_dependents();          // only now: this CTA was resident during the reduce, the next kernel's need not be
 #endif
@@ -162,11 +189,10 @@ decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int 
   for (int base = 0; base < rows; base += kTailThreads / kLanes) {
     const int r = base + threadIdx.x / kLanes;
     const int row = min(r, rows - 1);
-    const int32_t st = state[row];
     float conf;
     int32_t tok;
     const bool ok = finalize_row<kLanes>(partials + ((int64_t)b * rows + row) * splits, splits, sub,
-                                         st, mask_id, conf, tok);
+                                         s_state[row], mask_id, conf, tok);
     if (sub == 0 && r < rows) {
       conf_out[(int64_t)b * rows + row] = conf;
       tok_out[(int64_t)b * rows + row] = tok;
@@ -175,22 +201,32 @@ decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int 
       if (!ok && decide_status) atomicOr(decide_status + b, SPIFFY_DEV_NONFINITE);
     }
   }
-  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll 1
   for (int node = warp; node < N; node += kTailThreads / 32) {
     const uint64_t bits = unmask_rule(s_conf + node * L, s_state + node * L, L, mask_id, rule, top_s,
                                       tau, lane);
+    int32_t next[2];  // the node's next state
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int l = lane + 32 * h;
+      next[h] = l < L ? walk_next_token(s_state, s_top, bits, node, L, l) : 0;
+    }
+    // a node with nothing to unmask ends the walk
+    const int link = table && bits != 0 ? child_of(s_kids[node], s_hash, s_state, next, N, L, lane) : kNoLink;
     if (lane == 0) {
       bits_out[(int64_t)b * N + node] = bits;
       n_unmask_out[(int64_t)b * N + node] = __popcll(bits);
       s_bits[node] = bits;
+      if (table) s_link[node] = link;
     }
   }
-  __syncthreads();
-  const bool bad = walk_link_children(N, L, parent_cap, s_state, s_top, s_off, s_idx, s_bits, s_link,
-                                      warp, kTailThreads / 32, lane);
-  if (bad && lane == 0 && walk_status) atomicOr(walk_status + b, SPIFFY_DEV_BADGRAPH);
+  if (!table) {
+    __syncthreads();
+    good = !walk_link_children(N, L, parent_cap, s_state, s_top, s_off, s_idx, s_bits, s_link, warp, kTailThreads / 32,
+                               lane);
+  }
+  if (!good && walk_status) atomicOr(walk_status + b, SPIFFY_DEV_BADGRAPH);
   __syncthreads();
   if (warp == 0)
     walk_chase(N, L, s_state, s_top, s_bits, s_link, path + (int64_t)b * N,
@@ -310,6 +346,7 @@ spiffy_status launch_decide_finalize(const spiffy_decide_desc& d, const void* pa
 // runs under it, on one SM instead of many that the attention waits for: the tail, whatever there is to
 // merge (16 x 32 positions x 28 heads, x 19: 21.5 and 21.5, 27.0 and 27.7, 36.9 and 37.3).
 constexpr int kTailRows = 512, kTailPartials = 4096;
+constexpr size_t kTailSmem = 48 * 1024 - 1024;  // what the kernel declares itself comes on top
 spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits,
                                  const int32_t* block_tokens, float* conf, int32_t* top_tok,
                                  uint64_t* unmask_bits, int32_t* n_unmask,
@@ -322,7 +359,7 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
   const int64_t rows_of_one = (int64_t)d.n_nodes * d.block_len;
   int64_t chunk = 0;
   const int splits = decide_splits(d, &chunk);
-  if (rows_of_one > kTailRows || smem > 48 * 1024 || (!next && rows_of_one * splits > kTailPartials)) {
+  if (rows_of_one > kTailRows || smem > kTailSmem || (!next && rows_of_one * splits > kTailPartials)) {
     const spiffy_status st = decide_only(d, logits, block_tokens, conf, top_tok, unmask_bits,
                                          n_unmask, decide_status, ws, fresh, independent, next, stream);
     if (st != SPIFFY_OK) return st;

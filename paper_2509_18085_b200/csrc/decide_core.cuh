@@ -60,11 +60,10 @@ __device__ __forceinline__ uint64_t add_exp2(uint64_t acc, float x0, float x1, u
 __device__ __forceinline__ void merge(float& m, float& s, int& idx, float m2,
                                       float s2, int idx2) {
   if (m2 > m || (m2 == m && idx2 < idx)) idx = idx2;
-  const float M = fmaxf(m, m2);
-  const float f1 = (m == M) ? 1.f : ex2((m - M) * kLog2e);
-  const float f2 = (m2 == M) ? 1.f : ex2((m2 - M) * kLog2e);
-  s = __fmaf_rn(s, f1, __fmul_rn(s2, f2));  // spelled out: every instance rounds the same way
-  m = M;
+  // the sum that belongs to the larger maximum stays as it is
+  const float f = m == m2 ? 1.f : ex2(-fabsf(m - m2) * kLog2e);
+  s = m2 > m ? __fmaf_rn(s, f, s2) : __fmaf_rn(s2, f, s);  // spelled out: every instance rounds the same way
+  m = fmaxf(m, m2);
 }
 
 template <typename T>
@@ -371,11 +370,14 @@ __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int 
 // One warp applies the unmasking rule of Sec. 3.1 (Algorithm 1, step 3) to one
 // node; lane k owns positions k and k + 32.  conf: the node's L confidences,
 // -inf at unmasked positions.  Returns the bit mask of positions to unmask.
+// Few positions are taken one after the other, each the most confident of those left, the first of
+// several (a maximum and two votes); more than kRounds by their ranks.
 __device__ __forceinline__ uint64_t unmask_rule(const float* conf, const int32_t* state, int L,
                                                 int mask_id, int rule, int top_s, float tau,
                                                 int lane) {
+  constexpr int kRounds = 8;
   const unsigned full = 0xffffffffu;
-  bool masked[2], take[2];
+  bool masked[2];
   float c[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -383,9 +385,16 @@ __device__ __forceinline__ uint64_t unmask_rule(const float* conf, const int32_t
     masked[h] = l < L && state[min(l, L - 1)] == mask_id;
     c[h] = masked[h] ? conf[l] : -INFINITY;
   }
-  if (rule == SPIFFY_RULE_TOPS && top_s > 1) {
+  const bool tops = rule == SPIFFY_RULE_TOPS;
+  if (!tops) {  // strict, Sec. 3.1; an unusable row never passes
+    const uint64_t pass = (uint64_t)__ballot_sync(full, c[0] > tau && masked[0]) |
+                          (uint64_t)__ballot_sync(full, c[1] > tau && masked[1]) << 32;
+    if (pass) return pass;  // none: the single most confident position
+  }
+  if (tops && top_s > kRounds) {
     // rank among the masked positions by (confidence desc, position asc); the
     // confidence of an unmasked position is -inf and a masked one's is not
+    bool take[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int l = lane + 32 * h;
@@ -398,35 +407,20 @@ __device__ __forceinline__ uint64_t unmask_rule(const float* conf, const int32_t
       }
       take[h] = masked[h] && rank < top_s;
     }
-  } else {
-    // only the single most confident masked position matters (top-1, or the
-    // fallback of the threshold rule): a warp arg-max, ties to the lower position
-    float bc = (c[0] == c[0]) ? c[0] : -INFINITY;  // an unusable row never wins
-    int bp = lane;
-    if (c[1] > bc) {
-      bc = c[1];
-      bp = lane + 32;
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const float c2 = __shfl_xor_sync(full, bc, off);
-      const int p2 = __shfl_xor_sync(full, bp, off);
-      if (c2 > bc || (c2 == bc && p2 < bp)) {
-        bc = c2;
-        bp = p2;
-      }
-    }
-    const bool any_masked = __any_sync(full, masked[0] || masked[1]);
-    bool pass0 = false, pass1 = false;
-    if (rule != SPIFFY_RULE_TOPS) {
-      pass0 = masked[0] && c[0] > tau;  // strict, Sec. 3.1
-      pass1 = masked[1] && c[1] > tau;
-    }
-    const bool any_pass = __any_sync(full, pass0 || pass1);
-    take[0] = any_pass ? pass0 : (any_masked && masked[0] && bp == lane);
-    take[1] = any_pass ? pass1 : (any_masked && masked[1] && bp == lane + 32);
+    return (uint64_t)__ballot_sync(full, take[0]) | (uint64_t)__ballot_sync(full, take[1]) << 32;
   }
-  return (uint64_t)__ballot_sync(full, take[0]) | ((uint64_t)__ballot_sync(full, take[1]) << 32);
+  uint64_t bits = 0;
+#pragma unroll 1
+  for (int left = tops ? top_s : 1; left > 0; --left) {
+    const float best = warp_max(fmaxf(c[0], c[1]));  // an unusable row never wins
+    if (best == -INFINITY) break;                    // all taken
+    const unsigned lo = __ballot_sync(full, c[0] == best), hi = __ballot_sync(full, c[1] == best);
+    const int at = lo ? __ffs(lo) - 1 : __ffs(hi) + 31;
+    bits |= 1ull << at;
+    if (lane == at) c[0] = -INFINITY;
+    if (lane + 32 == at) c[1] = -INFINITY;
+  }
+  return bits;
 }
 
 }  // namespace

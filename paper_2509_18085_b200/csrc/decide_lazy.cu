@@ -49,7 +49,6 @@ struct __align__(16) LazyWord {
 };
 constexpr int kEnded = 0x7fffffff;
 constexpr int kPresent = 1;     // mark of a slice that has been written
-constexpr int kTableNodes = 64; // graphs up to here have their children in a table, and their likely walk guessed
 constexpr int kWalkCtas = 6;    // of the walk kernel per SM: 80 registers
 constexpr unsigned kPollsABatch = 64, kPollsToHelp = 1u << 12;
 
@@ -120,21 +119,6 @@ struct Graph {
   const int32_t* off;
   const int32_t* idx;
 };
-
-// A state, positions `lane` and `lane` + 32 (zeros beyond L): its still-masked positions, and a number that
-// equal states share.
-__device__ __forceinline__ uint64_t masked_of(const int32_t (&state)[2], int L, int mask_id, int lane) {
-  uint64_t masked = 0;
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-    masked |= (uint64_t)__ballot_sync(0xffffffffu, lane + 32 * h < L && state[h] == mask_id) << (32 * h);
-  return masked;
-}
-__device__ __forceinline__ uint32_t hash_of(const int32_t (&state)[2], int lane) {
-  const uint32_t a = ((uint32_t)state[0] + 0x9e3779b9u * (uint32_t)lane) * 0x85ebca6bu;
-  const uint32_t b = ((uint32_t)state[1] + 0x9e3779b9u * (uint32_t)(lane + 32)) * 0xc2b2ae35u;
-  return __reduce_xor_sync(0xffffffffu, (a ^ (a >> 15)) + (b ^ (b >> 13)));
-}
 
 // Item i of a node: a slice of one of its masked rows; the others are never read.
 struct Item {
@@ -239,18 +223,8 @@ lazy_walk_kernel(const __grid_constant__ LazyParams p) {
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   if (table) {
-    for (int m = 1 + warp; m < N; m += kReduceThreads / 32) {
-      const int e0 = g.off[m], e1 = g.off[m + 1];
-      if (e0 < 0 || e1 < e0 || e1 > p.parent_cap) {  // malformed offsets
-        s_bad = 1;
-        continue;
-      }
-      for (int e = e0 + lane; e < e1; e += 32) {
-        const int q = g.idx[e];
-        if (q < 0 || q >= m) s_bad = 1;  // ignored entry
-        else atomicOr(&s_kids[q][m >> 5], 1u << (m & 31));
-      }
-    }
+    for (int m = 1 + warp; m < N; m += kReduceThreads / 32)
+      if (!enter_parents(s_kids, g.off, g.idx, p.parent_cap, m, lane)) s_bad = 1;
     __syncthreads();
   }
   Partial* const slices = p.partials + (int64_t)b * N * L * p.splits;
@@ -395,24 +369,8 @@ lazy_walk_kernel(const __grid_constant__ LazyParams p) {
       }
       const uint64_t left = masked_of(next, L, p.mask_id, lane);
       int found = kNoLink;
-      if (table && go_on) {
-        // the first node (ascending) that lists `node` as a parent and equals its next state
-        const uint32_t hash = hash_of(next, lane);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int m0 = 32 * h;
-          if (m0 >= N || found != kNoLink) continue;
-          unsigned like = __ballot_sync(0xffffffffu, m0 + lane < N && s_hash[min(m0 + lane, N - 1)] == hash) & s_kids[node][h];
-          for (; like; like &= like - 1) {
-            const int32_t* sm = g.state + (m0 + __ffs(like) - 1) * L;
-            const bool eq = (lane >= L || sm[lane] == next[0]) && (lane + 32 >= L || sm[lane + 32] == next[1]);
-            if (__all_sync(0xffffffffu, eq)) {
-              found = m0 + __ffs(like) - 1;
-              break;
-            }
-          }
-        }
-      }
+      // the first node (ascending) that lists `node` as a parent and equals its next state
+      if (table && go_on) found = child_of(s_kids[node], s_hash, g.state, next, N, L, lane);
       if (lane == 0) {
         s_found = found;
         s_word = LazyWord{go_on, 0, left};

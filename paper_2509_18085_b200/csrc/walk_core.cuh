@@ -3,6 +3,7 @@
 // one as a parent and whose state equals the current node's next state; it stops
 // when there is none, or at a node with nothing left to unmask.
 //
+// A few nodes' children are found by a table (below), the others as follows.
 // Whether node m follows node p depends on p and m alone, not on the path, so
 // the links are found for all (parent, child) entries at once -- one warp per
 // child, lane k owning block positions k and k + 32 -- and the walk itself is a
@@ -14,6 +15,56 @@
 namespace spiffy {
 
 constexpr int kNoLink = 0x7fffffff;
+constexpr int kTableNodes = 64;  // graphs up to here have their children in a table: what lists a node as a parent, a bit each
+
+// A state, positions `lane` and `lane` + 32 (zeros beyond L): its still-masked positions, and a number that
+// equal states share.
+__device__ __forceinline__ uint64_t masked_of(const int32_t (&state)[2], int L, int mask_id, int lane) {
+  uint64_t masked = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    masked |= (uint64_t)__ballot_sync(0xffffffffu, lane + 32 * h < L && state[h] == mask_id) << (32 * h);
+  return masked;
+}
+__device__ __forceinline__ uint32_t hash_of(const int32_t (&state)[2], int lane) {
+  const uint32_t a = ((uint32_t)state[0] + 0x9e3779b9u * (uint32_t)lane) * 0x85ebca6bu;
+  const uint32_t b = ((uint32_t)state[1] + 0x9e3779b9u * (uint32_t)(lane + 32)) * 0xc2b2ae35u;
+  return __reduce_xor_sync(0xffffffffu, (a ^ (a >> 15)) + (b ^ (b >> 13)));
+}
+
+// One warp enters node m's parents into the table (all zero beforehand).  False on a lane that met a malformed
+// offset or entry, which is ignored.
+__device__ __forceinline__ bool enter_parents(uint32_t (*kids)[2], const int32_t* off, const int32_t* idx, int parent_cap,
+                                              int m, int lane) {
+  const int e0 = off[m], e1 = off[m + 1];
+  if (e0 < 0 || e1 < e0 || e1 > parent_cap) return false;
+  bool good = true;
+  for (int e = e0 + lane; e < e1; e += 32) {
+    const int q = idx[e];
+    if (q < 0 || q >= m) good = false;
+    else atomicOr(&kids[q][m >> 5], 1u << (m & 31));
+  }
+  return good;
+}
+
+// The first of the nodes in `kids` (a bit each) whose state is `next`, kNoLink if there is none; by one warp.
+__device__ __forceinline__ int child_of(const uint32_t (&kids)[2], const uint32_t* hashes, const int32_t* states,
+                                        const int32_t (&next)[2], int N, int L, int lane) {
+  const uint32_t hash = hash_of(next, lane);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int m0 = 32 * h;
+    if (m0 >= N) break;
+    unsigned like = __ballot_sync(0xffffffffu, m0 + lane < N && hashes[min(m0 + lane, N - 1)] == hash) & kids[h];
+    for (; like; like &= like - 1) {
+      const int m = m0 + __ffs(like) - 1;
+      const int32_t* sm = states + m * L;
+      if (__all_sync(0xffffffffu, (lane >= L || sm[lane] == next[0]) && (lane + 32 >= L || sm[lane + 32] == next[1])))
+        return m;
+    }
+  }
+  return kNoLink;
+}
 
 __device__ __forceinline__ int32_t walk_next_token(const int32_t* state, const int32_t* top,
                                                    uint64_t bits, int node, int L, int l) {

@@ -72,6 +72,27 @@ def test_one_call_equals_two_calls_and_the_oracle(B, N, L, V):
         assert int(dec.dev_status.sum()) == 0 and int(walk.dev_status.sum()) == 0
 
 
+@pytest.mark.parametrize("N,L,S", [(64, 8, 1), (64, 8, 8), (65, 7, 1), (33, 15, 3), (1, 64, 8), (2, 64, 9), (4, 40, 40)])
+def test_edges_of_the_table_of_children_and_of_the_rounds_of_the_rule(N, L, S):
+    """64 nodes have a table, 65 do not; up to 8 positions are taken in rounds, more by their ranks.  Among equal
+    confidences (equal rows) the lowest position is taken first, as the oracle does."""
+    logits, tokens, off, idx, mask = random_case(N, 2, N, L, 52, p_accept=0.9)
+    logits[:, :, 3::7] = logits[:, :, 2::7][:, :, :logits[:, :, 3::7].shape[2]]
+    for rule, tau in ((spiffy.RULE_TOPS, 0.0), (spiffy.RULE_THRESHOLD, 0.4)):
+        dec, walk = both(logits, tokens, off, idx, mask, rule, S, tau)
+        o, _ = oracle.verify_step(logits, tokens, off, idx, mask, rule, S, tau)
+        conf = dec.conf.cpu().numpy()
+        assert np.allclose(conf[tokens == mask], o.conf[tokens == mask], rtol=1e-5)
+        bits = G.bits_np(dec.unmask_bits)
+        for b in range(2):
+            for n in range(N):  # the rule on the call's own confidences, in which equal rows are equal
+                c = np.where(tokens[b, n] == mask, conf[b, n], -np.inf)
+                order = [int(l) for l in np.lexsort((np.arange(L), -c)) if c[l] > -np.inf]
+                over = [l for l in order if c[l] > np.float32(tau)]
+                take = order[:S] if rule == spiffy.RULE_TOPS else (over or order[:1])
+                assert int(bits[b, n]) == sum(1 << l for l in take)
+
+
 def test_deep_walks_happen_on_the_fused_kernel():
     logits, tokens, off, idx, mask = random_case(3, 40, 8, 16, 200, p_accept=1.0)
     dec, walk = both(logits, tokens, off, idx, mask, spiffy.RULE_TOPS)
