@@ -16,6 +16,7 @@
 // the walk in walk_core.cuh.
 #include "common.cuh"
 #include "decide_core.cuh"
+#include "sm100_ptx.cuh"
 #include "walk_core.cuh"
 
 namespace spiffy {
@@ -125,6 +126,145 @@ decide_finalize_kernel(const Partial* __restrict__ partials, int splits, int N,
 // 48 registers: with 56 and more, fewer reduce CTAs stay on the SM that the tail moves in on, and it comes
 // later (16 x 32 rows x 19 slices with an attention beside them 30.9 us, 30.8 so, 31.0 with 64).
 constexpr int kTailThreads = 1024;
+struct TailArgs {
+  int splits, N, L, mask_id, rule, top_s;
+  float tau;
+  const int32_t* block_tokens;
+  const int32_t* parent_off;
+  const int32_t* parent_idx;
+  int parent_cap;
+  float* conf;
+  int32_t* top_tok;
+  uint64_t* unmask_bits;
+  int32_t* n_unmask;
+  int32_t* decide_status;
+  int32_t* accepted_node;
+  int32_t* n_accepted;
+  int32_t* path;
+  int32_t* next_block;
+  int32_t* walk_status;
+};
+// A sequence's tail, by all threads of a CTA; `memory`: tail_smem_bytes().
+class Tail {
+ public:
+  __device__ __forceinline__ Tail(const TailArgs& a, int b, unsigned char* memory)
+      : a(a), b(b), rows(a.N * a.L), warp(threadIdx.x >> 5), lane(threadIdx.x & 31), warps(blockDim.x >> 5),
+        table(a.N <= kTableNodes) {
+    bits = reinterpret_cast<uint64_t*>(memory);
+    state = reinterpret_cast<int32_t*>(bits + a.N);
+    top = state + rows;
+    conf = reinterpret_cast<float*>(top + rows);
+    off = reinterpret_cast<int32_t*>(conf + rows);
+    idx = off + (a.N + 1);
+    link = idx + a.parent_cap;
+    __shared__ uint32_t s_kids[kTableNodes][2];
+    __shared__ uint32_t s_hash[kTableNodes];
+    kids = s_kids;
+    hash = s_hash;
+  }
+  // The graph on its way to shared memory.  kNow: read at L2, by a kernel that does not wait for the one before it.
+  template <bool kNow>
+  __device__ __forceinline__ void fetch() {
+    auto copy4 = [](void* dst, const void* src) {
+      if constexpr (kNow) {
+        *static_cast<int32_t*>(dst) = __ldcg(static_cast<const int32_t*>(src));
+        return;
+      }
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                       (uint32_t)__cvta_generic_to_shared(dst)),
+                   "l"(src)
+                   : "memory");
+    };
+    const int32_t* from_state = a.block_tokens + (int64_t)b * rows;
+    const int32_t* from_off = a.parent_off + (int64_t)b * (a.N + 1);
+    const int32_t* from_idx = a.parent_idx + (int64_t)b * a.parent_cap;
+    const int tid = threadIdx.x, step = blockDim.x;
+    for (int i = tid; i < rows; i += step) copy4(state + i, from_state + i);
+    for (int i = tid; i <= a.N; i += step) copy4(off + i, from_off + i);
+    for (int i = tid; i < a.parent_cap; i += step) copy4(idx + i, from_idx + i);
+    for (int i = tid; i < a.N; i += step) link[i] = kNoLink;
+    for (int i = tid; i < 2 * kTableNodes; i += step) (&kids[0][0])[i] = 0u;
+  }
+  // ... has arrived: children and hashes, complete behind the next barrier of the CTA.
+  __device__ __forceinline__ void arrived() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (!table) return;
+#pragma unroll 1
+    for (int n = warp; n < a.N; n += warps) {
+      const int32_t mine[2] = {lane < a.L ? state[n * a.L + lane] : 0, lane + 32 < a.L ? state[n * a.L + lane + 32] : 0};
+      const uint32_t h = hash_of(mine, lane);
+      if (lane == 0) hash[n] = h;
+      if (n > 0) good &= enter_parents(kids, off, idx, a.parent_cap, n, lane);
+    }
+  }
+  // Steps 1 and 2: kLanes threads a row merge its slices, `splits` from partials + row * splits on.
+  template <int kLanes, class Source>
+  __device__ __forceinline__ void merge_rows(const Partial* partials, Source source) {
+    const int sub = threadIdx.x & (kLanes - 1), step = blockDim.x / kLanes;
+    for (int base = 0; base < rows; base += step) {
+      const int r = base + threadIdx.x / kLanes;
+      const int row = min(r, rows - 1);
+      float c;
+      int32_t tok;
+      const bool ok = finalize_row<kLanes>(partials + (int64_t)row * a.splits, a.splits, sub, state[row], a.mask_id, c, tok,
+                                           source);
+      if (sub == 0 && r < rows) {
+        a.conf[(int64_t)b * rows + row] = c;
+        a.top_tok[(int64_t)b * rows + row] = tok;
+        conf[row] = c;
+        top[row] = tok;
+        if (!ok && a.decide_status) atomicOr(a.decide_status + b, SPIFFY_DEV_NONFINITE);
+      }
+    }
+  }
+  // Steps 3 to 5.
+  __device__ __forceinline__ void walk() {
+    const int N = a.N, L = a.L;
+    __syncthreads();
+#pragma unroll 1
+    for (int node = warp; node < N; node += warps) {
+      const uint64_t take = unmask_rule(conf + node * L, state + node * L, L, a.mask_id, a.rule, a.top_s, a.tau, lane);
+      int32_t next[2];  // the node's next state
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int l = lane + 32 * h;
+        next[h] = l < L ? walk_next_token(state, top, take, node, L, l) : 0;
+      }
+      // a node with nothing to unmask ends the walk
+      const int child = table && take != 0 ? child_of(kids[node], hash, state, next, N, L, lane) : kNoLink;
+      if (lane == 0) {
+        a.unmask_bits[(int64_t)b * N + node] = take;
+        a.n_unmask[(int64_t)b * N + node] = __popcll(take);
+        bits[node] = take;
+        if (table) link[node] = child;
+      }
+    }
+    if (!table) {
+      __syncthreads();
+      good = !walk_link_children(N, L, a.parent_cap, state, top, off, idx, bits, link, warp, warps, lane);
+    }
+    if (!good && a.walk_status) atomicOr(a.walk_status + b, SPIFFY_DEV_BADGRAPH);
+    __syncthreads();
+    if (warp == 0)
+      walk_chase(N, L, state, top, bits, link, a.path + (int64_t)b * N, a.next_block + (int64_t)b * L, a.accepted_node + b,
+                 a.n_accepted + b, lane);
+  }
+  int32_t* state;
+
+ private:
+  const TailArgs& a;
+  const int b, rows, warp, lane, warps;
+  const bool table;
+  bool good = true;  // no malformed offset or entry met
+  uint64_t* bits;
+  int32_t *top, *off, *idx;
+  float* conf;
+  int* link;
+  uint32_t (*kids)[2];
+  uint32_t* hash;
+};
+
 template <int kLanes>  // threads per row: all N * L rows are merged in one pass when kLanes * N * L <= 1024
 __global__ void __launch_bounds__(kTailThreads + 256, 1)  // 48 registers
 decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int L,
@@ -136,101 +276,93 @@ decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int 
                    int parent_cap, int32_t* __restrict__ accepted_node,
                    int32_t* __restrict__ n_accepted, int32_t* __restrict__ path,
                    int32_t* __restrict__ next_block, int32_t* __restrict__ walk_status, int early_trigger) {
-  extern __shared__ __align__(8) unsigned char tail_smem[];
+  extern __shared__ __align__(16) unsigned char tail_smem[];
 #if __CUDA_ARCH__ >= 900
   if (early_trigger) pdl_launch_dependents();  // an independent kernel comes next, and takes the SMs the reduce leaves
 #endif
-  const int b = blockIdx.x;
-  const int rows = N * L;
-  uint64_t* s_bits = reinterpret_cast<uint64_t*>(tail_smem);
-  int32_t* s_state = reinterpret_cast<int32_t*>(s_bits + N);
-  int32_t* s_top = s_state + rows;
-  float* s_conf = reinterpret_cast<float*>(s_top + rows);
-  int32_t* s_off = reinterpret_cast<int32_t*>(s_conf + rows);
-  int32_t* s_idx = s_off + (N + 1);
-  int* s_link = s_idx + parent_cap;
-  __shared__ uint32_t s_kids[kTableNodes][2];
-  __shared__ uint32_t s_hash[kTableNodes];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool table = N <= kTableNodes;
-  bool good = true;  // no malformed offset or entry met
-  {
-    const int32_t* state = block_tokens + (int64_t)b * rows;
-    auto copy4 = [](void* dst, const void* src) {
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
-                       (uint32_t)__cvta_generic_to_shared(dst)),
-                   "l"(src)
-                   : "memory");
-    };
-    const int32_t* off = parent_off + (int64_t)b * (N + 1);
-    const int32_t* idx = parent_idx + (int64_t)b * parent_cap;
-    for (int i = threadIdx.x; i < rows; i += kTailThreads) copy4(s_state + i, state + i);
-    for (int i = threadIdx.x; i <= N; i += kTailThreads) copy4(s_off + i, off + i);
-    for (int i = threadIdx.x; i < parent_cap; i += kTailThreads) copy4(s_idx + i, idx + i);
-    for (int i = threadIdx.x; i < N; i += kTailThreads) s_link[i] = kNoLink;
-    if (threadIdx.x < 2 * kTableNodes) (&s_kids[0][0])[threadIdx.x] = 0u;
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncthreads();
-  if (table) {
-#pragma unroll 1
-    for (int n = warp; n < N; n += kTailThreads / 32) {
-      const int32_t mine[2] = {lane < L ? s_state[n * L + lane] : 0, lane + 32 < L ? s_state[n * L + lane + 32] : 0};
-      const uint32_t hash = hash_of(mine, lane);
-      if (lane == 0) s_hash[n] = hash;
-      if (n > 0) good &= enter_parents(s_kids, s_off, s_idx, parent_cap, n, lane);
-    }
-  }
+  const TailArgs a = {splits, N, L, mask_id, rule, top_s, tau, block_tokens, parent_off, parent_idx, parent_cap, conf_out,
+                      tok_out, bits_out, n_unmask_out, decide_status, accepted_node, n_accepted, path, next_block, walk_status};
+  Tail tail(a, (int)blockIdx.x, tail_smem);
+  tail.template fetch<false>();
+  tail.arrived();
 #if __CUDA_ARCH__ >= 900
   cudaGridDependencySynchronize();  // the reduce kernel's partials are visible
   pdl_launch_dependents();          // only now: this CTA was resident during the reduce, the next kernel's need not be
 #endif
-  const int sub = threadIdx.x & (kLanes - 1);
-  for (int base = 0; base < rows; base += kTailThreads / kLanes) {
-    const int r = base + threadIdx.x / kLanes;
-    const int row = min(r, rows - 1);
-    float conf;
-    int32_t tok;
-    const bool ok = finalize_row<kLanes>(partials + ((int64_t)b * rows + row) * splits, splits, sub,
-                                         s_state[row], mask_id, conf, tok);
-    if (sub == 0 && r < rows) {
-      conf_out[(int64_t)b * rows + row] = conf;
-      tok_out[(int64_t)b * rows + row] = tok;
-      s_conf[row] = conf;
-      s_top[row] = tok;
-      if (!ok && decide_status) atomicOr(decide_status + b, SPIFFY_DEV_NONFINITE);
-    }
-  }
-  __syncthreads();
-#pragma unroll 1
-  for (int node = warp; node < N; node += kTailThreads / 32) {
-    const uint64_t bits = unmask_rule(s_conf + node * L, s_state + node * L, L, mask_id, rule, top_s,
-                                      tau, lane);
-    int32_t next[2];  // the node's next state
+  tail.template merge_rows<kLanes>(partials + (int64_t)blockIdx.x * N * L * splits, CompleteSlices{});
+  tail.walk();
+}
+
+// The same for few slices beside a CUDA-core attention (SPIFFY_INDEPENDENT), reduce included: a cluster of
+// kSmallCtas CTAs per sequence, whose groups of kReduceThreads threads take the slices of masked rows in turn;
+// the partial results go straight into the shared memory of the first CTA, which does the rest.  One launch
+// instead of two, and no partial result waits for a kernel to end and another to read it from L2.  Bound: the
+// launch, a trip for the tokens and one for each round of slices, the steps of the tail.  Two groups a CTA: larger
+// ones find no room beside an attention that fills the machine (2 x 32 positions x 32 heads over 4000 keys
+// 127.2 us, with four groups 133.9, without this kernel 130.1; 4 x 2 x 8 positions x 12 heads over 300 10.8, 14.8
+// and 13.7), and the smallest gain nothing by them (4 x 8 rows of one slice 6.3, 6.2 and 9.2).
+constexpr int kSmallCtas = 8, kSmallGroups = 2, kSmallRows = 64;
+template <typename T>
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallGroups* kReduceThreads)
+decide_small_kernel(const __grid_constant__ TailArgs a, const T* __restrict__ logits, int64_t row_stride, int V,
+                    int64_t chunk, int next, StatusClear clear) {
+  extern __shared__ __align__(16) unsigned char tail_smem[];
+  __shared__ int16_t list[kSmallRows];  // the masked rows
+  __shared__ int n_masked;
+  const int b = (int)blockIdx.x / kSmallCtas, rank = (int)blockIdx.x % kSmallCtas, tid = threadIdx.x;
+  const int rows = a.N * a.L, group = tid / kReduceThreads;
+  sm100::cluster_arrive_relaxed();  // the first CTA is there when all are
+#if __CUDA_ARCH__ >= 900
+  if (next) pdl_launch_dependents();
+#endif
+  if (tid < 32) {
+    int32_t token[kSmallRows / 32];
+    int n = 0;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int l = lane + 32 * h;
-      next[h] = l < L ? walk_next_token(s_state, s_top, bits, node, L, l) : 0;
+    for (int h = 0; h < kSmallRows / 32; ++h)  // all on their way at once
+      token[h] = 32 * h < rows ? __ldcg(a.block_tokens + (int64_t)b * rows + min(tid + 32 * h, rows - 1)) : 0;
+#pragma unroll
+    for (int h = 0; h < kSmallRows / 32; ++h) {
+      const bool masked = tid + 32 * h < rows && token[h] == a.mask_id;
+      const unsigned vote = __ballot_sync(0xffffffffu, masked);
+      if (masked) list[n + __popc(vote & ((1u << tid) - 1u))] = (int16_t)(tid + 32 * h);
+      n += __popc(vote);
     }
-    // a node with nothing to unmask ends the walk
-    const int link = table && bits != 0 ? child_of(s_kids[node], s_hash, s_state, next, N, L, lane) : kNoLink;
-    if (lane == 0) {
-      bits_out[(int64_t)b * N + node] = bits;
-      n_unmask_out[(int64_t)b * N + node] = __popcll(bits);
-      s_bits[node] = bits;
-      if (table) s_link[node] = link;
-    }
+    if (tid == 0) n_masked = n;
   }
-  if (!table) {
-    __syncthreads();
-    good = !walk_link_children(N, L, parent_cap, s_state, s_top, s_off, s_idx, s_bits, s_link, warp, kTailThreads / 32,
-                               lane);
+  Partial* slots = reinterpret_cast<Partial*>(tail_smem);
+  Tail tail(a, b, tail_smem + (size_t)rows * a.splits * sizeof(Partial));
+  if (rank == 0) {
+    if (tid == 0 && clear.batch) clear.run(b);
+    tail.template fetch<true>();
   }
-  if (!good && walk_status) atomicOr(walk_status + b, SPIFFY_DEV_BADGRAPH);
   __syncthreads();
-  if (warp == 0)
-    walk_chase(N, L, s_state, s_top, s_bits, s_link, path + (int64_t)b * N,
-               next_block + (int64_t)b * L, accepted_node + b, n_accepted + b, lane);
+  // the first CTA, which has the graph to prepare, comes last
+  const int items = n_masked * a.splits, first = (rank + kSmallCtas - 1) % kSmallCtas * kSmallGroups + group;
+  const uint32_t leader = sm100::map_to_cta(sm100::smem_u32(slots), 0);
+  bool all_here = false;
+  for (int i = first; i < items; i += kSmallCtas * kSmallGroups) {
+    const int nth = i / a.splits, split = i - nth * a.splits, row = list[nth];
+    const Partial r = reduce_slice<T, kSmallGroups>(logits + ((int64_t)b * rows + row) * row_stride, V, chunk, split,
+                                               static_cast<Partial*>(nullptr));
+    if (!all_here) sm100::cluster_wait();
+    all_here = true;
+    if (tid % kReduceThreads == 0)
+      asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(leader + (uint32_t)(row * a.splits + split) * 16u),
+                   "r"(__float_as_uint(r.m)), "r"(__float_as_uint(r.s)), "r"((uint32_t)r.idx), "r"(0u)
+                   : "memory");
+  }
+  if (!all_here) sm100::cluster_wait();
+  sm100::cluster_arrive();
+  if (rank != 0) return;
+  tail.arrived();
+  sm100::cluster_wait();  // every slice is here
+  tail.template merge_rows<4>(slots, SharedSlices{});
+  tail.walk();
+#if __CUDA_ARCH__ >= 900
+  cudaGridDependencySynchronize();  // complete no sooner than the attention
+  pdl_launch_dependents();
+#endif
 }
 
 size_t tail_smem_bytes(const spiffy_decide_desc& d, int parent_cap) {
@@ -347,6 +479,13 @@ spiffy_status launch_decide_finalize(const spiffy_decide_desc& d, const void* pa
 // merge (16 x 32 positions x 28 heads, x 19: 21.5 and 21.5, 27.0 and 27.7, 36.9 and 37.3).
 constexpr int kTailRows = 512, kTailPartials = 4096;
 constexpr size_t kTailSmem = 48 * 1024 - 1024;  // what the kernel declares itself comes on top
+// Beside a CUDA-core attention (`independent`) up to kSmallSlices slices a sequence take one launch of a cluster.
+// fp32, the step with one launch and with two, us: 4 x 8 rows of one slice 6.3 and 9.2, 4 x 16 over 500 keys 29.0
+// and 31.9, 2 x 32 over 4000 keys x 32 heads 127.2 and 130.1, 4 x 2 x 32 so 501 and 505, 2 x 8 x 8 90.8 and 94.2,
+// 3 x 8 of two 6.7 and 8.9; beyond, 3 x 8 rows of five slices 9.9 and 8.2, 8 x 32 of one 19.4 and 12.3.
+// A decision in front of an attention or by itself is no sooner done in one launch (bf16, 4 x 8 rows of one
+// slice 7.2 and 7.2 us with the attention, 4 x 16 9.3 and 7.3).
+constexpr int kSmallSlices = 64, kSmallBatch = 8;
 spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits,
                                  const int32_t* block_tokens, float* conf, int32_t* top_tok,
                                  uint64_t* unmask_bits, int32_t* n_unmask,
@@ -365,6 +504,23 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
     if (st != SPIFFY_OK) return st;
     return launch_walk(d, block_tokens, parent_off, parent_idx, parent_cap, top_tok, unmask_bits,
                        accepted_node, n_accepted, path, next_block, walk_status, fresh, stream);
+  }
+  const size_t small_smem = smem + (size_t)rows_of_one * splits * sizeof(Partial);
+  if (independent && rows_of_one <= kSmallRows && rows_of_one * splits <= kSmallSlices && small_smem <= kTailSmem &&
+      d.batch <= kSmallBatch) {
+    const TailArgs a = {splits, (int)d.n_nodes, (int)d.block_len, (int)d.mask_token_id, (int)d.rule, (int)d.top_s,
+                        d.threshold, block_tokens, parent_off, parent_idx, (int)parent_cap, conf, top_tok, unmask_bits,
+                        n_unmask, decide_status, accepted_node, n_accepted, path, next_block, walk_status};
+    auto run = [&](auto kernel, auto* typed) {
+      return launch_pdl(kernel, dim3(kSmallCtas * d.batch), dim3(kSmallGroups * kReduceThreads), small_smem, stream, a, typed,
+                        (int64_t)d.row_stride, (int)d.vocab, chunk, (int)next,
+                        status_clear(d, fresh, decide_status, walk_status));
+    };
+    const cudaError_t e = d.logits_dtype == SPIFFY_BF16
+                              ? run(decide_small_kernel<__nv_bfloat16>, static_cast<const __nv_bfloat16*>(logits))
+                              : run(decide_small_kernel<float>, static_cast<const float*>(logits));
+    count_launch();
+    return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
   }
   Partial* partials = static_cast<Partial*>(ws);
   const spiffy_status st = launch_reduce(d, logits, block_tokens, partials, splits, chunk, 1, independent,

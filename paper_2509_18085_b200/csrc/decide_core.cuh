@@ -179,9 +179,10 @@ __device__ __forceinline__ float warp_max(float x) {
 // gets the sum of exp((x - maximum) / T).  `tag`, if not 0, goes into the result's spare word
 // in the one 16-byte access that writes it: a reader that polls for the tag has the rest with it.
 // `out` may be null: thread 0 has the result anyway.  `keep`, in shared memory, gets the slice's
-// vectors, number i at kept_at(i).
+// vectors, number i at kept_at(i).  kGroups: the CTA is that many groups of kReduceThreads threads, each
+// with a slice of its own (named barriers 1 ...); "thread 0" is then the group's first.
 __device__ __forceinline__ int kept_at(int i) { return i ^ ((i >> 3) & 7); }  // no bank conflicts at stride 8 either
-template <typename T>
+template <typename T, int kGroups = 1>
 __device__ __forceinline__ Partial reduce_slice(const T* __restrict__ base, int V, int64_t chunk,
                                              int split, Partial* __restrict__ out,
                                              const float k = kLog2e, const int tag = 0, uint4* keep = nullptr) {
@@ -192,7 +193,12 @@ __device__ __forceinline__ Partial reduce_slice(const T* __restrict__ base, int 
   const int nvec = begin < end ? (int)((end - begin) / EPV) : 0;  // <= kReduceThreads * kUnroll
   const int ntail = begin < end ? (int)(end - begin) - nvec * EPV : 0;  // < EPV, last slice only
   const uint4* p = reinterpret_cast<const uint4*>(base + begin);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int group = kGroups == 1 ? 0 : (int)threadIdx.x / kReduceThreads;
+  const int tid = (int)threadIdx.x - group * kReduceThreads, warp = tid >> 5, lane = tid & 31;
+  auto sync = [&]() {
+    if constexpr (kGroups == 1) __syncthreads();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kReduceThreads) : "memory");
+  };
 
   // 1. the thread's vectors t, t + kReduceThreads, ...; thread 0 also takes the ragged tail
   uint4 v[kUnroll];
@@ -214,11 +220,13 @@ __device__ __forceinline__ Partial reduce_slice(const T* __restrict__ base, int 
   for (int e = 0; e < EPV; ++e) m = fmaxf(m, tail[e]);
   const float mine = m;
   m = warp_max(m);
-  __shared__ float warp_m[kReduceThreads / 32], warp_s[kReduceThreads / 32];
-  __shared__ int slice_idx;
+  __shared__ float warp_ms[kGroups][kReduceThreads / 32], warp_ss[kGroups][kReduceThreads / 32];
+  __shared__ int slice_idxs[kGroups];
+  float *const warp_m = warp_ms[group], *const warp_s = warp_ss[group];
+  int& slice_idx = slice_idxs[group];
   if (lane == 0) warp_m[warp] = m;
   if (tid == 0) slice_idx = 0x7fffffff;
-  __syncthreads();
+  sync();
   m = warp_m[0];
 #pragma unroll
   for (int w = 1; w < kReduceThreads / 32; ++w) m = fmaxf(m, warp_m[w]);
@@ -253,7 +261,7 @@ __device__ __forceinline__ Partial reduce_slice(const T* __restrict__ base, int 
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
   if (lane == 0) warp_s[warp] = s;
-  __syncthreads();
+  sync();
   Partial r = {m, s, 0, tag};
   if (tid == 0) {
     s = warp_s[0];
@@ -280,12 +288,15 @@ __device__ __forceinline__ int4 load16(const void* p) {
 // How finalize_row comes by a row's slices.  Complete: they are all there, written by an earlier kernel.
 // They are read at L2, as this CTA may have been resident while that kernel wrote them.
 struct CompleteSlices {
-  static constexpr bool kWaits = false;
+  static constexpr bool kWaits = false, kShared = false;
+};
+struct SharedSlices {  // ... in this CTA's shared memory
+  static constexpr bool kWaits = false, kShared = true;
 };
 // They are being written: a slice is there when its spare word is `tag`.  At most `polls` looks at a batch
 // of slices; `missing` when they ran out, and the row's results mean nothing.
 struct TaggedSlices {
-  static constexpr bool kWaits = true;
+  static constexpr bool kWaits = true, kShared = false;
   int tag;
   unsigned polls;
   bool missing = false;
@@ -302,7 +313,7 @@ template <int kLanes, class Source = CompleteSlices>
 __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int splits, int sub,
                                              int32_t state, int mask_id, float& conf, int32_t& tok,
                                              Source&& from = Source{}) {
-  constexpr bool kWaits = std::remove_reference_t<Source>::kWaits;
+  constexpr bool kWaits = std::remove_reference_t<Source>::kWaits, kShared = std::remove_reference_t<Source>::kShared;
   constexpr int kAcc = 8 / kLanes;
   float m[kAcc], s[kAcc];
   int idx[kAcc];
@@ -325,7 +336,8 @@ __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int 
         const int k = sub + kLanes * (t0 + u);
         q[u] = Partial{-INFINITY, 0.f, 0x7fffffff, 0};
         if (k < splits && state == mask_id) {  // the slices of an unmasked row were never written
-          const int4 w = kWaits ? load16(p + k) : __ldcg(reinterpret_cast<const int4*>(p + k));
+          const int4* at = reinterpret_cast<const int4*>(p + k);
+          const int4 w = kShared ? *at : kWaits ? load16(at) : __ldcg(at);
           q[u] = Partial{__int_as_float(w.x), __int_as_float(w.y), w.z, w.w};
         }
       }

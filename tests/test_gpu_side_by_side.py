@@ -22,6 +22,10 @@ pytestmark = pytest.mark.gpu
     # a call of two launches, the second by pairs and by one M-tile per block; beside the fused tail and not
     (5, 8, 32, 256, 32, 32, 128, 1000, "bf16"), (1, 18, 60, 100, 150, 50, 128, 1000, "bf16"),
     (2, 3, 32, 500, 5, 5, 128, 2864, "f32"),
+    # fp32: the decision in one launch, up to 64 slices a sequence and 8 sequences, and just beyond
+    (1, 1, 1, 60, 1, 1, 64, 52, "f32"), (8, 4, 16, 60, 4, 4, 64, 1000, "f32"), (9, 4, 16, 60, 4, 4, 64, 1000, "f32"),
+    (1, 3, 21, 60, 4, 4, 64, 4096, "f32"), (1, 1, 64, 60, 4, 4, 64, 4096, "f32"), (2, 1, 64, 60, 4, 4, 64, 4100, "f32"),
+    (3, 4, 4, 60, 4, 4, 64, 16384, "f32"), (1, 64, 1, 60, 4, 4, 64, 300, "f32"), (1, 65, 1, 60, 4, 4, 64, 300, "f32"),
 ])
 def test_same_bits_as_one_after_the_other(B, N, L, P, Hq, Hkv, d, V, dtype):
     cfg = W.Config("t", B, N, L, P, Hq, Hkv, d, dtype, V, spiffy.RULE_THRESHOLD)
