@@ -19,16 +19,17 @@
 // output word 0 giving u_s, word 1 giving u' and u = (word + 0.5) / 2^32: the
 // noise follows the state of the block, never the node's index.
 //
-// A vocabulary of several slices takes two kernels.  The reduce is the greedy
+// A vocabulary of several slices takes three kernels.  The reduce is the greedy
 // decision's (one pass over the logits, HBM-bound) with the exponent scaled by
 // 1 / T.  The select kernel, one CTA per row, picks the slice from the partial
 // results (one generator call per slice), re-reads that one slice (16 KB, mostly
-// still in L2), inverts its running sum, and the last CTA of a node to finish
-// applies the rule.  A vocabulary of one slice: the select kernel reduces it itself
-// and keeps it in shared memory, which spares a launch and three trips through L2,
-// and a kernel of one CTA per sequence applies the rule, as nothing came before
-// that could have cleared the nodes' arrival counters (49 masked rows of 64 x
-// 2251: 8.6 -> 5.5 us; 3144 of 4608 x 4064: 40.9 -> 28.9).
+// still in L2) and inverts its running sum.  The rule kernel, a warp per node, is
+// resident by then, its tokens read.  (The last CTA of a node to finish applied the
+// rule before: a fence, an arrival counter and a trip for the confidences more.
+// 8 x 32 rows x 16 slices 16.8 -> 15.9 us, 4 x 512 x 8 46.1 -> 43.5, 32 x 8 8.6 -> 8.4.)
+// A vocabulary of one slice: the select kernel reduces it itself and keeps it in
+// shared memory, which spares a launch and three trips through L2 (49 masked rows of
+// 64 x 2251: 8.6 -> 5.5 us; 3144 of 4608 x 4064: 40.9 -> 28.9).
 #include <type_traits>
 
 #include "common.cuh"
@@ -88,23 +89,18 @@ __device__ __forceinline__ void merge_t(float& m, float& s, float m2, float s2, 
   m = M;
 }
 
-// grid = (splits, B*N*L); one CTA reduces one vocabulary slice of one row and
-// the first CTA of row i clears node i's arrival counter for the select kernel.
+// grid = (splits, B*N*L); one CTA reduces one vocabulary slice of one row.
 template <typename T>
 __global__ void __launch_bounds__(kReduceThreads, 9)
 decide_sampled_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V, int64_t chunk,
-                             int splits, int nodes, const int32_t* __restrict__ block_tokens, int mask_id,
-                             float k, Partial* __restrict__ partials, int* __restrict__ node_count,
-                             StatusClear clear) {
+                             int splits, const int32_t* __restrict__ block_tokens, int mask_id,
+                             float k, Partial* __restrict__ partials, StatusClear clear) {
 #if __CUDA_ARCH__ >= 900
   cudaGridDependencySynchronize();
 #endif
   const int row = blockIdx.y;
   const int32_t token = block_tokens[row];  // ahead of the clearing: every CTA waits for it first
-  if (blockIdx.x == 0 && threadIdx.x == kReduceThreads - 1 && row < nodes) {  // at least as many as sequences
-    node_count[row] = 0;
-    if (row < clear.batch) clear.run(row);
-  }
+  if (blockIdx.x == 0 && threadIdx.x == kReduceThreads - 1 && row < clear.batch) clear.run(row);
   if (token != mask_id) return;  // already unmasked: never read
   reduce_slice(logits + (int64_t)row * row_stride, V, chunk, (int)blockIdx.x,
                partials + (int64_t)row * splits + blockIdx.x, k);
@@ -141,16 +137,15 @@ struct SliceChoice {
 
 // grid = B*N*L rows; kReduceThreads threads; thread t holds the vectors
 // 8 t ... 8 t + 7 of the chosen slice, i.e. a contiguous run of entries.  kWhole: the row is one
-// slice, reduced here, and the rule is left to decide_sampled_rule_kernel.
+// slice, reduced here.
 template <typename T, bool kWhole>
 __global__ void __launch_bounds__(kReduceThreads, 5)  // 96 registers
 decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, int V, int64_t chunk,
                              int splits, int N, int L, const int32_t* __restrict__ block_tokens,
-                             int mask_id, int rule, int top_s, float tau, float inv_t,
-                             uint32_t seed_lo, uint32_t seed_hi, Partial* partials,
-                             int* __restrict__ node_count, float* __restrict__ conf_out,
-                             int32_t* __restrict__ tok_out, uint64_t* __restrict__ bits_out,
-                             int32_t* __restrict__ n_unmask_out, int32_t* __restrict__ dev_status) {
+                             int mask_id, float inv_t,
+                             uint32_t seed_lo, uint32_t seed_hi, const Partial* partials,
+                             float* __restrict__ conf_out, int32_t* __restrict__ tok_out,
+                             int32_t* __restrict__ dev_status) {
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr uint32_t NI = Elem<T>::kNegInf;
   const int row = blockIdx.x;
@@ -179,13 +174,11 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
   }
 #if __CUDA_ARCH__ >= 900
   pdl_launch_dependents();
-  if (!kWhole) cudaGridDependencySynchronize();  // the reduce kernel's partials and cleared counters are visible
+  if (!kWhole) cudaGridDependencySynchronize();  // the reduce kernel's partials are visible
 #endif
   const float k = inv_t * kLog2e;
   __shared__ SliceChoice choice;
   __shared__ double warp_total[kReduceThreads / 32];
-  __shared__ int is_last;
-  __shared__ float sconf[64];
   __shared__ uint4 kept[kWhole ? kReduceThreads * kUnroll : 1];  // the row, when it is one slice
   if (state == mask_id) {  // the whole CTA takes the same branch
     if (kWhole) {
@@ -239,7 +232,6 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
         conf_out[row] = __int_as_float(0x7fc00000);  // NaN: never wins the rule
         tok_out[row] = 0;
         if (!kWhole && dev_status) atomicOr(dev_status + b, SPIFFY_DEV_NONFINITE);
-        __threadfence();
       }
     } else {
       // level 2: the chosen slice, entries in ascending order over (thread, vector, element)
@@ -342,59 +334,58 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
         }
         conf_out[row] = fminf(1.0f, ex2((x_pick - c.row_m) * k) / c.row_s);
         tok_out[row] = (int32_t)begin + pick;
-        __threadfence();
       }
     }
   } else if (tid == 0) {
     conf_out[row] = -INFINITY;
     tok_out[row] = state;
-    __threadfence();
-  }
-  if (kWhole) return;
-  // the last row of a node to arrive applies the rule to the node
-  __syncthreads();
-  if (tid == 0) is_last = atomicAdd(node_count + node, 1) == L - 1;
-  __syncthreads();
-  if (!is_last || warp != 0) return;
-  __threadfence();
-  for (int i = lane; i < L; i += 32) sconf[i] = __ldcg(conf_out + (int64_t)node * L + i);
-  __syncwarp();
-  const uint64_t bits = unmask_rule(sconf, block_tokens + (int64_t)node * L, L, mask_id, rule, top_s, tau, lane);
-  if (lane == 0) {
-    bits_out[node] = bits;
-    n_unmask_out[node] = __popcll(bits);
   }
 }
 
-// grid = sequences, a warp per node: one CTA per sequence, so that the status word, which may arrive
-// with arbitrary contents (fresh), has one writer.
-constexpr int kRuleThreads = 512;
+// A warp per node; grid = sequences * ctas, CTA c of a sequence taking its nodes 16 c, 16 c + 1, ....  Where the
+// status word may arrive with arbitrary contents (kStatus: nothing came before that could have cleared it) it
+// has one writer: one CTA per sequence, for all nodes.
+constexpr int kRuleThreads = 512, kRuleWarps = kRuleThreads / 32;
+template <bool kStatus>
 __global__ void __launch_bounds__(kRuleThreads)
-decide_sampled_rule_kernel(const float* __restrict__ conf, int N, int L, const int32_t* __restrict__ block_tokens,
+decide_sampled_rule_kernel(const float* __restrict__ conf, int N, int L, int ctas, const int32_t* __restrict__ block_tokens,
                            int mask_id, int rule, int top_s, float tau, uint64_t* __restrict__ bits_out,
                            int32_t* __restrict__ n_unmask_out, int32_t* __restrict__ dev_status, int fresh) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b = blockIdx.x;
-  __shared__ float sconf[kRuleThreads / 32][64];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b = (int)blockIdx.x / ctas, first = ((int)blockIdx.x - b * ctas) * kRuleWarps + warp;
+  __shared__ float sconf[kRuleWarps][64];
+  __shared__ int32_t stoken[kRuleWarps][64];
+  auto tokens_of = [&](int n) {
+    const int32_t* t = block_tokens + ((int64_t)b * N + n) * L;
+    for (int i = lane; i < L; i += 32) stoken[warp][i] = t[i];
+  };
 #if __CUDA_ARCH__ >= 900
   pdl_launch_dependents();
+#endif
+  // The select kernel started behind one that had waited, or waited before it let this one start: the tokens are
+  // complete.
+  if (first < N) tokens_of(first);
+#if __CUDA_ARCH__ >= 900
   cudaGridDependencySynchronize();
 #endif
   bool bad = false;
-  for (int n = warp; n < N; n += kRuleThreads / 32) {
+  for (int n = first; n < N; n += kStatus ? kRuleWarps : N) {
     const int64_t node = (int64_t)b * N + n;
+    if (n != first) tokens_of(n);
     for (int i = lane; i < L; i += 32) {
       const float c = __ldcg(conf + node * L + i);
       bad |= c != c;  // the mark of a row without a usable distribution
       sconf[warp][i] = c;
     }
     __syncwarp();
-    const uint64_t bits = unmask_rule(sconf[warp], block_tokens + node * L, L, mask_id, rule, top_s, tau, lane);
+    const uint64_t bits = unmask_rule(sconf[warp], stoken[warp], L, mask_id, rule, top_s, tau, lane);
     if (lane == 0) {
       bits_out[node] = bits;
       n_unmask_out[node] = __popcll(bits);
     }
     __syncwarp();
   }
+  if (!kStatus) return;
   bad = __syncthreads_or(bad);
   if (threadIdx.x == 0 && dev_status) {
     const int32_t flag = bad ? SPIFFY_DEV_NONFINITE : 0;
@@ -411,7 +402,7 @@ size_t partial_bytes(const spiffy_decide_desc& d) {
 }  // namespace
 
 size_t decide_sampled_workspace_bytes(const spiffy_decide_desc& d) {
-  return partial_bytes(d) + (size_t)d.batch * d.n_nodes * sizeof(int);
+  return partial_bytes(d);
 }
 
 spiffy_status launch_decide_sampled(const spiffy_decide_desc& d, float temperature, uint64_t seed,
@@ -422,7 +413,7 @@ spiffy_status launch_decide_sampled(const spiffy_decide_desc& d, float temperatu
   const int splits = decide_splits(d, &chunk);
   const int rows = d.batch * d.n_nodes * d.block_len;
   Partial* partials = static_cast<Partial*>(ws);
-  int* node_count = reinterpret_cast<int*>(static_cast<char*>(ws) + partial_bytes(d));
+  const Partial* cpartials = partials;
   const float inv_t = 1.0f / temperature;
   const uint32_t lo = (uint32_t)(seed & 0xffffffffu), hi = (uint32_t)(seed >> 32);
   cudaError_t e;
@@ -432,21 +423,23 @@ spiffy_status launch_decide_sampled(const spiffy_decide_desc& d, float temperatu
     cudaError_t r = cudaSuccess;
     if (!whole) {
       r = launch_pdl(decide_sampled_reduce_kernel<T>, dim3(splits, rows), dim3(kReduceThreads), (size_t)0, stream,
-                     typed, (int64_t)d.row_stride, (int)d.vocab, chunk, splits, (int)(d.batch * d.n_nodes), block_tokens,
-                     (int)d.mask_token_id, inv_t * kLog2e, partials, node_count, status_clear(d, fresh, dev_status, nullptr));
+                     typed, (int64_t)d.row_stride, (int)d.vocab, chunk, splits, block_tokens,
+                     (int)d.mask_token_id, inv_t * kLog2e, partials, status_clear(d, fresh, dev_status, nullptr));
       count_launch();
       if (r != cudaSuccess) return r;
     }
     r = launch_pdl(whole ? decide_sampled_select_kernel<T, true> : decide_sampled_select_kernel<T, false>, dim3(rows),
                    dim3(kReduceThreads), (size_t)0, stream, typed, (int64_t)d.row_stride, (int)d.vocab, chunk, splits,
-                   (int)d.n_nodes, (int)d.block_len, block_tokens, (int)d.mask_token_id, (int)d.rule, (int)d.top_s,
-                   d.threshold, inv_t, lo, hi, partials, node_count, conf, top_tok, unmask_bits, n_unmask, dev_status);
+                   (int)d.n_nodes, (int)d.block_len, block_tokens, (int)d.mask_token_id, inv_t, lo, hi, cpartials, conf,
+                   top_tok, dev_status);
     count_launch();
-    if (r != cudaSuccess || !whole) return r;
+    if (r != cudaSuccess) return r;
     const float* cconf = conf;
-    r = launch_pdl(decide_sampled_rule_kernel, dim3(d.batch), dim3(kRuleThreads), (size_t)0, stream, cconf,
-                   (int)d.n_nodes, (int)d.block_len, block_tokens, (int)d.mask_token_id, (int)d.rule, (int)d.top_s,
-                   d.threshold, unmask_bits, n_unmask, dev_status, fresh ? 1 : 0);
+    const int ctas = whole ? 1 : (d.n_nodes + kRuleWarps - 1) / kRuleWarps;
+    r = launch_pdl(whole ? decide_sampled_rule_kernel<true> : decide_sampled_rule_kernel<false>, dim3(d.batch * ctas),
+                   dim3(kRuleThreads), (size_t)0, stream, cconf, (int)d.n_nodes, (int)d.block_len, ctas, block_tokens,
+                   (int)d.mask_token_id, (int)d.rule, (int)d.top_s, d.threshold, unmask_bits, n_unmask, dev_status,
+                   fresh ? 1 : 0);
     count_launch();
     return r;
   };
