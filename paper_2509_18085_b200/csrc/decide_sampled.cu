@@ -210,19 +210,14 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
           }
         }
       }
+      // the row's maximum and sum, in a fixed order; the best slice, the first of equal ones
+      const float row_m = warp_max(rm), top = warp_max(best);
+      rs *= rm == row_m ? 1.f : ex2((rm - row_m) * k);
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {  // fixed order
-        merge_t(rm, rs, __shfl_xor_sync(0xffffffffu, rm, off), __shfl_xor_sync(0xffffffffu, rs, off), k);
-        const float s2 = __shfl_xor_sync(0xffffffffu, best, off);
-        const int i2 = __shfl_xor_sync(0xffffffffu, bs, off);
-        const uint32_t w2 = __shfl_xor_sync(0xffffffffu, bw, off);
-        const float m2 = __shfl_xor_sync(0xffffffffu, bm, off);
-        const float z2 = __shfl_xor_sync(0xffffffffu, bz, off);
-        if (i2 != 0x7fffffff && (bs == 0x7fffffff || s2 > best || (s2 == best && i2 < bs))) {
-          best = s2; bs = i2; bw = w2; bm = m2; bz = z2;
-        }
-      }
-      if (lane == 0) choice = SliceChoice{bs, bw, bm, bz, rm, rs};
+      for (int off = 16; off > 0; off >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, off);
+      const int slice = (int)__reduce_min_sync(0xffffffffu, best == top ? (unsigned)bs : 0x7fffffffu);
+      const unsigned has = __ballot_sync(0xffffffffu, bs == slice);
+      if (lane == __ffs(has) - 1) choice = SliceChoice{slice, bw, bm, bz, row_m, rs};
     }
     __syncthreads();
     const SliceChoice c = choice;
