@@ -26,6 +26,7 @@ constexpr int kVecs = 8;       // 128-bit vectors per thread
 constexpr int kMaxK = 4;       // vocabulary ranks
 constexpr int kBuildThreads = 1024;  // a warp per block position
 constexpr int kRelated = 64;         // formulas whose subset relation fits its table
+constexpr int kAtHand = 4;
 constexpr int kFormulaBytes = 4096;  // shared memory for what is known about so many
 constexpr int kGraphInts = 6144;     // shared-memory copy of the draft graph (24 KB)
 
@@ -257,8 +258,8 @@ __device__ bool strict_subset(const BuildArgs& g, int a, int c) {
 // position's slices and takes its logarithms, a second step sorts the positions, and one warp, a formula a
 // lane, does the rest without another barrier, in loops that are not unrolled.  32 positions x 16 slices, ten
 // formulas: 4600 cycles to the wait and 14200 behind it with 1024 threads at eight barriers, formulas looked up
-// through generic pointers pair by pair, logarithms inside the chains and merges by shuffles; 4500 and 7900
-// now (the call 13.0 -> 9.8 us).  The whole chain gone through once beforehand, to have its instructions at
+// through generic pointers pair by pair, logarithms inside the chains and merges by shuffles; 4500 and 7000
+// now (the call 13.0 -> 9.4 us).  The whole chain gone through once beforehand, to have its instructions at
 // hand, takes longer than the top-k kernel leaves time for (22 us).
 __global__ void __launch_bounds__(kBuildThreads)
 draft_build_kernel(BuildArgs g) {
@@ -357,6 +358,21 @@ draft_build_kernel(BuildArgs g) {
       if (lane == 0) fs.subsets[c][w % (kRelated / 32)] = word;
     }
     __syncthreads();
+  }
+  // Of up to 32 formulas of up to four candidates and children each, lane q of the first two warps has those of
+  // formula q at hand: places in by_rank_log (-1: no more), indices in fs.local.
+  bool at_hand = false;
+  int place[kAtHand], kid[kAtHand], n_places = 0, needed = 0x7fffffff;
+  if (one_warp && D <= 32 && warp <= 1) {
+    const int q = min(lane, D - 1), e0 = f_off[q], k0 = c_off[q], n_kids = c_off[q + 1] - k0;
+    n_places = f_off[q + 1] - e0;
+    needed = fs.ranks_needed[q];
+    at_hand = __all_sync(0xffffffffu, n_places <= kAtHand && n_kids <= kAtHand);
+#pragma unroll
+    for (int u = 0; u < kAtHand; ++u) {
+      place[u] = u < n_places && needed <= 64 ? f_i[e0 + u] * kMaxK + f_j[e0 + u] : -1;
+      kid[u] = u < n_kids ? c_idx[k0 + u] : kRelated;
+    }
   }
 #if __CUDA_ARCH__ >= 900
   cudaGridDependencySynchronize();  // the top-k kernel's partial results are visible, the outputs free
@@ -475,39 +491,68 @@ draft_build_kernel(BuildArgs g) {
     // Two warps with the same numbers: what follows from them is written by one or the other.
     if (warp > 1) return;
     const bool lists = warp == 0, drafts = warp == 1 || warps == 1;
-#pragma unroll 1
-    for (int q = lane; q < D; q += 32) {  // 3. local scores: geometric means of the candidates' probabilities
-      const int e0 = f_off[q], e1 = f_off[q + 1];
+    if (at_hand) {  // 3. and 4. as below, the look-ups all at once
       float x = -INFINITY, lg = -INFINITY;
-      if (fs.ranks_needed[q] <= masked) {
-        float logsum = 0.f;
-#pragma unroll 2
-        for (int e = e0; e < e1; ++e) logsum += by_rank_log[f_i[e] * kMaxK + f_j[e]];
-        x = expf(logsum / (float)(e1 - e0));  // 0 where a candidate has no probability
+      if (needed <= masked) {
+        float v[kAtHand];
+#pragma unroll
+        for (int u = 0; u < kAtHand; ++u) v[u] = place[u] >= 0 ? by_rank_log[max(place[u], 0)] : 0.f;
+        x = expf((((v[0] + v[1]) + v[2]) + v[3]) / (float)n_places);
         lg = x > 0.f ? logf(fmaxf(x, 1e-45f)) : -INFINITY;
       }
-      fs.local[q] = x;
-      fs.log[q] = lg;
-    }
-    __syncwarp();
-#pragma unroll 1
-    for (int q = lane; q < D; q += 32) {  // 4. score = GM(local, GM(children's)); without buildable children local
-      float x = fs.local[q];
-      if (x != -INFINITY) {
-        float logsum = 0.f;
-        int n = 0;
-        const int e1 = c_off[q + 1];
-#pragma unroll 2
-        for (int e = c_off[q]; e < e1; ++e) {
-          const int y = c_idx[e];
-          if (fs.local[y] == -INFINITY) continue;
-          logsum += fs.log[y];
-          ++n;
-        }
-        if (n > 0) x = sqrtf(x * expf(logsum / (float)n));
+      if (lane < D) {
+        fs.local[lane] = x;
+        fs.log[lane] = lg;
       }
-      fs.total[q] = x;
-      if (lists) g.score[(int64_t)b * D + q] = x;
+      __syncwarp();
+      int n = 0;
+      float sum = 0.f;
+#pragma unroll
+      for (int u = 0; u < kAtHand; ++u) {
+        const bool counts = fs.local[kid[u]] != -INFINITY;
+        sum += counts ? fs.log[kid[u]] : 0.f;
+        n += counts;
+      }
+      if (x != -INFINITY && n > 0) x = sqrtf(x * expf(sum / (float)n));
+      if (lane < D) {
+        fs.total[lane] = x;
+        if (lists) g.score[(int64_t)b * D + lane] = x;
+      }
+    } else {
+#pragma unroll 1
+      for (int q = lane; q < D; q += 32) {  // 3. local scores: geometric means of the candidates' probabilities
+        const int e0 = f_off[q], e1 = f_off[q + 1];
+        float x = -INFINITY, lg = -INFINITY;
+        if (fs.ranks_needed[q] <= masked) {
+          float logsum = 0.f;
+#pragma unroll 2
+          for (int e = e0; e < e1; ++e) logsum += by_rank_log[f_i[e] * kMaxK + f_j[e]];
+          x = expf(logsum / (float)(e1 - e0));  // 0 where a candidate has no probability
+          lg = x > 0.f ? logf(fmaxf(x, 1e-45f)) : -INFINITY;
+        }
+        fs.local[q] = x;
+        fs.log[q] = lg;
+      }
+      __syncwarp();
+#pragma unroll 1
+      for (int q = lane; q < D; q += 32) {  // 4. score = GM(local, GM(children's)); without buildable children local
+        float x = fs.local[q];
+        if (x != -INFINITY) {
+          float logsum = 0.f;
+          int n = 0;
+          const int e1 = c_off[q + 1];
+#pragma unroll 2
+          for (int e = c_off[q]; e < e1; ++e) {
+            const int y = c_idx[e];
+            if (fs.local[y] == -INFINITY) continue;
+            logsum += fs.log[y];
+            ++n;
+          }
+          if (n > 0) x = sqrtf(x * expf(logsum / (float)n));
+        }
+        fs.total[q] = x;
+        if (lists) g.score[(int64_t)b * D + q] = x;
+      }
     }
     __syncwarp();
     uint64_t keep_bits = 0;  // 5. the D* best (score desc, formula index asc) keep their formula order
