@@ -436,7 +436,8 @@ spiffy_status spiffy_accept_walk(const spiffy_decide_desc* desc,
  * fp32 entries a row comes in; any number under SPIFFY_INDEPENDENT_NEXT), the
  * merge of the slices, the unmasking rule and the walk run in one kernel per
  * sequence, one launch fewer than the two separate calls; otherwise this is the
- * two calls.
+ * two calls.  Under SPIFFY_INDEPENDENT up to 64 slices a sequence (N * L <= 64,
+ * at most 8 sequences) are one launch in all, the reduce included.
  * Workspace: spiffy_unmask_decide_workspace(desc).
  */
 spiffy_status spiffy_decide_walk(const spiffy_decide_desc* desc, const void* logits,

@@ -200,7 +200,7 @@ graph_attention_simt_kernel(const SimtParams p, const T* __restrict__ q, const T
     stage_wait();     // V of this tile
     __syncthreads();  // ... of every thread; K has been read
     if (t + 1 < t1) stage_tile(sk, kp, kb, t + 1);
-#pragma unroll 2
+#pragma unroll 4  // 1 to 2 % over two (64 x 32 positions x 32 heads on 8 over 4000 keys 3175 us, 3132 so)
     for (int c4 = 0; c4 < kKeys / 4; ++c4) {
       float4 pv[R];
 #pragma unroll

@@ -190,7 +190,7 @@ spiffy_status launch_attention_tc_dual(const spiffy_attn_desc& d0, const AttnPro
 //   - Every kernel waits, and none is complete before it has waited, so that a kernel which
 //     is complete, or has been waited for, stands for all that came before it in the stream.
 //   - Before its wait a kernel writes nothing in global memory and reads nothing, except:
-//     (a) The walk, tail and sampled selection kernels read the block's tokens, the first two
+//     (a) The walk, tail, sampled selection and rule kernels read the block's tokens, the first two
 //         the parent lists as well.  Each comes behind a kernel of its own call that waited
 //         before it let its dependents start (the reduces do, and the finalize kernel is
 //         itself launched behind one), so whatever wrote those arrays ahead of the call is
@@ -200,7 +200,8 @@ spiffy_status launch_attention_tc_dual(const spiffy_attn_desc& d0, const AttnPro
 //         the root kernel, which waited.
 //     (b) The draft-build kernel reads the draft formulas, constants of the model, and the block, as the
 //         top-k kernel in front of it waited before it let it start.
-//     (c) The reduce under SPIFFY_INDEPENDENT and the attention under SPIFFY_ATTN_INDEPENDENT
+//     (c) The reduce, or the one kernel that few slices take, under SPIFFY_INDEPENDENT and the attention
+//         under SPIFFY_ATTN_INDEPENDENT
 //         read their inputs, write their outputs and wait last.  What precedes them is, by the
 //         flags' contract, a call that touches none of these; its kernels started, in turn,
 //         behind one that had waited before it triggered (the CUDA-core attention; the reduce
