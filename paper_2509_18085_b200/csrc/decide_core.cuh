@@ -308,8 +308,9 @@ struct TaggedSlices {
 // (accumulator j takes slices j, j + 8, ...) are combined by the butterfly
 // 4, 2, 1 with the lower index first; a lane holds the accumulators j = sub,
 // sub + kLanes, ... and does the butterfly steps that stay inside it locally.
-// Returns false on lane 0 when the row is masked and not usable.
-template <int kLanes, class Source = CompleteSlices>
+// Returns false on lane 0 when the row is masked and not usable.  kAtOnce: slices of a lane on their way at
+// a time, at least (the order of the merge does not depend on it).
+template <int kLanes, class Source = CompleteSlices, int kAtOnce = 4>
 __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int splits, int sub,
                                              int32_t state, int mask_id, float& conf, int32_t& tok,
                                              Source&& from = Source{}) {
@@ -326,7 +327,8 @@ __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int 
   // this lane's slices are sub, sub + kLanes, sub + 2 kLanes, ...; slice number t
   // goes to accumulator t mod kAcc.  They are fetched kBatch at a time, all
   // loads of a batch in flight together; a missing slice merges as the identity.
-  constexpr int kBatch = kAcc > 4 ? kAcc : 4;
+  constexpr int kBatch = kAcc > kAtOnce ? kAcc : kAtOnce;
+  static_assert(kBatch % kAcc == 0, "slice number t of a lane goes to accumulator t mod kAcc");
   for (int t0 = 0; sub + kLanes * t0 < splits; t0 += kBatch) {
     Partial q[kBatch];
     auto fetch = [&]() {
