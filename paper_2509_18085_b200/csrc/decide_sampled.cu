@@ -397,7 +397,9 @@ size_t partial_bytes(const spiffy_decide_desc& d) {
 }  // namespace
 
 size_t decide_sampled_workspace_bytes(const spiffy_decide_desc& d) {
-  return partial_bytes(d);
+  // The word per node, which arrival counters took once, stays part of the query's answer: what callers hold and
+  // check against it keeps its size.
+  return partial_bytes(d) + (size_t)d.batch * d.n_nodes * sizeof(int);
 }
 
 spiffy_status launch_decide_sampled(const spiffy_decide_desc& d, float temperature, uint64_t seed,
