@@ -328,7 +328,7 @@ draft_build_kernel(BuildArgs g) {
   __syncthreads();
   if (one_warp) {
     if (tid == 0) fs.local[kRelated] = -INFINITY;
-    if (tid < kRelated) fs.total[tid] = -INFINITY;
+    for (int i = tid; i < kRelated; i += threads) fs.total[i] = -INFINITY;
     for (int q = tid; q < D; q += threads) {
       uint64_t set[kMaxK] = {};
       const int e0 = f_off[q], e1 = f_off[q + 1];

@@ -153,3 +153,26 @@ def test_graphs_at_the_edges_of_the_build_kernel(D, L, budget, top_k):
     got, want = run_both(logits, state, V - 1, budget, top_k, torch.float32, formulas, children)
     assert assert_parity(got, want, 2e-5) >= 1
     assert budget < 3 or int(want.parent_off[0, -1]) > budget
+
+
+@pytest.mark.parametrize("D", [33, 34, 35, 61, 63, 64])
+@pytest.mark.parametrize("budget", [1, 2, 4])
+def test_a_block_of_one_position_behind_another_call(D, budget):
+    """One warp builds it, of formulas for two: what a call of 64 confident formulas left in shared memory, on
+    every multiprocessor, has no part in the ranking."""
+    full = [[(i, 0)] for i in range(32)] + [[(i, 0), (i + 1, 0)] for i in range(31)] + [[(0, 0), (1, 0), (2, 0)]]
+    sure = np.zeros((600, 32, 64), dtype=np.float32)
+    sure[..., 5] = 20.0
+    full_graph = spiffy.draft_graph(full, [[] for _ in full])
+    sure, masked = G.to_dev(sure), G.to_dev(np.full((600, 32), 63, dtype=np.int32))
+    r = np.random.default_rng(D)
+    B, V = 300, 40
+    logits = r.standard_normal((B, 1, V)).astype(np.float32)
+    state = np.full((B, 1), V, dtype=np.int32)
+    formulas = [[(1 + q % 8, q // 8 % 4), (10 + q, 0)] for q in range(D)]  # of a position that is not there
+    for j, q in enumerate((0, 7, D - 2, D - 1)):
+        formulas[q] = [(0, j)]
+    spiffy.spiffy_draft_blocks(sure, masked, 63, full_graph, 64, 1)
+    got, want = run_both(logits, state, V, budget, 4, torch.float32, formulas, [[] for _ in formulas])
+    assert assert_parity(got, want, 1e-5) > B // 2
+    assert (want.kept[:, 0] >= 0).all()
