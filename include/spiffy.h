@@ -317,7 +317,9 @@ spiffy_status spiffy_unmask_decide_static(const spiffy_decide_desc* desc,
  *      sum_{w <= v in s*} exp(z_w) reaches u' Z_s*   (inversion inside the slice);
  * conf is its probability softmax(z)[top_tok]; the unmasking rule then runs on
  * conf exactly as in spiffy_unmask_decide, and every other argument, layout and
- * status bit is that call's.  One pass over the logits plus one slice per row:
+ * status bit is that call's.  A masked row that is not finite gets conf = NaN and
+ * top_tok = 0; the rule passes over it, except that of a node whose masked rows
+ * are all so the first is taken (decoding always advances).  One pass over the logits plus one slice per row:
  * the cost of the greedy decision, not of V random numbers per row.
  * The uniforms come from the counter-based generator Philox4x32-10 (Salmon,
  * Moraes, Dror, Shaw, SC 2011):

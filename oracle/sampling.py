@@ -110,8 +110,11 @@ def draw_token(z, u_slice, u_inside, slice_width):
 def apply_rule(conf, tokens, mask_id, rule, top_s, threshold):
     """Sec. 3.1 on given confidences: the top_s most confident masked positions
     (ties to the lower position), or every masked position above the threshold
-    and, if there is none, the most confident one.  Returns (bits, count,
-    margin): margin is how far a confidence is from changing the outcome."""
+    and, if there is none, the most confident one.  A NaN marks a row without a
+    usable distribution: it is passed over; of a node that has no other masked
+    row the first masked position is taken, so that decoding always advances.
+    Returns (bits, count, margin): margin is how far a confidence is from
+    changing the outcome."""
     B, N, L = tokens.shape
     bits = np.zeros((B, N), dtype=np.uint64)
     count = np.zeros((B, N), dtype=np.int32)
@@ -120,6 +123,11 @@ def apply_rule(conf, tokens, mask_id, rule, top_s, threshold):
         for n in range(N):
             masked = [l for l in range(L) if tokens[b, n, l] == mask_id]
             if not masked:
+                continue
+            first = masked[0]
+            masked = [l for l in masked if not np.isnan(conf[b, n, l])]
+            if not masked:
+                bits[b, n], count[b, n] = np.uint64(1) << np.uint64(first), 1
                 continue
             ranked = sorted(masked, key=lambda l: (-conf[b, n, l], l))
             c = [conf[b, n, l] for l in ranked]

@@ -384,55 +384,60 @@ __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int 
 // One warp applies the unmasking rule of Sec. 3.1 (Algorithm 1, step 3) to one
 // node; lane k owns positions k and k + 32.  conf: the node's L confidences,
 // -inf at unmasked positions.  Returns the bit mask of positions to unmask.
+// kMarks: a NaN marks a masked row without a usable distribution (the sampled decision's; the greedy
+// one's confidences are numbers).  It is passed over, and where a node has no other masked row the first
+// masked position is taken, so that decoding always advances.
 // Few positions are taken one after the other, each the most confident of those left, the first of
 // several (a maximum and two votes); more than kRounds by their ranks.
+template <bool kMarks = false>
 __device__ __forceinline__ uint64_t unmask_rule(const float* conf, const int32_t* state, int L,
                                                 int mask_id, int rule, int top_s, float tau,
                                                 int lane) {
   constexpr int kRounds = 8;
   const unsigned full = 0xffffffffu;
-  bool masked[2];
-  float c[2];
+  auto masked = [&](int l) { return l < L && state[min(l, L - 1)] == mask_id; };
+  float c[2];  // -inf: not to be taken
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int l = lane + 32 * h;
-    masked[h] = l < L && state[min(l, L - 1)] == mask_id;
-    c[h] = masked[h] ? conf[l] : -INFINITY;
+    c[h] = masked(l) ? conf[l] : -INFINITY;
+    if (kMarks && c[h] != c[h]) c[h] = -INFINITY;
   }
   const bool tops = rule == SPIFFY_RULE_TOPS;
-  if (!tops) {  // strict, Sec. 3.1; an unusable row never passes
-    const uint64_t pass = (uint64_t)__ballot_sync(full, c[0] > tau && masked[0]) |
-                          (uint64_t)__ballot_sync(full, c[1] > tau && masked[1]) << 32;
-    if (pass) return pass;  // none: the single most confident position
-  }
+  uint64_t bits = 0;
+  if (!tops)  // strict, Sec. 3.1
+    bits = (uint64_t)__ballot_sync(full, c[0] > tau) | (uint64_t)__ballot_sync(full, c[1] > tau) << 32;
   if (tops && top_s > kRounds) {
-    // rank among the masked positions by (confidence desc, position asc); the
-    // confidence of an unmasked position is -inf and a masked one's is not
+    // rank among the usable positions by (confidence desc, position asc)
     bool take[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int l = lane + 32 * h;
       int rank = 0;
-      if (masked[h]) {
+      if (c[h] != -INFINITY) {
         for (int j = 0; j < L; ++j) {
-          const float cj = conf[j];
+          const float cj = conf[j];  // a NaN is ahead of nothing
           rank += (cj > c[h] || (cj == c[h] && j < l)) ? 1 : 0;
         }
       }
-      take[h] = masked[h] && rank < top_s;
+      take[h] = c[h] != -INFINITY && rank < top_s;
     }
-    return (uint64_t)__ballot_sync(full, take[0]) | (uint64_t)__ballot_sync(full, take[1]) << 32;
-  }
-  uint64_t bits = 0;
+    bits = (uint64_t)__ballot_sync(full, take[0]) | (uint64_t)__ballot_sync(full, take[1]) << 32;
+  } else if (!bits) {  // the threshold rule: the single most confident position, where none passes
 #pragma unroll 1
-  for (int left = tops ? top_s : 1; left > 0; --left) {
-    const float best = warp_max(fmaxf(c[0], c[1]));  // an unusable row never wins
-    if (best == -INFINITY) break;                    // all taken
-    const unsigned lo = __ballot_sync(full, c[0] == best), hi = __ballot_sync(full, c[1] == best);
-    const int at = lo ? __ffs(lo) - 1 : __ffs(hi) + 31;
-    bits |= 1ull << at;
-    if (lane == at) c[0] = -INFINITY;
-    if (lane + 32 == at) c[1] = -INFINITY;
+    for (int left = tops ? top_s : 1; left > 0; --left) {
+      const float best = warp_max(fmaxf(c[0], c[1]));
+      if (best == -INFINITY) break;  // all taken
+      const unsigned lo = __ballot_sync(full, c[0] == best), hi = __ballot_sync(full, c[1] == best);
+      const int at = lo ? __ffs(lo) - 1 : __ffs(hi) + 31;
+      bits |= 1ull << at;
+      if (lane == at) c[0] = -INFINITY;
+      if (lane + 32 == at) c[1] = -INFINITY;
+    }
+  }
+  if (kMarks && !bits) {  // no usable row
+    const uint64_t any = (uint64_t)__ballot_sync(full, masked(lane)) | (uint64_t)__ballot_sync(full, masked(lane + 32)) << 32;
+    bits = any & (0ull - any);
   }
   return bits;
 }

@@ -224,7 +224,7 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
     const bool usable = c.slice != 0x7fffffff && fabsf(c.row_m) < INFINITY && c.row_s > 0.f && c.row_s < INFINITY;
     if (!usable) {
       if (tid == 0) {
-        conf_out[row] = __int_as_float(0x7fc00000);  // NaN: never wins the rule
+        conf_out[row] = __int_as_float(0x7fc00000);  // NaN: the rule passes over it
         tok_out[row] = 0;
         if (!kWhole && dev_status) atomicOr(dev_status + b, SPIFFY_DEV_NONFINITE);
       }
@@ -373,7 +373,7 @@ decide_sampled_rule_kernel(const float* __restrict__ conf, int N, int L, int cta
       sconf[warp][i] = c;
     }
     __syncwarp();
-    const uint64_t bits = unmask_rule(sconf[warp], stoken[warp], L, mask_id, rule, top_s, tau, lane);
+    const uint64_t bits = unmask_rule<true>(sconf[warp], stoken[warp], L, mask_id, rule, top_s, tau, lane);
     if (lane == 0) {
       bits_out[node] = bits;
       n_unmask_out[node] = __popcll(bits);

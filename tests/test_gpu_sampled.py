@@ -153,6 +153,27 @@ def test_unusable_rows_set_the_status_bit_and_spare_the_rest():
     assert np.array_equal(dec2.top_tok.cpu().numpy()[sure], o.top_tok[sure])
 
 
+@pytest.mark.parametrize("rule,s", [(spiffy.RULE_TOPS, 1), (spiffy.RULE_TOPS, 2), (spiffy.RULE_TOPS, 8),
+                                    (spiffy.RULE_TOPS, 9), (spiffy.RULE_TOPS, 70), (spiffy.RULE_THRESHOLD, 1)])
+@pytest.mark.parametrize("L,V", [(1, 52), (5, 52), (32, 52), (33, 52), (64, 52), (64, 9000)])
+def test_unusable_rows_are_unmasked_only_where_there_is_nothing_else(L, V, rule, s):
+    """Some rows of a node without a distribution, all of them, all but one, an unmasked position in front: the
+    rule on the call's own confidences, where such a row is a NaN."""
+    logits, tokens, mask = case(L, 2, 6, L, V, "f32", p_unmasked=0.0)
+    logits[:, 1, ::3, V // 2] = np.nan
+    logits[:, 2:4, :, 1] = np.nan
+    logits[:, 4, :L - 1] = -np.inf
+    logits[:, 5, L // 2:, 0] = np.inf
+    tokens[:, 3, 0] = 7
+    dec = spiffy.spiffy_unmask_decide_sampled(G.to_dev(logits), G.to_dev(tokens), mask, rule, 1.0, 3, s, 0.02)
+    conf = dec.conf.cpu().numpy()
+    assert np.isnan(conf[:, 2]).all() and not np.isnan(conf[:, 0]).any()
+    bits, count, _ = S.apply_rule(conf, tokens, mask, rule, s, np.float32(0.02))
+    assert np.array_equal(G.bits_np(dec.unmask_bits), bits)
+    assert np.array_equal(dec.n_unmask.cpu().numpy(), count)
+    assert (count[tokens.min(axis=2) == mask] >= 1).all()  # decoding advances
+
+
 def test_argument_checks():
     logits, tokens, mask = case(1, 1, 2, 4, 64, "f32")
     lg, tk = G.to_dev(logits), G.to_dev(tokens)

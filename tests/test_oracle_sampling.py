@@ -152,6 +152,20 @@ def test_rule_agrees_with_the_verification_oracle(rule, S_, tau):
     assert np.array_equal(bits, o.unmask_bits) and np.array_equal(count, o.n_unmask)
 
 
+@pytest.mark.parametrize("rule,S_,want", [(oracle.RULE_TOPS, 1, [[4], [1], [2]]), (oracle.RULE_TOPS, 2, [[2, 4], [1], [2]]),
+                                          (oracle.RULE_TOPS, 9, [[2, 3, 4], [1], [2]]),
+                                          (oracle.RULE_THRESHOLD, 1, [[2, 4], [1], [2]]),
+                                          (oracle.RULE_THRESHOLD, 9, [[2, 4], [1], [2]])])
+def test_rule_passes_over_rows_without_a_distribution(rule, S_, want):
+    """NaN confidences among others, at every masked position, and all but one, which is below the threshold."""
+    nan, out = np.nan, -np.inf
+    conf = np.array([[[nan, out, 0.6, 0.2, 0.9], [out, nan, nan, nan, nan], [nan, nan, 0.1, nan, out]]])
+    state = np.where(np.isneginf(conf), 3, 29).astype(np.int32)
+    bits, count, _ = S.apply_rule(conf, state, 29, rule, S_, 0.5)
+    assert [[l for l in range(5) if int(b) >> l & 1] for b in bits[0]] == want
+    assert count[0].tolist() == [len(w) for w in want]
+
+
 def test_noise_follows_the_state_not_the_node():
     r = np.random.default_rng(2)
     row = r.standard_normal((1, 1, 6, 50)).astype(np.float32)
