@@ -609,7 +609,8 @@ size_t spiffy_draft_blocks_workspace(const spiffy_draft_desc* desc);
  *               D*+1 nodes in the layout spiffy_accept_walk reads: node a is a
  *               parent of node c when a's candidate set is a strict subset of
  *               c's (Eqs. draft-graph-2/3; node 0 is the empty set)
- *   dev_status  [B]: SPIFFY_DEV_NONFINITE for an unusable logits row,
+ *   dev_status  [B]: SPIFFY_DEV_NONFINITE for an unusable logits row (its
+ *               candidates count as of probability 0: ranks behind the others'),
  *               SPIFFY_DEV_BADGRAPH when parent_cap was too small (lists cut)
  */
 spiffy_status spiffy_draft_blocks(const spiffy_draft_desc* desc, const void* logits,

@@ -297,7 +297,6 @@ draft_build_kernel(BuildArgs g) {
   const int npairs = g.formula_off[D], nkids = g.child_off[D];
   const int f_mine = tid <= D ? g.formula_off[tid] : 0, c_mine = tid <= D ? g.child_off[tid] : 0;
   const int32_t t0 = lane < L ? state[lane] : ~g.mask_id, t1 = lane + 32 < L ? state[lane + 32] : ~g.mask_id;
-  for (int l = tid; l < 64; l += threads) pos_of_rank[l] = 0;  // ranks that rows without a distribution leave out
   for (int i = tid; i < 64 * kMaxK; i += threads) {
     by_rank_log[i] = -INFINITY;
     by_rank_tok[i] = 0;
@@ -453,6 +452,7 @@ draft_build_kernel(BuildArgs g) {
         }
       }
       p_top = mine == -INFINITY ? 0.f : ex2((mine - M) * kLog2e) / s;
+      if (!(p_top >= 0.f)) p_top = 0.f;  // a row without a distribution: behind the others, a rank of its own
       cand_tok[h] = mine_tok;
       cand_log[h] = p_top > 0.f ? logf(fmaxf(p_top, 1e-45f)) : -INFINITY;
       if (lane == 0 && (!(fabsf(M) < INFINITY) || !(s > 0.f) || !(s < INFINITY)) && g.dev_status)

@@ -176,3 +176,29 @@ def test_a_block_of_one_position_behind_another_call(D, budget):
     got, want = run_both(logits, state, V, budget, 4, torch.float32, formulas, [[] for _ in formulas])
     assert assert_parity(got, want, 1e-5) > B // 2
     assert (want.kept[:, 0] >= 0).all()
+
+
+@pytest.mark.parametrize("L,V", [(6, 300), (40, 300), (33, 20000)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
+def test_rows_without_a_distribution_come_last(L, V, bad):
+    """Their positions have the last ranks, lower positions first, as if every token had the probability 0; a row
+    of equal logits takes the same rank, and the drafts of the other positions come out alike."""
+    r = np.random.default_rng(L)
+    B = 20
+    logits = (r.standard_normal((B, L, V)) * 3).astype(np.float32)
+    spoiled = r.random((B, L)) < 0.4
+    spoiled[:, 0], spoiled[:, 1:5] = True, False
+    flat = logits.copy()
+    flat[spoiled] = 0.0
+    if bad == -float("inf"):
+        logits[spoiled] = bad
+    else:
+        logits[spoiled, V // 2] = bad
+    state = np.full((B, L), V, dtype=np.int32)
+    graph = spiffy.draft_graph(FORMULAS, CHILDREN)
+    want = spiffy.spiffy_draft_blocks(G.to_dev(flat), G.to_dev(state), V, graph, 10, 3)
+    for _ in range(3):
+        got = spiffy.spiffy_draft_blocks(G.to_dev(logits), G.to_dev(state), V, graph, 10, 3)
+        for f in ("tokens", "kept", "score", "parent_off", "parent_idx"):
+            assert torch.equal(getattr(got, f), getattr(want, f)), f
+        assert got.dev_status.tolist() == [spiffy.DEV_NONFINITE] * B and int(want.dev_status.sum()) == 0
