@@ -248,8 +248,8 @@ __device__ bool strict_subset(const BuildArgs& g, int a, int c) {
   return true;
 }
 
-// grid = B sequences, a warp per block position (at most kBuildThreads); dynamic shared memory, see
-// build_smem_bytes.
+// grid = B sequences, build_threads() threads: a warp per block position, two positions a warp beyond 32;
+// dynamic shared memory, see build_smem_bytes.
 //
 // A chain of small steps in one CTA: what bounds it is how many dependent accesses it is long and how many
 // instructions it meets for the first time (some five cycles each), not how much it does.  All that does not
@@ -383,7 +383,7 @@ draft_build_kernel(BuildArgs g) {
   int cand_tok[2] = {};
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const int l = warp + h * warps;  // two rounds are enough for 64 positions, as there are min(L, 32) warps
+    const int l = warp + h * warps;  // two rounds are enough for 64 positions, as there are min(L, 32) warps at least
     if (l >= L) break;
     const TopPartial* p = g.partials + ((int64_t)b * L + l) * g.splits;
     const bool is_masked = (masked_bits >> l & 1ull) != 0ull;
@@ -490,7 +490,7 @@ draft_build_kernel(BuildArgs g) {
   if (one_warp) {
     // Two warps with the same numbers: what follows from them is written by one or the other.
     if (warp > 1) return;
-    const bool lists = warp == 0, drafts = warp == 1 || warps == 1;
+    const bool lists = warp == 0, drafts = warp == 1;
     if (at_hand) {  // 3. and 4. as below, the look-ups all at once
       float x = -INFINITY, lg = -INFINITY;
       if (needed <= masked) {
@@ -720,6 +720,13 @@ int64_t draft_chunk(const spiffy_draft_desc& d, int* splits) {
   return chunk;
 }
 
+// A warp per block position, and 16 at least, for the formulas: 1024 of them and one position take 47 us with 512
+// threads, 77 with 1024 before the kernel's chain was shortened and 372 with a warp for the one position (4 positions: 57, 84,
+// 131; 64 formulas and one position 8.6, 11.0, 20.0; ten formulas 5.9, 8.9, 6.6; eight positions or more alike).
+int build_threads(const spiffy_draft_desc& d) {
+  return std::min(kBuildThreads, std::max(kBuildThreads / 2, 32 * d.block_len));
+}
+
 size_t build_smem_bytes(const spiffy_draft_desc& d) {
   return std::max(d.n_formulas <= kRelated ? (size_t)kFormulaBytes : (size_t)0,
                   (size_t)d.n_formulas * 12 + (size_t)(d.budget + 1) * 8);  // a graph of few formulas may be too long to stage
@@ -761,8 +768,7 @@ spiffy_status launch_draft(const spiffy_draft_desc& d, const void* logits, const
   g.state = state; g.formula_off = formula_off; g.formula_i = formula_i; g.formula_j = formula_j;
   g.child_off = child_off; g.child_idx = child_idx; g.tokens = tokens; g.kept = kept; g.score = score;
   g.parent_off = parent_off; g.parent_idx = parent_idx; g.dev_status = dev_status; g.fill_parents = fresh ? 1 : 0;
-  e = launch_pdl(draft_build_kernel, dim3(d.batch), dim3(32 * std::min<int>(d.block_len, kBuildThreads / 32)),
-                 build_smem_bytes(d), stream, g);
+  e = launch_pdl(draft_build_kernel, dim3(d.batch), dim3(build_threads(d)), build_smem_bytes(d), stream, g);
   count_launch();
   return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
 }

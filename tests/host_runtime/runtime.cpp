@@ -89,6 +89,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
   if (name.find("decide_reduce_kernel") != std::string::npos) more = " early " + i(8);
   if (name.find("accept_walk_kernel") != std::string::npos) more = " lists " + p(3) + " staged " + i(13);
   if (name.find("decide_tail_kernel") != std::string::npos) more = " lists " + p(14) + " early " + i(22);
+  if (name.find("draft_build_kernel") != std::string::npos) more = " threads " + std::to_string(c->blockDim.x);
   if (name.find("graph_attention") != std::string::npos) {
     unsigned cluster = 1;
     for (unsigned k = 0; k < c->numAttrs; ++k)
@@ -128,8 +129,10 @@ int lmhead_grid(const spiffy_decide_desc&) { return 0; }
 size_t lmhead_workspace_bytes(const spiffy_decide_desc&, int, int) { return 0; }
 spiffy_status launch_lmhead_decide(const spiffy_decide_desc&, int, const void*, const void*, const int32_t*, float*,
                                    int32_t*, uint64_t*, int32_t*, int32_t*, void*, bool, cudaStream_t) { return SPIFFY_ECUDA; }
+#ifdef REAL_ATTENTION
 size_t draft_workspace_bytes(const spiffy_draft_desc&) { return 0; }
 spiffy_status launch_draft(const spiffy_draft_desc&, const void*, const int32_t*, const int32_t*, const int32_t*,
                            const int32_t*, const int32_t*, const int32_t*, int32_t*, int32_t*, float*, int32_t*, int32_t*,
                            int32_t*, void*, bool, cudaStream_t) { return SPIFFY_ECUDA; }
+#endif
 }  // namespace spiffy

@@ -15,7 +15,7 @@ from paper_2509_18085_b200 import workloads as W
 from paper_2509_18085_b200.step import VerifyStep, inputs_from_workload
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-UNITS = ["step_host", "decide", "walk", "stage", "api"]
+UNITS = ["step_host", "decide", "walk", "draft", "stage", "api"]
 
 
 @pytest.fixture(scope="module")
@@ -172,6 +172,18 @@ def test_fused_tail_up_to_4096_partial_results(host, N, L, V, dtype, flags):
                                    ctypes.c_void_p(STREAM)) == spiffy.OK
     kernels = [re.search("(decide_reduce|decide_tail|decide_finalize|accept_walk)_kernel", line).group(1) for line in host.fake_log().decode().splitlines()]
     assert kernels == (["decide_reduce", "decide_tail"] if fused else ["decide_reduce", "decide_finalize", "accept_walk"])
+
+
+@pytest.mark.parametrize("D,L", [(1, 1), (64, 1), (1000, 1), (300, 4), (10, 15), (1000, 17), (10, 32), (10, 33), (1024, 64)])
+def test_drafting_has_threads_for_positions_and_formulas(host, D, L):
+    """A warp per position, two positions a warp beyond 32; on short blocks 512 threads for the formulas all the same."""
+    d = spiffy.DraftDesc(1, L, 1000, spiffy.F32, 1000, 999, D, 1, 1, 8)
+    p = ctypes.c_void_p(1 << 20)
+    host.fake_reset(b"", 0, 0)
+    assert host.spiffy_draft_blocks(ctypes.byref(d), *[p] * 14, ctypes.c_size_t(1 << 40), ctypes.c_void_p(STREAM)) == spiffy.OK
+    (build,) = [line for line in host.fake_log().decode().splitlines() if "draft_build" in line]
+    threads = int(re.search(r"threads (\d+)", build).group(1))
+    assert 512 <= threads <= 1024 and threads % 32 == 0 and threads >= 32 * min(L, 32)
 
 
 def test_a_step_object_describes_each_input_anew(monkeypatch):
