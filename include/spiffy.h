@@ -106,7 +106,9 @@ typedef enum { SPIFFY_RULE_TOPS = 0, SPIFFY_RULE_THRESHOLD = 1 } spiffy_rule;
  * another and follow one another in a stream: the later one may start while the
  * earlier one runs, and what follows in the stream still follows both.
  * SPIFFY_INDEPENDENT: the call before this one is an attention call on the
- * CUDA-core kernel and writes none of this call's inputs.
+ * CUDA-core kernel and writes none of this call's inputs.  The workspace, and with
+ * SPIFFY_FRESH_STATUS the status words, are written while it may still run; the
+ * results once it is complete, so that they may lie in memory that it reads.
  * SPIFFY_INDEPENDENT_NEXT: the next call is an attention call with
  * SPIFFY_ATTN_INDEPENDENT.  It starts as the vocabulary reduce lets go of the
  * multiprocessors (a tensor-core attention needs whole ones) and runs beside the

@@ -200,9 +200,9 @@ spiffy_status launch_attention_tc_dual(const spiffy_attn_desc& d0, const AttnPro
 //         the root kernel, which waited.
 //     (b) The draft-build kernel reads the draft formulas, constants of the model, and the block, as the
 //         top-k kernel in front of it waited before it let it start.
-//     (c) The reduce, or the one kernel that few slices take, under SPIFFY_INDEPENDENT and the attention
-//         under SPIFFY_ATTN_INDEPENDENT
-//         read their inputs, write their outputs and wait last.  What precedes them is, by the
+//     (c) The reduce under SPIFFY_INDEPENDENT and the attention under SPIFFY_ATTN_INDEPENDENT
+//         read their inputs, write their outputs and wait last; the one kernel that few slices
+//         take under SPIFFY_INDEPENDENT reads its inputs, waits and writes.  What precedes them is, by the
 //         flags' contract, a call that touches none of these; its kernels started, in turn,
 //         behind one that had waited before it triggered (the CUDA-core attention; the reduce
 //         of a plain decision), so everything ahead of that call is complete.  The second launch

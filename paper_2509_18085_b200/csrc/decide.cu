@@ -149,7 +149,9 @@ struct TailArgs {
   int32_t* next_block;
   int32_t* walk_status;
 };
-// A sequence's tail, by all threads of a CTA; `memory`: tail_smem_bytes().
+// A sequence's tail, by all threads of a CTA; `memory`: tail_smem_bytes().  kHold: the results stay in shared
+// memory until publish().
+template <bool kHold>
 class Tail {
  public:
   __device__ __forceinline__ Tail(const TailArgs& a, int b, unsigned char* memory)
@@ -164,8 +166,10 @@ class Tail {
     link = idx + a.parent_cap;
     __shared__ uint32_t s_kids[kTableNodes][2];
     __shared__ uint32_t s_hash[kTableNodes];
+    __shared__ int32_t s_flags[kHold ? 4 : 1];
     kids = s_kids;
     hash = s_hash;
+    flags = s_flags;
   }
   // The graph on its way to shared memory.  kNow: read at L2, by a kernel that does not wait for the one before it.
   template <bool kNow>
@@ -189,6 +193,7 @@ class Tail {
     for (int i = tid; i < a.parent_cap; i += step) copy4(idx + i, from_idx + i);
     for (int i = tid; i < a.N; i += step) link[i] = kNoLink;
     for (int i = tid; i < 2 * kTableNodes; i += step) (&kids[0][0])[i] = 0u;
+    if (kHold && tid < 2) flags[tid] = 0;
   }
   // ... has arrived: children and hashes, complete behind the next barrier of the CTA.
   __device__ __forceinline__ void arrived() {
@@ -215,11 +220,13 @@ class Tail {
       const bool ok = finalize_row<kLanes>(partials + (int64_t)row * a.splits, a.splits, sub, state[row], a.mask_id, c, tok,
                                            source);
       if (sub == 0 && r < rows) {
-        a.conf[(int64_t)b * rows + row] = c;
-        a.top_tok[(int64_t)b * rows + row] = tok;
+        if (!kHold) {
+          a.conf[(int64_t)b * rows + row] = c;
+          a.top_tok[(int64_t)b * rows + row] = tok;
+        }
         conf[row] = c;
         top[row] = tok;
-        if (!ok && a.decide_status) atomicOr(a.decide_status + b, SPIFFY_DEV_NONFINITE);
+        if (!ok) report(0, a.decide_status, SPIFFY_DEV_NONFINITE);
       }
     }
   }
@@ -239,8 +246,10 @@ class Tail {
       // a node with nothing to unmask ends the walk
       const int child = table && take != 0 ? child_of(kids[node], hash, state, next, N, L, lane) : kNoLink;
       if (lane == 0) {
-        a.unmask_bits[(int64_t)b * N + node] = take;
-        a.n_unmask[(int64_t)b * N + node] = __popcll(take);
+        if (!kHold) {
+          a.unmask_bits[(int64_t)b * N + node] = take;
+          a.n_unmask[(int64_t)b * N + node] = __popcll(take);
+        }
         bits[node] = take;
         if (table) link[node] = child;
       }
@@ -249,11 +258,52 @@ class Tail {
       __syncthreads();
       good = !walk_link_children(N, L, a.parent_cap, state, top, off, idx, bits, link, warp, warps, lane);
     }
-    if (!good && a.walk_status) atomicOr(a.walk_status + b, SPIFFY_DEV_BADGRAPH);
+    if (!good) report(1, a.walk_status, SPIFFY_DEV_BADGRAPH);
     __syncthreads();
-    if (warp == 0)
+    if (warp != 0) return;
+    if (kHold) {
+      int hops;
+      const int end = walk_follow(N, link, link, lane, hops);
+      if (lane == 0) flags[2] = end, flags[3] = hops;
+    } else {
       walk_chase(N, L, state, top, bits, link, a.path + (int64_t)b * N, a.next_block + (int64_t)b * L, a.accepted_node + b,
                  a.n_accepted + b, lane);
+    }
+  }
+  // kHold, 256 threads, up to 64 rows: the results to where they belong once the kernel before is complete, whose
+  // memory that may have been.  What a thread writes is in its registers by then (4 x 16 rows of one slice beside an
+  // attention over 500 keys 20.0 us; read from shared memory behind the wait 21.3, written ahead of it 19.9).
+  __device__ __forceinline__ void publish(bool fresh) {
+    __syncthreads();
+    const int N = a.N, L = a.L, part = (int)threadIdx.x / 64, i = (int)threadIdx.x % 64, end = flags[2], hops = flags[3];
+    int32_t *one = nullptr, *two = nullptr;
+    int32_t first = 0, second = 0;
+    uint64_t set = 0;
+    if (part == 0) {
+      if (i < rows) one = reinterpret_cast<int32_t*>(a.conf) + b * rows + i, first = __float_as_int(conf[i]);
+      if (i == 0) two = a.accepted_node + b, second = end;
+      if (i == 1) two = a.n_accepted + b, second = hops;
+    } else if (part == 1) {
+      if (i < rows) one = a.top_tok + b * rows + i, first = top[i];
+      if (i < 2) two = i == 0 ? a.decide_status : a.walk_status, second = flags[i];
+      if (two) two += b;
+      if (!fresh && second == 0) two = nullptr;
+    } else if (part == 2) {
+      if (i < N) one = a.n_unmask + b * N + i, set = bits[i], first = __popcll(set);
+    } else {
+      if (i < N) one = a.path + b * N + i, first = i <= hops ? link[i] : -1;
+      if (i < L) two = a.next_block + b * L + i, second = walk_next_token(state, top, bits[end], end, L, i);
+    }
+#if __CUDA_ARCH__ >= 900
+    cudaGridDependencySynchronize();
+    pdl_launch_dependents();
+#endif
+    if (one) *one = first;
+    if (part == 2 && i < N) a.unmask_bits[b * N + i] = set;
+    if (two) {
+      if (part == 1 && !fresh) atomicOr(two, second);
+      else *two = second;
+    }
   }
   int32_t* state;
 
@@ -262,6 +312,11 @@ class Tail {
   const int b, rows, warp, lane, warps;
   const bool table;
   bool good = true;  // no malformed offset or entry met
+  int32_t* flags;    // kHold: status bits of the decision and of the walk, the node it ends on, the hops
+  __device__ __forceinline__ void report(int which, int32_t* status, int32_t flag) {
+    if (kHold) atomicOr(flags + which, flag);
+    else if (status) atomicOr(status + b, flag);
+  }
   uint64_t* bits;
   int32_t *top, *off, *idx;
   float* conf;
@@ -287,7 +342,7 @@ decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int 
 #endif
   const TailArgs a = {splits, N, L, mask_id, rule, top_s, tau, block_tokens, parent_off, parent_idx, parent_cap, conf_out,
                       tok_out, bits_out, n_unmask_out, decide_status, accepted_node, n_accepted, path, next_block, walk_status};
-  Tail tail(a, (int)blockIdx.x, tail_smem);
+  Tail<false> tail(a, (int)blockIdx.x, tail_smem);
   tail.template fetch<false>();
   tail.arrived();
 #if __CUDA_ARCH__ >= 900
@@ -300,17 +355,19 @@ decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int 
 
 // The same for few slices beside a CUDA-core attention (SPIFFY_INDEPENDENT), reduce included: a cluster of
 // kSmallCtas CTAs per sequence, whose groups of kReduceThreads threads take the slices of masked rows in turn;
-// the partial results go straight into the shared memory of the first CTA, which does the rest.  One launch
+// the partial results go straight into the shared memory of the first CTA, which does the rest, writes its
+// results once the attention is complete and keeps them in shared memory until then.  One launch
 // instead of two, and no partial result waits for a kernel to end and another to read it from L2.  Bound: the
 // launch, a trip for the tokens and one for each round of slices, the steps of the tail.  Two groups a CTA: larger
 // ones find no room beside an attention that fills the machine (2 x 32 positions x 32 heads over 4000 keys
 // 127.2 us, with four groups 133.9, without this kernel 130.1; 4 x 2 x 8 positions x 12 heads over 300 10.8, 14.8
-// and 13.7), and the smallest gain nothing by them (4 x 8 rows of one slice 6.3, 6.2 and 9.2).
+// and 13.7), and the smallest gain nothing by them (4 x 8 rows of one slice 6.3, 6.2 and 9.2; all with the results
+// written ahead of the wait).
 constexpr int kSmallCtas = 8, kSmallGroups = 2, kSmallRows = 64;
 template <typename T>
 __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallGroups* kReduceThreads)
 decide_small_kernel(const __grid_constant__ TailArgs a, const T* __restrict__ logits, int64_t row_stride, int V,
-                    int64_t chunk, int next, StatusClear clear) {
+                    int64_t chunk, int next, int fresh) {
   extern __shared__ __align__(16) unsigned char tail_smem[];
   __shared__ int16_t list[kSmallRows];  // the masked rows
   __shared__ int n_masked;
@@ -336,11 +393,8 @@ decide_small_kernel(const __grid_constant__ TailArgs a, const T* __restrict__ lo
     if (tid == 0) n_masked = n;
   }
   Partial* slots = reinterpret_cast<Partial*>(tail_smem);
-  Tail tail(a, b, tail_smem + (size_t)rows * a.splits * sizeof(Partial));
-  if (rank == 0) {
-    if (tid == 0 && clear.batch) clear.run(b);
-    tail.template fetch<true>();
-  }
+  Tail<true> tail(a, b, tail_smem + (size_t)rows * a.splits * sizeof(Partial));
+  if (rank == 0) tail.template fetch<true>();
   __syncthreads();
   // the first CTA, which has the graph to prepare, comes last
   const int items = n_masked * a.splits, first = (rank + kSmallCtas - 1) % kSmallCtas * kSmallGroups + group;
@@ -364,10 +418,7 @@ decide_small_kernel(const __grid_constant__ TailArgs a, const T* __restrict__ lo
   sm100::cluster_wait();  // every slice is here
   tail.template merge_rows<4>(slots, SharedSlices{});
   tail.walk();
-#if __CUDA_ARCH__ >= 900
-  cudaGridDependencySynchronize();  // complete no sooner than the attention
-  pdl_launch_dependents();
-#endif
+  tail.publish(fresh);
 }
 
 size_t tail_smem_bytes(const spiffy_decide_desc& d, int parent_cap) {
@@ -485,9 +536,9 @@ spiffy_status launch_decide_finalize(const spiffy_decide_desc& d, const void* pa
 constexpr int kTailRows = 512, kTailPartials = 4096;
 constexpr size_t kTailSmem = 48 * 1024 - 1024;  // what the kernel declares itself comes on top
 // Beside a CUDA-core attention (`independent`) up to kSmallSlices slices a sequence take one launch of a cluster.
-// fp32, the step with one launch and with two, us: 4 x 8 rows of one slice 6.3 and 9.2, 4 x 16 over 500 keys 29.0
-// and 31.9, 2 x 32 over 4000 keys x 32 heads 127.2 and 130.1, 4 x 2 x 32 so 501 and 505, 2 x 8 x 8 90.8 and 94.2,
-// 3 x 8 of two 6.7 and 8.9; beyond, 3 x 8 rows of five slices 9.9 and 8.2, 8 x 32 of one 19.4 and 12.3.
+// fp32, the step with one launch and with two, us: 4 x 8 rows of one slice 7.4 and 9.8, 4 x 16 over 500 keys 20.1
+// and 22.7, 2 x 32 over 4000 keys x 32 heads 125.6 and 128.5, 4 x 2 x 32 so 491 and 496, 2 x 8 x 8 over 4000 x 16
+// 125.9 and 128.7, 3 x 8 of two 9.8 and 12.8; beyond, 3 x 8 rows of five slices 9.9 and 8.2, 8 x 32 of one 19.4 and 12.3.
 // A decision in front of an attention or by itself is no sooner done in one launch (bf16, 4 x 8 rows of one
 // slice 7.2 and 7.2 us with the attention, 4 x 16 9.3 and 7.3).
 constexpr int kSmallSlices = 64, kSmallBatch = 8;
@@ -518,8 +569,7 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
                         n_unmask, decide_status, accepted_node, n_accepted, path, next_block, walk_status};
     auto run = [&](auto kernel, auto* typed) {
       return launch_pdl(kernel, dim3(kSmallCtas * d.batch), dim3(kSmallGroups * kReduceThreads), small_smem, stream, a, typed,
-                        (int64_t)d.row_stride, (int)d.vocab, chunk, (int)next,
-                        status_clear(d, fresh, decide_status, walk_status));
+                        (int64_t)d.row_stride, (int)d.vocab, chunk, (int)next, (int)fresh);
     };
     const cudaError_t e = d.logits_dtype == SPIFFY_BF16
                               ? run(decide_small_kernel<__nv_bfloat16>, static_cast<const __nv_bfloat16*>(logits))

@@ -108,13 +108,11 @@ __device__ __forceinline__ bool walk_link_children(int N, int L, int parent_cap,
   return __any_sync(full, bad);
 }
 
-// Called by one warp after the links are complete (a block-wide sync after
-// walk_link_children).
-__device__ __forceinline__ void walk_chase(int N, int L, const int32_t* state, const int32_t* top,
-                                           const uint64_t* ubits, const int* link, int32_t* pth,
-                                           int32_t* next_block, int32_t* accepted_node,
-                                           int32_t* n_accepted, int lane) {
-  int cur = 0, hops = 0;
+// Called by one warp after the links are complete (a block-wide sync after walk_link_children): the
+// node the walk ends on, the hops to it in `hops`, and the path, hops + 1 entries, in `pth`.
+__device__ __forceinline__ int walk_follow(int N, const int* link, int32_t* pth, int lane, int& hops) {
+  int cur = 0;
+  hops = 0;
   if (lane == 0) {
     // `link` may be the path array itself: a link is read before the slot at or
     // below its node is reused for the path (hop h is stored at index h <= node)
@@ -125,15 +123,32 @@ __device__ __forceinline__ void walk_chase(int N, int L, const int32_t* state, c
       m = link[cur];
       pth[++hops] = cur;
     }
+  }
+  hops = __shfl_sync(0xffffffffu, hops, 0);
+  return __shfl_sync(0xffffffffu, cur, 0);
+}
+
+// ... and what it says about the node `cur` it ends on.
+__device__ __forceinline__ void walk_end(int cur, int hops, int L, const int32_t* state, const int32_t* top,
+                                         const uint64_t* ubits, int32_t* next_block, int32_t* accepted_node,
+                                         int32_t* n_accepted, int lane) {
+  if (lane == 0) {
     *accepted_node = cur;
     *n_accepted = hops;
   }
-  cur = __shfl_sync(0xffffffffu, cur, 0);
-  hops = __shfl_sync(0xffffffffu, hops, 0);
-  for (int i = hops + 1 + lane; i < N; i += 32) pth[i] = -1;
   const uint64_t bits = ubits[cur];
   if (lane < L) next_block[lane] = walk_next_token(state, top, bits, cur, L, lane);
   if (lane + 32 < L) next_block[lane + 32] = walk_next_token(state, top, bits, cur, L, lane + 32);
+}
+
+__device__ __forceinline__ void walk_chase(int N, int L, const int32_t* state, const int32_t* top,
+                                           const uint64_t* ubits, const int* link, int32_t* pth,
+                                           int32_t* next_block, int32_t* accepted_node,
+                                           int32_t* n_accepted, int lane) {
+  int hops;
+  const int cur = walk_follow(N, link, pth, lane, hops);
+  for (int i = hops + 1 + lane; i < N; i += 32) pth[i] = -1;
+  walk_end(cur, hops, L, state, top, ubits, next_block, accepted_node, n_accepted, lane);
 }
 
 }  // namespace spiffy

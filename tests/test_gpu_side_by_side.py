@@ -64,6 +64,33 @@ def test_late_in_a_block(N, V, dtype):
                 assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("N,L", [(4, 8), (1, 64), (9, 16)])  # in one launch, in two
+def test_results_may_lie_where_the_attention_reads(N, L):
+    """SPIFFY_INDEPENDENT is about the decision's inputs: its results may replace keys that the attention in front,
+    which takes far longer, has yet to read."""
+    cfg = W.Config("t", 2, N, L, 6000, 8, 8, 128, "f32", 1000, spiffy.RULE_THRESHOLD)
+    x, apart = inputs_from_workload(W.make(cfg, 8)), VerifyStep(cfg)
+    apart.attention(x)
+    apart.decide_accept(x)
+    want, keys, step = _results(apart), x.k_prefix.clone(), VerifyStep(cfg)
+    room, at = x.k_prefix.view(-1), x.k_prefix.numel()
+
+    def moved(t):  # from the last keys backwards
+        nonlocal at
+        at -= -(-t.numel() * t.element_size() // 64) * 16
+        return room[at:at + t.numel() * t.element_size() // 4].view(t.dtype).view(t.shape)
+
+    for results in (step.decision, step.walk):
+        for f in dataclasses.fields(results):
+            if f.name != "dev_status":  # OR-ed into what is there
+                setattr(results, f.name, moved(getattr(results, f.name)))
+    for _ in range(3):
+        x.k_prefix.copy_(keys)
+        step.run(x)
+        for a, b in zip(_results(step), want):
+            assert torch.equal(a, b)
+
+
 def _results(s):
     out = [s.attn_out, s.attn_status] + list(_fields(s.decision)) + list(_fields(s.walk))
     return [t.clone().view(torch.uint8) for t in out]
