@@ -123,7 +123,7 @@ decide_finalize_kernel(const Partial* __restrict__ partials, int splits, int N,
 // lists) does not depend on the reduce kernel; ahead of the wait it is copied to
 // shared memory and, for up to kTableNodes nodes, made a table of children with
 // hashes of the states, which saves a step of its own for the links.
-// grid = B, kTailThreads threads, dynamic shared memory tail_smem_bytes().
+// grid = B, kTailThreads threads or fewer, dynamic shared memory tail_smem_bytes().
 // Bound: a chain of short steps.  Behind the wait, 3 x 100 rows x 7 slices, two positions a node: 2640 cycles
 // for the merge, 1640 for the rule, 1020 for links and 1010 for the chase when the rule ranked positions one
 // by one and links were a step of their own with an exchange through atomics; 2040, 2110 for rule and links,
@@ -325,7 +325,7 @@ class Tail {
   uint32_t* hash;
 };
 
-template <int kLanes>  // threads per row: all N * L rows are merged in one pass when kLanes * N * L <= 1024
+template <int kLanes>  // threads per row: all N * L rows are merged in one pass when there are kLanes * N * L threads
 __global__ void __launch_bounds__(kTailThreads + 256, 1)  // 48 registers
 decide_tail_kernel(const Partial* __restrict__ partials, int splits, int N, int L,
                    const int32_t* __restrict__ block_tokens, int mask_id, int rule, int top_s,
@@ -534,6 +534,13 @@ spiffy_status launch_decide_finalize(const spiffy_decide_desc& d, const void* pa
 // runs under it, on one SM instead of many that the attention waits for: the tail, whatever there is to
 // merge (16 x 32 positions x 28 heads, x 19: 21.5 and 21.5, 27.0 and 27.7, 36.9 and 37.3).
 constexpr int kTailRows = 512, kTailPartials = 4096;
+// The tail's threads.  With 1024, at 48 registers, an SM holds one CTA: best while each sequence has an SM of its own.
+// Beyond, several smaller ones to an SM.  us with 256, 512 and 1024: 600 sequences x 64 rows of one slice 61.4 66.6
+// 74.8, 2000 x 32 106.5 119.3 145.9, 300 x 128 64.4 66.8 71.3, 200 x 256 88.5 87.6 91.2, 150 x 432 117.2 111.4 113.6.
+int tail_threads(int batch, int rows) {
+  if (batch <= sm_count()) return kTailThreads;
+  return rows <= kTailThreads / 8 ? kTailThreads / 4 : kTailThreads / 2;
+}
 constexpr size_t kTailSmem = 48 * 1024 - 1024;  // what the kernel declares itself comes on top
 // Beside a CUDA-core attention (`independent`) up to kSmallSlices slices a sequence take one launch of a cluster.
 // fp32, the step with one launch and with two, us: 4 x 8 rows of one slice 7.4 and 9.8, 4 x 16 over 500 keys 20.1
@@ -582,17 +589,17 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
                                          status_clear(d, fresh, decide_status, walk_status), stream);
   if (st != SPIFFY_OK) return st;
   const Partial* cpart = partials;
-  const int rows = d.n_nodes * d.block_len;
+  const int rows = d.n_nodes * d.block_len, threads = tail_threads(d.batch, rows);
   auto launch = [&](auto kernel) {
-    return launch_pdl(kernel, dim3(d.batch), dim3(kTailThreads), smem, stream, cpart, splits,
+    return launch_pdl(kernel, dim3(d.batch), dim3(threads), smem, stream, cpart, splits,
                       (int)d.n_nodes, (int)d.block_len, block_tokens, (int)d.mask_token_id,
                       (int)d.rule, (int)d.top_s, d.threshold, conf, top_tok, unmask_bits, n_unmask,
                       decide_status, parent_off, parent_idx, (int)parent_cap, accepted_node,
                       n_accepted, path, next_block, walk_status, (int)next);
   };
-  const cudaError_t e = rows <= kTailThreads / 8   ? launch(decide_tail_kernel<8>)
-                        : rows <= kTailThreads / 4 ? launch(decide_tail_kernel<4>)
-                                                   : launch(decide_tail_kernel<2>);
+  const cudaError_t e = rows <= threads / 8   ? launch(decide_tail_kernel<8>)
+                        : rows <= threads / 4 ? launch(decide_tail_kernel<4>)
+                                              : launch(decide_tail_kernel<2>);
   count_launch();
   return e == cudaSuccess ? SPIFFY_OK : SPIFFY_ECUDA;
 }

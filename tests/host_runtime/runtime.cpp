@@ -88,7 +88,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
   std::string more;
   if (name.find("decide_reduce_kernel") != std::string::npos) more = " early " + i(8);
   if (name.find("accept_walk_kernel") != std::string::npos) more = " lists " + p(3) + " staged " + i(13);
-  if (name.find("decide_tail_kernel") != std::string::npos) more = " lists " + p(14) + " early " + i(22);
+  if (name.find("decide_tail_kernel") != std::string::npos) more = " threads " + std::to_string(c->blockDim.x) + " lists " + p(14) + " early " + i(22);
   if (name.find("draft_build_kernel") != std::string::npos) more = " threads " + std::to_string(c->blockDim.x);
   if (name.find("graph_attention") != std::string::npos) {
     unsigned cluster = 1;

@@ -55,6 +55,16 @@ def random_case(seed, B, N, L, V, p_accept=0.7, dtype="f32"):
     return logits, tokens, off, idx, mask
 
 
+@pytest.mark.parametrize("B,N,L,V", [(149, 4, 8, 52), (200, 8, 16, 36), (149, 3, 43, 36), (149, 6, 64, 20), (149, 65, 2, 20)])
+def test_more_sequences_than_multiprocessors(B, N, L, V):
+    """The tail with 256 threads and with 512: 32, 128, 129, 384 and 130 rows a sequence."""
+    logits, tokens, off, idx, mask = random_case(B + N, B, N, L, V)
+    for rule, S, tau in ((spiffy.RULE_TOPS, 1, 0.0), (spiffy.RULE_TOPS, 3, 0.0), (spiffy.RULE_THRESHOLD, 1, 0.5)):
+        _, walk = both(logits, tokens, off, idx, mask, rule, S, tau)
+        if (rule, S) == (spiffy.RULE_TOPS, 1):
+            assert int(walk.n_accepted.sum()) > B // 4
+
+
 @pytest.mark.parametrize("B,N,L,V", [(3, 8, 32, 5000), (2, 16, 32, 1000), (5, 3, 7, 36), (1, 2, 64, 300),
                                      (2, 9, 64, 132), (1, 1, 1, 16)])
 def test_one_call_equals_two_calls_and_the_oracle(B, N, L, V):

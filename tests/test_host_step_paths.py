@@ -174,6 +174,18 @@ def test_fused_tail_up_to_4096_partial_results(host, N, L, V, dtype, flags):
     assert kernels == (["decide_reduce", "decide_tail"] if fused else ["decide_reduce", "decide_finalize", "accept_walk"])
 
 
+@pytest.mark.parametrize("B,N,L,fit", [(1, 4, 8, 1), (148, 8, 8, 1), (149, 16, 27, 2), (149, 8, 16, 4), (600, 8, 8, 4), (65535, 1, 1, 4)])
+def test_tails_of_more_sequences_than_multiprocessors_share_them(host, B, N, L, fit):
+    """65536 registers at 48 a thread, 148 multiprocessors."""
+    d = spiffy.DecideDesc(B, N, L, 1024, spiffy.BF16, 1024, 1023, spiffy.RULE_TOPS, 1, 0.9)
+    p = ctypes.c_void_p(1 << 20)
+    host.fake_reset(b"", 0, 0)
+    assert host.spiffy_decide_walk(ctypes.byref(d), p, p, p, p, 4, *[p] * 11, ctypes.c_size_t(1 << 40),
+                                   ctypes.c_void_p(STREAM)) == spiffy.OK
+    (tail,) = [line for line in host.fake_log().decode().splitlines() if "decide_tail" in line]
+    assert 65536 // (48 * int(re.search(r"threads (\d+)", tail).group(1))) >= fit
+
+
 @pytest.mark.parametrize("D,L", [(1, 1), (64, 1), (1000, 1), (300, 4), (10, 15), (1000, 17), (10, 32), (10, 33), (1024, 64)])
 def test_drafting_has_threads_for_positions_and_formulas(host, D, L):
     """A warp per position, two positions a warp beyond 32; on short blocks 512 threads for the formulas all the same."""
