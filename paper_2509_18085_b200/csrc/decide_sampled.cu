@@ -339,7 +339,8 @@ decide_sampled_select_kernel(const T* __restrict__ logits, int64_t row_stride, i
 
 // A warp per node; grid = sequences * ctas, CTA c of a sequence taking its nodes 16 c, 16 c + 1, ....  Where the
 // status word may arrive with arbitrary contents (kStatus: nothing came before that could have cleared it) it
-// has one writer: one CTA per sequence, for all nodes.
+// has one writer: one CTA per sequence, for all nodes.  A warp's next node is then fetched while the rule is applied
+// to this one (rows of one slice, us: 500 x 1 33.5 -> 19.2, 4000 x 8 421 -> 281, 300 x 4 29.5 -> 20.0).
 constexpr int kRuleThreads = 512, kRuleWarps = kRuleThreads / 32;
 template <bool kStatus>
 __global__ void __launch_bounds__(kRuleThreads)
@@ -350,9 +351,19 @@ decide_sampled_rule_kernel(const float* __restrict__ conf, int N, int L, int cta
   const int b = (int)blockIdx.x / ctas, first = ((int)blockIdx.x - b * ctas) * kRuleWarps + warp;
   __shared__ float sconf[kRuleWarps][64];
   __shared__ int32_t stoken[kRuleWarps][64];
+  int32_t token[2] = {};
+  float c[2] = {};
   auto tokens_of = [&](int n) {
-    const int32_t* t = block_tokens + ((int64_t)b * N + n) * L;
-    for (int i = lane; i < L; i += 32) stoken[warp][i] = t[i];
+    const int32_t* from = block_tokens + ((int64_t)b * N + n) * L;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (lane + 32 * h < L) token[h] = from[lane + 32 * h];
+  };
+  auto confidences_of = [&](int n) {
+    const float* from = conf + ((int64_t)b * N + n) * L;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (lane + 32 * h < L) c[h] = __ldcg(from + lane + 32 * h);
   };
 #if __CUDA_ARCH__ >= 900
   pdl_launch_dependents();
@@ -363,16 +374,22 @@ decide_sampled_rule_kernel(const float* __restrict__ conf, int N, int L, int cta
 #if __CUDA_ARCH__ >= 900
   cudaGridDependencySynchronize();
 #endif
+  if (first < N) confidences_of(first);
   bool bad = false;
-  for (int n = first; n < N; n += kStatus ? kRuleWarps : N) {
-    const int64_t node = (int64_t)b * N + n;
-    if (n != first) tokens_of(n);
-    for (int i = lane; i < L; i += 32) {
-      const float c = __ldcg(conf + node * L + i);
-      bad |= c != c;  // the mark of a row without a usable distribution
-      sconf[warp][i] = c;
+  for (int n = first; n < N;) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      bad |= c[h] != c[h];  // the mark of a row without a usable distribution
+      sconf[warp][lane + 32 * h] = c[h];
+      stoken[warp][lane + 32 * h] = token[h];
     }
     __syncwarp();
+    const int64_t node = (int64_t)b * N + n;
+    n = kStatus ? n + kRuleWarps : N;
+    if (n < N) {  // on their way beside the rule
+      tokens_of(n);
+      confidences_of(n);
+    }
     const uint64_t bits = unmask_rule<true>(sconf[warp], stoken[warp], L, mask_id, rule, top_s, tau, lane);
     if (lane == 0) {
       bits_out[node] = bits;

@@ -174,6 +174,21 @@ def test_unusable_rows_are_unmasked_only_where_there_is_nothing_else(L, V, rule,
     assert (count[tokens.min(axis=2) == mask] >= 1).all()  # decoding advances
 
 
+@pytest.mark.parametrize("N,L,V", [(15, 33, 52), (16, 1, 52), (17, 64, 52), (33, 5, 52), (100, 32, 52), (17, 33, 9000)])
+def test_rule_of_more_nodes_than_warps(N, L, V):
+    """Each node by its own rows and tokens, the next one fetched meanwhile; a row without a distribution in the
+    last node of one sequence."""
+    logits, tokens, mask = case(N, 3, N, L, V, "f32", p_unmasked=0.4)
+    tokens[1, N - 1, 0] = mask
+    logits[1, N - 1, 0, 7] = np.nan
+    for rule, s in ((spiffy.RULE_TOPS, 1), (spiffy.RULE_TOPS, 3), (spiffy.RULE_THRESHOLD, 1)):
+        dec = spiffy.spiffy_unmask_decide_sampled(G.to_dev(logits), G.to_dev(tokens), mask, rule, 1.0, 3, s, 0.1)
+        bits, count, _ = S.apply_rule(dec.conf.cpu().numpy(), tokens, mask, rule, s, np.float32(0.1))
+        assert np.array_equal(G.bits_np(dec.unmask_bits), bits)
+        assert np.array_equal(dec.n_unmask.cpu().numpy(), count)
+        assert dec.dev_status.tolist() == [0, spiffy.DEV_NONFINITE, 0]
+
+
 def test_argument_checks():
     logits, tokens, mask = case(1, 1, 2, 4, 64, "f32")
     lg, tk = G.to_dev(logits), G.to_dev(tokens)
