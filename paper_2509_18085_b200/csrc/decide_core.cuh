@@ -388,7 +388,10 @@ __device__ __forceinline__ bool finalize_row(const Partial* __restrict__ p, int 
 // one's confidences are numbers).  It is passed over, and where a node has no other masked row the first
 // masked position is taken, so that decoding always advances.
 // Few positions are taken one after the other, each the most confident of those left, the first of
-// several (a maximum and two votes); more than kRounds by their ranks.
+// several (a maximum and two votes, whatever L); more than kRounds, or a quarter of the block, by their ranks
+// (a look at every position, whatever S).  Rounds and ranks, decision and walk, us: 2 x 33 nodes x 12 positions, six
+// of them taken 8.95 8.35, eight 9.44 8.40; 4 x 64 x 8, two 10.3 10.5, four 11.0 10.5, eight 11.4 10.5; 16 x 32, eight
+// 7.4 7.2; 8 x 64, eight 7.2 8.4.
 template <bool kMarks = false>
 __device__ __forceinline__ uint64_t unmask_rule(const float* conf, const int32_t* state, int L,
                                                 int mask_id, int rule, int top_s, float tau,
@@ -407,7 +410,7 @@ __device__ __forceinline__ uint64_t unmask_rule(const float* conf, const int32_t
   uint64_t bits = 0;
   if (!tops)  // strict, Sec. 3.1
     bits = (uint64_t)__ballot_sync(full, c[0] > tau) | (uint64_t)__ballot_sync(full, c[1] > tau) << 32;
-  if (tops && top_s > kRounds) {
+  if (tops && (top_s > kRounds || L <= 4 * top_s)) {
     // rank among the usable positions by (confidence desc, position asc)
     bool take[2];
 #pragma unroll

@@ -5,7 +5,7 @@ import pytest
 import torch
 
 import oracle
-from oracle import toy
+from oracle import sampling, toy
 from paper_2509_18085_b200 import spiffy
 from paper_2509_18085_b200 import workloads as W
 
@@ -237,3 +237,16 @@ def test_degenerate_shapes():
     assert np.array_equal(dec.top_tok.cpu().numpy(), o.top_tok)
     assert np.array_equal(G.bits_np(dec.unmask_bits), o.unmask_bits)
     assert dec.n_unmask.cpu().numpy().tolist() == o.n_unmask.tolist() and o.n_unmask[0, 1] == 0
+
+
+@pytest.mark.parametrize("L,S", [(1, 1), (4, 1), (5, 1), (8, 2), (9, 2), (32, 8), (33, 8), (33, 9), (64, 8), (64, 16), (64, 70)])
+def test_rule_by_rounds_and_by_ranks(L, S):
+    """Both sides of the line between the two, many confidences alike, on the call's own confidences."""
+    r = np.random.default_rng(L + S)
+    logits = r.integers(0, 2, (3, 5, L, 12)).astype(np.float32)
+    mask = 11
+    tokens = np.where(r.random((3, 5, L)) < 0.3, 2, mask).astype(np.int32)
+    dec = spiffy.spiffy_unmask_decide(G.to_dev(logits), G.to_dev(tokens), mask, spiffy.RULE_TOPS, S)
+    bits, count, _ = sampling.apply_rule(dec.conf.cpu().numpy(), tokens, mask, spiffy.RULE_TOPS, S, 0.0)
+    assert np.array_equal(G.bits_np(dec.unmask_bits), bits)
+    assert np.array_equal(dec.n_unmask.cpu().numpy(), count)
