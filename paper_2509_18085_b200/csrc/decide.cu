@@ -237,14 +237,16 @@ class Tail {
 #pragma unroll 1
     for (int node = warp; node < N; node += warps) {
       const uint64_t take = unmask_rule(conf + node * L, state + node * L, L, a.mask_id, a.rule, a.top_s, a.tau, lane);
-      int32_t next[2];  // the node's next state
+      int child = kNoLink;
+      if (table && take != 0) {  // a node with nothing to unmask ends the walk
+        int32_t next[2];         // the node's next state
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int l = lane + 32 * h;
-        next[h] = l < L ? walk_next_token(state, top, take, node, L, l) : 0;
+        for (int h = 0; h < 2; ++h) {
+          const int l = lane + 32 * h;
+          next[h] = l < L ? walk_next_token(state, top, take, node, L, l) : 0;
+        }
+        child = child_of(kids[node], hash, state, next, N, L, lane);
       }
-      // a node with nothing to unmask ends the walk
-      const int child = table && take != 0 ? child_of(kids[node], hash, state, next, N, L, lane) : kNoLink;
       if (lane == 0) {
         if (!kHold) {
           a.unmask_bits[(int64_t)b * N + node] = take;
