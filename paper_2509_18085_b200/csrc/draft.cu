@@ -720,10 +720,13 @@ int64_t draft_chunk(const spiffy_draft_desc& d, int* splits) {
   return chunk;
 }
 
-// A warp per block position, and 16 at least, for the formulas: 1024 of them and one position take 47 us with 512
-// threads, 77 with 1024 before the kernel's chain was shortened and 372 with a warp for the one position (4 positions: 57, 84,
-// 131; 64 formulas and one position 8.6, 11.0, 20.0; ten formulas 5.9, 8.9, 6.6; eight positions or more alike).
+// A warp per block position, and 16 at least, for the formulas: 64 of them and one position take 8.6 us with 512 threads, 11.0
+// with 1024 before the kernel's chain was shortened and 20.0 with a warp for the one position (ten formulas 5.9, 8.9, 6.6).
+// All threads work on graphs of more formulas than one warp takes, and their pairs of kept drafts: 1024, us with 512
+// and 1024: 65 formulas, one position 10.0 9.3; 200, eight 24.1 20.7; 1000, all kept, eight 1537 1085.  Not where two
+// blocks of 512 an SM have sequences to work on (100 formulas, 300 sequences 40.5 and 47.1).
 int build_threads(const spiffy_draft_desc& d) {
+  if (d.n_formulas > kRelated && d.batch <= sm_count()) return kBuildThreads;
   return std::min(kBuildThreads, std::max(kBuildThreads / 2, 32 * d.block_len));
 }
 

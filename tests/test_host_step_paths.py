@@ -198,6 +198,18 @@ def test_drafting_has_threads_for_positions_and_formulas(host, D, L):
     assert 512 <= threads <= 1024 and threads % 32 == 0 and threads >= 32 * min(L, 32)
 
 
+@pytest.mark.parametrize("B,D,L,threads", [(1, 64, 8, 512), (1, 65, 1, 1024), (148, 1000, 16, 1024), (149, 1000, 16, 512),
+                                           (149, 1000, 17, 544)])
+def test_drafting_of_large_graphs_has_all_threads(host, B, D, L, threads):
+    """While there is a multiprocessor for every sequence."""
+    d = spiffy.DraftDesc(B, L, 1000, spiffy.F32, 1000, 999, D, 1, 1, 8)
+    p = ctypes.c_void_p(1 << 20)
+    host.fake_reset(b"", 0, 0)
+    assert host.spiffy_draft_blocks(ctypes.byref(d), *[p] * 14, ctypes.c_size_t(1 << 40), ctypes.c_void_p(STREAM)) == spiffy.OK
+    (build,) = [line for line in host.fake_log().decode().splitlines() if "draft_build" in line]
+    assert int(re.search(r"threads (\d+)", build).group(1)) == threads
+
+
 def test_a_step_object_describes_each_input_anew(monkeypatch):
     """The parent lists of one graph are longer than the next one's: a descriptor kept from the first
     call would read past the end of the second call's arrays."""
