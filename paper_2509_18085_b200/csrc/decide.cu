@@ -536,12 +536,19 @@ spiffy_status launch_decide_finalize(const spiffy_decide_desc& d, const void* pa
 // runs under it, on one SM instead of many that the attention waits for: the tail, whatever there is to
 // merge (16 x 32 positions x 28 heads, x 19: 21.5 and 21.5, 27.0 and 27.7, 36.9 and 37.3).
 constexpr int kTailRows = 512, kTailPartials = 4096;
-// The tail's threads.  With 1024, at 48 registers, an SM holds one CTA: best while each sequence has an SM of its own.
-// Beyond, several smaller ones to an SM.  us with 256, 512 and 1024: 600 sequences x 64 rows of one slice 61.4 66.6
-// 74.8, 2000 x 32 106.5 119.3 145.9, 300 x 128 64.4 66.8 71.3, 200 x 256 88.5 87.6 91.2, 150 x 432 117.2 111.4 113.6.
-int tail_threads(int batch, int rows) {
-  if (batch <= sm_count()) return kTailThreads;
-  return rows <= kTailThreads / 8 ? kTailThreads / 4 : kTailThreads / 2;
+// The tail's threads: a warp per node and four threads a row, 256 at least.  At 48 registers 1024 of them take most of
+// an SM, where a CUDA-core attention beside the decision lets no such CTA in until it ends: the steps, us, with 1024
+// and so: 9 sequences x 4 x 8 rows over 500 keys x 8 heads 65.3 48.9, 32 x 2 x 4 over 300 45.9 34.8; before a
+// tensor-core attention 30 x 4 x 8 over 100 13.1 10.8; by itself 4 x 8 of 1024 entries 5.4 4.6, 16 x 8 x 8 7.9 7.1.  Fewer
+// than a warp per node are slower (64 x 2 7.4, with 512 8.2).
+// With more sequences than SMs several smaller ones to an SM, us with 256, 512 and 1024: 600 sequences x 64 rows of one
+// slice 61.4 66.6 74.8, 2000 x 32 106.5 119.3 145.9, 300 x 128 64.4 66.8 71.3, 200 x 256 88.5 87.6 91.2, 150 x 432 117.2
+// 111.4 113.6.
+int tail_threads(int batch, int N, int rows) {
+  const int most = batch <= sm_count() ? kTailThreads : rows <= kTailThreads / 8 ? kTailThreads / 4 : kTailThreads / 2;
+  int threads = kTailThreads / 4;
+  while (threads < most && (threads < 32 * N || threads < 4 * rows)) threads *= 2;
+  return threads;
 }
 constexpr size_t kTailSmem = 48 * 1024 - 1024;  // what the kernel declares itself comes on top
 // Beside a CUDA-core attention (`independent`) up to kSmallSlices slices a sequence take one launch of a cluster.
@@ -591,7 +598,7 @@ spiffy_status launch_decide_walk(const spiffy_decide_desc& d, const void* logits
                                          status_clear(d, fresh, decide_status, walk_status), stream);
   if (st != SPIFFY_OK) return st;
   const Partial* cpart = partials;
-  const int rows = d.n_nodes * d.block_len, threads = tail_threads(d.batch, rows);
+  const int rows = d.n_nodes * d.block_len, threads = tail_threads(d.batch, d.n_nodes, rows);
   auto launch = [&](auto kernel) {
     return launch_pdl(kernel, dim3(d.batch), dim3(threads), smem, stream, cpart, splits,
                       (int)d.n_nodes, (int)d.block_len, block_tokens, (int)d.mask_token_id,

@@ -186,6 +186,20 @@ def test_tails_of_more_sequences_than_multiprocessors_share_them(host, B, N, L, 
     assert 65536 // (48 * int(re.search(r"threads (\d+)", tail).group(1))) >= fit
 
 
+@pytest.mark.parametrize("B,N,L,threads", [(9, 4, 8, 256), (32, 8, 8, 256), (20, 9, 2, 512), (9, 5, 13, 512), (9, 16, 8, 512),
+                                           (9, 17, 1, 1024), (9, 3, 43, 1024), (120, 16, 32, 1024)])
+@pytest.mark.parametrize("flags", [0, spiffy.INDEPENDENT, spiffy.INDEPENDENT_NEXT])
+def test_a_tail_is_no_larger_than_its_graph_asks_for(host, B, N, L, threads, flags):
+    """A warp per node, four threads a row: the attention beside it leaves no room for more."""
+    d = spiffy.DecideDesc(B, N, L, 1024, spiffy.F32 | flags, 1024, 1023, spiffy.RULE_TOPS, 1, 0.9)
+    p = ctypes.c_void_p(1 << 20)
+    host.fake_reset(b"", 0, 0)
+    assert host.spiffy_decide_walk(ctypes.byref(d), p, p, p, p, 4, *[p] * 11, ctypes.c_size_t(1 << 40),
+                                   ctypes.c_void_p(STREAM)) == spiffy.OK
+    (tail,) = [line for line in host.fake_log().decode().splitlines() if "decide_tail" in line]
+    assert int(re.search(r"threads (\d+)", tail).group(1)) == threads
+
+
 @pytest.mark.parametrize("D,L", [(1, 1), (64, 1), (1000, 1), (300, 4), (10, 15), (1000, 17), (10, 32), (10, 33), (1024, 64)])
 def test_drafting_has_threads_for_positions_and_formulas(host, D, L):
     """A warp per position, two positions a warp beyond 32; on short blocks 512 threads for the formulas all the same."""
