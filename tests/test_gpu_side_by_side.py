@@ -91,6 +91,54 @@ def test_results_may_lie_where_the_attention_reads(N, L):
             assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("flags", [spiffy.INDEPENDENT, spiffy.INDEPENDENT | spiffy.INDEPENDENT_NEXT])
+@pytest.mark.parametrize("rule,S", [(spiffy.RULE_TOPS, 1), (spiffy.RULE_TOPS, 3), (spiffy.RULE_TOPS, 9), (spiffy.RULE_THRESHOLD, 1)])
+@pytest.mark.parametrize("B,N,L,V,dtype", [(8, 4, 16, 1000, "bf16"), (3, 8, 4, 16384, "bf16"), (2, 4, 8, 8000, "f32"),
+                                           (2, 64, 1, 300, "f32"), (1, 2, 32, 8192, "bf16"), (5, 3, 5, 12004, "f32")])
+def test_one_launch_with_odd_inputs(B, N, L, V, dtype, rule, S, flags):
+    """Behind an attention on the CUDA cores: rows that hold a NaN, an infinity or nothing but -inf, nodes with all
+    positions unmasked, malformed lists, status words that are OR-ed into or arrive with anything."""
+    cfg = W.Config("t", B, N, L, 40, 4, 4, 64, dtype, V, rule, S)
+    x = inputs_from_workload(W.make(cfg, 11))
+    x.logits[0, 0, L - 1, 1::2] = float("-inf")  # still a distribution
+    x.block_tokens[:, N // 2] = 5
+    spoiled = [0] * B
+    if B > 1:
+        x.logits[1, 0, 0, V // 2], spoiled[1] = float("nan"), spiffy.DEV_NONFINITE
+        x.block_tokens[1, 0, 0] = cfg.mask_id
+    if B > 2:
+        x.logits[2, N - 1, L - 1], spoiled[2] = float("-inf"), spiffy.DEV_NONFINITE
+        x.logits[2, 0, 0, 3] = float("inf")
+        x.block_tokens[2, N - 1, L - 1] = x.block_tokens[2, 0, 0] = cfg.mask_id
+    whole = torch.tensor([s == 0 for s in spoiled], device="cuda")
+    for lists in ("good", "entry", "offset"):
+        off, idx, bad = x.parent_off.clone(), x.parent_idx.clone(), 0
+        if lists != "good":
+            bad = spiffy.DEV_BADGRAPH
+            if lists == "entry":
+                off[0, 1:], idx[0, 0] = 1, N  # a node's one parent is a node that is not there
+                off[0, 1] = 0
+            else:
+                off[0, N - 1] = -3
+        args = (cfg.mask_id, cfg.rule, cfg.top_s, cfg.threshold)
+        dec = spiffy.spiffy_unmask_decide(x.logits, x.block_tokens, *args)
+        walk = spiffy.spiffy_accept_walk(x.block_tokens, off, idx, dec.top_tok, dec.unmask_bits)
+        assert dec.dev_status.tolist() == spoiled and walk.dev_status.tolist() == [bad] + [0] * (B - 1)
+        for kept in (True, False):
+            d, w = VerifyStep(cfg, attn_kernel=spiffy.ATTN_SIMT).decision, VerifyStep(cfg, attn_kernel=spiffy.ATTN_SIMT).walk
+            d.dev_status.fill_(64)
+            w.dev_status.fill_(32)
+            spiffy.spiffy_graph_attention(x.q, x.k_prefix, x.v_prefix, x.k_block, x.v_block, kernel=spiffy.ATTN_SIMT)
+            before = spiffy.launch_count()
+            got_d, got_w = spiffy.spiffy_decide_walk(x.logits, x.block_tokens, off, idx, *args, decision=d if kept else None,
+                                                     walk=w if kept else None, flags=flags)
+            assert spiffy.launch_count() - before == 1
+            assert got_d.dev_status.tolist() == [s | (64 if kept else 0) for s in spoiled]
+            assert got_w.dev_status.tolist() == [s | (32 if kept else 0) for s in [bad] + [0] * (B - 1)]
+            for a, b in zip(_fields(got_d)[:-1] + _fields(got_w)[:-1], _fields(dec)[:-1] + _fields(walk)[:-1]):
+                assert torch.equal(a[whole].view(torch.uint8), b[whole].view(torch.uint8))
+
+
 def _results(s):
     out = [s.attn_out, s.attn_status] + list(_fields(s.decision)) + list(_fields(s.walk))
     return [t.clone().view(torch.uint8) for t in out]

@@ -200,6 +200,22 @@ def test_a_tail_is_no_larger_than_its_graph_asks_for(host, B, N, L, threads, fla
     assert int(re.search(r"threads (\d+)", tail).group(1)) == threads
 
 
+@pytest.mark.parametrize("B,N,L,V,dtype,cap,small", [
+    (1, 1, 1, 100, spiffy.F32, 4, True), (8, 4, 16, 4096, spiffy.F32, 4, True), (9, 4, 16, 4096, spiffy.F32, 4, False),
+    (1, 8, 8, 8192, spiffy.BF16, 4, True), (1, 8, 8, 8200, spiffy.BF16, 4, False), (2, 13, 5, 1000, spiffy.BF16, 4, False),
+    (1, 2, 8, 16384, spiffy.F32, 4, True), (1, 2, 8, 16388, spiffy.F32, 4, False), (1, 4, 8, 1024, spiffy.F32, 11000, True),
+    (1, 4, 8, 1024, spiffy.F32, 12000, False)])
+@pytest.mark.parametrize("flags", [0, spiffy.INDEPENDENT, spiffy.INDEPENDENT_NEXT, spiffy.INDEPENDENT | spiffy.INDEPENDENT_NEXT])
+def test_up_to_64_slices_beside_an_attention_are_one_launch(host, B, N, L, V, dtype, cap, small, flags):
+    d = spiffy.DecideDesc(B, N, L, V, dtype | flags, V, V - 1, spiffy.RULE_TOPS, 1, 0.9)
+    p = ctypes.c_void_p(1 << 20)
+    host.fake_reset(b"", 0, 0)
+    assert host.spiffy_decide_walk(ctypes.byref(d), p, p, p, p, cap, *[p] * 11, ctypes.c_size_t(1 << 40),
+                                   ctypes.c_void_p(STREAM)) == spiffy.OK
+    log = host.fake_log().decode().splitlines()
+    assert (["decide_small" in line for line in log] == [True]) == (small and bool(flags & spiffy.INDEPENDENT))
+
+
 @pytest.mark.parametrize("D,L", [(1, 1), (64, 1), (1000, 1), (300, 4), (10, 15), (1000, 17), (10, 32), (10, 33), (1024, 64)])
 def test_drafting_has_threads_for_positions_and_formulas(host, D, L):
     """A warp per position, two positions a warp beyond 32; on short blocks 512 threads for the formulas all the same."""
