@@ -293,7 +293,8 @@ def run_part(args):
         out.update(gbs=by / sec / 1e9, frac_of_hbm=by / sec / 1e9 / peaks["hbm_gbs"], algorithmic_bytes=by,
                    masked_rows=masked_all)
         if args.part == "decide_walk_lazy":
-            # what the lazy call has to read: the still-masked rows of the nodes on the accepted path
+            # what the lazy call cannot do without: the still-masked rows of the nodes on the accepted path (it also
+            # reads slices of nodes that it guesses to come next, at most one node more per sequence and level)
             rows, hops = [], []
             for x, w in zip(sets, work):
                 walk = call(x)
@@ -305,7 +306,7 @@ def run_part(args):
             lazy_by = algorithmic_bytes(cfg, float(np.mean(rows)))[1]
             out.update(rows_on_path=float(np.mean(rows)), mean_accepted=float(np.mean(hops)),
                        lazy_algorithmic_bytes=lazy_by, lazy_gbs=lazy_by / sec / 1e9,
-                       note="gbs counts the eager call's bytes (every node); lazy_gbs the bytes this call reads")
+                       note="gbs counts the eager call's bytes (every node); lazy_gbs those of the accepted path, without wrong guesses")
     out["peaks"] = peaks["source"]
     print(json.dumps(out))
 

@@ -70,9 +70,9 @@ decide_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V,
 
 // grid = B*N nodes, 512 threads: eight threads per position merge the slices of
 // its row, then warp 0 applies the rule.
-// kAtOnce: slices of a thread on their way at a time; a further trip is 0.4 us or more.  Ten where there are more
-// than 32 slices a row (the 148 of the output projection: 0.5 to 1.3 us a call, 2 x 32 positions x 1024 x 32000
-// 31.6 -> 30.3, 8 x 32 x 4096 x 126464 193.0 -> 192.0); else four, which hold what there is.
+// kAtOnce: slices of a thread on their way at a time; a further trip is 0.4 us or more.  Ten for the output
+// projection with more than 32 slices a row (148: 0.5 to 1.3 us a call, 4 x 32 positions x 1024 x 32000 31.6 -> 30.3,
+// 8 x 32 x 4096 x 126464 193.0 -> 192.0).  Else four: one trip for the 32 slices of 131072 fp32 or 262144 bf16 entries.
 constexpr int kFinalizeThreads = 512;
 template <int kAtOnce>
 __global__ void __launch_bounds__(kFinalizeThreads)

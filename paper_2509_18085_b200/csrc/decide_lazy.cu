@@ -34,6 +34,12 @@
 // three and five): 28 us for one, 33 two, 38 three, 44 five; 1 x 16 x 32 x 152064 12.3 for none, then
 // 5 each.  Guesses more than one level ahead of the word cost more than they gave (32, 36, 39 and 42;
 // none accepted 16.4 for 12.3).
+// What guessing is worth depends on the guess: reducers look up from a wrong one after the slice at hand, or the next.
+// Without guesses / right / wrong / the one kernel from before, us, two drafts accepted: 1 x 8 x 32 x 126464 19.1 13.3
+// 20.3 25.1, 4 x 32 x 32 x 126464 35.7 28.7 41.8 38.5, 64 x 8 x 16 x 64000 74.9 69.8 85.3 75.1; none accepted, 4 x 32 x
+// 32, 14.0, 20.0 and 16.6.  One slice of a guess per reducer and then the word waited for: 31.5 for the 28.7, 38.1 for
+// 41.8, 17.3 for 20.0.  On drafted graphs of 4 x 32 x 32, one new token in five wrong, 16 of them on average: 32.6; with
+// one slice 34.5, with none 39.7, before 46.6.
 #include "common.cuh"
 #include "decide_core.cuh"
 #include "walk_core.cuh"
@@ -49,7 +55,7 @@ struct __align__(16) LazyWord {
 };
 constexpr int kEnded = 0x7fffffff;
 constexpr int kPresent = 1;     // mark of a slice that has been written
-constexpr int kWalkCtas = 6;    // of the walk kernel per SM: 80 registers
+constexpr int kWalkCtas = 6;    // of the walk kernel per SM: 80 registers, 208 bytes spilled; five of 96 spill as much, 1 to 2 % slower
 constexpr unsigned kPollsABatch = 64, kPollsToHelp = 1u << 12;
 
 struct LazyParams {
