@@ -73,9 +73,12 @@ decide_reduce_kernel(const T* __restrict__ logits, int64_t row_stride, int V,
 // kAtOnce: slices of a thread on their way at a time; a further trip is 0.4 us or more.  Ten for the output
 // projection with more than 32 slices a row (148: 0.5 to 1.3 us a call, 4 x 32 positions x 1024 x 32000 31.6 -> 30.3,
 // 8 x 32 x 4096 x 126464 193.0 -> 192.0).  Else four: one trip for the 32 slices of 131072 fp32 or 262144 bf16 entries.
+// With four, four CTAs to an SM at 32 registers: 100 nodes x 8 rows of one slice 6.6 us a call, with three (35
+// registers) 7.2; 200 x 2 5.1 and 5.6.  With ten, as many registers as it likes, 62: 1 x 4 x 8 positions x 512 x 16000
+// 11.0 us, at 40 registers 12.2.
 constexpr int kFinalizeThreads = 512;
 template <int kAtOnce>
-__global__ void __launch_bounds__(kFinalizeThreads)
+__global__ void __launch_bounds__(kFinalizeThreads, kAtOnce > 4 ? 1 : 4)
 decide_finalize_kernel(const Partial* __restrict__ partials, int splits, int N,
                        int L, const int32_t* __restrict__ block_tokens,
                        int mask_id, int rule, int top_s, float tau,
