@@ -555,9 +555,10 @@ int tail_threads(int batch, int N, int rows) {
 }
 constexpr size_t kTailSmem = 48 * 1024 - 1024;  // what the kernel declares itself comes on top
 // Beside a CUDA-core attention (`independent`) up to kSmallSlices slices a sequence take one launch of a cluster.
-// fp32, the step with one launch and with two, us: 4 x 8 rows of one slice 7.4 and 9.8, 4 x 16 over 500 keys 20.1
-// and 22.7, 2 x 32 over 4000 keys x 32 heads 125.6 and 128.5, 4 x 2 x 32 so 491 and 496, 2 x 8 x 8 over 4000 x 16
-// 125.9 and 128.7, 3 x 8 of two 9.8 and 12.8; beyond, 3 x 8 rows of five slices 9.9 and 8.2, 8 x 32 of one 19.4 and 12.3.
+// fp32, the step with one launch and with two, us: 4 x 8 rows of one slice 6.7 and 8.4, 4 x 16 over 500 keys 20.0
+// and 21.5, 2 x 32 over 4000 keys x 32 heads 125.2 and 127.3, 4 x 2 x 32 so 492 and 495, 2 x 8 x 8 over 4000 x 16
+// 76.3 and 78.5, 3 x 8 of two 7.1 and 8.0; beyond, 3 x 8 rows of five slices 10.2 and 8.5, 8 x 32 of one 19.4 and 12.3.
+// (12 sequences of 8 x 8 over 300 keys 55.5 and 57.4: the line for the batch could lie higher.)
 // A decision in front of an attention or by itself is no sooner done in one launch (bf16, 4 x 8 rows of one
 // slice 7.2 and 7.2 us with the attention, 4 x 16 9.3 and 7.3).
 constexpr int kSmallSlices = 64, kSmallBatch = 8;
