@@ -18,7 +18,8 @@ constexpr int kNoLink = 0x7fffffff;
 constexpr int kTableNodes = 64;  // graphs up to here have their children in a table: what lists a node as a parent, a bit each
 
 // A state, positions `lane` and `lane` + 32 (zeros beyond L): its still-masked positions, and a number that
-// equal states share.
+// equal states share (multipliers: the golden ratio's, and the two of MurmurHash3's 32-bit finaliser, which is in the
+// public domain; states of equal numbers are compared token by token, so that nothing rests on them).
 __device__ __forceinline__ uint64_t masked_of(const int32_t (&state)[2], int L, int mask_id, int lane) {
   uint64_t masked = 0;
 #pragma unroll
